@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
     tmem_slot[1] = 0;
     tmem_slot[2] = (base & 1023u) != 0 ? 1u : 0u;
     if (tmem_slot[2]) raise(p.status, XRL_ERR_UNSUPPORTED);
-    xform::init_barriers<H>(base);
+    xform::init_barriers<XC>(base);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
   const uint32_t tmem_base = *tmem_slot;
 
   uint32_t prod_it = 0, mma_it = 0, mma_lt = 0, epi_lt = 0;     // ring / accumulator positions, kept across layers
-  if (threadIdx.x == 0 && !aborted()) xform::load_w<H>(base, &p.map_w[0]);
+  if (threadIdx.x == 0 && !aborted()) xform::load_w<XC>(base, &p.map_w[0]);
 
   const int my_tiles = (num_tiles - int(blockIdx.x) + int(gridDim.x) - 1) / int(gridDim.x);
   const int blk_bits = 7 - p.br_shift;                           // blocks per 128-row tile = 2^blk_bits
@@ -141,20 +141,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
     // ---- transform phase: Z[zb] rows (and their half-score pairs) of this CTA's tiles --------------------
     if (!aborted()) {
       if (warp == 0) {
-        if (lane == 0 && !xform::produce_tiles<H>(base, &p.map_h, blockIdx.x, gridDim.x, num_tiles, prod_it)) {
+        if (lane == 0 && !xform::produce_tiles<XC>(base, &p.map_h, blockIdx.x, gridDim.x, num_tiles, prod_it)) {
           raise(p.status, XRL_ERR_TIMEOUT);
-          xform::drain_producer<H>(base, prod_it, uint32_t(l & 1));
+          xform::drain_producer<XC>(base, prod_it, uint32_t(l & 1));
           *abort_role = 1;
         }
       } else if (warp == 1) {
-        if (lane == 0 && !xform::mma_tiles<H>(base, tmem_base, blockIdx.x, gridDim.x, num_tiles, mma_it, mma_lt,
+        if (lane == 0 && !xform::mma_tiles<XC, H>(base, tmem_base, blockIdx.x, gridDim.x, num_tiles, mma_it, mma_lt,
                                               uint32_t(l & 1))) {
           raise(p.status, XRL_ERR_TIMEOUT);
           *abort_role = 1;
         }
       } else if (warp < 6) {
         float2* pairs = reinterpret_cast<float2*>(reinterpret_cast<char*>(p.Z[zb]) + size_t(H) * 2);
-        xform::epilogue_tiles<H>(smem, base, tmem_base, &p.map_zs[zb], pairs, p.z_row_bytes / 8, p.rows, K,
+        xform::epilogue_tiles<XC, H, false>(smem, base, tmem_base, &p.map_zs[zb], pairs, p.z_row_bytes / 8, p.rows, H / K,
                                  blockIdx.x, gridDim.x, num_tiles, epi_lt, threadIdx.x == 64, p.status);
       }
     }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
     __syncthreads();
     // every accumulator of the transform phase has been read, so all its MMAs have completed: W may be replaced.
     // (Issued only now: a thread's proxy fence waits for the copies it has in flight.)
-    if (threadIdx.x == 0 && l + 1 < p.layers && !aborted()) xform::load_w<H>(base, &p.map_w[l + 1]);
+    if (threadIdx.x == 0 && l + 1 < p.layers && !aborted()) xform::load_w<XC>(base, &p.map_w[l + 1]);
 
     // ---- attention phase: rows of the same tiles; the rings take the place of the A stages and staging ---
     if (!aborted() && warp < kAttWarps) {

@@ -1,7 +1,7 @@
 // Dense node transform of a graph-attention layer, Z = h W (paper Eq. 7, the "W h_j" term), on
 // the CUDA cores with fp32 accumulation.  This is the path for fp32 storage (whose tolerance a
-// single-pass reduced-precision tensor-core product cannot guarantee) and for hidden sizes the
-// tensor-core kernel is not built for.  The attention half-scores are taken from the accumulators in the
+// single-pass reduced-precision tensor-core product cannot guarantee) and for the bf16 models the
+// tensor-core kernel is kept off for (XRL_FORCE_SIMT_TRANSFORM).  The attention half-scores are taken from the accumulators in the
 // kernel's last step when one tile spans all H columns, the storage is fp32 and a head is 4, 8, ... 128 columns
 // wide (SCORES); otherwise from Z by k_scores.
 #include "xrl_internal.cuh"

@@ -80,7 +80,7 @@ struct xrl_ctx {
   Dims dims;
   int device = 0;
   bool weights_set = false;
-  bool use_umma = false;    // bf16 transform on the tensor cores (hidden 128 or 256)
+  bool use_umma = false;    // bf16 transform on the tensor cores (every hidden width the library takes)
   bool use_umma_embed = false;   // bf16 node update on the tensor cores
   DeviceBuf w0ext;          // W0 extended and transposed for the tensor-core node update
   size_t weight_floats = 0;

@@ -16,19 +16,25 @@ using namespace umma;
 constexpr int BM = 128;                 // rows per tile (UMMA M)
 constexpr int STAGE_BYTES = BM * 128;   // one A stage / one output staging tile: 128 rows x 128 B
 
-template <int H> struct Cfg {
-  static constexpr int KC = H / KCH;                    // K chunks (= output column chunks)
-  static constexpr int W_CHUNK_BYTES = H * 128;         // N rows x 128 B
+// NS: output columns a CTA computes (its slice of W, resident in shared memory); KP: input width padded to whole
+// 64-element chunks (the TMA unit fills what lies beyond the matrix with zeros).  NS = KP = H for hidden 128 and 256.
+template <int NS, int KP = NS> struct Cfg {
+  static_assert(NS % 32 == 0 && NS >= 32 && NS <= 256 && KP % KCH == 0, "tile shapes of tcgen05.mma and of the swizzle");
+  static constexpr int KC = KP / KCH;                   // K chunks
+  static constexpr int NC = (NS + KCH - 1) / KCH;       // output column chunks
+  static constexpr int W_CHUNK_BYTES = NS * 128;        // N rows x 128 B
   static constexpr int W_BYTES = KC * W_CHUNK_BYTES;
-  static constexpr int STAGES = (H == 256) ? 4 : 8;
-  static constexpr int TMEM_COLS = 2 * H;               // two fp32 accumulators of N = H columns
+  static constexpr int STAGES = W_BYTES > 64 * 1024 ? 4 : 8;
+  static constexpr int ACC_COLS = NS <= 32 ? 32 : NS <= 64 ? 64 : NS <= 128 ? 128 : 256;
+  static constexpr int TMEM_COLS = 2 * ACC_COLS;        // two fp32 accumulators of N columns, a power of two apart
   static constexpr int OFF_A = W_BYTES;
   static constexpr int OFF_OUT = OFF_A + STAGES * STAGE_BYTES;
   static constexpr int OFF_AVEC = OFF_OUT + 2 * STAGE_BYTES;
-  static constexpr int OFF_BAR = OFF_AVEC + 2 * H * 4;
+  static constexpr int OFF_BAR = OFF_AVEC + 2 * NS * 4;
   static constexpr int NUM_BARS = 1 + 2 * STAGES + 4;
   static constexpr int OFF_TMEM = OFF_BAR + NUM_BARS * 8;   // [0] TMEM base address, [1] abort flag
   static constexpr int SMEM_BYTES = OFF_TMEM + 16;
+  static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one SM");
 
   __device__ static uint32_t bar_w(uint32_t base) { return base + OFF_BAR; }
   __device__ static uint32_t bar_a_full(uint32_t base, int s) { return base + OFF_BAR + 8u * (1 + s); }
@@ -40,8 +46,7 @@ template <int H> struct Cfg {
 };
 
 // One thread: barriers of the layout above (128 epilogue threads free an accumulator).
-template <int H> __device__ __forceinline__ void init_barriers(uint32_t base) {
-  using C = Cfg<H>;
+template <typename C> __device__ __forceinline__ void init_barriers(uint32_t base) {
   mbar_init(C::bar_w(base), 1);
   for (int s = 0; s < C::STAGES; ++s) { mbar_init(C::bar_a_full(base, s), 1); mbar_init(C::bar_a_empty(base, s), 1); }
   for (int b = 0; b < 2; ++b) { mbar_init(C::bar_acc_full(base, b), 1); mbar_init(C::bar_acc_empty(base, b), 128); }
@@ -49,18 +54,16 @@ template <int H> __device__ __forceinline__ void init_barriers(uint32_t base) {
   fence_async_smem();
 }
 
-// One thread: W^T (K-major, H x H bf16) into the start of shared memory; completion on bar_w.
-template <int H> __device__ __forceinline__ void load_w(uint32_t base, const CUtensorMap* map_w) {
-  using C = Cfg<H>;
+// One thread: rows col0 .. col0 + NS - 1 of W^T (K-major bf16) into the start of shared memory; completion on bar_w.
+template <typename C> __device__ __forceinline__ void load_w(uint32_t base, const CUtensorMap* map_w, int col0 = 0) {
   mbar_expect_tx(C::bar_w(base), C::W_BYTES);
-  for (int kc = 0; kc < C::KC; ++kc) tma_load_2d(base + kc * C::W_CHUNK_BYTES, map_w, kc * KCH, 0, C::bar_w(base));
+  for (int kc = 0; kc < C::KC; ++kc) tma_load_2d(base + kc * C::W_CHUNK_BYTES, map_w, kc * KCH, col0, C::bar_w(base));
 }
 
 // One thread: the A tiles first, first + step, ... < num_tiles through the stage ring.  False on a timeout.
-template <int H>
+template <typename C>
 __device__ __forceinline__ bool produce_tiles(uint32_t base, const CUtensorMap* map_h, int first, int step,
                                               int num_tiles, uint32_t& it) {
-  using C = Cfg<H>;
   for (int tile = first; tile < num_tiles; tile += step) {
     for (int kc = 0; kc < C::KC; ++kc, ++it) {
       const int s = it % C::STAGES;
@@ -74,20 +77,18 @@ __device__ __forceinline__ bool produce_tiles(uint32_t base, const CUtensorMap* 
 }
 
 // After a producer timeout: let the loads already issued land before the CTA's shared memory goes away.
-template <int H> __device__ __forceinline__ void drain_producer(uint32_t base, uint32_t it, uint32_t w_parity) {
-  using C = Cfg<H>;
+template <typename C> __device__ __forceinline__ void drain_producer(uint32_t base, uint32_t it, uint32_t w_parity) {
   const uint32_t first = it > uint32_t(C::STAGES) ? it - C::STAGES : 0;
   for (uint32_t j = first; j < it; ++j) mbar_wait(C::bar_a_full(base, j % C::STAGES), (j / C::STAGES) & 1);
   mbar_wait(C::bar_w(base), w_parity);
 }
 
-// One thread: tcgen05.mma (M = 128, N = H, K = 16) over the same tiles, alternating between the two
+// One thread: tcgen05.mma (M = 128, N = NS, K = 16) over the same tiles, alternating between the two
 // accumulators; waits for W (phase w_parity of bar_w) first.  False on a timeout.
-template <int H>
+template <typename C, int NS>
 __device__ __forceinline__ bool mma_tiles(uint32_t base, uint32_t tmem_base, int first, int step, int num_tiles,
                                           uint32_t& it, uint32_t& lt, uint32_t w_parity) {
-  using C = Cfg<H>;
-  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(H >> 3) << 17) |
+  constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NS >> 3) << 17) |
                              (uint32_t(BM >> 4) << 24);   // fp32 accum, bf16 x bf16, K-major both
   if (!mbar_wait(C::bar_w(base), w_parity)) return false;
   tc_fence_after();
@@ -96,7 +97,7 @@ __device__ __forceinline__ bool mma_tiles(uint32_t base, uint32_t tmem_base, int
     const uint32_t use = lt >> 1;
     if (use > 0 && !mbar_wait(C::bar_acc_empty(base, buf), (use - 1) & 1)) return false;
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base + uint32_t(buf * H);
+    const uint32_t tmem_d = tmem_base + uint32_t(buf * C::ACC_COLS);
     for (int kc = 0; kc < C::KC; ++kc, ++it) {
       const int s = it % C::STAGES;
       if (!mbar_wait(C::bar_a_full(base, s), (it / C::STAGES) & 1)) return false;
@@ -117,16 +118,18 @@ __device__ __forceinline__ bool mma_tiles(uint32_t base, uint32_t tmem_base, int
 // per tile the half-scores from the fp32 accumulators, Z rounded to bf16 into a swizzled staging tile,
 // TMA store.  `leader` is one of the 128 threads; it owns the stores and waits for them at the end.
 // A timeout sets the abort word behind the tensor-memory slot and raises XRL_ERR_TIMEOUT.
-template <int H>
+// The CTA's NS columns are the matrix's columns col0 ... and their heads (of `d` columns, whole heads within the NS)
+// go to scores[row * score_stride + 0 ...]; columns and heads from `cols_left` on do not exist.  scores = nullptr: none are
+// taken.  ROUNDED: the half-scores are those of Z as stored (rounded), not of the accumulators.
+template <typename C, int NS, bool ROUNDED>
 __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uint32_t tmem_base,
                                                const CUtensorMap* map_z, float2* __restrict__ scores,
-                                               int score_stride, int rows, int K, int first, int step,
-                                               int num_tiles, uint32_t& lt, bool leader, int32_t* status) {
-  using C = Cfg<H>;
+                                               int score_stride, int rows, int d, int first, int step,
+                                               int num_tiles, uint32_t& lt, bool leader, int32_t* status,
+                                               int col0 = 0, int cols_left = NS) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;
   const int row_in_tile = q * 32 + lane;
-  const int d = H / K;                         // head width, a multiple of 8
   const float* avec = reinterpret_cast<const float*>(smem + C::OFF_AVEC);
   volatile uint32_t* abort_flag = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM) + 1;
   for (int tile = first; tile < num_tiles; tile += step, ++lt) {
@@ -139,21 +142,33 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
     epi_barrier();
     if (*abort_flag) break;
     tc_fence_after();
-    const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(buf * H);
+    const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(buf * C::ACC_COLS);
     const int64_t grow = int64_t(tile) * BM + row_in_tile;
     const bool live = grow < rows;
     float ss = 0.f, sd = 0.f;
     int head = 0, left = d;                    // columns left in the current head
-    for (int c = 0; c < C::KC; ++c) {          // 64 output columns per chunk
+    for (int c = 0; c < C::NC; ++c) {          // 64 output columns per chunk
       uint32_t v[2][32];
+      const bool half = NS % 64 != 0 && c == C::NC - 1;      // the last chunk holds 32 columns only
       tc_ld32(taddr + c * 64, v[0]);
-      tc_ld32(taddr + c * 64 + 32, v[1]);
+      if (!half) {
+        tc_ld32(taddr + c * 64 + 32, v[1]);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 32; ++t) v[1][t] = 0u;
+      }
       tc_wait_ld();
+      if (ROUNDED) {                           // Z as it will be stored
+#pragma unroll
+        for (int t = 0; t < 64; ++t)
+          v[t >> 5][t & 31] = __float_as_uint(__bfloat162float(__float2bfloat16_rn(__uint_as_float(v[t >> 5][t & 31]))));
+      }
       // half-scores from the fp32 accumulators, eight columns at a time
 #pragma unroll
       for (int g = 0; g < 8; ++g) {
+        if (half && g >= 4) break;
         const float4* as = reinterpret_cast<const float4*>(avec + c * 64 + g * 8);
-        const float4* ad = reinterpret_cast<const float4*>(avec + H + c * 64 + g * 8);
+        const float4* ad = reinterpret_cast<const float4*>(avec + NS + c * 64 + g * 8);
         const float4 s0 = as[0], s1 = as[1], d0 = ad[0], d1 = ad[1];
         const uint32_t* z = &v[g >> 2][(g & 3) * 8];
         ss = fmaf(__uint_as_float(z[0]), s0.x, ss); sd = fmaf(__uint_as_float(z[0]), d0.x, sd);
@@ -166,7 +181,7 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
         ss = fmaf(__uint_as_float(z[7]), s1.w, ss); sd = fmaf(__uint_as_float(z[7]), d1.w, sd);
         left -= 8;
         if (left == 0) {
-          if (live) scores[grow * score_stride + head] = make_float2(ss, sd);
+          if (live && scores != nullptr && c * 64 + g * 8 < cols_left) scores[grow * score_stride + head] = make_float2(ss, sd);
           ss = 0.f; sd = 0.f; ++head; left = d;
         }
       }
@@ -186,8 +201,8 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
       }
       fence_async_smem();
       epi_barrier();
-      if (leader) {
-        tma_store_2d(map_z, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, c * 64, tile * BM);
+      if (leader && c * 64 < cols_left) {
+        tma_store_2d(map_z, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, col0 + c * 64, tile * BM);
         tma_commit();
       }
     }

@@ -1,0 +1,34 @@
+"""The tensor-core kernels of Eq. 6 and of the node transform at every hidden width they are built for: widths that end
+inside a 64-column chunk, widths above 256 (column slices), heads that cross a slice's end, row counts around a tile."""
+import pytest
+
+from workloads import configs, dags
+import gpu_util
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,K", [(32, 2), (64, 1), (96, 3), (160, 4), (192, 6), (224, 7), (288, 3), (320, 8), (352, 1),
+                                 (384, 3), (416, 13), (448, 7), (480, 2), (512, 8), (512, 2)])
+@pytest.mark.parametrize("nodes", [1, 127, 129])
+def test_bf16_widths(xo, H, K, nodes):
+    import paper_2304_14698_b200 as xrl
+    rng = dags.make_rng(H + nodes)
+    m = dict(T=21, S=8, H=H, K=K, L=2, Hm=24, Dg=1, dtype="bf16", A_max=2)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, True) for n in (nodes, 1)]
+    batch = dags.flatten(graphs, [0, 2], 2)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 3)
+    st, packed = xo.pack(batch)
+    assert st == 0
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        for layer in range(m["L"] + 1):
+            got = xrl.xrl_debug_node_features(ag.ctx, ag.batch, layer, H)
+            want = xo.encode(m, blob, batch, packed, dump_layer=layer, want_nodes=True)
+            gpu_util.assert_close(got, want["nodes"], "bf16", f"nodes after stage {layer}")
+        assert ag.device_status() == 0
+    finally:
+        ag.close()
