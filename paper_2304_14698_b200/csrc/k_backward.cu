@@ -382,11 +382,10 @@ k_scores_bwd_rows(ZView<T> zv, const float* __restrict__ ds_src, const float* __
   }
 }
 
-// ---- dW += A^T B over a range of rows: A [rows x Ka] (storage type), B [rows x Nb] fp32 -------------------
+// ---- dW += A^T B over a range of rows: A [rows x Ka], B [rows x Nb], fp32, any shapes (the heads' weights) ----------
 // 64 x 64 output tile per CTA, the rows cut into chunks along grid.z, partial products added with atomics.
-template <typename TA>
 __global__ void __launch_bounds__(256)
-k_atb(const TA* __restrict__ A, int lda, const float* __restrict__ Bm, int ldb, float* __restrict__ Cout, int ldc,
+k_atb(const float* __restrict__ A, int lda, const float* __restrict__ Bm, int ldb, float* __restrict__ Cout, int ldc,
       int rows, int Ka, int Nb, int rows_per_chunk, float* __restrict__ colsum_out) {
   __shared__ float As[16][64 + 1];
   __shared__ float Bs[16][64 + 1];
@@ -401,7 +400,7 @@ k_atb(const TA* __restrict__ A, int lda, const float* __restrict__ Bm, int ldb, 
     for (int t = tid; t < 16 * 64; t += 256) {
       const int rr = t >> 6, cc = t & 63;
       const int r = r0 + rr;
-      As[rr][cc] = (r < r_end && a0 + cc < Ka) ? to_float(A[size_t(r) * lda + a0 + cc]) : 0.f;
+      As[rr][cc] = (r < r_end && a0 + cc < Ka) ? A[size_t(r) * lda + a0 + cc] : 0.f;
       Bs[rr][cc] = (r < r_end && b0 + cc < Nb) ? Bm[size_t(r) * ldb + b0 + cc] : 0.f;
     }
     __syncthreads();
@@ -432,6 +431,85 @@ k_atb(const TA* __restrict__ A, int lda, const float* __restrict__ Bm, int ldb, 
     for (int v = 0; v < 4; ++v) {
       const int ka = a0 + ty * 4 + u, nb = b0 + tx * 4 + v;
       if (ka < Ka && nb < Nb && acc[u][v] != 0.f) atomicAdd(&Cout[size_t(ka) * ldc + nb], acc[u][v]);
+    }
+}
+
+// ---- the same product for the layers' weights: dW [H x H] += A^T B, A = h_in [rows x H], B = dz [rows x H] fp32 --------
+// TILE x TILE outputs per CTA, 8 x 8 per thread (two 4-wide groups in each direction: conflict-free 16-byte reads of
+// shared memory), 16 rows per step with the next step's pieces already in registers.  The product reduces over the
+// rows, so all parallelism beyond the H x H / TILE^2 tiles comes from cutting the rows into chunks (grid.z) whose
+// results meet in vector atomics; 64-row tiles of 4 x 4 outputs per thread with chunks of 2,048 rows left half the SMs
+// without work at 36 k rows (0.333 ms per layer at H = 128; now 0.031, with dh = dz W^T 0.065 -> 0.029).  Bound by FFMA issue.  fp32 FMA chains as before, shorter ones per chunk.
+constexpr int kAtbRows = 16;
+template <typename TA, int TILE>
+__global__ void __launch_bounds__((TILE / 8) * (TILE / 8))
+k_atb_tile(const TA* __restrict__ A, const float* __restrict__ Bm, float* __restrict__ Cout, int rows, int H,
+           int rows_per_chunk, bool vec) {
+  constexpr int NTX = TILE / 8, NT = NTX * NTX;
+  constexpr int PIECES = kAtbRows * TILE / 4 / NT;     // 4-wide pieces per thread, operand and step
+  __shared__ __align__(16) float As[kAtbRows][TILE];
+  __shared__ __align__(16) float Bs[kAtbRows][TILE];
+  const int tid = threadIdx.x, ty = tid / NTX, tx = tid % NTX;
+  const int a0 = blockIdx.x * TILE, b0 = blockIdx.y * TILE;
+  const int r_begin = blockIdx.z * rows_per_chunk, r_end = min(rows, r_begin + rows_per_chunk);
+  float acc[8][8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+#pragma unroll
+    for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+  Chunk<TA, 4> ra[PIECES];
+  float4 rb[PIECES];
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int it = 0; it < PIECES; ++it) {
+      const int idx = tid + it * NT, rr = r0 + idx / (TILE / 4), c = (idx % (TILE / 4)) * 4;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) ra[it].v[t] = TA(0.f);
+      rb[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (rr < r_end) {
+        if (a0 + c < H) ra[it] = *reinterpret_cast<const Chunk<TA, 4>*>(A + size_t(rr) * H + a0 + c);
+        if (b0 + c < H) rb[it] = *reinterpret_cast<const float4*>(Bm + size_t(rr) * H + b0 + c);
+      }
+    }
+  };
+  if (r_begin < r_end) fetch(r_begin);
+  for (int r0 = r_begin; r0 < r_end; r0 += kAtbRows) {
+#pragma unroll
+    for (int it = 0; it < PIECES; ++it) {
+      const int idx = tid + it * NT, rr = idx / (TILE / 4), c = (idx % (TILE / 4)) * 4;
+      *reinterpret_cast<float4*>(&As[rr][c]) =
+          make_float4(to_float(ra[it].v[0]), to_float(ra[it].v[1]), to_float(ra[it].v[2]), to_float(ra[it].v[3]));
+      *reinterpret_cast<float4*>(&Bs[rr][c]) = rb[it];
+    }
+    __syncthreads();
+    if (r0 + kAtbRows < r_end) fetch(r0 + kAtbRows);
+#pragma unroll
+    for (int rr = 0; rr < kAtbRows; ++rr) {
+      float a[8], b[8];
+      *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(&As[rr][ty * 4]);
+      *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(&As[rr][TILE / 2 + ty * 4]);
+      *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(&Bs[rr][tx * 4]);
+      *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(&Bs[rr][TILE / 2 + tx * 4]);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const int m = a0 + (u < 4 ? ty * 4 + u : TILE / 2 + ty * 4 + u - 4), n = b0 + g * (TILE / 2) + tx * 4;
+      if (m >= H || n >= H) continue;
+      float* o = Cout + size_t(m) * H + n;
+      if (vec) {
+        atomicAdd(reinterpret_cast<float4*>(o), make_float4(acc[u][4 * g], acc[u][4 * g + 1], acc[u][4 * g + 2], acc[u][4 * g + 3]));
+      } else {                                         // (the caller's gradient buffer may sit on any 4-byte boundary)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) atomicAdd(o + t, acc[u][4 * g + t]);
+      }
     }
 }
 
@@ -1068,7 +1146,7 @@ void atb_f32(const float* A, int lda, const float* Bm, int ldb, float* Cout, int
   if (rows <= 0 || Ka <= 0 || Nb <= 0) return;
   const int chunk = chunk_rows(rows, 1024);
   dim3 g(unsigned((Ka + 63) / 64), unsigned((Nb + 63) / 64), unsigned((rows + chunk - 1) / chunk));
-  k_atb<float><<<g, 256, 0, st>>>(A, lda, Bm, ldb, Cout, ldc, rows, Ka, Nb, chunk, colsum_out);
+  k_atb<<<g, 256, 0, st>>>(A, lda, Bm, ldb, Cout, ldc, rows, Ka, Nb, chunk, colsum_out);
 }
 // weights' gradients of one head from its per-row buffers; returns the launches
 int mlp_weight_grads(const float* X, int in, int rows, int hid, int hid2, const float* Y1, const float* Y2,
@@ -1247,8 +1325,15 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   const size_t zrow = z_row_bytes(d);
   const int grid_rows = int(std::min<int64_t>((int64_t(N) + 7) / 8, int64_t(kNumSMs) * 8));
   const int grid_cols = int(std::min<int64_t>((int64_t(N) + 255) / 256, int64_t(kNumSMs) * 2));
-  const int chunk = chunk_rows(N, 2048);
-  dim3 g_atb(unsigned((H + 63) / 64), unsigned((H + 63) / 64), unsigned((N + chunk - 1) / chunk));
+  // dW on CUDA cores: 128-wide tiles where they fit H (one CTA of 256 threads per SM: 160 registers; held to 128
+  // registers and two CTAs the launch takes 35.6 us instead of 33.6 at 36 k rows), else 64-wide ones (six CTAs of 64
+  // threads per SM); the rows in as many chunks as fill the SMs, at least 64 rows each
+  const bool wide_atb = H % 128 == 0;
+  const int atb_side = wide_atb ? H / 128 : (H + 63) / 64;
+  const int atb_chunks = std::max(1, (wide_atb ? 1 : 6) * kNumSMs / (atb_side * atb_side));
+  const int chunk = std::max(64, int(((int64_t(N) + atb_chunks - 1) / atb_chunks + 15) & ~int64_t(15)));
+  dim3 g_atb(unsigned(atb_side), unsigned(atb_side), unsigned((N + chunk - 1) / chunk));
+  const bool vec = (reinterpret_cast<uintptr_t>(gW) & 15) == 0;
   dim3 g_gwt(unsigned((N + 63) / 64), unsigned((H + 63) / 64));
   // tensor-core products: about two waves of CTAs over the rows, chunks of a multiple of 32 rows, at least 512
   const int tiles = (H / 128) * (H / 128);
@@ -1295,8 +1380,15 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
       k_atb_mma<<<g_atb_mma, 256, 0, st>>>(static_cast<const bf16*>(h_in), dzb, gW, N, H, chunk_mma);          \
       k_gwt_mma<<<g_gwt_mma, 256, 0, st>>>(dzb, static_cast<const bf16*>(lw.W), dh_in, N, H, gwt_tpc);                  \
     } else {                                                                                                   \
-      k_atb<TY_><<<g_atb, 256, 0, st>>>(static_cast<const TY_*>(h_in), H, dz, H, gW, H, N, H, H, chunk, nullptr);       \
-      k_gwt<TY_><<<g_gwt, 256, 0, st>>>(dz, static_cast<const TY_*>(lw.W), dh_in, N, H, H);                    \
+      if (wide_atb)                                                                                            \
+        k_atb_tile<TY_, 128><<<g_atb, 256, 0, st>>>(static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);  \
+      else                                                                                                     \
+        k_atb_tile<TY_, 64><<<g_atb, 64, 0, st>>>(static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);    \
+      /* from 8,192 rows on the 128 x 128 tiles of the forward product have CTAs for every SM */               \
+      if (N >= 8192 && H > 64)                                                                                 \
+        launch_rows_times_matrix(d, dz, lw.Wt, dh_in, N, st);                                                  \
+      else                                                                                                     \
+        k_gwt<TY_><<<g_gwt, 256, 0, st>>>(dz, static_cast<const TY_*>(lw.W), dh_in, N, H, H);                  \
     }                                                                                                          \
   } while (0)
   if (d.dtype == XRL_BF16) BWD_BODY(bf16); else BWD_BODY(float);

@@ -113,9 +113,11 @@ __device__ __forceinline__ void load4<bf16>(const bf16* p, bool ok, float (&v)[4
   v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xFFFF0000u);
 }
 
-template <typename T, bool SCORES>
+// (TA, TW, TZ: element types of the rows, of the matrix and of the result: the reverse pass multiplies fp32 gradients
+// with matrices in the storage type)
+template <typename TA, typename TW, typename TZ, bool SCORES>
 __global__ void __launch_bounds__(256)
-k_xform_simt128(const T* __restrict__ h, const T* __restrict__ W, T* __restrict__ Z, int H, int rows,
+k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restrict__ Z, int H, int rows,
                 const float* __restrict__ a_src, const float* __restrict__ a_dst, float2* __restrict__ scores, int K) {
   __shared__ __align__(16) float As[TK][TM];
   __shared__ __align__(16) float Bs[TK][TN];
@@ -132,20 +134,20 @@ k_xform_simt128(const T* __restrict__ h, const T* __restrict__ W, T* __restrict_
   const int a_row = tid >> 1, a_k = (tid & 1) * 4;      // 128 rows x 8 k: one 4-vector per thread
   const int b_k = tid >> 5, b_c = (tid & 31) * 4;       // 8 k x 128 cols
   const bool a_ok = row0 + a_row < rows;
-  const T* a_ptr = h + size_t(a_ok ? row0 + a_row : 0) * H + a_k;
+  const TA* a_ptr = h + size_t(a_ok ? row0 + a_row : 0) * H + a_k;
   const bool b_ok = col0 + b_c < H;                     // H is a multiple of 4
-  const T* b_ptr = W + size_t(b_k) * H + (b_ok ? col0 + b_c : 0);
+  const TW* b_ptr = W + size_t(b_k) * H + (b_ok ? col0 + b_c : 0);
   float ra[4], rb[4];
-  load4<T>(a_ptr, a_ok, ra);
-  load4<T>(b_ptr, b_ok, rb);
+  load4<TA>(a_ptr, a_ok, ra);
+  load4<TW>(b_ptr, b_ok, rb);
   for (int k0 = 0; k0 < H; k0 += TK) {
 #pragma unroll
     for (int t = 0; t < 4; ++t) As[a_k + t][a_row] = ra[t];
     *reinterpret_cast<float4*>(&Bs[b_k][b_c]) = make_float4(rb[0], rb[1], rb[2], rb[3]);
     __syncthreads();
     if (k0 + TK < H) {                                    // next slice in flight during the arithmetic
-      load4<T>(a_ptr + k0 + TK, a_ok, ra);
-      load4<T>(b_ptr + size_t(k0 + TK) * H, b_ok, rb);
+      load4<TA>(a_ptr + k0 + TK, a_ok, ra);
+      load4<TW>(b_ptr + size_t(k0 + TK) * H, b_ok, rb);
     }
 #pragma unroll
     for (int k = 0; k < TK; ++k) {
@@ -193,7 +195,7 @@ k_xform_simt128(const T* __restrict__ h, const T* __restrict__ W, T* __restrict_
       const int c = col0 + jg * 64 + tx * 4;
       if (c >= H) continue;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) Z[size_t(r) * H + c + j] = T(acc[i][jg * 4 + j]);
+      for (int j = 0; j < 4; ++j) Z[size_t(r) * H + c + j] = TZ(acc[i][jg * 4 + j]);
     }
   }
 }
@@ -380,18 +382,18 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
   if (rows >= 8192) {
     dim3 g128(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
     if (d.dtype == XRL_BF16) {
-      k_xform_simt128<bf16, false><<<g128, 256, 0, st>>>(static_cast<const bf16*>(h) + off,
+      k_xform_simt128<bf16, bf16, bf16, false><<<g128, 256, 0, st>>>(static_cast<const bf16*>(h) + off,
                                                          static_cast<const bf16*>(lw.W),
                                                          static_cast<bf16*>(Z) + off, d.H, int(rows), nullptr, nullptr,
                                                          nullptr, d.K);
     } else if (fuse_scores(d, lw, TN, scores)) {
-      k_xform_simt128<float, true><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
+      k_xform_simt128<float, float, float, true><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
                                                          static_cast<const float*>(lw.W),
                                                          static_cast<float*>(Z) + off, d.H, int(rows), lw.a_src, lw.a_dst,
                                                          sc, d.K);
       return 1;
     } else {
-      k_xform_simt128<float, false><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
+      k_xform_simt128<float, float, float, false><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
                                                           static_cast<const float*>(lw.W),
                                                           static_cast<float*>(Z) + off, d.H, int(rows), nullptr, nullptr,
                                                           nullptr, d.K);
@@ -417,6 +419,19 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
                                                     nullptr, d.K);
   }
   return 1 + launch_scores(d, Z, lw, scores, win, st);
+}
+
+// out [rows x H] fp32 = G [rows x H] fp32 times Wt [H x H] (storage type, row-major): the reverse pass's dh = dz W^T
+// with W^T as stored by xrl_set_weights; fp32 FMA chains in the order of the columns.
+int launch_rows_times_matrix(const Dims& d, const float* G, const void* Wt, float* out, int rows, cudaStream_t st) {
+  dim3 g(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
+  if (d.dtype == XRL_BF16)
+    k_xform_simt128<float, bf16, float, false><<<g, 256, 0, st>>>(G, static_cast<const bf16*>(Wt), out, d.H, rows, nullptr,
+                                                                  nullptr, nullptr, d.K);
+  else
+    k_xform_simt128<float, float, float, false><<<g, 256, 0, st>>>(G, static_cast<const float*>(Wt), out, d.H, rows, nullptr,
+                                                                   nullptr, nullptr, d.K);
+  return 1;
 }
 
 }  // namespace xrl

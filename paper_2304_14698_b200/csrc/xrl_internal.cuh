@@ -61,7 +61,7 @@ __device__ __forceinline__ float to_float(bf16 x) { return __bfloat162float(x); 
 // ---- device-side weights ------------------------------------------------------------------
 struct LayerWeights {
   const void* W;        // storage type, [H x H] row-major [in x out]
-  const void* Wt;       // bf16 only: transpose [out x in] (K-major B operand of the tensor-core path)
+  const void* Wt;       // transpose [out x in] (K-major B operand of the tensor-core path; the reverse pass)
   const float* a_src;   // [H]
   const float* a_dst;   // [H]
   const float* b;       // [H]
@@ -146,6 +146,7 @@ int launch_embed(const Dims& d, const int32_t* rowptr, const int32_t* col, const
 // scores: [N][K] pairs {s_src, s_dst} (float2), both already multiplied by log2(e)
 int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void* Z, float* scores,
                       Window win, cudaStream_t st);
+int launch_rows_times_matrix(const Dims& d, const float* G, const void* Wt, float* out, int rows, cudaStream_t st);
 bool embed_umma_supported(const Dims& d);
 int embed_umma_kpad(const Dims& d);
 void build_w0ext(const Dims& d, const void* W0_store, const float* b0, void* out, cudaStream_t st);

@@ -1,0 +1,49 @@
+"""The dense products of the training step's reverse pass at the sizes where their tiles end: widths that are not a
+multiple of the tile, row counts around a chunk and past the line from which whole 128-row tiles are used, and a
+gradient buffer that is not 16-byte aligned."""
+import numpy as np
+import pytest
+
+from workloads import dags
+import gpu_util
+from test_gpu_ppo import BF16_ENTRYWISE, GRAD_TOL, _check_grad, _transitions
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,K,dtype,nodes", [(32, 2, "fp32", 63), (96, 3, "fp32", 2100), (128, 4, "fp32", 2050),
+                                             (160, 4, "fp32", 257), (384, 3, "fp32", 65), (64, 2, "bf16", 127),
+                                             (192, 6, "bf16", 2100), (384, 3, "bf16", 65), (128, 4, "bf16", 129),
+                                             (256, 8, "bf16", 1), (512, 8, "bf16", 131)])
+def test_gradient_at_the_edges_of_the_tiles(xo, H, K, dtype, nodes):
+    import torch
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3)
+    rng = dags.make_rng(H + nodes)
+    sizes = [nodes, nodes + 3, nodes, 1, nodes + 1]
+    graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in sizes]
+    batch = dags.flatten(graphs, [0, 3, 5], 3)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 7)
+    st, packed = xo.pack(batch)
+    assert st == 0
+    action, logp_old, adv, ret = _transitions(xo, m, blob, batch, packed, 5)
+    want = xo.ppo_grad(m, blob, batch, packed, action, logp_old, adv, ret)
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        f32 = lambda a: torch.from_numpy(np.asarray(a, np.float32)).cuda()
+        buf = torch.full((len(blob) + 4,), 7.0, device="cuda")
+        loss = torch.empty(4, device="cuda")
+        for shift in (0, 1):
+            grad = buf[shift:shift + len(blob)]
+            xrl.xrl_ppo_grad(ag.ctx, ag.batch, torch.from_numpy(batch["mask"]).cuda(), torch.from_numpy(action).cuda(),
+                             f32(logp_old), f32(adv), f32(ret), loss, grad)
+            torch.cuda.synchronize()
+            assert ag.device_status() == 0
+            gpu_util.assert_close(loss.cpu().numpy(), want["loss"], dtype, "loss")
+            _check_grad(m, grad.cpu().numpy().astype(np.float64), want["grad"], GRAD_TOL[dtype], f"shift {shift}",
+                        entrywise=BF16_ENTRYWISE if dtype == "bf16" else None)
+    finally:
+        ag.close()
