@@ -7,8 +7,8 @@
 // (nothing is recomputed here); the reverse of Eq. 7 runs row-wise kernels (a warp per destination row:
 // k_aggregate_bwd_rows, k_scores_bwd_rows) with generic fallbacks (k_aggregate_bwd, k_scores_bwd) for head
 // counts that do not divide 32; the two dense products of a layer, dW = h_in^T dz and dh_in = dz W^T, run on
-// the tensor cores (mma.sync bf16, fp32 accumulate: k_atb_mma, k_gwt_mma) for bf16 models of hidden 128, 256
-// or 512 and on CUDA-core tiles (k_atb, k_gwt) otherwise.  Gradients are fp32; sums over rows are collected
+// the tensor cores (k_bwd_umma.cu) for bf16 models of hidden 128, 256 or 512 and on CUDA-core tiles (k_atb_tile,
+// k_gwt and the forward product's kernel) otherwise.  Gradients are fp32; sums over rows are collected
 // with floating-point atomics, so the last bits of a gradient depend on the order in which the hardware
 // serves them.  Activations saved by the forward pass are read in their storage type.  On the tensor-core
 // path the half-score terms (ds a) are added into the bf16 copy of dz that the products read (`dzb`) only:
@@ -547,195 +547,6 @@ k_gwt(const float* __restrict__ G, const TW* __restrict__ W, float* __restrict__
     for (int v = 0; v < 4; ++v) {
       const int r = r0 + ty * 4 + u, k = k0 + tx * 4 + v;
       if (r < rows && k < Hk) out[size_t(r) * Hk + k] = acc[u][v];
-    }
-}
-
-// ---- the two products of a layer's reverse pass on the tensor cores (bf16 models, H a multiple of 128) --------
-// mma.sync m16n8k16, bf16 operands, fp32 accumulators; a CTA of 8 warps (4 x 2) takes a 128 x 128 tile of the
-// result, a warp 32 x 64.  Operand tiles sit in shared memory in 16-byte pieces whose position within a row is
-// XOR-ed with the row number, so that the eight rows one ldmatrix reads fall into different banks.
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// out [rows x H] fp32 = G [rows x H] bf16 times W^T, W [H x H] bf16 row-major [in x out]: out[r][k] = sum_n G[r][n] W[k][n]
-// A CTA takes tiles_per_cta consecutive tiles of 128 rows (kGwtTiles when that still leaves several waves of
-// CTAs, else one); its loop runs over (tile, 64-wide step of n) pairs, so
-// that the first pieces of the next tile are already on their way while the last step of the current tile is
-// multiplied and its 64 KB of results are stored.
-constexpr int kGwtTiles = 4;
-__global__ void __launch_bounds__(256, 2)
-k_gwt_mma(const bf16* __restrict__ G, const bf16* __restrict__ W, float* __restrict__ out, int rows, int H,
-          int tiles_per_cta) {
-  __shared__ __align__(128) bf16 As[128 * 64];      // [row r][64 n], 8 pieces of 16 bytes per row
-  __shared__ __align__(128) bf16 Bs[128 * 64];      // [row k][64 n]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = warp >> 1, wn = warp & 1;
-  // consecutive CTAs take the column tiles of the same rows, so that the rows' second reading comes from L2
-  const int ncol = H / 128;
-  const int k0 = int(blockIdx.x % ncol) * 128;
-  const int tile0 = int(blockIdx.x / ncol) * tiles_per_cta, ntiles = (rows + 127) / 128;
-  const int nk = H / 64, total = min(tiles_per_cta, ntiles - tile0) * nk;
-  float acc[2][8][4];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 8; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  const uint32_t as_base = uint32_t(__cvta_generic_to_shared(As)), bs_base = uint32_t(__cvta_generic_to_shared(Bs));
-  // the next step's pieces travel from global memory to registers while the current step is multiplied
-  uint4 va[4], vb[4];
-  auto fetch = [&](int step) {
-    const int r0 = (tile0 + step / nk) * 128, n0 = (step % nk) * 64;
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + 256 * it, row = idx >> 3, ch = idx & 7;
-      va[it] = make_uint4(0, 0, 0, 0);
-      if (r0 + row < rows) va[it] = *reinterpret_cast<const uint4*>(G + size_t(r0 + row) * H + n0 + ch * 8);
-      vb[it] = *reinterpret_cast<const uint4*>(W + size_t(k0 + row) * H + n0 + ch * 8);
-    }
-  };
-  if (total > 0) fetch(0);
-  for (int step = 0; step < total; ++step) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int idx = tid + 256 * it, row = idx >> 3, ch = idx & 7;
-      const int phys = (row * 8 + (ch ^ (row & 7))) * 8;
-      *reinterpret_cast<uint4*>(As + phys) = va[it];
-      *reinterpret_cast<uint4*>(Bs + phys) = vb[it];
-    }
-    __syncthreads();
-    if (step + 1 < total) fetch(step + 1);
-#pragma unroll
-    for (int kk = 0; kk < 64; kk += 16) {
-      uint32_t af[2][4];
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const int row = wm * 32 + mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-        const int ch = (kk >> 3) + (lane >> 4);
-        ldsm_x4(af[mt], as_base + uint32_t((row * 8 + (ch ^ (row & 7))) * 16));
-      }
-#pragma unroll
-      for (int np = 0; np < 4; ++np) {
-        uint32_t bf[4];
-        const int row = wn * 64 + np * 16 + (lane & 7) + (lane >> 4) * 8;
-        const int ch = (kk >> 3) + ((lane >> 3) & 1);
-        ldsm_x4(bf, bs_base + uint32_t((row * 8 + (ch ^ (row & 7))) * 16));
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          mma_bf16(acc[mt][2 * np], af[mt], bf[0], bf[1]);
-          mma_bf16(acc[mt][2 * np + 1], af[mt], bf[2], bf[3]);
-        }
-      }
-    }
-    __syncthreads();
-    if (step % nk == nk - 1) {                       // the tile is complete: store it, start the next from zero
-      const int r0 = (tile0 + step / nk) * 128;
-      const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-          const int r = r0 + wm * 32 + mt * 16 + g, c = k0 + wn * 64 + nt * 8 + 2 * t;
-          if (r < rows)
-            *reinterpret_cast<float2*>(out + size_t(r) * H + c) = make_float2(acc[mt][nt][0], acc[mt][nt][1]);
-          if (r + 8 < rows)
-            *reinterpret_cast<float2*>(out + size_t(r + 8) * H + c) = make_float2(acc[mt][nt][2], acc[mt][nt][3]);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) acc[mt][nt][q] = 0.f;
-        }
-    }
-  }
-}
-
-// dW [H x H] fp32 += A^T B over the rows [chunk z], A = h_in [rows x H] bf16, B = dz [rows x H] bf16
-__global__ void __launch_bounds__(256, 2)
-k_atb_mma(const bf16* __restrict__ A, const bf16* __restrict__ Bm, float* __restrict__ dW, int rows, int H,
-          int rows_per_chunk) {
-  __shared__ __align__(128) bf16 As[32 * 128];      // [row r][128 m], 16 pieces of 16 bytes per row
-  __shared__ __align__(128) bf16 Bs[32 * 128];      // [row r][128 n]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = warp >> 1, wn = warp & 1;
-  const int m0 = blockIdx.x * 128, n0 = blockIdx.y * 128;
-  const int r_begin = blockIdx.z * rows_per_chunk, r_end = min(rows, r_begin + rows_per_chunk);
-  float acc[2][8][4];
-#pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 8; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  const uint32_t as_base = uint32_t(__cvta_generic_to_shared(As)), bs_base = uint32_t(__cvta_generic_to_shared(Bs));
-  uint4 va[2], vb[2];
-  auto fetch = [&](int rr) {
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      const int idx = tid + 256 * it, row = idx >> 4, ch = idx & 15;
-      va[it] = make_uint4(0, 0, 0, 0); vb[it] = make_uint4(0, 0, 0, 0);
-      if (rr + row < r_end) {
-        va[it] = *reinterpret_cast<const uint4*>(A + size_t(rr + row) * H + m0 + ch * 8);
-        vb[it] = *reinterpret_cast<const uint4*>(Bm + size_t(rr + row) * H + n0 + ch * 8);
-      }
-    }
-  };
-  if (r_begin < r_end) fetch(r_begin);
-  for (int rr = r_begin; rr < r_end; rr += 32) {
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      const int idx = tid + 256 * it, row = idx >> 4, ch = idx & 15;
-      const int phys = (row * 16 + (ch ^ (row & 7))) * 8;
-      *reinterpret_cast<uint4*>(As + phys) = va[it];
-      *reinterpret_cast<uint4*>(Bs + phys) = vb[it];
-    }
-    __syncthreads();
-    if (rr + 32 < r_end) fetch(rr + 32);
-#pragma unroll
-    for (int kk = 0; kk < 32; kk += 16) {
-      uint32_t af[2][4];
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        // the stored rows are the products' k index: transposed 8 x 8 loads give the (m, k) fragments
-        const int row = kk + (lane & 7) + (lane >> 4) * 8;
-        const int ch = ((wm * 32 + mt * 16) >> 3) + ((lane >> 3) & 1);
-        ldsm_x4_trans(af[mt], as_base + uint32_t((row * 16 + (ch ^ (row & 7))) * 16));
-      }
-#pragma unroll
-      for (int np = 0; np < 4; ++np) {
-        uint32_t bf[4];
-        const int row = kk + (lane & 7) + ((lane >> 3) & 1) * 8;
-        const int ch = ((wn * 64 + np * 16) >> 3) + (lane >> 4);
-        ldsm_x4_trans(bf, bs_base + uint32_t((row * 16 + (ch ^ (row & 7))) * 16));
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          mma_bf16(acc[mt][2 * np], af[mt], bf[0], bf[1]);
-          mma_bf16(acc[mt][2 * np + 1], af[mt], bf[2], bf[3]);
-        }
-      }
-    }
-    __syncthreads();
-  }
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int m = m0 + wm * 32 + mt * 16 + g, n = n0 + wn * 64 + nt * 8 + 2 * t;
-      float* o = dW + size_t(m) * H + n;
-      if (acc[mt][nt][0] != 0.f) atomicAdd(o, acc[mt][nt][0]);
-      if (acc[mt][nt][1] != 0.f) atomicAdd(o + 1, acc[mt][nt][1]);
-      if (acc[mt][nt][2] != 0.f) atomicAdd(o + size_t(8) * H, acc[mt][nt][2]);
-      if (acc[mt][nt][3] != 0.f) atomicAdd(o + size_t(8) * H + 1, acc[mt][nt][3]);
     }
 }
 
@@ -1315,7 +1126,7 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
 int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores,
                          const void* h_in, const void* h_out, const float* dh_out, float* dh_in, float* dz,
                          float* ds, void* dz_store, const LayerWeights& lw, float* gW, float* ga_src, float* ga_dst,
-                         float* gb, int32_t N, cudaStream_t st) {
+                         float* gb, int32_t N, int32_t* status, cudaStream_t st) {
   if (N <= 0) return 0;
   const int H = d.H, K = d.K;
   cudaMemsetAsync(dz, 0, sizeof(float) * size_t(N) * H, st);
@@ -1335,18 +1146,10 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   dim3 g_atb(unsigned(atb_side), unsigned(atb_side), unsigned((N + chunk - 1) / chunk));
   const bool vec = (reinterpret_cast<uintptr_t>(gW) & 15) == 0;
   dim3 g_gwt(unsigned((N + 63) / 64), unsigned((H + 63) / 64));
-  // tensor-core products: about two waves of CTAs over the rows, chunks of a multiple of 32 rows, at least 512
-  const int tiles = (H / 128) * (H / 128);
-  const int want_chunks = std::max(1, 2 * kNumSMs / std::max(1, tiles));
-  const int chunk_mma = std::max(512, int(((int64_t(N) + want_chunks - 1) / want_chunks + 31) & ~int64_t(31)));
-  dim3 g_atb_mma(unsigned(H / 128), unsigned(H / 128), unsigned((N + chunk_mma - 1) / chunk_mma));
-  const int row_tiles = (N + 127) / 128;
-  const int gwt_tpc = int64_t(row_tiles) * (H / 128) >= int64_t(kGwtTiles) * 4 * kNumSMs ? kGwtTiles : 1;
-  dim3 g_gwt_mma(unsigned((row_tiles + gwt_tpc - 1) / gwt_tpc) * unsigned(H / 128));
   const int NF = H / 32;
   const bool rows_kernels = (32 % K == 0) && (NF == 1 || NF == 2 || NF == 4 || NF == 8 || NF == 16);
   // bf16 models of hidden 128, 256 or 512 take both products on the tensor cores, from a bf16 copy of dz
-  const bool mma = rows_kernels && d.dtype == XRL_BF16 && H % 128 == 0 && dz_store != nullptr;
+  const bool mma = rows_kernels && bwd_umma_supported(d) && dz_store != nullptr;
   bf16* dzb = mma ? static_cast<bf16*>(dz_store) : nullptr;
 #define BWD_ROWS(TY_, NF_)                                                                                     \
   do {                                                                                                         \
@@ -1377,8 +1180,7 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
                                                                        dz, ga_src, ga_dst, N, H, K);           \
     }                                                                                                          \
     if (mma) {                                                                                                 \
-      k_atb_mma<<<g_atb_mma, 256, 0, st>>>(static_cast<const bf16*>(h_in), dzb, gW, N, H, chunk_mma);          \
-      k_gwt_mma<<<g_gwt_mma, 256, 0, st>>>(dzb, static_cast<const bf16*>(lw.W), dh_in, N, H, gwt_tpc);                  \
+      if (launch_bwd_umma(d, h_in, dzb, lw.W, dh_in, gW, N, status, st) < 0) return -1;                        \
     } else {                                                                                                   \
       if (wide_atb)                                                                                            \
         k_atb_tile<TY_, 128><<<g_atb, 256, 0, st>>>(static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);  \

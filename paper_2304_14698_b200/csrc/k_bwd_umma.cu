@@ -1,0 +1,353 @@
+// The two dense products of an attention layer's reverse pass (paper Section 3.3.4's gradient through Eq. 7) on the
+// 5th-generation tensor cores, for bf16 models: with dz the gradient of Z = h W in bf16,
+//   dh = dz W^T   the transform kernel's roles and tiles (xrl_xform_umma.cuh) with W itself as the K-major operand
+//                 and an fp32 result;
+//   dW += h^T dz  reduces over the rows, so both operands are used as they lie in memory: a 64-row block of h and one
+//                 of dz come in as TMA boxes of 64 columns, which tcgen05.mma reads as MN-major operands, and
+//                 the whole H x H result (H = 256: all 512 columns of tensor memory) stays in tensor memory
+//                 while the CTA walks its range of rows.  The CTAs' results meet in the gradient by TMA
+//                 reductions (fp32 add in L2).
+// Both are bound by HBM: 6 H bytes per row (dh: 2 H in, 4 H out) and 4 H bytes per row (dW).
+//
+// Every wait on an mbarrier is bounded; on expiry the kernel records XRL_ERR_TIMEOUT, drains its own copies in
+// flight, frees its tensor memory and returns.
+#include "xrl_xform_umma.cuh"
+
+namespace xrl {
+
+using namespace umma;
+using namespace xform;
+
+namespace {
+
+constexpr int kThreads = 192;            // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+
+__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
+}
+
+// 32 fp32 columns of a thread's row into a staging tile of 128 rows x 128 bytes, 128-byte swizzle
+__device__ __forceinline__ void stage_row(uint8_t* tile, int row, const uint32_t (&v)[32]) {
+  uint8_t* p = tile + row * 128;
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    *reinterpret_cast<uint4*>(p + ((j ^ (row & 7)) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+}
+
+// ---- dh = dz W^T ---------------------------------------------------------------------------------------------
+template <int NS, int KP>
+__global__ void __launch_bounds__(kThreads, 1)
+k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_w,
+          const __grid_constant__ CUtensorMap map_o, int rows, int H, int slices, int32_t* status) {
+  using C = Cfg<NS, KP>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const uint32_t base = smem_u32(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int num_tiles = (rows + BM - 1) / BM;
+  const int slice = int(blockIdx.x) % slices, first = int(blockIdx.x) / slices, step = int(gridDim.x) / slices;
+  const int col0 = slice * NS, cols = min(NS, H - col0);
+  if ((base & 1023u) != 0) {
+    if (threadIdx.x == 0) raise(status, XRL_ERR_UNSUPPORTED);
+    return;
+  }
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM);
+  if (threadIdx.x == 0) {
+    tmem_slot[1] = 0;
+    init_barriers<C>(base);
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  if (warp == 0) {
+    if (lane == 0) {
+      load_w<C>(base, &map_w, col0);
+      uint32_t it = 0;
+      if (!produce_tiles<C>(base, &map_g, first, step, num_tiles, it)) {
+        raise(status, XRL_ERR_TIMEOUT);
+        drain_producer<C>(base, it, 0);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      uint32_t it = 0, lt = 0;
+      if (!mma_tiles<C, NS>(base, tmem_base, first, step, num_tiles, it, lt, 0)) raise(status, XRL_ERR_TIMEOUT);
+    }
+  } else {
+    const int q = warp & 3, row_in_tile = q * 32 + lane;
+    const bool leader = threadIdx.x == 64;
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+    uint32_t lt = 0;
+    for (int tile = first; tile < num_tiles; tile += step, ++lt) {
+      const int buf = lt & 1;
+      uint32_t okw = 1;
+      if (lane == 0) okw = mbar_wait(C::bar_acc_full(base, buf), (lt >> 1) & 1) ? 1u : 0u;
+      okw = __shfl_sync(0xFFFFFFFFu, okw, 0);
+      if (!okw && lane == 0) { *abort_flag = 1; raise(status, XRL_ERR_TIMEOUT); }
+      epi_barrier();
+      if (*abort_flag) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(buf * C::ACC_COLS);
+#pragma unroll 2
+      for (int c = 0; c < NS / 32; ++c) {
+        uint32_t v[32];
+        tc_ld32(taddr + c * 32, v);
+        tc_wait_ld();
+        if (leader) tma_wait_read<1>();          // the store issued two chunks ago has read this staging tile
+        epi_barrier();
+        stage_row(smem + C::OFF_OUT + (c & 1) * STAGE_BYTES, row_in_tile, v);
+        fence_async_smem();
+        epi_barrier();
+        if (leader && c * 32 < cols) {
+          tma_store_2d(&map_o, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, col0 + c * 32, tile * BM);
+          tma_commit();
+        }
+      }
+      tc_fence_before();
+      mbar_arrive(C::bar_acc_empty(base, buf));
+    }
+    if (leader) tma_wait_all();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                 ::"r"(tmem_base), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+  }
+}
+
+// ---- dW += h^T dz ----------------------------------------------------------------------------------------------
+// S: side of the square of dW a CTA accumulates (128: H = 128; 256: H = 256, and a quarter of H = 512).
+constexpr int RB = 64;                   // rows per stage
+template <int S> struct WCfg {
+  static constexpr int CHUNK = RB * 128;                 // 64 rows x 64 columns
+  static constexpr int OPERAND = (S / 64) * CHUNK;       // one operand of a stage
+  static constexpr int STAGES = S == 256 ? 3 : 5;
+  static constexpr int OFF_OUT = STAGES * 2 * OPERAND;
+  static constexpr int OFF_BAR = OFF_OUT + 2 * STAGE_BYTES;
+  static constexpr int OFF_TMEM = OFF_BAR + 8 * (2 * STAGES + 1);
+  static constexpr int SMEM_BYTES = OFF_TMEM + 16;
+  static constexpr int HALVES = S / 128;                 // M = 128 rows of dW per instruction
+  static constexpr int TMEM_COLS = HALVES * S;
+  static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one SM");
+};
+
+// Shared-memory matrix descriptor of an MN-major, 128-byte-swizzled operand: rows (the reduction index) of 128 bytes,
+// 8-row groups 1,024 bytes apart, 64-column chunks `chunk` bytes apart.
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t chunk) {
+  return uint64_t((addr & 0x3FFFFu) >> 4) | (uint64_t(chunk >> 4) << 16) | (uint64_t(1024 >> 4) << 32) |
+         (uint64_t(1) << 46) | (uint64_t(2) << 61);
+}
+
+template <int S>
+__global__ void __launch_bounds__(kThreads, 1)
+k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_g,
+          const __grid_constant__ CUtensorMap map_o, float* __restrict__ dW, int rows, int H, int side, bool use_tma,
+          int32_t* status) {
+  using C = WCfg<S>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const uint32_t base = smem_u32(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((base & 1023u) != 0) {
+    if (threadIdx.x == 0) raise(status, XRL_ERR_UNSUPPORTED);
+    return;
+  }
+  // CTA = (range of 64-row blocks, square of dW); the squares of a range side by side
+  const int squares = side * side, part = int(blockIdx.x) / squares, parts = int(gridDim.x) / squares;
+  const int a0 = (int(blockIdx.x) % squares) / side * S, b0 = int(blockIdx.x) % side * S;
+  const int blocks = (rows + RB - 1) / RB;
+  const int blk0 = int(int64_t(blocks) * part / parts), blk1 = int(int64_t(blocks) * (part + 1) / parts);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM);
+  auto bar_full = [&](int s) { return base + C::OFF_BAR + 8u * s; };
+  auto bar_empty = [&](int s) { return base + C::OFF_BAR + 8u * (C::STAGES + s); };
+  const uint32_t bar_done = base + C::OFF_BAR + 8u * (2 * C::STAGES);
+  if (threadIdx.x == 0) {
+    tmem_slot[1] = 0;
+    for (int s = 0; s < C::STAGES; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+    mbar_init(bar_done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const int nblk = blk1 - blk0;            // >= 1: the launch has at most one part per block
+
+  if (warp == 0) {
+    if (lane == 0) {
+      bool ok = true;
+      int i = 0;
+      for (; i < nblk; ++i) {
+        const int s = i % C::STAGES, round = i / C::STAGES;
+        if (round > 0 && !mbar_wait(bar_empty(s), (round - 1) & 1)) { ok = false; break; }
+        mbar_expect_tx(bar_full(s), 2 * C::OPERAND);
+        const uint32_t at = base + s * 2 * C::OPERAND;
+        for (int c = 0; c < S / 64; ++c) {
+          tma_load_2d(at + c * C::CHUNK, &map_h, a0 + c * 64, (blk0 + i) * RB, bar_full(s));
+          tma_load_2d(at + C::OPERAND + c * C::CHUNK, &map_g, b0 + c * 64, (blk0 + i) * RB, bar_full(s));
+        }
+      }
+      if (!ok) {                           // let the loads already issued land before the shared memory goes away
+        raise(status, XRL_ERR_TIMEOUT);
+        for (int j = i > C::STAGES ? i - C::STAGES : 0; j < i; ++j) mbar_wait(bar_full(j % C::STAGES), (j / C::STAGES) & 1);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // fp32 accumulators, bf16 x bf16, both operands MN-major (bits 15, 16), M = 128, N = S
+      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (uint32_t(S >> 3) << 17) |
+                                 (uint32_t(128 >> 4) << 24);
+      bool ok = true;
+      for (int i = 0; i < nblk; ++i) {
+        const int s = i % C::STAGES;
+        if (!mbar_wait(bar_full(s), (i / C::STAGES) & 1)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t at = base + s * 2 * C::OPERAND;
+#pragma unroll
+        for (int ks = 0; ks < RB / 16; ++ks)             // 16 rows = two 8-row groups per instruction
+#pragma unroll
+          for (int m = 0; m < C::HALVES; ++m)
+            tc_mma(tmem_base + uint32_t(m * S), smem_desc_mn(at + m * 2 * C::CHUNK + ks * 2048, C::CHUNK),
+                   smem_desc_mn(at + C::OPERAND + ks * 2048, C::CHUNK), idesc, (i | ks) != 0 ? 1u : 0u);
+        tc_commit(bar_empty(s));
+      }
+      if (ok) tc_commit(bar_done);
+      else raise(status, XRL_ERR_TIMEOUT);
+    }
+  } else {
+    const int q = warp & 3, row = q * 32 + lane;
+    const bool leader = threadIdx.x == 64;
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+    // the whole range is multiplied first: the limit of one wait, several times over
+    uint32_t okw = 1;
+    if (lane == 0) {
+      okw = 0;
+      for (int t = 0; t < 4 && !okw; ++t) okw = mbar_wait(bar_done, 0) ? 1u : 0u;
+    }
+    okw = __shfl_sync(0xFFFFFFFFu, okw, 0);
+    if (!okw && lane == 0) { *abort_flag = 1; raise(status, XRL_ERR_TIMEOUT); }
+    epi_barrier();
+    if (!*abort_flag) {
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16);
+      for (int c = 0; c < C::HALVES * (S / 32); ++c) {
+        const int m = c / (S / 32), cc = c % (S / 32);
+        uint32_t v[32];
+        tc_ld32(taddr + m * S + cc * 32, v);
+        tc_wait_ld();
+        if (use_tma) {
+          if (leader) tma_wait_read<1>();
+          epi_barrier();
+          stage_row(smem + C::OFF_OUT + (c & 1) * STAGE_BYTES, row, v);
+          fence_async_smem();
+          epi_barrier();
+          if (leader) {
+            tma_reduce_add_2d(&map_o, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, b0 + cc * 32, a0 + m * 128);
+            tma_commit();
+          }
+        } else {
+          float* o = dW + size_t(a0 + m * 128 + row) * H + b0 + cc * 32;
+#pragma unroll
+          for (int t = 0; t < 32; ++t) atomicAdd(o + t, __uint_as_float(v[t]));
+        }
+      }
+      if (leader) tma_wait_all();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                 ::"r"(tmem_base), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+  }
+}
+
+// 2-D fp32 tensor [rows x cols] row-major, box [128 rows x 32 columns], 128-byte swizzle
+bool make_map_f32(CUtensorMap* m, void* ptr, uint64_t rows, uint64_t cols) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {cols, rows};
+  cuuint64_t strides[1] = {cols * 4};
+  cuuint32_t box[2] = {32, 128};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+         CUDA_SUCCESS;
+}
+
+template <int NS, int KP>
+int launch_dh(int H, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
+  using C = Cfg<NS, KP>;
+  static bool attr_set[64] = {};
+  if (!ensure_dynamic_smem(k_dh_umma<NS, KP>, C::SMEM_BYTES, attr_set)) return -1;
+  CUtensorMap mg, mw, mo;
+  if (!make_map(&mg, dzb, uint64_t(rows), H, BM) || !make_map(&mw, W, H, H, NS) || !make_map_f32(&mo, dh, uint64_t(rows), H))
+    return -1;
+  const int slices = (H + NS - 1) / NS, tiles = (rows + BM - 1) / BM, groups = kNumSMs / slices;
+  k_dh_umma<NS, KP><<<(tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st>>>(mg, mw, mo, rows, H, slices,
+                                                                                                 status);
+  return 1;
+}
+
+template <int S>
+int launch_dw(int H, const void* h, const void* dzb, float* dW, int32_t rows, int32_t* status, cudaStream_t st) {
+  using C = WCfg<S>;
+  static bool attr_set[64] = {};
+  if (!ensure_dynamic_smem(k_dw_umma<S>, C::SMEM_BYTES, attr_set)) return -1;
+  const bool aligned = (reinterpret_cast<uintptr_t>(dW) & 15) == 0;    // the caller's buffer may sit on any 4-byte boundary
+  CUtensorMap mh, mg, mo;
+  if (!make_map(&mh, h, uint64_t(rows), H, RB) || !make_map(&mg, dzb, uint64_t(rows), H, RB)) return -1;
+  if (aligned) { if (!make_map_f32(&mo, dW, H, H)) return -1; }
+  else mo = mh;
+  const int side = H / S, squares = side * side;
+  // at least eight blocks per CTA: every CTA ends with a reduction of its whole square of dW into the gradient
+  const int blocks = (rows + RB - 1) / RB, want = (blocks + 7) / 8, most = kNumSMs / squares;
+  k_dw_umma<S><<<(want < most ? want : most) * squares, kThreads, C::SMEM_BYTES, st>>>(
+      mh, mg, mo, dW, rows, H, side, aligned, status);
+  return 1;
+}
+
+}  // namespace
+
+// bf16 models of hidden 128, 256 or 512 (the widths whose dz is kept in bf16 for these products)
+bool bwd_umma_supported(const Dims& d) {
+  return d.dtype == XRL_BF16 && (d.H == 128 || d.H == 256 || d.H == 512) && encode_fn() != nullptr;
+}
+// dh [rows x H] = dzb W^T and dW [H x H] += h^T dzb.  Returns kernels launched, or -1.
+int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W, float* dh, float* dW, int32_t rows,
+                    int32_t* status, cudaStream_t st) {
+  if (rows <= 0) return 0;
+  int a, b;
+  switch (d.H) {
+    case 128:
+      a = launch_dw<128>(128, h, dzb, dW, rows, status, st);
+      b = launch_dh<128, 128>(128, dzb, W, dh, rows, status, st);
+      break;
+    case 256:
+      a = launch_dw<256>(256, h, dzb, dW, rows, status, st);
+      b = launch_dh<256, 256>(256, dzb, W, dh, rows, status, st);
+      break;
+    case 512:
+      a = launch_dw<256>(512, h, dzb, dW, rows, status, st);
+      b = launch_dh<128, 512>(512, dzb, W, dh, rows, status, st);
+      break;
+    default: return -1;
+  }
+  return a < 0 || b < 0 ? -1 : a + b;
+}
+
+}  // namespace xrl

@@ -1155,7 +1155,7 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
     float* ga_src = grad + (lw.a_src - wb);
     const int k = launch_gat_layer_bwd(d, gat_rowptr, gat_col, zs[l], ss[l], hs[l], hs[l + 1], dh_cur,
                              dh_nxt, dz, ds, dz_store, lw, ga_src - H * H, ga_src, grad + (lw.a_dst - wb),
-                             grad + (lw.b - wb), b->N, st);
+                             grad + (lw.b - wb), b->N, ctx->status.as<int32_t>(), st);
     if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
     n += k;
     std::swap(dh_cur, dh_nxt);
