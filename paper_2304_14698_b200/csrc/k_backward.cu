@@ -200,11 +200,14 @@ __device__ __forceinline__ void atomic_add_chunk(float* p, const float (&v)[NF])
   }
 }
 
-template <typename T, int NF>
+// GATHER: nothing is scattered; every entry's (alpha, de) goes to its place in the transposed lists `tl` and the masked
+// gradient dpre replaces dh_out (unless it arrives masked), for k_dz_gather to collect.
+template <typename T, int NF, bool GATHER>
 __global__ void __launch_bounds__(256)
 k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, ZView<T> zv,
-                     const T* __restrict__ h_out, const float* __restrict__ dh_out, float* __restrict__ dz,
-                     float* __restrict__ ds_src, float* __restrict__ ds_dst, float* __restrict__ db, int N, int K) {
+                     const T* __restrict__ h_out, float* __restrict__ dh_out, bool masked, float* __restrict__ dz,
+                     float* __restrict__ ds_src, float* __restrict__ ds_dst, float* __restrict__ db, int N, int K,
+                     BwdLists tl) {
   constexpr int H = 32 * NF;
   __shared__ float sm_db[H];
   for (int c = threadIdx.x; c < H; c += blockDim.x) sm_db[c] = 0.f;
@@ -224,12 +227,14 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
       load_chunk<T, NF>(h_out + size_t(i) * H + lane * NF, ho);
 #pragma unroll
       for (int f = 0; f < NF; ++f) { dp[f] = ho[f] > 0.f ? g[f] : 0.f; dbr[f] += dp[f]; }
+      if (GATHER && !masked) store_chunk<NF>(dh_out + size_t(i) * H + lane * NF, dp);
     }
     bool live = false;
 #pragma unroll
     for (int f = 0; f < NF; ++f) live = live || dp[f] != 0.f;
-    if (!__any_sync(0xFFFFFFFFu, live)) continue;     // a row whose units are all off: nothing flows (ds is zeroed)
+    if (!GATHER && !__any_sync(0xFFFFFFFFu, live)) continue;   // a row whose units are all off: nothing flows (ds is zeroed)
     const int32_t e0 = rowptr[i], deg = rowptr[i + 1] - e0;
+    const int32_t self_entry = GATHER ? tl.rowptr[i] + i : 0;
     const float sd = zv.pair(i, k).y;
     // One sweep over the row's neighbours and the row itself (entry `deg`) takes, per head, the score e_t, the
     // product dal_t = dpre . z_t, and with a running maximum the sums  sum_t 2^(e_t - mx)  and
@@ -294,10 +299,15 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
     const float inv = 1.f / sum;
     const float dot = dotu * inv;
     float dsd = 0.f;
-    auto scatter = [&](int32_t j, float eraw, float dal) {
+    auto scatter = [&](int32_t j, int t, float eraw, float dal) {
       const float al = exp2f(lrelu(eraw) - mx) * inv;
       const float de = al * (dal - dot) * (eraw > 0.f ? 1.f : 0.2f);
       dsd += de;
+      if (GATHER) {
+        const int32_t at = t < deg ? tl.inv[e0 + t] : self_entry;
+        if (leader) tl.entry[size_t(at) * K + k] = make_float2(al, de);
+        return;
+      }
       if (leader && de != 0.f) atomicAdd(&ds_src[size_t(j) * K + k], de);
       if (live) {
         float v[NF];
@@ -308,7 +318,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
     };
 #pragma unroll
     for (int t = 0; t < kCache; ++t)
-      if (t <= deg) scatter(__shfl_sync(0xFFFFFFFFu, c0, t), ce[t], cd[t]);
+      if (t <= deg) scatter(__shfl_sync(0xFFFFFFFFu, c0, t), t, ce[t], cd[t]);
     for (int base = 0; base <= deg; base += 32) {
       const int idx = base + lane;
       const int32_t cj = base == 0 ? c0 : (idx < deg ? col[e0 + idx] : i);
@@ -317,7 +327,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
         const int32_t j = __shfl_sync(0xFFFFFFFFu, cj, t);
         float eraw, dal;
         score_and_product(j, eraw, dal);
-        scatter(j, eraw, dal);
+        scatter(j, base + t, eraw, dal);
       }
     }
     if (leader) ds_dst[size_t(i) * K + k] = dsd;
@@ -935,14 +945,20 @@ k_graph_bwd(const float* __restrict__ emb, const float* __restrict__ dlogit, Mlp
   }
 }
 
-// the readout is a plain sum: every node receives its graph's gradient (four columns per thread; H % 4 == 0)
-__global__ void k_readout_bwd(const float* __restrict__ dr, const int32_t* __restrict__ seg_id,
+// the readout is a plain sum: every node receives its graph's gradient, masked by the ReLU of its features (four columns
+// per thread; H % 4 == 0)
+template <typename T>
+__global__ void k_readout_bwd(const float* __restrict__ dr, const int32_t* __restrict__ seg_id, const T* __restrict__ h,
                               float* __restrict__ dh, int64_t n_quads, int H) {
   const int q = H >> 2;
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_quads; t += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = t / q;
     const int c = int(t - i * q);
-    reinterpret_cast<float4*>(dh)[t] = reinterpret_cast<const float4*>(dr + size_t(seg_id[i]) * H)[c];
+    const float4 g = reinterpret_cast<const float4*>(dr + size_t(seg_id[i]) * H)[c];
+    float ho[4];
+    load_chunk<T, 4>(h + 4 * t, ho);
+    reinterpret_cast<float4*>(dh)[t] = make_float4(ho[0] > 0.f ? g.x : 0.f, ho[1] > 0.f ? g.y : 0.f, ho[2] > 0.f ? g.z : 0.f,
+                                                   ho[3] > 0.f ? g.w : 0.f);
   }
 }
 
@@ -1115,22 +1131,32 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
   const int64_t ne = N * (d.H / 4);
   if (ne > 0) {
     const unsigned grid = unsigned(std::min<int64_t>((ne + 255) / 256, int64_t(kNumSMs) * 64));
-    k_readout_bwd<<<grid, 256, 0, st>>>(dr, seg_id, dh, ne, d.H);
+    if (d.dtype == XRL_BF16) k_readout_bwd<bf16><<<grid, 256, 0, st>>>(dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
+    else k_readout_bwd<float><<<grid, 256, 0, st>>>(dr, seg_id, static_cast<const float*>(hL), dh, ne, d.H);
     ++n;
   }
   return n;
 }
 
+static bool bwd_rows_kernels(const Dims& d) {
+  const int NF = d.H / 32;
+  return (32 % d.K == 0) && (NF == 1 || NF == 2 || NF == 4 || NF == 8 || NF == 16);
+}
+bool bwd_leaves_masked(const Dims& d) { return bwd_rows_kernels(d) && bwd_umma_supported(d); }
+
 // One attention layer backwards: dh_out -> (dW, da_src, da_dst, db) and dh_in.  Z / scores hold the layer's
 // forward transform of h_in; dz [N x H] and ds [2 N K] are scratch.
 int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores,
-                         const void* h_in, const void* h_out, const float* dh_out, float* dh_in, float* dz,
-                         float* ds, void* dz_store, const LayerWeights& lw, float* gW, float* ga_src, float* ga_dst,
-                         float* gb, int32_t N, int32_t* status, cudaStream_t st) {
+                         const void* h_in, const void* h_out, float* dh_out, bool masked, float* dh_in, float* dz,
+                         float* ds, void* dz_store, const BwdLists* lists, const LayerWeights& lw, float* gW, float* ga_src,
+                         float* ga_dst, float* gb, int32_t N, int32_t* status, cudaStream_t st) {
   if (N <= 0) return 0;
   const int H = d.H, K = d.K;
-  cudaMemsetAsync(dz, 0, sizeof(float) * size_t(N) * H, st);
-  cudaMemsetAsync(ds, 0, sizeof(float) * size_t(N) * K * 2, st);
+  const bool gather = lists != nullptr;      // dz by producer from the lists (every entry written, nothing to clear)
+  if (!gather) {
+    cudaMemsetAsync(dz, 0, sizeof(float) * size_t(N) * H, st);
+    cudaMemsetAsync(ds, 0, sizeof(float) * size_t(N) * K * 2, st);
+  }
   float* ds_src = ds;
   float* ds_dst = ds + size_t(N) * K;
   const size_t zrow = z_row_bytes(d);
@@ -1147,16 +1173,25 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   const bool vec = (reinterpret_cast<uintptr_t>(gW) & 15) == 0;
   dim3 g_gwt(unsigned((N + 63) / 64), unsigned((H + 63) / 64));
   const int NF = H / 32;
-  const bool rows_kernels = (32 % K == 0) && (NF == 1 || NF == 2 || NF == 4 || NF == 8 || NF == 16);
+  const bool rows_kernels = bwd_rows_kernels(d);
   // bf16 models of hidden 128, 256 or 512 take both products on the tensor cores, from a bf16 copy of dz
   const bool mma = rows_kernels && bwd_umma_supported(d) && dz_store != nullptr;
   bf16* dzb = mma ? static_cast<bf16*>(dz_store) : nullptr;
 #define BWD_ROWS(TY_, NF_)                                                                                     \
   do {                                                                                                         \
-    k_aggregate_bwd_rows<TY_, NF_><<<grid_rows, 256, 0, st>>>(rowptr, col, zv, static_cast<const TY_*>(h_out), \
-                                                              dh_out, dz, ds_src, ds_dst, gb, N, K);           \
+    k_aggregate_bwd_rows<TY_, NF_, false><<<grid_rows, 256, 0, st>>>(                                          \
+        rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, dz, ds_src, ds_dst, gb, N, K, BwdLists{});  \
     k_scores_bwd_rows<TY_, NF_><<<grid_rows, 256, 0, st>>>(zv, ds_src, ds_dst, lw.a_src, lw.a_dst, dz, dzb,    \
                                                            ga_src, ga_dst, N, K);                              \
+  } while (0)
+#define BWD_GATHER(TY_, NF_)                                                                                   \
+  do {                                                                                                         \
+    if (launch_rows_gather(d, *lists, rowptr, col, Z, scores, h_out, dh_out, masked, ds_dst, gb, N, status, st) < 0) \
+      k_aggregate_bwd_rows<TY_, NF_, true><<<grid_rows, 256, 0, st>>>(                                         \
+          rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, nullptr, nullptr, ds_dst, gb, N, K, *lists); \
+    if (launch_dz_gather(d, *lists, dh_out, Z, zrow, ds_dst, lw, mma ? dz_store : static_cast<void*>(dz), ga_src, ga_dst, \
+                         N, status, st) < 0)                                                                   \
+      return -1;                                                                                               \
   } while (0)
 #define BWD_BODY(TY_)                                                                                          \
   do {                                                                                                         \
@@ -1165,7 +1200,9 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
     zv.pairs = d.zmerged ? reinterpret_cast<const float2*>(static_cast<const char*>(Z) + size_t(H) * sizeof(TY_)) \
                          : reinterpret_cast<const float2*>(scores);                                          \
     zv.pair_stride = d.zmerged ? int(zrow / 8) : K;                                                            \
-    if (rows_kernels) {                                                                                        \
+    if (gather) {                                                                                              \
+      if (NF == 4) BWD_GATHER(TY_, 4); else BWD_GATHER(TY_, 8);                                                \
+    } else if (rows_kernels) {                                                                                 \
       switch (NF) {                                                                                            \
         case 1: BWD_ROWS(TY_, 1); break;                                                                       \
         case 2: BWD_ROWS(TY_, 2); break;                                                                       \
@@ -1195,6 +1232,7 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   } while (0)
   if (d.dtype == XRL_BF16) BWD_BODY(bf16); else BWD_BODY(float);
 #undef BWD_ROWS
+#undef BWD_GATHER
 #undef BWD_BODY
   return 4;
 }

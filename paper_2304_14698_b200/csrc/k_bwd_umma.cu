@@ -1,13 +1,13 @@
 // The two dense products of an attention layer's reverse pass (paper Section 3.3.4's gradient through Eq. 7) on the
 // 5th-generation tensor cores, for bf16 models: with dz the gradient of Z = h W in bf16,
 //   dh = dz W^T   the transform kernel's roles and tiles (xrl_xform_umma.cuh) with W itself as the K-major operand
-//                 and an fp32 result;
+//                 and an fp32 result, which leaves masked by the ReLU of h (what the next layer down needs);
 //   dW += h^T dz  reduces over the rows, so both operands are used as they lie in memory: a 64-row block of h and one
 //                 of dz come in as TMA boxes of 64 columns, which tcgen05.mma reads as MN-major operands, and
 //                 the whole H x H result (H = 256: all 512 columns of tensor memory) stays in tensor memory
 //                 while the CTA walks its range of rows.  The CTAs' results meet in the gradient by TMA
 //                 reductions (fp32 add in L2).
-// Both are bound by HBM: 6 H bytes per row (dh: 2 H in, 4 H out) and 4 H bytes per row (dW).
+// Both are bound by HBM: 8 H bytes per row (dh: 4 H in, 4 H out) and 4 H bytes per row (dW).
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records XRL_ERR_TIMEOUT, drains its own copies in
 // flight, frees its tensor memory and returns.
@@ -39,7 +39,8 @@ __device__ __forceinline__ void stage_row(uint8_t* tile, int row, const uint32_t
 template <int NS, int KP>
 __global__ void __launch_bounds__(kThreads, 1)
 k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_w,
-          const __grid_constant__ CUtensorMap map_o, int rows, int H, int slices, int32_t* status) {
+          const __grid_constant__ CUtensorMap map_o, const bf16* __restrict__ h, int rows, int H, int slices,
+          int32_t* status) {
   using C = Cfg<NS, KP>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
@@ -84,6 +85,21 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
     const bool leader = threadIdx.x == 64;
     volatile uint32_t* abort_flag = tmem_slot + 1;
     uint32_t lt = 0;
+    // The features whose ReLU masks the result: this thread's row of a tile, 32 columns (64 bytes) per chunk, asked for a
+    // whole tile ahead (2 NS bytes of them in registers: asked for one chunk ahead the four warps wait for them,
+    // 0.448 instead of 0.351 ms at 990 k rows and hidden 256).
+    uint4 hn[NS / 32][4];
+    auto features = [&](int tile, int c, uint4 (&f)[4]) {
+      const int64_t r = int64_t(tile) * BM + row_in_tile;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        f[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (tile < num_tiles && r < rows && c * 32 < cols)
+          f[j] = __ldg(reinterpret_cast<const uint4*>(h + size_t(r) * H + col0 + c * 32) + j);
+      }
+    };
+#pragma unroll
+    for (int c = 0; c < NS / 32; ++c) features(first, c, hn[c]);
     for (int tile = first; tile < num_tiles; tile += step, ++lt) {
       const int buf = lt & 1;
       uint32_t okw = 1;
@@ -94,11 +110,19 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
       if (*abort_flag) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(buf * C::ACC_COLS);
-#pragma unroll 2
+#pragma unroll
       for (int c = 0; c < NS / 32; ++c) {
         uint32_t v[32];
         tc_ld32(taddr + c * 32, v);
         tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float f[8];
+          unpack(hn[c][j], f);
+#pragma unroll
+          for (int t = 0; t < 8; ++t) v[8 * j + t] = f[t] > 0.f ? v[8 * j + t] : 0u;
+        }
+        features(tile + step, c, hn[c]);
         if (leader) tma_wait_read<1>();          // the store issued two chunks ago has read this staging tile
         epi_barrier();
         stage_row(smem + C::OFF_OUT + (c & 1) * STAGE_BYTES, row_in_tile, v);
@@ -290,7 +314,7 @@ bool make_map_f32(CUtensorMap* m, void* ptr, uint64_t rows, uint64_t cols) {
 }
 
 template <int NS, int KP>
-int launch_dh(int H, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
+int launch_dh(int H, const void* h, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
   using C = Cfg<NS, KP>;
   static bool attr_set[64] = {};
   if (!ensure_dynamic_smem(k_dh_umma<NS, KP>, C::SMEM_BYTES, attr_set)) return -1;
@@ -298,8 +322,8 @@ int launch_dh(int H, const void* dzb, const void* W, float* dh, int32_t rows, in
   if (!make_map(&mg, dzb, uint64_t(rows), H, BM) || !make_map(&mw, W, H, H, NS) || !make_map_f32(&mo, dh, uint64_t(rows), H))
     return -1;
   const int slices = (H + NS - 1) / NS, tiles = (rows + BM - 1) / BM, groups = kNumSMs / slices;
-  k_dh_umma<NS, KP><<<(tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st>>>(mg, mw, mo, rows, H, slices,
-                                                                                                 status);
+  k_dh_umma<NS, KP><<<(tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st>>>(
+      mg, mw, mo, static_cast<const bf16*>(h), rows, H, slices, status);
   return 1;
 }
 
@@ -327,7 +351,7 @@ int launch_dw(int H, const void* h, const void* dzb, float* dW, int32_t rows, in
 bool bwd_umma_supported(const Dims& d) {
   return d.dtype == XRL_BF16 && (d.H == 128 || d.H == 256 || d.H == 512) && encode_fn() != nullptr;
 }
-// dh [rows x H] = dzb W^T and dW [H x H] += h^T dzb.  Returns kernels launched, or -1.
+// dh [rows x H] = dzb W^T where h > 0, else 0, and dW [H x H] += h^T dzb.  Returns kernels launched, or -1.
 int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W, float* dh, float* dW, int32_t rows,
                     int32_t* status, cudaStream_t st) {
   if (rows <= 0) return 0;
@@ -335,15 +359,15 @@ int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W
   switch (d.H) {
     case 128:
       a = launch_dw<128>(128, h, dzb, dW, rows, status, st);
-      b = launch_dh<128, 128>(128, dzb, W, dh, rows, status, st);
+      b = launch_dh<128, 128>(128, h, dzb, W, dh, rows, status, st);
       break;
     case 256:
       a = launch_dw<256>(256, h, dzb, dW, rows, status, st);
-      b = launch_dh<256, 256>(256, dzb, W, dh, rows, status, st);
+      b = launch_dh<256, 256>(256, h, dzb, W, dh, rows, status, st);
       break;
     case 512:
       a = launch_dw<256>(512, h, dzb, dW, rows, status, st);
-      b = launch_dh<128, 512>(512, dzb, W, dh, rows, status, st);
+      b = launch_dh<128, 512>(512, h, dzb, W, dh, rows, status, st);
       break;
     default: return -1;
   }

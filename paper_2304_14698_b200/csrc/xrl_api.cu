@@ -1115,8 +1115,15 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   const size_t h_bytes = up(sb * Nmax * H), f_bytes = up(4 * Nmax * H), ds_bytes = up(8 * Nmax * size_t(c.heads));
   const size_t heads_bytes = up(4 * ppo_heads_workspace_floats(d, c.max_graphs, c.max_envs));
   const size_t z_bytes = up(Nmax * z_row_bytes(d));
+  // dz by producer: transposed neighbour lists (N + 1, E, E ints; scratch), one {alpha, score gradient} per entry and head
+  const bool gather = bwd_gather_supported(d);
+  const size_t Emax = size_t(c.max_edges) * (c.neighbourhood ? 2 : 1);
+  const size_t t_rows = up(4 * (Nmax + 1)), t_slots = up(4 * (Emax + 1)),
+               t_scratch = up(4 * (Nmax + scan_workspace_ints(int64_t(Nmax) + 1))),
+               t_entries = up(8 * size_t(c.heads) * (Nmax + Emax + 4));
+  const size_t lists_bytes = gather ? t_rows + 2 * t_slots + t_scratch + t_entries : 0;
   if (!ctx->bw.p) {
-    if (ctx->bw.alloc(size_t(L + 2) * h_bytes + size_t(L) * (z_bytes + ds_bytes) + 3 * f_bytes + ds_bytes +
+    if (ctx->bw.alloc(lists_bytes + size_t(L + 2) * h_bytes + size_t(L) * (z_bytes + ds_bytes) + 3 * f_bytes + ds_bytes +
                       heads_bytes) != cudaSuccess) {
       cudaGetLastError();
       ctx->bw.p = nullptr;
@@ -1136,7 +1143,16 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   float* dh_b = reinterpret_cast<float*>(p); p += f_bytes;
   float* dz = reinterpret_cast<float*>(p); p += f_bytes;
   float* ds = reinterpret_cast<float*>(p); p += ds_bytes;
-  float* heads_ws = reinterpret_cast<float*>(p);
+  float* heads_ws = reinterpret_cast<float*>(p); p += heads_bytes;
+  BwdLists lists{};
+  int32_t* lists_scratch = nullptr;
+  if (gather) {
+    lists.rowptr = reinterpret_cast<int32_t*>(p); p += t_rows;
+    lists.col = reinterpret_cast<int32_t*>(p); p += t_slots;
+    lists.inv = reinterpret_cast<int32_t*>(p); p += t_slots;
+    lists_scratch = reinterpret_cast<int32_t*>(p); p += t_scratch;
+    lists.entry = reinterpret_cast<float2*>(p);
+  }
   XRL_CUDA(cudaMemsetAsync(grad, 0, 4 * ctx->weight_floats, st));
   XRL_CUDA(cudaMemsetAsync(loss_out, 0, 16, st));
   if (b->B == 0 || b->num_envs == 0) return XRL_OK;
@@ -1148,13 +1164,16 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
                         heads_ws, loss_out, dh_a, logp_out, ctx->status.as<int32_t>(), st);
   const int32_t* gat_rowptr = c.neighbourhood ? b->rowptr_nbr.as<int32_t>() : b->rowptr.as<int32_t>();
   const int32_t* gat_col = c.neighbourhood ? b->col_nbr.as<int32_t>() : b->col.as<int32_t>();
+  if (gather && L > 0)
+    n += launch_bwd_lists(gat_rowptr, gat_col, b->N, b->E * (c.neighbourhood ? 2 : 1), lists, lists_scratch, st);
   float* dh_cur = dh_a;
   float* dh_nxt = dh_b;
   for (int l = L - 1; l >= 0 && b->N > 0; --l) {
     const LayerWeights& lw = ctx->dw.layer[l];
     float* ga_src = grad + (lw.a_src - wb);
     const int k = launch_gat_layer_bwd(d, gat_rowptr, gat_col, zs[l], ss[l], hs[l], hs[l + 1], dh_cur,
-                             dh_nxt, dz, ds, dz_store, lw, ga_src - H * H, ga_src, grad + (lw.a_dst - wb),
+                             l == L - 1 || bwd_leaves_masked(d),   // (the readout's reverse masks too)
+                             dh_nxt, dz, ds, dz_store, gather ? &lists : nullptr, lw, ga_src - H * H, ga_src, grad + (lw.a_dst - wb),
                              grad + (lw.b - wb), b->N, ctx->status.as<int32_t>(), st);
     if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
     n += k;

@@ -1,6 +1,7 @@
 """The dense products of the training step's reverse pass at the sizes where their tiles end: widths that are not a
 multiple of the tile, row counts around a chunk and past the line from which whole 128-row tiles are used, and a
-gradient buffer that is not 16-byte aligned."""
+gradient buffer that is not 16-byte aligned; and its lists by producer, on nodes with more readers or producers than a
+warp's list holds."""
 import numpy as np
 import pytest
 
@@ -16,13 +17,37 @@ pytestmark = pytest.mark.gpu
                                              (192, 6, "bf16", 2100), (384, 3, "bf16", 65), (128, 4, "bf16", 129),
                                              (256, 8, "bf16", 1), (512, 8, "bf16", 131)])
 def test_gradient_at_the_edges_of_the_tiles(xo, H, K, dtype, nodes):
-    import torch
-    import paper_2304_14698_b200 as xrl
     m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3)
     rng = dags.make_rng(H + nodes)
     sizes = [nodes, nodes + 3, nodes, 1, nodes + 1]
     graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in sizes]
-    batch = dags.flatten(graphs, [0, 3, 5], 3)
+    _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
+
+
+def _star(rng, m, readers, producers, repeats):
+    """Node 0 is read by `readers` nodes, the last node reads `producers` of them (and node 1 `repeats` times)."""
+    n = readers + 2
+    src = [0] * readers + list(range(1, producers + 1)) + [1] * repeats
+    dst = list(range(1, readers + 1)) + [n - 1] * (producers + repeats)
+    g = dags.random_dag(rng, n, m["T"], 8, m["dtype"] == "bf16")
+    g["edge_src"], g["edge_dst"] = np.array(src, np.int32), np.array(dst, np.int32)
+    return g
+
+
+@pytest.mark.parametrize("H,K,dtype,both", [(128, 2, "fp32", False), (128, 4, "fp32", False), (128, 16, "fp32", True),
+                                            (256, 8, "fp32", False), (128, 8, "bf16", False), (256, 2, "bf16", False),
+                                            (256, 4, "bf16", True), (256, 8, "bf16", False), (256, 16, "bf16", False)])
+def test_gradient_with_long_lists(xo, H, K, dtype, both):
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3, both_ways=both)
+    rng = dags.make_rng(H + K)
+    graphs = [_star(rng, m, *v) for v in ((94, 2, 0), (95, 94, 1), (96, 95, 0), (97, 96, 3), (200, 150, 40))]
+    _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
+
+
+def _compare(xo, batch, m):
+    import torch
+    import paper_2304_14698_b200 as xrl
+    dtype = m["dtype"]
     batch["model"] = m
     blob, _ = gpu_util.default_weights(batch, 7)
     st, packed = xo.pack(batch)
