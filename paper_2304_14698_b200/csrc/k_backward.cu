@@ -17,7 +17,7 @@
 // the smaller one.
 #include <algorithm>
 
-#include "xrl_internal.cuh"
+#include "xrl_agg_tma.cuh"
 
 namespace xrl {
 
@@ -581,97 +581,130 @@ k_embed_inputs(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ c
 }
 
 // ---- Eq. 6, reverse: dW0 += x^T dpre, db0 += dpre, x_i = [edge sum | one-hot op | own shape] -------------
-// A CTA takes a range of rows, R at a time: the tile's masked gradients dpre [R x H], its dense inputs
-// [R x 16] (computed beforehand by k_embed_inputs) and its operator ids come into shared memory with wide
-// coalesced loads, eight requested per thread before the first is used; then a thread owns one column and
-// every P-th row of the tile (P threads share a column): the sixteen dense products accumulate in its
-// registers, the one-hot block in the P-th of P shared-memory copies [T x H] of that part of dW0 (a plain add
-// per row and column: nobody else touches that copy's column; shared-memory atomics cost far more here than
-// the adds themselves).  Registers and the copies go to global memory once per CTA.
-constexpr int kEmbedBwdThreads = 512;
+// A warp owns 64 columns (two per lane) and walks its share of the rows eight at a time: the next eight rows' gradients
+// (256 bytes each), operators and dense inputs (k_embed_inputs; one coalesced 512-byte load) are asked for before the
+// current eight are used, so no barrier and no staging of the gradients stands between memory and the multiplies.  The
+// sixteen dense products accumulate in registers, the one-hot block in the warp's own shared-memory copy [T x 64] of
+// that part of dW0 (a plain add per row and column: nobody else touches the copy; shared-memory float atomics cost far
+// more than the adds).  Bound by issue: 16 packed FMA and as many others per row and 64 columns.  Staging 64-row tiles of all
+// columns for 512 threads between two barriers took 0.94 ms at 990 k rows and hidden 256, this takes 0.45 (1.0 GB: 0.16 ms).
+constexpr int kEmbBwdRows = 8;                     // rows in flight per warp
+struct EmbBwdStage { float x[kEmbBwdRows][2 * kS]; int32_t op[kEmbBwdRows]; };
 template <typename T>
-__global__ void __launch_bounds__(kEmbedBwdThreads)
+__global__ void __launch_bounds__(128)
 k_embed_bwd(const float* __restrict__ xs, const int32_t* __restrict__ op, const T* __restrict__ h0,
-            const float* __restrict__ dh0, float* __restrict__ dW0, float* __restrict__ db0, int N, int H, int Tn,
-            int R, int P) {
-  extern __shared__ float sm_embed[];
-  float* oh = sm_embed;                            // [P][Tn x H]
-  float* dpt = oh + size_t(P) * Tn * H;            // [R x H]
-  float* xt = dpt + size_t(R) * H;                 // [R x 16]
-  int32_t* opt = reinterpret_cast<int32_t*>(xt + size_t(R) * 2 * kS);   // [R]
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int t = tid; t < P * Tn * H; t += nt) oh[t] = 0.f;
-  const int part = tid / H, c = tid - part * H;    // threads beyond P x H only help with the loads
-  float* my_oh = oh + size_t(min(part, P - 1)) * Tn * H;
-  const int rows_per_cta = (N + gridDim.x - 1) / gridDim.x;
-  const int r0 = blockIdx.x * rows_per_cta, r1 = min(N, r0 + rows_per_cta);
-  const int qpr = H >> 2;                          // 16-byte pieces per row
-  const int step_r = nt / qpr, step_q = nt - step_r * qpr;   // what a stride of nt pieces does to (row, piece)
-  float acc[2 * kS], dbr = 0.f;
+            const float* __restrict__ dh0, bool masked, float* __restrict__ dW0, float* __restrict__ db0, int N, int H, int Tn) {
+  extern __shared__ __align__(16) float sm_embed[];
+  const int warps = blockDim.x >> 5, wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  EmbBwdStage& stg = reinterpret_cast<EmbBwdStage*>(sm_embed)[wib];
+  float* oh = sm_embed + warps * (sizeof(EmbBwdStage) / sizeof(float)) + size_t(wib) * Tn * 64;   // [Tn x 64]
+  for (int t = lane; t < Tn * 64; t += 32) oh[t] = 0.f;
+  const int c = blockIdx.y * 64 + 2 * lane;        // H is a multiple of 32: the last group may hold 32 columns only
+  const bool on = c < H;
+  // packed fp32 (two products per instruction): acc[c][t] = inputs 2t, 2t + 1 of column c
+  aggtma::F2 acc[2][kS];
 #pragma unroll
-  for (int s = 0; s < 2 * kS; ++s) acc[s] = 0.f;
-  for (int t0 = r0; t0 < r1; t0 += R) {
-    const int rows = min(R, r1 - t0);
-    __syncthreads();                               // the previous tile has been consumed (and oh is zeroed)
-    constexpr int kBatch = 8;
-    int r = tid / qpr, q = tid - r * qpr;
-    while (r < rows) {
-      float4 g[kBatch];
-      Chunk<T, 4> hc[kBatch];
-      int rr[kBatch], qq[kBatch];
+  for (int t = 0; t < kS; ++t) acc[0][t] = acc[1][t] = aggtma::make_f2(0.f, 0.f);
+  const int64_t step = int64_t(gridDim.x) * warps * kEmbBwdRows;
+  float2 g[kEmbBwdRows], gn[kEmbBwdRows];
+  float4 xn;
+  int32_t on_op = 0;
+  auto fetch = [&](int64_t r0) {
+    const float* p = dh0 + size_t(r0) * H + c;
+    const T* q = h0 + size_t(r0) * H + c;
+    const bool whole = on && r0 + kEmbBwdRows <= N;
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        rr[u] = r; qq[u] = q;
-        if (r < rows) {
-          g[u] = *reinterpret_cast<const float4*>(dh0 + size_t(t0 + r) * H + 4 * q);
-          hc[u] = *reinterpret_cast<const Chunk<T, 4>*>(h0 + size_t(t0 + r) * H + 4 * q);
-        }
-        r += step_r; q += step_q;
-        if (q >= qpr) { q -= qpr; ++r; }
+    for (int u = 0; u < kEmbBwdRows; ++u) {
+      const bool live = whole || (on && r0 + u < N);
+      gn[u] = make_float2(0.f, 0.f);
+      if (live) gn[u] = __ldg(reinterpret_cast<const float2*>(p + u * H));
+      if (!masked && live) {
+        float ho[2];
+        load_chunk<T, 2>(q + u * H, ho);
+        if (!(ho[0] > 0.f)) gn[u].x = 0.f;
+        if (!(ho[1] > 0.f)) gn[u].y = 0.f;
       }
-#pragma unroll
-      for (int u = 0; u < kBatch; ++u)
-        if (rr[u] < rows)
-          *reinterpret_cast<float4*>(dpt + size_t(rr[u]) * H + 4 * qq[u]) =
-              make_float4(to_float(hc[u].v[0]) > 0.f ? g[u].x : 0.f, to_float(hc[u].v[1]) > 0.f ? g[u].y : 0.f,
-                          to_float(hc[u].v[2]) > 0.f ? g[u].z : 0.f, to_float(hc[u].v[3]) > 0.f ? g[u].w : 0.f);
     }
-    for (int idx = tid; idx < rows * 4; idx += nt)
-      reinterpret_cast<float4*>(xt)[idx] = reinterpret_cast<const float4*>(xs + size_t(t0) * 2 * kS)[idx];
-    for (int idx = tid; idx < rows; idx += nt) opt[idx] = min(max(op[t0 + idx], 0), Tn - 1);   // (pack reports bad ids)
-    __syncthreads();
-    if (part < P) {
-      for (int rw = part; rw < rows; rw += P) {
-        const float dp = dpt[size_t(rw) * H + c];
-        if (dp == 0.f) continue;
-        const float4* xr = reinterpret_cast<const float4*>(xt + size_t(rw) * 2 * kS);
+    // lane t: piece t of the eight rows' inputs (four 16-byte pieces per row)
+    xn = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 + (lane >> 2) < N) xn = __ldg(reinterpret_cast<const float4*>(xs + size_t(r0) * 2 * kS) + lane);
+    if (lane < kEmbBwdRows) on_op = r0 + lane < N ? min(max(__ldg(op + r0 + lane), 0), Tn - 1) * 64 : 0;   // (pack reports bad ids)
+  };
+  int64_t r0 = (int64_t(blockIdx.x) * warps + wib) * kEmbBwdRows;
+  if (r0 < N) fetch(r0);
+  for (; r0 < N; r0 += step) {
+    __syncwarp();                                  // the previous eight rows' inputs have been read
+    reinterpret_cast<float4*>(&stg.x[0][0])[lane] = xn;
+    if (lane < kEmbBwdRows) stg.op[lane] = on_op;
+#pragma unroll
+    for (int u = 0; u < kEmbBwdRows; ++u) g[u] = gn[u];
+    __syncwarp();
+    if (r0 + step < N) fetch(r0 + step);
+    // two rows at a time: everything they read from shared memory is asked for before their sums are stored (the
+    // compiler keeps reads behind stores that may alias them); rows past the end hold zeros
+#pragma unroll
+    for (int u = 0; u < kEmbBwdRows; u += 2) {
+      ulonglong2 x[2][4];                          // pairs of inputs as they lie
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        x[0][v] = reinterpret_cast<const ulonglong2*>(stg.x[u])[v];
+        x[1][v] = reinterpret_cast<const ulonglong2*>(stg.x[u + 1])[v];
+      }
+      const int2 o = *reinterpret_cast<const int2*>(&stg.op[u]);
+      float2* p0 = reinterpret_cast<float2*>(oh + o.x) + lane;
+      float2* p1 = reinterpret_cast<float2*>(oh + o.y) + lane;
+      float2 v0 = *p0, v1 = *p1;
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        const aggtma::F2 ga = aggtma::make_f2(g[u + w].x, g[u + w].x), gb = aggtma::make_f2(g[u + w].y, g[u + w].y);
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const float4 x = xr[v];
-          acc[4 * v] = fmaf(x.x, dp, acc[4 * v]);
-          acc[4 * v + 1] = fmaf(x.y, dp, acc[4 * v + 1]);
-          acc[4 * v + 2] = fmaf(x.z, dp, acc[4 * v + 2]);
-          acc[4 * v + 3] = fmaf(x.w, dp, acc[4 * v + 3]);
+          const aggtma::F2 xa{x[w][v].x}, xb{x[w][v].y};
+          aggtma::fma2(acc[0][2 * v], xa, ga); aggtma::fma2(acc[0][2 * v + 1], xb, ga);
+          aggtma::fma2(acc[1][2 * v], xa, gb); aggtma::fma2(acc[1][2 * v + 1], xb, gb);
         }
-        my_oh[size_t(opt[rw]) * H + c] += dp;
-        dbr += dp;
       }
+      v0.x += g[u].x; v0.y += g[u].y;
+      if (o.x == o.y) v1 = v0;
+      v1.x += g[u + 1].x; v1.y += g[u + 1].y;
+      *p0 = v0;
+      *p1 = v1;
     }
   }
-  if (part < P) {
-#pragma unroll
-    for (int s = 0; s < kS; ++s) {
-      if (acc[s] != 0.f) atomicAdd(&dW0[size_t(s) * H + c], acc[s]);
-      if (acc[kS + s] != 0.f) atomicAdd(&dW0[size_t(kS + Tn + s) * H + c], acc[kS + s]);
-    }
-    if (dbr != 0.f) atomicAdd(&db0[c], dbr);
-  }
+  // the CTA's warps share the columns: their registers meet in shared memory, one input at a time, and go to global memory
+  // once per CTA
   __syncthreads();
-  for (int t = tid; t < Tn * H; t += nt) {
-    float v = 0.f;
-    for (int pp = 0; pp < P; ++pp) v += oh[size_t(pp) * Tn * H + t];
-    if (v != 0.f) atomicAdd(&dW0[size_t(kS) * H + t], v);
+  const float* oh0 = sm_embed + warps * (sizeof(EmbBwdStage) / sizeof(float));
+  float* red = sm_embed + warps * (sizeof(EmbBwdStage) / sizeof(float)) + size_t(warps) * Tn * 64;  // [warps][64]
+  const int cc = blockIdx.y * 64 + int(threadIdx.x & 63);
+#pragma unroll
+  for (int s = 0; s < 2 * kS; ++s) {
+    float lo, hi, v[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      aggtma::split_f2(acc[e][s >> 1], lo, hi);
+      v[e] = s & 1 ? hi : lo;
+    }
+    reinterpret_cast<float2*>(red + wib * 64)[lane] = make_float2(v[0], v[1]);
+    __syncthreads();
+    for (int k = threadIdx.x; k < 64; k += blockDim.x) {
+      float t = 0.f;
+      for (int w = 0; w < warps; ++w) t += red[w * 64 + k];
+      const int col = blockIdx.y * 64 + k;
+      if (col < H && t != 0.f) atomicAdd(dW0 + size_t(s < kS ? s : kS + Tn + (s - kS)) * H + col, t);
+    }
+    __syncthreads();
   }
+  // the one-hot block; every row has one operator, so the block's columns sum to the bias gradient
+  float bias = 0.f;
+  for (int t = threadIdx.x; t < Tn * 64; t += blockDim.x) {       // (a thread keeps one column: blockDim is 64 or 128)
+    float v = 0.f;
+    for (int w = 0; w < warps; ++w) v += oh0[size_t(w) * Tn * 64 + t];
+    const int col = blockIdx.y * 64 + (t & 63);
+    if (col < H && v != 0.f) atomicAdd(&dW0[size_t(kS + (t >> 6)) * H + col], v);
+    bias += v;
+  }
+  if (cc < H && bias != 0.f) atomicAdd(&db0[cc], bias);
 }
 
 // ---- the heads' MLPs: Linear(in, hid), ReLU, [Linear(hid, hid2), ReLU,] Linear(last, 1) ---------------------
@@ -1237,34 +1270,24 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   return 4;
 }
 
-// Eq. 6 in reverse keeps P copies of the one-hot block of W0's gradient ([T x H]) and a tile of R rows in shared
-// memory: as many copies as threads share a column (at most 4), then the largest tile that still fits
-static size_t embed_bwd_bytes(const Dims& d, int R, int P) {
-  return sizeof(float) * (size_t(P) * d.T * d.H + size_t(R) * d.H + size_t(R) * 2 * kS) + sizeof(int32_t) * R;
-}
-static void embed_bwd_shape(const Dims& d, int* R, int* P) {
-  constexpr size_t kCeiling = size_t(227) * 1024;
-  *R = 0; *P = 1;
-  for (int p = std::min(4, std::max(1, kEmbedBwdThreads / d.H)); p >= 1; --p)
-    for (int r = 64; r >= 16; r >>= 1)
-      if (embed_bwd_bytes(d, r, p) <= kCeiling) { *R = r; *P = p; return; }
-  if (embed_bwd_bytes(d, 8, 1) <= kCeiling) *R = 8;
-}
+// The model shapes Eq. 6's reverse takes: a copy of the one-hot block of W0's gradient ([T x H]) and eight rows of all
+// columns within one SM's shared memory (the kernel itself keeps 64 columns of it per warp).
 size_t embed_bwd_smem_bytes(const Dims& d) {
-  int R, P;
-  embed_bwd_shape(d, &R, &P);
-  return embed_bwd_bytes(d, std::max(R, 8), P);
+  return sizeof(float) * (size_t(d.T) * d.H + 8 * size_t(d.H) + 8 * 2 * kS) + sizeof(int32_t) * 8;
 }
 
 int launch_embed_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, const int32_t* op, const void* shape,
-                     const void* eattr, const void* h0, const float* dh0, float* xs, float* gW0, float* gb0, int32_t N,
-                     cudaStream_t st) {
+                     const void* eattr, const void* h0, const float* dh0, bool masked, float* xs, float* gW0, float* gb0,
+                     int32_t N, cudaStream_t st) {
   if (N <= 0) return 0;
-  int R, P;
-  embed_bwd_shape(d, &R, &P);
-  if (R == 0) return -1;
-  const size_t smem = embed_bwd_bytes(d, R, P);
-  const int grid = int(std::min<int64_t>((int64_t(N) + R - 1) / R, int64_t(kNumSMs)));
+  // four warps per CTA, two where their copies would not fit (T <= 256: two always do); CTAs for every SM's shared memory (at most 16 warps' worth)
+  const size_t per_warp = sizeof(EmbBwdStage) + sizeof(float) * (size_t(d.T) * 64 + 64), room = size_t(220) * 1024;
+  const int warps = 4 * per_warp <= room ? 4 : 2;
+  const size_t smem = warps * per_warp;
+  const int groups = (d.H + 63) / 64;
+  const int per_sm = int(std::max<size_t>(1, std::min<size_t>(16 / warps, room / (smem + 1024))));
+  const int64_t want = (int64_t(N) + warps * kEmbBwdRows - 1) / (warps * kEmbBwdRows);
+  const dim3 grid(unsigned(std::min<int64_t>(want, std::max(1, kNumSMs * per_sm / groups))), unsigned(groups));
   const unsigned grid_x = unsigned((int64_t(N) + 255) / 256);
   // the opt-in is the kernel's ceiling for every later launch: ask for all an SM has, once per device
   constexpr int kSmemCeiling = 227 * 1024;
@@ -1273,15 +1296,13 @@ int launch_embed_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, c
     if (!ensure_dynamic_smem(k_embed_bwd<bf16>, kSmemCeiling, attr)) return -1;
     k_embed_inputs<bf16><<<grid_x, 256, 0, st>>>(rowptr, col, static_cast<const bf16*>(shape),
                                                  static_cast<const bf16*>(eattr), xs, N);
-    k_embed_bwd<bf16><<<grid, kEmbedBwdThreads, smem, st>>>(xs, op, static_cast<const bf16*>(h0), dh0, gW0, gb0, N,
-                                                            d.H, d.T, R, P);
+    k_embed_bwd<bf16><<<grid, 32 * warps, smem, st>>>(xs, op, static_cast<const bf16*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
   } else {
     static bool attr[64] = {};
     if (!ensure_dynamic_smem(k_embed_bwd<float>, kSmemCeiling, attr)) return -1;
     k_embed_inputs<float><<<grid_x, 256, 0, st>>>(rowptr, col, static_cast<const float*>(shape),
                                                   static_cast<const float*>(eattr), xs, N);
-    k_embed_bwd<float><<<grid, kEmbedBwdThreads, smem, st>>>(xs, op, static_cast<const float*>(h0), dh0, gW0, gb0, N,
-                                                             d.H, d.T, R, P);
+    k_embed_bwd<float><<<grid, 32 * warps, smem, st>>>(xs, op, static_cast<const float*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
   }
   return 2;
 }
