@@ -2,70 +2,17 @@
 // invalid-action masking and No-Op (Sections 3.3.2, 3.3.3), and the categorical draw.
 // Every reduction runs in a fixed order (no floating-point atomics), so results are
 // reproducible run to run.
-#include "xrl_internal.cuh"
+#include <algorithm>
+
+#include "xrl_heads.cuh"
 
 namespace xrl {
+
+using namespace heads;
 
 namespace {
 
 constexpr int kRoThreads = 256;
-
-// sum_k x[k] * W[k * ld + c]: the weight loads are issued DEPTH (then eight) at a time so that their
-// latencies overlap; the additions keep the order k = 0, 1, 2, ...  DEPTH = 32 is for launches of few
-// CTAs, which are bound by the latency of these loads; with many CTAs per SM the registers it takes cost
-// more occupancy than the depth gains, and DEPTH = 8 is used.
-template <int DEPTH>
-__device__ __forceinline__ float column_dot(const float* x, int in, const float* __restrict__ W, int ld,
-                                            int c, float acc) {
-  int k = 0;
-  if (DEPTH > 8) {
-    for (; k + DEPTH <= in; k += DEPTH) {
-      float w[DEPTH];
-#pragma unroll
-      for (int t = 0; t < DEPTH; ++t) w[t] = __ldg(W + size_t(k + t) * ld + c);
-#pragma unroll
-      for (int t = 0; t < DEPTH; ++t) acc = fmaf(x[k + t], w[t], acc);
-    }
-  }
-  for (; k + 8 <= in; k += 8) {
-    float w[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) w[t] = __ldg(W + size_t(k + t) * ld + c);
-#pragma unroll
-    for (int t = 0; t < 8; ++t) acc = fmaf(x[k + t], w[t], acc);
-  }
-  for (; k < in; ++k) acc = fmaf(x[k], __ldg(W + size_t(k) * ld + c), acc);
-  return acc;
-}
-
-// y[c] = bias[c] + sum_k x[k] W[k * ld + c] for c < ncols, for every thread block shape: with fewer columns
-// than threads the k range is cut into P = blockDim / CP contiguous parts (CP = columns per pass, a power of
-// two), the parts are computed by different thread groups and added in part order.  Every thread of the
-// block calls it; `part` is blockDim floats of scratch; emit(c, y) runs once per column.
-template <int DEPTH, typename Emit>
-__device__ __forceinline__ void dense_columns(const float* x, int in, const float* __restrict__ W, int ld,
-                                              int ncols, const float* __restrict__ bias, float* part, Emit emit) {
-  const int nt = blockDim.x, tid = threadIdx.x;
-  int CP = 32;
-  while (CP < ncols && CP < nt) CP <<= 1;
-  const int P = nt / CP, cl = tid % CP, p = tid / CP;
-  if (P == 1) {                                  // as many columns as threads (or more): no split, no barriers
-    for (int c = tid; c < ncols; c += nt) emit(c, column_dot<DEPTH>(x, in, W, ld, c, bias[c]));
-    return;
-  }
-  const int k0 = int((int64_t(in) * p) / P), k1 = int((int64_t(in) * (p + 1)) / P);
-  for (int c0 = 0; c0 < ncols; c0 += CP) {
-    const int c = c0 + cl;
-    part[tid] = (c < ncols) ? column_dot<DEPTH>(x + k0, k1 - k0, W + size_t(k0) * ld, ld, c, 0.f) : 0.f;
-    __syncthreads();
-    if (p == 0 && c < ncols) {
-      float y = bias[c];
-      for (int q = 0; q < P; ++q) y += part[q * CP + cl];
-      emit(c, y);
-    }
-    __syncthreads();
-  }
-}
 
 // ---- readout, stage 1: column sums of one chunk of consecutive rows of one graph -------------
 template <typename T>
@@ -112,231 +59,148 @@ k_readout(const T* __restrict__ h, const int32_t* __restrict__ chunk_row0,
   }
 }
 
-// ---- Eq. 8: emb_g = ReLU(Wg^T [ sum of the graph's chunk sums | g0_g ] + bg) -------------------
-template <int DEPTH>
-__global__ void __launch_bounds__(1024)
-k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ graph_chunk_off,
-                const float* __restrict__ g0, const float* __restrict__ Wg,
-                const float* __restrict__ bg, float* __restrict__ emb, int H, int Dg) {
-  extern __shared__ float u[];                   // [H + Dg], then blockDim floats of scratch
-  float* part = u + H + Dg;
-  const int32_t g = blockIdx.x;
-  const int32_t c0 = graph_chunk_off[g], c1 = graph_chunk_off[g + 1];
-  for (int c = threadIdx.x; c < H; c += blockDim.x) {
-    float s = 0.f;
-    for (int32_t ch = c0; ch < c1; ++ch) s += partial[size_t(ch) * H + c];
-    u[c] = s;
-  }
-  for (int t = threadIdx.x; t < Dg; t += blockDim.x) u[H + t] = g0 ? g0[size_t(g) * Dg + t] : 0.f;
-  __syncthreads();
-  dense_columns<DEPTH>(u, H + Dg, Wg, H, H, bg, part,
-                [&](int c, float y) { emb[size_t(g) * H + c] = fmaxf(y, 0.f); });
-}
-
-// Eq. 8 from the partial sums written by the aggregate kernel fused with the readout: per graph, the
-// partial of the block in which the graph starts (if it does not start at the block's first row), then
-// the partials of the following 32-row blocks whose first row belongs to the graph, in order.
-template <int DEPTH>
-__global__ void __launch_bounds__(1024)
-k_global_update_blocks(const float* __restrict__ partial, const int32_t* __restrict__ node_off,
-                       int32_t nblocks, int bshift, const float* __restrict__ g0, const float* __restrict__ Wg,
-                       const float* __restrict__ bg, float* __restrict__ emb, int H, int Dg) {
-  extern __shared__ __align__(16) float u[];     // [H + Dg], then (16-byte aligned) 4 blockDim floats of scratch
-  float* part = u + ((H + Dg + 3) & ~3);
-  const int32_t g = blockIdx.x;
-  const int32_t start = node_off[g], end = node_off[g + 1];
-  // With more threads than columns the blocks' partial sums are added in P interleaved parts (part p takes the
-  // blocks b0 + p, b0 + p + P, ...), and the parts in order: a fixed order for a given launch shape.
-  const int P = int(blockDim.x) >= 2 * H ? int(blockDim.x) / H : 1;
-  if (P > 1 && (H & 3) == 0) {
-    // four columns per thread (16-byte loads) and 4 P interleaved parts: with 1,024 threads and H = 256 a thread
-    // adds every 16th block, so that a graph of 70 blocks costs one round of loads instead of five
-    const int HV = H >> 2, PV = int(blockDim.x) / HV;
-    const int cv = threadIdx.x % HV, p = threadIdx.x / HV;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    int32_t b0 = 0, b1 = -1;
-    if (end > start) {
-      b0 = start >> bshift;
-      if (start & ((1 << bshift) - 1)) ++b0;
-      b1 = (end - 1) >> bshift;
-    }
-    if (p < PV)
-      for (int32_t b = b0 + p; b <= b1; b += PV) {
-        const float4 v = *reinterpret_cast<const float4*>(partial + size_t(b) * H + 4 * cv);
-        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-      }
-    if (p < PV) *reinterpret_cast<float4*>(part + size_t(p) * H + 4 * cv) = s;
-    __syncthreads();
-    if (int(threadIdx.x) < H) {
-      const int c = threadIdx.x;
-      float t = (end > start && (start & ((1 << bshift) - 1))) ? partial[size_t(nblocks + g) * H + c] : 0.f;
-      for (int q = 0; q < PV; ++q) t += part[q * H + c];
-      u[c] = t;
-    }
-  } else if (P == 1) {
-    for (int c = threadIdx.x; c < H; c += blockDim.x) {
-      float s = 0.f;
+// ---- Eq. 8: emb_g = ReLU(Wg^T [ sum of the graph's partial sums | g0_g ] + bg), GP graphs per CTA -------------------
+// Where a graph's partial sums lie: BLOCKS = false: rows off[g] .. off[g + 1] - 1 of `partial` (readout chunks).
+// BLOCKS = true, after the aggregate kernel fused with the readout: off = node offsets; the partial of the block in which
+// the graph starts (if it does not start at the block's first row), then the partials of the following blocks whose first
+// row belongs to the graph.  The rows are added in P interleaved parts, four columns per thread, and the parts in order: a
+// fixed order for a given launch shape.  U_out (optional): the sums with g0 behind them, [B x (H + Dg)].
+template <int GP, bool BLOCKS>
+__global__ void __launch_bounds__(kThreads)
+k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ off, int32_t nblocks, int bshift,
+                const float* __restrict__ g0, const float* __restrict__ Wg, const float* __restrict__ bg,
+                float* __restrict__ emb, float* __restrict__ U_out, int H, int Dg, int B) {
+  extern __shared__ __align__(16) float u[];     // [GP][xs], then scratch
+  const int xs = row_stride(H + Dg), nt = blockDim.x, tid = threadIdx.x;
+  float* part = u + GP * xs;
+  const int32_t first = blockIdx.x * GP;
+  const int HV = H >> 2, NG = nt / HV, P = NG >= GP ? NG / GP : 1;
+  const int cv = tid % HV, grp = tid / HV;
+  auto range = [&](int32_t g, int32_t& b0, int32_t& b1) {         // rows b0 .. b1 of `partial`
+    const int32_t start = off[g], end = off[g + 1];
+    if (BLOCKS) {
+      b0 = 0; b1 = -1;
       if (end > start) {
-        int32_t b0 = start >> bshift;
-        if (start & ((1 << bshift) - 1)) { s += partial[size_t(nblocks + g) * H + c]; ++b0; }
-        const int32_t b1 = (end - 1) >> bshift;
-        for (int32_t b = b0; b <= b1; ++b) s += partial[size_t(b) * H + c];
+        b0 = start >> bshift;
+        if (start & ((1 << bshift) - 1)) ++b0;
+        b1 = (end - 1) >> bshift;
       }
-      u[c] = s;
+    } else {
+      b0 = start; b1 = end - 1;
     }
-  } else {
-    const int c = threadIdx.x % H, p = threadIdx.x / H;
-    float s = 0.f;
-    int32_t b0 = 0, b1 = -1;
-    if (end > start) {
-      b0 = start >> bshift;
-      if (start & ((1 << bshift) - 1)) ++b0;
-      b1 = (end - 1) >> bshift;
+  };
+  if (grp < NG)
+    for (int t = grp; t < GP * P; t += NG) {
+      const int gl = t / P, p = t - gl * P;
+      if (first + gl >= B) break;
+      int32_t b0, b1;
+      range(first + gl, b0, b1);
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int32_t b = b0 + p; b <= b1; b += 8 * P) {
+        float4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (b + q * P <= b1) v[q] = *reinterpret_cast<const float4*>(partial + size_t(b + q * P) * H + 4 * cv);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { s.x += v[q].x; s.y += v[q].y; s.z += v[q].z; s.w += v[q].w; }
+      }
+      *reinterpret_cast<float4*>(part + size_t(t) * H + 4 * cv) = s;
     }
-    if (p < P)
-      for (int32_t b = b0 + p; b <= b1; b += P) s += partial[size_t(b) * H + c];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (p == 0) {
-      float t = (end > start && (start & ((1 << bshift) - 1))) ? partial[size_t(nblocks + g) * H + c] : 0.f;
-      for (int q = 0; q < P; ++q) t += part[q * H + c];
-      u[c] = t;
+  __syncthreads();
+  for (int i = tid; i < GP * xs; i += nt) {
+    const int gl = i / xs, c = i - gl * xs;
+    const int32_t g = first + gl;
+    float v = 0.f;
+    if (g < B && c < H) {
+      if (BLOCKS) {
+        const int32_t start = off[g];
+        if (off[g + 1] > start && (start & ((1 << bshift) - 1))) v = partial[size_t(nblocks + g) * H + c];
+      }
+      for (int q = 0; q < P; ++q) v += part[size_t(gl * P + q) * H + c];
+    } else if (g < B && c < H + Dg) {
+      v = g0 ? g0[size_t(g) * Dg + (c - H)] : 0.f;
     }
+    u[i] = v;
+    if (U_out != nullptr && g < B && c < H + Dg) U_out[size_t(g) * (H + Dg) + c] = v;
   }
-  for (int t = threadIdx.x; t < Dg; t += blockDim.x) u[H + t] = g0 ? g0[size_t(g) * Dg + t] : 0.f;
   __syncthreads();
-  dense_columns<DEPTH>(u, H + Dg, Wg, H, H, bg, part,
-                [&](int c, float y) { emb[size_t(g) * H + c] = fmaxf(y, 0.f); });
+  dense_rows<GP>(u, xs, H + Dg, Wg, H, H, bg, part, [&](int g, int c, float y) {
+    if (first + g < B) emb[size_t(first + g) * H + c] = fmaxf(y, 0.f);
+  });
 }
 
-// Block-wide sum in a fixed order (lanes of a warp by a shuffle tree, then the warps' sums by one warp's
-// shuffle tree): the same for the same blockDim, two barriers.  Every thread contributes v and gets the sum;
-// `scratch` holds at least 32 floats.  blockDim is a multiple of 32.
-__device__ float block_sum(float v, float* scratch) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  float r = lane < nw ? scratch[lane] : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
-  __syncthreads();
-  return r;
-}
-__device__ float block_max(float v, float* scratch) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-  if (lane == 0) scratch[wid] = v;
-  __syncthreads();
-  float r = lane < nw ? scratch[lane] : -INFINITY;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xFFFFFFFFu, r, o));
-  __syncthreads();
-  return r;
-}
-
-// A head's MLP (Section 3.3.2): out = w2 . ReLU(W1^T x + b1) + b2, or with a second hidden width hid2 > 0
-// out = w2 . ReLU(Wh^T ReLU(W1^T x + b1) + bh) + b2.  x (length `in`) and y1 (hid floats, used only when
-// hid2 > 0) are in shared memory; all threads return the result.
-struct Mlp { const float *W1, *b1, *Wh, *bh, *w2, *b2; int hid, hid2; };
-template <int DEPTH>
-__device__ float mlp_scalar(const float* x, int in, const Mlp& m, float* y1, float* scratch) {
-  float contrib = 0.f;
-  if (m.hid2 <= 0) {
-    dense_columns<DEPTH>(x, in, m.W1, m.hid, m.hid, m.b1, scratch, [&](int c, float y) { contrib += fmaxf(y, 0.f) * m.w2[c]; });
-  } else {
-    dense_columns<DEPTH>(x, in, m.W1, m.hid, m.hid, m.b1, scratch, [&](int c, float y) { y1[c] = fmaxf(y, 0.f); });
-    __syncthreads();
-    dense_columns<DEPTH>(y1, m.hid, m.Wh, m.hid2, m.hid2, m.bh, scratch,
-                  [&](int c, float y) { contrib += fmaxf(y, 0.f) * m.w2[c]; });
-  }
-  return block_sum(contrib, scratch) + m.b2[0];
-}
-
-// ---- policy MLP: one scalar score per graph -----------------------------------------------------
-template <int DEPTH>
-__global__ void __launch_bounds__(1024)
-k_policy_logit(const float* __restrict__ emb, const Mlp mlp, float* __restrict__ logit, int H) {
-  extern __shared__ float sm[];                  // [H] + [blockDim] + [hid]
-  float* x = sm;
-  float* scratch = sm + H;
-  float* y1 = scratch + blockDim.x;
-  const int32_t g = blockIdx.x;
-  for (int c = threadIdx.x; c < H; c += blockDim.x) x[c] = emb[size_t(g) * H + c];
-  __syncthreads();
-  const float v = mlp_scalar<DEPTH>(x, H, mlp, y1, scratch);
-  if (threadIdx.x == 0) logit[g] = v;
-}
-
-// The rest of a head's MLP behind its first layer: y1 = ReLU(W1^T x + b1) is given (hid floats in shared
-// memory); all threads return the result.
-template <int DEPTH>
+// The rest of a head's MLP behind its first layer: y1 = ReLU(W1^T x + b1) is given (hid floats in shared memory, on a
+// 16-byte boundary; y2: hid2 floats); all threads return the result.
 __device__ float mlp_tail(const float* y1, const Mlp& m, float* scratch) {
   float contrib = 0.f;
   if (m.hid2 <= 0) {
     for (int c = threadIdx.x; c < m.hid; c += blockDim.x) contrib += y1[c] * m.w2[c];
   } else {
-    dense_columns<DEPTH>(y1, m.hid, m.Wh, m.hid2, m.hid2, m.bh, scratch,
-                  [&](int c, float y) { contrib += fmaxf(y, 0.f) * m.w2[c]; });
+    dense_rows<1>(y1, 0, m.hid, m.Wh, m.hid2, m.hid2, m.bh, scratch,
+                  [&](int, int c, float y) { contrib += fmaxf(y, 0.f) * m.w2[c]; });
   }
   return block_sum(contrib, scratch) + m.b2[0];
 }
 
-// ---- steps of few graphs and environments: policy scores and the value head's first layer in one launch ------
-// CTAs [0, B) are k_policy_logit.  CTAs B + e * VC + ch compute chunk ch (hid / VC columns) of the value head's
-// first layer for environment e: y1[e] = ReLU(W1^T [emb(current) | mean of the valid candidates' emb] + b1), the
-// candidate mean taken inside the CTA (part p of the threads adds candidates p, p + P, ... in order, the parts
-// in order).  The 2H x hid weights are then read by VC CTAs instead of by the one CTA of the environment.
-template <int DEPTH>
-__global__ void __launch_bounds__(1024)
+// ---- policy scores of all graphs and the value head's first layer, in one launch ----------------------------------
+// CTAs [0, policy_ctas): policy MLP of GP graphs each, one scalar per graph.  y1_out / y2_out (optional): its hidden
+// activations.  CTAs policy_ctas + e * VC + ch compute chunk ch (hid / VC columns) of the value head's first layer for
+// environment e, y1v[e] = ReLU(W1^T [emb(current) | mean of the valid candidates' emb] + b1), the candidate mean taken
+// inside the CTA: the 2H x hid weights are then read by VC CTAs instead of by the one CTA of the environment.
+template <int GP>
+__global__ void __launch_bounds__(kThreads)
 k_policy_value_hidden(const float* __restrict__ emb, const Mlp pm, float* __restrict__ logit, int H, int32_t B,
+                      int policy_ctas, float* __restrict__ y1_out, float* __restrict__ y2_out,
                       const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask, int A, const Mlp vm,
                       float* __restrict__ y1v, int VC) {
-  extern __shared__ float sm[];                  // policy: [H] + [blockDim] + [hid]; value: [2H] + [blockDim]
+  extern __shared__ __align__(16) float sm[];
   const int nt = blockDim.x, tid = threadIdx.x;
-  if (int32_t(blockIdx.x) < B) {
-    float* x = sm;
-    float* scratch = sm + H;
-    float* y1 = scratch + nt;
-    const int32_t g = blockIdx.x;
-    for (int c = tid; c < H; c += nt) x[c] = emb[size_t(g) * H + c];
+  if (int(blockIdx.x) < policy_ctas) {
+    const int xs = row_stride(H), ys = row_stride(pm.hid), zs = row_stride(pm.hid2);
+    float* x = sm;                               // [GP][xs]
+    float* y1 = x + GP * xs;                     // [GP][ys]
+    float* y2 = y1 + GP * ys;                    // [GP][zs]
+    float* part = y2 + GP * zs;                  // [GP * nt]
+    const int32_t first = blockIdx.x * GP;
+    for (int i = tid; i < GP * xs; i += nt) {
+      const int g = i / xs, c = i - g * xs;
+      x[i] = first + g < B && c < H ? emb[size_t(first + g) * H + c] : 0.f;
+    }
     __syncthreads();
-    const float v = mlp_scalar<DEPTH>(x, H, pm, y1, scratch);
-    if (tid == 0) logit[g] = v;
+    dense_rows<GP>(x, xs, H, pm.W1, pm.hid, pm.hid, pm.b1, part, [&](int g, int c, float y) {
+      y1[g * ys + c] = fmaxf(y, 0.f);
+      if (y1_out != nullptr && first + g < B) y1_out[size_t(first + g) * pm.hid + c] = fmaxf(y, 0.f);
+    });
+    const float* last = y1;
+    int ls = ys, width = pm.hid;
+    if (pm.hid2 > 0) {
+      dense_rows<GP>(y1, ys, pm.hid, pm.Wh, pm.hid2, pm.hid2, pm.bh, part, [&](int g, int c, float y) {
+        y2[g * zs + c] = fmaxf(y, 0.f);
+        if (y2_out != nullptr && first + g < B) y2_out[size_t(first + g) * pm.hid2 + c] = fmaxf(y, 0.f);
+      });
+      last = y2; ls = zs; width = pm.hid2;
+    }
+    const int lane = tid & 31, warp = tid >> 5;  // a warp per graph
+    if (warp < GP && first + warp < B) {
+      float v = 0.f;
+      for (int c = lane; c < width; c += 32) v = fmaf(last[warp * ls + c], pm.w2[c], v);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if (lane == 0) logit[first + warp] = v + pm.b2[0];
+    }
     return;
   }
   float* u = sm;                                 // [2H]
-  float* scratch = sm + 2 * H;                   // [blockDim]
-  const int32_t e = (int32_t(blockIdx.x) - B) / VC, ch = (int32_t(blockIdx.x) - B) % VC;
+  float* scratch = sm + 2 * H;                   // [4 blockDim]
+  const int32_t e = (int32_t(blockIdx.x) - policy_ctas) / VC, ch = (int32_t(blockIdx.x) - policy_ctas) % VC;
   const int32_t cur = env_off[e];
-  const int32_t C = env_off[e + 1] - cur - 1;
-  const uint8_t* mk = mask + size_t(e) * A;
-  float cnt = 0.f;
-  for (int a = tid; a < C && a < A; a += nt) cnt += mk[a] ? 1.f : 0.f;
-  const float nv = block_sum(cnt, scratch);
-  const int P = nt >= 2 * H ? nt / H : 1;
-  {
-    const int c = tid % H, p = tid / H;
-    float s = 0.f;
-    if (p < P && tid < P * H)
-      for (int a = p; a < C && a < A; a += P)
-        if (mk[a]) s += emb[size_t(cur + 1 + a) * H + c];
-    scratch[tid] = s;
-    __syncthreads();
-    if (tid < H) {
-      float t = 0.f;
-      for (int q = 0; q < P; ++q) t += scratch[q * H + tid];
-      u[tid] = emb[size_t(cur) * H + tid];
-      u[H + tid] = nv > 0.f ? t / nv : 0.f;
-    }
-    __syncthreads();
-  }
+  value_input(emb, cur, env_off[e + 1] - cur - 1, mask + size_t(e) * A, A, H, u, scratch);
   const int CW = (vm.hid + VC - 1) / VC, c_lo = ch * CW, ncols = min(CW, vm.hid - c_lo);
   if (ncols > 0)
-    dense_columns<DEPTH>(u, 2 * H, vm.W1 + c_lo, vm.hid, ncols, vm.b1 + c_lo, scratch,
-                  [&](int c, float y) { y1v[size_t(e) * vm.hid + c_lo + c] = fmaxf(y, 0.f); });
+    dense_rows<1>(u, 0, 2 * H, vm.W1 + c_lo, vm.hid, ncols, vm.b1 + c_lo, scratch,
+                  [&](int, int c, float y) { y1v[size_t(e) * vm.hid + c_lo + c] = fmaxf(y, 0.f); });
 }
 
 // ---- Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11) -----------------------------------------
@@ -415,87 +279,69 @@ __device__ int32_t sample_row(const float* __restrict__ p, int A1, uint64_t seed
   return act;
 }
 
-// ---- sum of the valid candidates' embeddings of one environment, 32 columns per CTA ---------------
-// 1024 threads = 32 columns x 32 parts; part p adds candidates p, p + 32, ... in order, the parts are
-// then added in order: a fixed summation order, so the result is reproducible.
+// ---- per environment: masked softmax, the value MLP behind its first layer, optional draw ----------------------------
+// A thread keeps its entries' scores in registers up to kKeep per thread; the rest is read again.
+constexpr int kKeep = 2;
 __global__ void __launch_bounds__(1024)
-k_candidate_sum(const float* __restrict__ emb, const int32_t* __restrict__ env_off,
-                const uint8_t* __restrict__ mask, float* __restrict__ cand_sum, int H, int A) {
-  __shared__ float part[32][33];
-  const int32_t e = blockIdx.x;
-  const int c = blockIdx.y * 32 + (threadIdx.x & 31), p = threadIdx.x >> 5;
-  const int32_t cur = env_off[e];
-  const int32_t C = env_off[e + 1] - cur - 1;
-  const uint8_t* mk = mask + size_t(e) * A;
-  float s = 0.f;
-  if (c < H)
-    for (int a = p; a < C; a += 32)
-      if (mk[a]) s += emb[size_t(cur + 1 + a) * H + c];
-  part[p][threadIdx.x & 31] = s;
-  __syncthreads();
-  if (p == 0 && c < H) {
-    float t = 0.f;
-    for (int q = 0; q < 32; ++q) t += part[q][threadIdx.x & 31];
-    cand_sum[size_t(e) * H + c] = t;
-  }
-}
-
-// ---- per environment: masked softmax, candidate mean, value MLP, optional draw -----------------
-template <int DEPTH>
-__global__ void __launch_bounds__(1024)
-k_env_policy(const float* __restrict__ emb, const float* __restrict__ logit,
-             const float* __restrict__ cand_sum,
-             const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask,
-             const Mlp vmlp, float* __restrict__ probs,
-             float* __restrict__ value, int32_t* __restrict__ action, int H, int A,
-             uint64_t seed, uint64_t step, int32_t* status, const float* __restrict__ y1_pre) {
-  extern __shared__ unsigned long long sm64[];   // [nt + 1] u64, then floats
+k_env_policy(const float* __restrict__ logit, const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask,
+             const Mlp vmlp, float* __restrict__ probs, float* __restrict__ value, int32_t* __restrict__ action, int A,
+             uint64_t seed, uint64_t step, int32_t* status, const float* __restrict__ y1v) {
+  extern __shared__ __align__(16) unsigned long long sm64[];   // [nt + 2] u64, then floats
   const int nt = blockDim.x, tid = threadIdx.x;
-  float* scratch = reinterpret_cast<float*>(sm64 + nt + 1);   // [nt]
-  float* u = scratch + nt;                                    // [2H]
-  float* y1 = u + 2 * H;                                      // [hid]
+  float* scratch = reinterpret_cast<float*>(sm64 + nt + 2);   // [nt]
+  float* y1 = scratch + nt;                                   // [hid]
   const int32_t e = blockIdx.x;
   const int32_t cur = env_off[e];
   const int32_t C = env_off[e + 1] - cur - 1;
   const uint8_t* mk = mask + size_t(e) * A;
   float* pr = probs + size_t(e) * (A + 1);
+  // the value head's first layer is asked for before the softmax needs its barriers
+  for (int c = tid; c < vmlp.hid; c += nt) y1[c] = __ldg(y1v + size_t(e) * vmlp.hid + c);
 
   // masked softmax over the valid candidates and No-Op (index A, scored by the current graph)
+  auto score = [&](int a) -> float {             // -inf: excluded
+    if (a == A) return logit[cur];
+    return a < C && mk[a] ? logit[cur + 1 + a] : -INFINITY;
+  };
+  float kept[kKeep];
   float mx = -INFINITY;
-  for (int a = tid; a <= A; a += nt) {
-    bool valid = (a == A);
-    if (a < A && mk[a]) {
-      if (a >= C) raise(status, XRL_ERR_INVALID_ARG); else valid = true;
+#pragma unroll
+  for (int t = 0; t < kKeep; ++t) {
+    const int a = tid + t * nt;
+    kept[t] = -INFINITY;
+    if (a <= A) {
+      if (a < A && a >= C && mk[a]) raise(status, XRL_ERR_INVALID_ARG);
+      kept[t] = score(a);
+      mx = fmaxf(mx, kept[t]);
     }
-    if (valid) mx = fmaxf(mx, logit[a == A ? cur : cur + 1 + a]);
+  }
+  for (int a = tid + kKeep * nt; a <= A; a += nt) {
+    if (a < A && a >= C && mk[a]) raise(status, XRL_ERR_INVALID_ARG);
+    mx = fmaxf(mx, score(a));
   }
   mx = block_max(mx, scratch);
   float se = 0.f;
-  for (int a = tid; a <= A; a += nt) {
+  bool drop[kKeep];                              // an excluded entry is exactly 0 whatever the maximum is
+#pragma unroll
+  for (int t = 0; t < kKeep; ++t) {
+    const int a = tid + t * nt;
+    drop[t] = a > A || (a < A && !(a < C && mk[a]));
+    kept[t] = drop[t] ? 0.f : expf(kept[t] - mx);
+    se += kept[t];
+  }
+  for (int a = tid + kKeep * nt; a <= A; a += nt) {
     const bool valid = (a == A) || (a < C && mk[a]);
-    const float ex = valid ? expf(logit[a == A ? cur : cur + 1 + a] - mx) : 0.f;
+    const float ex = valid ? expf(score(a) - mx) : 0.f;
     pr[a] = ex;
     se += ex;
   }
   const float denom = block_sum(se, scratch);
-  for (int a = tid; a <= A; a += nt) pr[a] = pr[a] / denom;     // each thread rewrites its own entries
+#pragma unroll
+  for (int t = 0; t < kKeep; ++t)
+    if (tid + t * nt <= A) pr[tid + t * nt] = kept[t] / denom;
+  for (int a = tid + kKeep * nt; a <= A; a += nt) pr[a] = pr[a] / denom;     // each thread rewrites its own entries
 
-  float v;
-  if (y1_pre != nullptr) {
-    // the value head's first layer was computed by k_policy_value_hidden: the rest of the MLP
-    for (int c = tid; c < vmlp.hid; c += nt) y1[c] = y1_pre[size_t(e) * vmlp.hid + c];
-    __syncthreads();
-    v = mlp_tail<DEPTH>(y1, vmlp, scratch);
-  } else {
-    // value head input: [ emb(current) | mean of emb over the valid candidates ]
-    for (int c = tid; c < H; c += nt) u[c] = emb[size_t(cur) * H + c];
-    float cnt = 0.f;
-    for (int a = tid; a < C; a += nt) cnt += mk[a] ? 1.f : 0.f;
-    const float nv = block_sum(cnt, scratch);
-    for (int c = tid; c < H; c += nt) u[H + c] = nv > 0.f ? cand_sum[size_t(e) * H + c] / nv : 0.f;
-    __syncthreads();
-    v = mlp_scalar<DEPTH>(u, 2 * H, vmlp, y1, scratch);
-  }
+  const float v = mlp_tail(y1, vmlp, scratch);
   if (tid == 0) value[e] = v;
 
   if (action != nullptr) {
@@ -545,11 +391,15 @@ __global__ void k_round_weights(const float* __restrict__ src, T* __restrict__ d
   if (dst_t != nullptr) dst_t[size_t(c) * rows + r] = v;
 }
 
-// Launches with at most a few CTAs per SM are bound by the latency of their weight loads.
-bool few_ctas(int64_t ctas) { return ctas <= 4 * kNumSMs; }
-// With fewer CTAs than SMs every CTA has an SM to itself and the chain of dependent weight loads of one thread
-// is the whole run time: 1,024 threads cut every column's sum into four parts (dense_columns) instead of one.
-int head_threads(int64_t ctas) { return ctas <= kNumSMs ? 1024 : 256; }
+// Graphs per CTA: as few as leave every CTA an SM of its own (each then waits for its weights once, and every weight is
+// loaded once for all of a CTA's graphs), at most 16, within the shared memory that `bytes(GP)` says.  Measured (Eq. 8 and
+// the policy scores, hidden 256): 2,945 graphs 0.081 + 0.058 ms with a CTA of 256 threads per graph, 1,024 graphs 0.048 +
+// 0.030 ms.
+template <typename Bytes> int graphs_per_cta(int64_t B, Bytes bytes) {
+  int gp = 1;
+  while (gp < 16 && (B + gp - 1) / gp > kNumSMs && bytes(2 * gp) <= size_t(200) * 1024) gp <<= 1;
+  return gp;
+}
 
 int pow2_threads(int want) {          // power of two in [32, 1024] (block_sum needs a power of two)
   int t = 32;
@@ -576,27 +426,72 @@ int launch_readout(const Dims& d, const void* h, const int32_t* chunk_row0, cons
   return 1;
 }
 
-int launch_global_update(const Dims& d, const float* partial, const int32_t* graph_chunk_off,
-                         const float* g0, const DevWeights& w, float* emb, int32_t B, cudaStream_t st) {
-  if (B <= 0) return 0;
-  const int nt = head_threads(B);
-  const size_t smem = sizeof(float) * size_t(d.H + d.Dg + nt);
-  if (few_ctas(B)) k_global_update<32><<<B, nt, smem, st>>>(partial, graph_chunk_off, g0, w.Wg, w.bg, emb, d.H, d.Dg);
-  else k_global_update<8><<<B, nt, smem, st>>>(partial, graph_chunk_off, g0, w.Wg, w.bg, emb, d.H, d.Dg);
+namespace {
+template <int GP, bool BLOCKS>
+int global_update(const Dims& d, const float* partial, const int32_t* off, int32_t nblocks, int shift, const float* g0,
+                  const DevWeights& w, float* emb, float* U_out, int32_t B, size_t smem, cudaStream_t st) {
+  static bool attr[64] = {};
+  if (smem > 48 * 1024 && !ensure_dynamic_smem(k_global_update<GP, BLOCKS>, 227 * 1024, attr)) return -1;
+  k_global_update<GP, BLOCKS><<<(B + GP - 1) / GP, kThreads, smem, st>>>(partial, off, nblocks, shift, g0, w.Wg, w.bg, emb,
+                                                                         U_out, d.H, d.Dg, B);
   return 1;
+}
+template <bool BLOCKS>
+int launch_update(const Dims& d, const float* partial, const int32_t* off, int32_t nblocks, int shift, const float* g0,
+                  const DevWeights& w, float* emb, float* U_out, int32_t B, cudaStream_t st) {
+  if (B <= 0) return 0;
+  // rows of u, then scratch: the parts of the block sums (max(groups, GP) rows of H), the parts of the dense map
+  auto bytes = [&](int gp) {
+    const size_t rows = size_t(std::max(kThreads / (d.H / 4), gp)) * d.H, parts = size_t(gp) * kThreads;
+    return sizeof(float) * (size_t(gp) * row_stride(d.H + d.Dg) + std::max(rows, parts));
+  };
+  const int gp = graphs_per_cta(B, bytes);
+#define UPDATE_CASE(G_) case G_: return global_update<G_, BLOCKS>(d, partial, off, nblocks, shift, g0, w, emb, U_out, B, bytes(G_), st);
+  switch (gp) { UPDATE_CASE(1) UPDATE_CASE(2) UPDATE_CASE(4) UPDATE_CASE(8) default: UPDATE_CASE(16) }
+#undef UPDATE_CASE
+}
+template <int GP>
+int policy_value(const Dims& d, const Mlp& pm, const Mlp& vm, const float* emb, float* logit, int32_t B, float* y1_out,
+                 float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v, int VC, size_t smem,
+                 cudaStream_t st) {
+  static bool attr[64] = {};
+  if (smem > 48 * 1024 && !ensure_dynamic_smem(k_policy_value_hidden<GP>, 227 * 1024, attr)) return -1;
+  const int pc = (B + GP - 1) / GP;
+  k_policy_value_hidden<GP><<<pc + num_envs * VC, kThreads, smem, st>>>(emb, pm, logit, d.H, B, pc, y1_out, y2_out, env_off,
+                                                                        mask, d.A, vm, y1v, VC);
+  return 1;
+}
+}  // namespace
+
+int launch_global_update(const Dims& d, const float* partial, const int32_t* graph_chunk_off,
+                         const float* g0, const DevWeights& w, float* emb, int32_t B, cudaStream_t st, float* U_out) {
+  return launch_update<false>(d, partial, graph_chunk_off, 0, 0, g0, w, emb, U_out, B, st);
 }
 
 int launch_global_update_blocks(const Dims& d, const float* partial, const int32_t* node_off, int32_t nblocks,
                                 int block_shift, const float* g0, const DevWeights& w, float* emb, int32_t B,
                                 cudaStream_t st) {
-  if (B <= 0) return 0;
-  const int nt = head_threads(B);
-  const size_t smem = sizeof(float) * size_t(d.H + d.Dg + 3 + 4 * nt);   // the block sums' parts take 4 floats per thread
-  if (few_ctas(B))
-    k_global_update_blocks<32><<<B, nt, smem, st>>>(partial, node_off, nblocks, block_shift, g0, w.Wg, w.bg, emb, d.H, d.Dg);
-  else
-    k_global_update_blocks<8><<<B, nt, smem, st>>>(partial, node_off, nblocks, block_shift, g0, w.Wg, w.bg, emb, d.H, d.Dg);
-  return 1;
+  return launch_update<true>(d, partial, node_off, nblocks, block_shift, g0, w, emb, nullptr, B, st);
+}
+
+// Policy scores of all graphs (logit [B]; y1_out / y2_out optional) and, for num_envs > 0, the first layer of the value
+// head (y1v [num_envs x Hm]).
+int launch_policy_value_hidden(const Dims& d, const DevWeights& w, const float* emb, float* logit, int32_t B, float* y1_out,
+                               float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v,
+                               cudaStream_t st) {
+  const Mlp pm{w.pW1, w.pb1, w.pWh, w.pbh, w.pw2, w.pb2, d.Hm, d.Hm2};
+  const Mlp vm{w.vW1, w.vb1, w.vWh, w.vbh, w.vw2, w.vb2, d.Hm, d.Hm2};
+  auto bytes = [&](int gp) {
+    const size_t policy = size_t(gp) * (row_stride(d.H) + row_stride(d.Hm) + row_stride(d.Hm2) + kThreads);
+    return sizeof(float) * std::max(policy, size_t(2 * d.H + 4 * kThreads));
+  };
+  const int gp = graphs_per_cta(B, bytes);
+  // the value CTAs of an environment share its first layer: eight while they find SMs of their own beside the others'
+  const int VC = num_envs <= 8 ? 8 : num_envs <= 32 ? 4 : num_envs <= 128 ? 2 : 1;
+#define POLICY_CASE(G_) \
+  case G_: return policy_value<G_>(d, pm, vm, emb, logit, B, y1_out, y2_out, env_off, mask, num_envs, y1v, VC, bytes(G_), st);
+  switch (gp) { POLICY_CASE(1) POLICY_CASE(2) POLICY_CASE(4) POLICY_CASE(8) default: POLICY_CASE(16) }
+#undef POLICY_CASE
 }
 
 int launch_heads(const Dims& d, const DevWeights& w, const float* emb, const int32_t* env_off,
@@ -604,40 +499,15 @@ int launch_heads(const Dims& d, const DevWeights& w, const float* emb, const int
                  float* value, int32_t* action, uint64_t seed, uint64_t step, int32_t* status,
                  cudaStream_t st) {
   if (B <= 0 || num_envs <= 0) return 0;
-  const Mlp pm{w.pW1, w.pb1, w.pWh, w.pbh, w.pw2, w.pb2, d.Hm, d.Hm2};
   const Mlp vm{w.vW1, w.vb1, w.vWh, w.vbh, w.vw2, w.vb2, d.Hm, d.Hm2};
-  float* cand_sum = logit_ws + B;                 // [num_envs x H], behind the per-graph logits
-  // Steps of few graphs and environments with a short action space (the paper's own sizes): two launches, the
-  // value head's first layer spread over kValueChunks CTAs per environment next to the policy CTAs.
-  constexpr int kValueChunks = 8;
-  if (B + num_envs * kValueChunks <= kNumSMs && d.A <= 256 && d.Hm <= d.H) {
-    const int nt = 1024;
-    const size_t sm1 = sizeof(float) * size_t(2 * d.H + nt + d.Hm);
-    float* y1v = cand_sum;                        // [num_envs x Hm] (Hm <= H): the candidate sums are not needed here
-    k_policy_value_hidden<32><<<B + num_envs * kValueChunks, nt, sm1, st>>>(emb, pm, logit_ws, d.H, B, env_off, mask,
-                                                                         d.A, vm, y1v, kValueChunks);
-    const size_t smem = sizeof(unsigned long long) * size_t(nt + 1) + sizeof(float) * size_t(nt + 2 * d.H + d.Hm);
-    k_env_policy<32><<<num_envs, nt, smem, st>>>(emb, logit_ws, cand_sum, env_off, mask, vm, probs, value, action,
-                                                 d.H, d.A, seed, step, status, y1v);
-    return 2;
-  }
-  const int pnt = head_threads(B);
-  const size_t psm = sizeof(float) * size_t(d.H + pnt + d.Hm);
-  if (few_ctas(B)) k_policy_logit<32><<<B, pnt, psm, st>>>(emb, pm, logit_ws, d.H);
-  else k_policy_logit<8><<<B, pnt, psm, st>>>(emb, pm, logit_ws, d.H);
-  k_candidate_sum<<<dim3(num_envs, (d.H + 31) / 32), 1024, 0, st>>>(emb, env_off, mask, cand_sum, d.H, d.A);
-  int want = d.H > d.A + 1 ? d.H : d.A + 1;
-  if (want < 256) want = 256;               // enough threads to split the value head's dense map
-  if (num_envs <= kNumSMs) want = 1024;     // (an SM per environment: see head_threads)
+  float* y1v = logit_ws + B;                      // [num_envs x Hm], behind the per-graph logits
+  if (launch_policy_value_hidden(d, w, emb, logit_ws, B, nullptr, nullptr, env_off, mask, num_envs, y1v, st) < 0) return -1;
+  int want = std::max({d.A + 1, d.Hm, 256});      // enough threads to split the value head's dense map
+  if (num_envs <= kNumSMs && d.Hm2 > 0) want = 1024;     // (an SM per environment: more parts, shorter chains)
   const int nt = pow2_threads(want);
-  const size_t smem = sizeof(unsigned long long) * size_t(nt + 1) + sizeof(float) * size_t(nt + 2 * d.H + d.Hm);
-  if (few_ctas(num_envs))
-    k_env_policy<32><<<num_envs, nt, smem, st>>>(emb, logit_ws, cand_sum, env_off, mask, vm, probs, value, action,
-                                                 d.H, d.A, seed, step, status, nullptr);
-  else
-    k_env_policy<8><<<num_envs, nt, smem, st>>>(emb, logit_ws, cand_sum, env_off, mask, vm, probs, value, action,
-                                                d.H, d.A, seed, step, status, nullptr);
-  return 3;
+  const size_t smem = sizeof(unsigned long long) * size_t(nt + 2) + sizeof(float) * size_t(nt + d.Hm);
+  k_env_policy<<<num_envs, nt, smem, st>>>(logit_ws, env_off, mask, vm, probs, value, action, d.A, seed, step, status, y1v);
+  return 2;
 }
 
 int launch_sample(const float* probs, int32_t num_envs, int32_t A1, uint64_t seed, uint64_t step,

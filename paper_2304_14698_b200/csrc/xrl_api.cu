@@ -663,7 +663,8 @@ xrl_status xrl_create(const xrl_model_config* cfg, int32_t device, xrl_ctx** out
     const size_t slots = slots_fused > size_t(ctx->max_chunks) ? slots_fused : size_t(ctx->max_chunks);
     A(ctx->partial, 4 * slots * H);
   }
-  A(ctx->logits, 4 * (size_t(cfg->max_graphs) + size_t(cfg->max_envs) * H));   // logits, then candidate sums
+  // logits, then the value head's first layer per environment
+  A(ctx->logits, 4 * (size_t(cfg->max_graphs) + size_t(cfg->max_envs) * size_t(cfg->mlp_hidden)));
   A(ctx->status, 16);          // [0] the device status word; [2], [3] the all-layers kernel's barrier counters
   if (e == cudaSuccess) e = cudaMemset(ctx->status.p, 0, 16);
   if (e != cudaSuccess) {
@@ -921,6 +922,7 @@ xrl_status xrl_encode(xrl_ctx* ctx, const xrl_batch* b, const float* g0, float* 
   else
     k = launch_global_update(ctx->dims, ctx->partial.as<float>(), b->d_graph_chunk_off, g0, ctx->dw,
                              graph_emb, b->B, st);
+  if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
   ctx->prof.end(FAM_HEADS, slot, k, st);
   n += k;
   ctx->launches_encode = n;
@@ -1039,6 +1041,7 @@ xrl_status xrl_encode_delta(xrl_ctx* ctx, const xrl_batch* b, const int32_t* bas
   n_launch += k;
   slot = pf.begin(st);
   k = launch_global_update(d, ctx->partial.as<float>(), b->d_graph_chunk_off, g0, ctx->dw, graph_emb, b->B, st);
+  if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
   pf.end(FAM_HEADS, slot, k, st);
   n_launch += k;
   ctx->launches_encode = n_launch;
@@ -1089,6 +1092,7 @@ xrl_status xrl_policy_value(xrl_ctx* ctx, const xrl_batch* b, const float* graph
   ctx->launches_heads = launch_heads(ctx->dims, ctx->dw, graph_emb, b->d_env_off, mask, b->B, b->num_envs,
                                      ctx->logits.as<float>(), probs, value, action, seed, step,
                                      ctx->status.as<int32_t>(), st);
+  if (ctx->launches_heads < 0) { ctx->launches_heads = 0; cudaGetLastError(); return XRL_ERR_CUDA; }
   ctx->prof.end(FAM_HEADS, slot, int(ctx->launches_heads), st);
   XRL_CUDA(cudaGetLastError());
   return XRL_OK;

@@ -205,7 +205,11 @@ int launch_delta_fill(const DeltaIn& in, int32_t n, int32_t t, const int32_t* li
 int launch_delta_remap(int32_t N, int32_t L, const int32_t* level, const int32_t* rank, const int32_t* base,
                        int32_t* remap, cudaStream_t st);
 int launch_global_update(const Dims& d, const float* partial, const int32_t* graph_chunk_off,
-                         const float* g0, const DevWeights& w, float* emb, int32_t B, cudaStream_t st);
+                         const float* g0, const DevWeights& w, float* emb, int32_t B, cudaStream_t st,
+                         float* U_out = nullptr);
+int launch_policy_value_hidden(const Dims& d, const DevWeights& w, const float* emb, float* logit, int32_t B, float* y1_out,
+                               float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v,
+                               cudaStream_t st);
 int launch_heads(const Dims& d, const DevWeights& w, const float* emb, const int32_t* env_off,
                  const uint8_t* mask, int32_t B, int32_t num_envs, float* logit_ws, float* probs,
                  float* value, int32_t* action, uint64_t seed, uint64_t step, int32_t* status,
