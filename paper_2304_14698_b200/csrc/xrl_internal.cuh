@@ -219,7 +219,8 @@ int launch_sample(const float* probs, int32_t num_envs, int32_t A1, uint64_t see
 // ---- reverse pass (Section 3.3.4) --------------------------------------------------------------------
 size_t ppo_heads_workspace_floats(const Dims& d, int64_t B, int64_t num_envs);
 int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const float* w_base, const void* hL,
-                     const int32_t* node_off, const int32_t* seg_id, const float* g0, const int32_t* env_off,
+                     const float* partial, const int32_t* graph_chunk_off, const int32_t* seg_id, const float* g0,
+                     const int32_t* env_off,
                      const uint8_t* mask, const int32_t* action, const float* logp_old, const float* adv,
                      const float* ret, float eps, float c1, float c2, int32_t B, int32_t num_envs, int64_t N,
                      float* ws, float* loss, float* dh, float* logp_out, int32_t* status, cudaStream_t st);
