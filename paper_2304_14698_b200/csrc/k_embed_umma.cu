@@ -122,7 +122,7 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
     const int row_in_tile = q * 32 + lane;
     const bool leader = (threadIdx.x == 32);
     volatile uint32_t* abort_flag = tmem_slot + 1;
-    uint32_t lt = 0;
+    uint32_t lt = 0, stores = 0;
     for (int tile = first; tile < num_tiles; tile += step, ++lt) {
       const int buf = lt & 1;
       uint32_t okw = 1;
@@ -143,9 +143,11 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
           for (int t = 0; t < 32; ++t) v[1][t] = 0u;
         }
         tc_wait_ld();
+        if (c * 64 >= cols) continue;            // columns that do not exist (the same for all threads)
+        // the two staging tiles alternate from store to store, across tiles too (a tile may have an odd number of chunks)
         if (leader) tma_wait_read<1>();
         epi_barrier();
-        uint8_t* stage = smem + C::OFF_OUT + (c & 1) * CHUNK_BYTES + row_in_tile * 128;
+        uint8_t* stage = smem + C::OFF_OUT + (stores & 1) * CHUNK_BYTES + row_in_tile * 128;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const uint32_t* z = &v[j >> 2][(j & 3) * 8];
@@ -158,10 +160,11 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
         }
         fence_async_smem();
         epi_barrier();
-        if (leader && c * 64 < cols) {
-          tma_store_2d(&map_h, base + C::OFF_OUT + (c & 1) * CHUNK_BYTES, col0 + c * 64, tile * BM);
+        if (leader) {
+          tma_store_2d(&map_h, base + C::OFF_OUT + (stores & 1) * CHUNK_BYTES, col0 + c * 64, tile * BM);
           tma_commit();
         }
+        ++stores;
       }
       tc_fence_before();
       mbar_arrive(bar_acc_empty(buf));

@@ -132,6 +132,7 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
   const int row_in_tile = q * 32 + lane;
   const float* avec = reinterpret_cast<const float*>(smem + C::OFF_AVEC);
   volatile uint32_t* abort_flag = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM) + 1;
+  uint32_t stores = 0;
   for (int tile = first; tile < num_tiles; tile += step, ++lt) {
     const int buf = lt & 1;
     // one lane per warp waits; the four warps agree on the outcome before touching a barrier
@@ -185,10 +186,12 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
           ss = 0.f; sd = 0.f; ++head; left = d;
         }
       }
-      // staging tile (c & 1) must no longer be read by the store issued two chunks ago
+      if (c * 64 >= cols_left) continue;       // columns that do not exist: nothing to stage (the same for all threads)
+      // the two staging tiles alternate from store to store, across tiles too (a tile may have an odd number of chunks):
+      // this one must no longer be read by the store issued two stores ago
       if (leader) tma_wait_read<1>();
       epi_barrier();
-      uint8_t* stage = smem + C::OFF_OUT + (c & 1) * STAGE_BYTES + row_in_tile * 128;
+      uint8_t* stage = smem + C::OFF_OUT + (stores & 1) * STAGE_BYTES + row_in_tile * 128;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {            // 16-byte chunk j of this row, swizzled by the row
         const uint32_t* z = &v[j >> 2][(j & 3) * 8];
@@ -201,10 +204,11 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
       }
       fence_async_smem();
       epi_barrier();
-      if (leader && c * 64 < cols_left) {
-        tma_store_2d(map_z, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, col0 + c * 64, tile * BM);
+      if (leader) {
+        tma_store_2d(map_z, base + C::OFF_OUT + (stores & 1) * STAGE_BYTES, col0 + c * 64, tile * BM);
         tma_commit();
       }
+      ++stores;
     }
     tc_fence_before();
     mbar_arrive(C::bar_acc_empty(base, buf));   // 128 arrivals free the accumulator

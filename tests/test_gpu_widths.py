@@ -32,3 +32,31 @@ def test_bf16_widths(xo, H, K, nodes):
         assert ag.device_status() == 0
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K", [(64, 2), (192, 6), (320, 2)])
+def test_bf16_widths_with_many_tiles_per_cta(xo, H, K):
+    """Output tiles with an odd number of 64-column chunks, several tiles per CTA: the staging buffers of one tile's last
+    store and the next tile's first must not be the same."""
+    import paper_2304_14698_b200 as xrl
+    rng = dags.make_rng(H)
+    m = dict(T=21, S=8, H=H, K=K, L=1, Hm=24, Dg=1, dtype="bf16", A_max=64)
+    g = dags.random_dag(rng, 1500, m["T"], 8, True)
+    batch = dags.flatten([g] * 50, [0, 50], 64)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 4)
+    one = dags.flatten([g], [0, 1], 64)
+    st, packed = xo.pack(one)
+    assert st == 0
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        for layer in (0, 1):
+            got = xrl.xrl_debug_node_features(ag.ctx, ag.batch, layer, H).reshape(50, 1500, H)
+            want = xo.encode(m, blob, one, packed, dump_layer=layer, want_nodes=True)["nodes"]
+            for i in range(50):
+                gpu_util.assert_close(got[i], want, "bf16", f"copy {i} after stage {layer}")
+                assert (got[i] == got[0]).all()
+    finally:
+        ag.close()
