@@ -174,6 +174,11 @@ xrl_status xrl_pack_flat(xrl_ctx* ctx, int32_t where, int32_t num_graphs, const 
                          const int32_t* edge_src, const int32_t* edge_dst, const int32_t* env_off,
                          int32_t num_envs, void* stream, xrl_batch** out);
 
+/* Host helper for callers of the pack calls whose features are float: n values of src (HOST float) rounded to bf16 bit
+ * patterns in dst (HOST), nearest even, by the integer rule bits = (u + 0x7FFF + ((u >> 16) & 1)) >> 16 on the float's
+ * 32-bit pattern u.  Needs no device.  Errors: INVALID_ARG. */
+xrl_status xrl_round_features(const float* src, uint16_t* dst, int64_t n);
+
 xrl_status xrl_batch_free(xrl_ctx* ctx, xrl_batch* batch);
 /* All four outputs HOST. */
 xrl_status xrl_batch_info(const xrl_batch* batch, int64_t* num_nodes, int64_t* num_edges,

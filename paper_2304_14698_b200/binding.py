@@ -26,7 +26,7 @@ EXPORTED_SYMBOLS = [
     "xrl_policy_value", "xrl_sample", "xrl_last_device_status", "xrl_launch_counts", "xrl_version",
     "xrl_profile", "xrl_profile_read", "xrl_pack_csr_static", "xrl_encode_delta", "xrl_delta_rows", "xrl_get_weights",
     "xrl_graph_begin", "xrl_graph_launch", "xrl_batch_set_edge_attr", "xrl_ppo_grad", "xrl_gae",
-    "xrl_grad_weigh", "xrl_grad_unweigh", "xrl_init_weights",
+    "xrl_grad_weigh", "xrl_grad_unweigh", "xrl_init_weights", "xrl_round_features",
 ]
 PROFILE_FAMILIES = ["pack", "node_update", "transform", "aggregate", "readout", "heads", "aggregate_readout",
                     "layers_fused"]
@@ -75,6 +75,7 @@ def load_library():
         "xrl_init_weights": [vp, u64],
         "xrl_pack": [vp, C.POINTER(_Graph), i32, vp, i32, vp, C.POINTER(vp)],
         "xrl_pack_flat": [vp, i32, i32, vp, vp, vp, vp, vp, vp, vp, i32, vp, C.POINTER(vp)],
+        "xrl_round_features": [vp, vp, i64],
         "xrl_batch_free": [vp, vp],
         "xrl_batch_info": [vp, C.POINTER(i64), C.POINTER(i64), C.POINTER(i32), C.POINTER(i32)],
         "xrl_batch_export": [vp, vp, vp, vp, vp, vp, vp],
@@ -145,6 +146,14 @@ def to_bf16_bits(x: np.ndarray) -> np.ndarray:
     return u.astype(np.uint16).reshape(x.shape)
 
 
+def xrl_round_features(x: np.ndarray) -> np.ndarray:
+    """The same in the library (a step's features are rounded on every pack from host memory)."""
+    x = np.ascontiguousarray(x, dtype=np.float32)
+    out = np.empty(x.shape, np.uint16)
+    _check(load_library().xrl_round_features(_np_ptr(x), _np_ptr(out), x.size), "xrl_round_features")
+    return out
+
+
 # ---- one function per C entry point ---------------------------------------------------------
 
 def xrl_version() -> str:
@@ -191,7 +200,7 @@ def xrl_pack(ctx, graphs, env_off, dtype, stream=None, batch=None):
         op = np.ascontiguousarray(g["op"], dtype=np.int32)
         shp = np.ascontiguousarray(g["shape"], dtype=np.float32)
         if dtype in ("bf16", XRL_BF16):
-            shp = to_bf16_bits(shp)
+            shp = xrl_round_features(shp)
         es = np.ascontiguousarray(g["edge_src"], dtype=np.int32)
         ed = np.ascontiguousarray(g["edge_dst"], dtype=np.int32)
         keep += [op, shp, es, ed]
@@ -468,7 +477,7 @@ class Agent:
 
     def storage_shape(self, shape_f32):
         """Host float32 shape features -> the array xrl_pack_flat expects for this model's dtype."""
-        return to_bf16_bits(shape_f32) if self.m["dtype"] == "bf16" else \
+        return xrl_round_features(shape_f32) if self.m["dtype"] == "bf16" else \
             np.ascontiguousarray(shape_f32, dtype=np.float32)
 
     def pack(self, batch):

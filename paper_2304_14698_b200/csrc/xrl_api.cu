@@ -113,8 +113,16 @@ struct xrl_batch {
   cudaStream_t stream = nullptr;
   // device
   DeviceBuf meta;           // n_nodes[B] n_edges[B] env_off[Ne+1] graph_chunk_off[B+1] chunk_row0[] chunk_row1[]
-  DeviceBuf node_off, edge_off, seg_id, graph_env, rowptr, col, op, shape;
-  DeviceBuf edge_src, edge_dst, deg, tmp_eid, long_rows, long_count, scan_ws, coarse;
+  DeviceBuf node_off, edge_off, seg_id, graph_env, rowptr, col;
+  // shape | op | edge_src | edge_dst of the packed batch, back to back (one copy brings them from the staging buffer):
+  // place_bulk sets the pieces for the batch at hand
+  DeviceBuf bulk;
+  struct Piece { void* p = nullptr; template <typename T> T* as() const { return static_cast<T*>(p); } } op, shape, edge_src, edge_dst;
+  void place_bulk(size_t N, size_t E, size_t shape_row) {
+    char* q = static_cast<char*>(bulk.p);
+    shape.p = q; op.p = q + shape_row * N; edge_src.p = q + (shape_row + 4) * N; edge_dst.p = q + (shape_row + 4) * N + 4 * E;
+  }
+  DeviceBuf deg, tmp_eid, long_rows, long_count, scan_ws, coarse;
   // contexts with attributes on the edges: slot -> input edge, the attributes as given and in slot order
   DeviceBuf eid, eattr_in, eattr;
   bool has_eattr = false;
@@ -201,8 +209,7 @@ xrl_status alloc_batch(xrl_ctx* ctx, xrl_batch** out) {
   A(b->node_off, 4 * (B + 1)); A(b->edge_off, 4 * (B + 1));
   A(b->seg_id, 4 * N); A(b->graph_env, 4 * B);
   A(b->rowptr, 4 * (N + 1)); A(b->col, 4 * E);
-  A(b->op, 4 * N); A(b->shape, sb * N * kS);
-  A(b->edge_src, 4 * E); A(b->edge_dst, 4 * E);
+  A(b->bulk, (4 + sb * kS) * N + 8 * E);
   A(b->deg, 4 * N); A(b->tmp_eid, 8 * E + 8);
   A(b->long_rows, 4 * (E / 32 + 1)); A(b->long_count, 4); A(b->coarse, 4 * (E / 1024 + 2));
   A(b->scan_ws, 4 * scan_workspace_ints(int64_t(N > B ? N : B) + 1));
@@ -330,6 +337,7 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
 
   // ---- bulk arrays -------------------------------------------------------------------------------
   const size_t sb = storage_bytes(c.dtype);
+  b->place_bulk(size_t(N), size_t(E), sb * kS);
   const int32_t *d_src, *d_dst;
   // page-locked caller memory and a large batch of graphs that the per-graph packer takes: ranges of
   // graphs are copied and packed one after the other on the batch's own stream (see xrl_batch::nparts)
@@ -370,9 +378,9 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
     d_src = b->edge_src.as<int32_t>();
     d_dst = b->edge_dst.as<int32_t>();
   } else if (graphs || where == XRL_MEM_HOST) {
-    char* p_op = b->h_bulk;
-    char* p_shape = p_op + 4 * size_t(N);
-    char* p_src = p_shape + sb * kS * size_t(N);
+    char* p_shape = b->h_bulk;                     // in the device buffer's order: one copy
+    char* p_op = p_shape + sb * kS * size_t(N);
+    char* p_src = p_op + 4 * size_t(N);
     char* p_dst = p_src + 4 * size_t(E);
     if (graphs) {
       size_t no = 0, eo = 0;
@@ -392,14 +400,8 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
       if (N) { memcpy(p_op, op, 4 * size_t(N)); memcpy(p_shape, shape, sb * kS * size_t(N)); }
       if (E) { memcpy(p_src, edge_src, 4 * size_t(E)); memcpy(p_dst, edge_dst, 4 * size_t(E)); }
     }
-    if (N) {
-      XRL_CUDA(cudaMemcpyAsync(b->op.p, p_op, 4 * size_t(N), cudaMemcpyHostToDevice, st));
-      XRL_CUDA(cudaMemcpyAsync(b->shape.p, p_shape, sb * kS * size_t(N), cudaMemcpyHostToDevice, st));
-    }
-    if (E) {
-      XRL_CUDA(cudaMemcpyAsync(b->edge_src.p, p_src, 4 * size_t(E), cudaMemcpyHostToDevice, st));
-      XRL_CUDA(cudaMemcpyAsync(b->edge_dst.p, p_dst, 4 * size_t(E), cudaMemcpyHostToDevice, st));
-    }
+    const size_t bytes = (4 + sb * kS) * size_t(N) + 8 * size_t(E);
+    if (bytes) XRL_CUDA(cudaMemcpyAsync(b->bulk.p, b->h_bulk, bytes, cudaMemcpyHostToDevice, st));
     d_src = b->edge_src.as<int32_t>();
     d_dst = b->edge_dst.as<int32_t>();
   } else {
@@ -806,13 +808,23 @@ xrl_status xrl_pack_flat(xrl_ctx* ctx, int32_t where, int32_t num_graphs, const 
                      env_off, num_envs, stream, out);
 }
 
+xrl_status xrl_round_features(const float* src, uint16_t* dst, int64_t n) {
+  if (n < 0 || (n > 0 && (!src || !dst))) return XRL_ERR_INVALID_ARG;
+  for (int64_t i = 0; i < n; ++i) {
+    uint32_t u;
+    memcpy(&u, src + i, 4);
+    dst[i] = uint16_t((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
+  }
+  return XRL_OK;
+}
+
 xrl_status xrl_batch_free(xrl_ctx* ctx, xrl_batch* b) {
   if (!b) return XRL_OK;
   if (ctx && b->ctx != ctx) return XRL_ERR_STATE;
   cudaSetDevice(b->ctx->device);
   cudaDeviceSynchronize();
   DeviceBuf* bufs[] = {&b->meta, &b->node_off, &b->edge_off, &b->seg_id, &b->graph_env, &b->rowptr,
-                       &b->col, &b->op, &b->shape, &b->edge_src, &b->edge_dst, &b->deg, &b->tmp_eid,
+                       &b->col, &b->bulk, &b->deg, &b->tmp_eid,
                        &b->long_rows, &b->long_count, &b->scan_ws, &b->coarse, &b->eid, &b->eattr_in,
                        &b->eattr, &b->rowptr_out, &b->col_out, &b->rowptr_nbr, &b->col_nbr};
   for (DeviceBuf* d : bufs) d->release();
