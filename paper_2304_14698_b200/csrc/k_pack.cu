@@ -225,7 +225,8 @@ k_pack_graph(int32_t* __restrict__ node_off, int32_t* __restrict__ edge_off,
              int32_t* __restrict__ seg_id, int32_t* __restrict__ rowptr, int32_t* __restrict__ col,
              int32_t* status, int32_t g_first, int32_t* __restrict__ eid,
              const int32_t* __restrict__ n_nodes, const int32_t* __restrict__ n_edges,
-             const int32_t* __restrict__ env_off, int32_t num_envs, int32_t* __restrict__ graph_env) {
+             const int32_t* __restrict__ env_off, int32_t num_envs, int32_t* __restrict__ graph_env,
+             int32_t* __restrict__ op_copy, const uint4* __restrict__ shape, uint4* __restrict__ shape_copy, int32_t pieces) {
   extern __shared__ __align__(16) int32_t psm[];
   int32_t* deg = psm;                         // [cap_n + 1] in-degree, then exclusive row starts
   int32_t* cur = psm + cap_n + 1;             // [cap_n]     row cursors
@@ -270,7 +271,13 @@ k_pack_graph(int32_t* __restrict__ node_off, int32_t* __restrict__ edge_off,
     cur[i] = 0;
     seg_id[nb + i] = g;
     const int32_t o = op[nb + i];
+    if (op_copy != nullptr) op_copy[nb + i] = o;
     if (o < 0 || o >= T) raise(status, XRL_ERR_BAD_GRAPH);
+  }
+  // the caller's device arrays into the batch's (shape rows as 16-byte pieces): instead of two copies beside this kernel
+  if (shape_copy != nullptr) {
+    const size_t first = size_t(nb) * pieces;
+    for (int32_t i = tid; i < n * pieces; i += NT) shape_copy[first + i] = __ldg(shape + first + i);
   }
   __syncthreads();
   // edges four at a time per thread: the loads of a batch are issued before any of them is used
@@ -469,7 +476,9 @@ int launch_pack_graphs(const PackIn& in, const PackOut& out, int T, int32_t g0, 
     k_pack_graph<NT_, OFF_><<<g1 - g0, NT_, smem, st>>>(out.node_off, out.edge_off, in.op, in.edge_src,           \
                                                         in.edge_dst, T, in.B, in.max_n, out.seg_id, out.rowptr,   \
                                                         out.col, status, g0, out.eid, in.n_nodes, in.n_edges,     \
-                                                        in.env_off, in.num_envs, out.graph_env);                  \
+                                                        in.env_off, in.num_envs, out.graph_env, out.op_copy,      \
+                                                        static_cast<const uint4*>(in.shape),                      \
+                                                        static_cast<uint4*>(out.shape_copy), in.shape_pieces);    \
   } while (0)
   if (graph_threads(in.max_n) == 1024) {
     if (offsets) PACK_GRAPH(1024, true, attr1024o); else PACK_GRAPH(1024, false, attr1024);

@@ -362,6 +362,7 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
       XRL_CUDA(cudaEventCreateWithFlags(&b->ev_part[p], cudaEventDisableTiming));
   }
   b->nparts = 0;
+  bool pack_copies = false;
   if (parts > 0) {
     d_src = b->edge_src.as<int32_t>();
     d_dst = b->edge_dst.as<int32_t>();
@@ -405,7 +406,15 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
     d_src = b->edge_src.as<int32_t>();
     d_dst = b->edge_dst.as<int32_t>();
   } else {
-    if (N) {
+    // the per-graph packer reads the operators anyway and copies the features with them (16-byte pieces: both sides on
+    // such a boundary): two launches fewer, paper_step 0.126 -> 0.118 ms, and 75 us instead of 62 + 23 for 2 M nodes of
+    // 1,000-node graphs.  Not for graphs of thousands of nodes, where one or two CTAs fill an SM and wait for their own
+    // copies (4.1 M nodes of 4,000-node graphs: 247 us against 171 + 35)
+    PackIn probe{};
+    probe.B = num_graphs; probe.max_n = max_n; probe.max_m = max_m;
+    pack_copies = pack_per_graph(probe) && max_n < 2048 && (reinterpret_cast<uintptr_t>(shape) & 15) == 0 &&
+                  (reinterpret_cast<uintptr_t>(b->shape.p) & 15) == 0;
+    if (N && !pack_copies) {
       XRL_CUDA(cudaMemcpyAsync(b->op.p, op, 4 * size_t(N), cudaMemcpyDeviceToDevice, st));
       XRL_CUDA(cudaMemcpyAsync(b->shape.p, shape, sb * kS * size_t(N), cudaMemcpyDeviceToDevice, st));
     }
@@ -427,6 +436,10 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
   po.long_rows = b->long_rows.as<int32_t>(); po.long_count = b->long_count.as<int32_t>();
   po.scan_ws = b->scan_ws.as<int32_t>(); po.coarse = b->coarse.as<int32_t>();
   po.eid = c.edge_attributes ? b->eid.as<int32_t>() : nullptr;
+  if (pack_copies) {
+    in.op = op; in.shape = shape; in.shape_pieces = int32_t(sb * kS / 16);
+    po.op_copy = b->op.as<int32_t>(); po.shape_copy = b->shape.p;
+  }
   b->has_eattr = false;                          // attributes belong to one packing of the batch
   if (parts == 0) {
     const size_t slot = ctx->prof.begin(st);
@@ -437,6 +450,7 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
       rin.edge_src = in.edge_dst; rin.edge_dst = in.edge_src;
       PackOut rpo = po;
       rpo.rowptr = b->rowptr_out.as<int32_t>(); rpo.col = b->col_out.as<int32_t>(); rpo.eid = nullptr;
+      rpo.op_copy = nullptr; rpo.shape_copy = nullptr;
       ctx->launches_pack += launch_pack(rin, rpo, c.num_op_types, ctx->status.as<int32_t>(), st);
       ctx->launches_pack += launch_merge_csr(po.rowptr, po.col, rpo.rowptr, rpo.col, in.N,
                                              b->rowptr_nbr.as<int32_t>(), b->col_nbr.as<int32_t>(), st);

@@ -112,10 +112,15 @@ struct PackIn {
   int32_t max_n, max_m;                           // largest node / edge count of one graph
   const int32_t *n_nodes, *n_edges, *env_off;     // device copies of the metadata
   const int32_t *op, *edge_src, *edge_dst;        // device
+  const void* shape = nullptr;                    // with PackOut::shape_copy: [N] rows of shape_pieces x 16 bytes
+  int32_t shape_pieces = 0;
 };
 struct PackOut {
   int32_t *node_off, *edge_off, *seg_id, *graph_env, *rowptr, *col;
   int32_t *deg, *tmp_eid /* [2E]: (edge id, producer) pairs */, *long_rows, *long_count, *scan_ws, *coarse;   // scratch
+  // optional (the per-graph packer only): copies of the caller's op and shape arrays
+  int32_t* op_copy = nullptr;
+  void* shape_copy = nullptr;
   int32_t* eid = nullptr;   // optional output [E]: the input edge in each CSR slot (attributes on edges)
 };
 int launch_pack(const PackIn& in, const PackOut& out, int T, int32_t* status, cudaStream_t st);
