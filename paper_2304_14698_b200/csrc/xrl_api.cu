@@ -27,7 +27,15 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-constexpr int32_t kReadoutChunkRows = 512;
+// Rows a CTA of the readout adds: short chunks where the batch has few of them (a chain of loads per CTA and few CTAs:
+// 124 k rows, hidden 192: 24 us with 512-row chunks), long ones where there are plenty and every chunk is one more partial sum
+// to add per graph and one more list entry to send.
+constexpr int64_t kReadoutFewRows = int64_t(1) << 17;
+int32_t readout_chunk_rows(int64_t N) { return N <= kReadoutFewRows ? 128 : 512; }
+int64_t readout_max_chunks(int64_t max_nodes, int64_t max_graphs) {
+  const int64_t few = (max_nodes < kReadoutFewRows ? max_nodes : kReadoutFewRows) / 128, many = max_nodes / 512;
+  return max_graphs + (few > many ? few : many) + 1;
+}
 
 struct DeviceBuf {
   void* p = nullptr;
@@ -314,14 +322,15 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
   int32_t* m_c0 = m_gco + (Bz + 1);
   int32_t* m_c1 = m_c0 + ctx->max_chunks;
   int32_t chunks = 0, row = 0;
+  const int32_t chunk_rows = readout_chunk_rows(N);
   for (int32_t g = 0; g < num_graphs; ++g) {
     const int32_t n = graphs ? graphs[g].num_nodes : n_nodes[g];
     m_nn[g] = n;
     m_ne[g] = graphs ? graphs[g].num_edges : n_edges[g];
     m_gco[g] = chunks;
-    for (int32_t r = 0; r < n; r += kReadoutChunkRows) {
+    for (int32_t r = 0; r < n; r += chunk_rows) {
       m_c0[chunks] = row + r;
-      m_c1[chunks] = row + (r + kReadoutChunkRows < n ? r + kReadoutChunkRows : n);
+      m_c1[chunks] = row + (r + chunk_rows < n ? r + chunk_rows : n);
       ++chunks;
     }
     row += n;
@@ -657,7 +666,7 @@ xrl_status xrl_create(const xrl_model_config* cfg, int32_t device, xrl_ctx** out
   ctx->use_umma_embed = embed_umma_supported(ctx->dims) && getenv("XRL_FORCE_SIMT_TRANSFORM") == nullptr;
   // Z rows carry their half-score pairs when both kernels that touch them support it
   ctx->dims.zmerged = (ctx->use_umma && cfg->dtype == XRL_BF16 && aggregate_tma_shape(ctx->dims)) ? 1 : 0;
-  ctx->max_chunks = int32_t(cfg->max_graphs + cfg->max_nodes / kReadoutChunkRows + 1);
+  ctx->max_chunks = int32_t(readout_max_chunks(cfg->max_nodes, cfg->max_graphs));
   const size_t sb = storage_bytes(cfg->dtype), N = size_t(cfg->max_nodes), H = size_t(cfg->hidden);
   const size_t F0 = size_t(2 * kS + cfg->num_op_types);
   cudaError_t e = cudaSuccess;
