@@ -117,7 +117,7 @@ struct xrl_ctx {
 struct xrl_batch {
   xrl_ctx* ctx = nullptr;
   bool packed = false;
-  int32_t B = 0, num_envs = 0, N = 0, E = 0, num_chunks = 0;
+  int32_t B = 0, num_envs = 0, N = 0, E = 0, num_chunks = 0, max_n = 0;   // max_n: nodes of the largest graph
   cudaStream_t stream = nullptr;
   // device
   DeviceBuf meta;           // n_nodes[B] n_edges[B] env_off[Ne+1] graph_chunk_off[B+1] chunk_row0[] chunk_row1[]
@@ -511,7 +511,7 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
   XRL_CUDA(cudaGetLastError());
 
   b->B = num_graphs; b->num_envs = num_envs; b->N = int32_t(N); b->E = int32_t(E);
-  b->num_chunks = chunks; b->stream = st; b->packed = true;
+  b->num_chunks = chunks; b->max_n = max_n; b->stream = st; b->packed = true;
   return XRL_OK;
 }
 
@@ -1005,14 +1005,17 @@ xrl_status xrl_encode_delta(xrl_ctx* ctx, const xrl_batch* b, const int32_t* bas
   Profiler& pf = ctx->prof;
   int n_launch = 0;
   size_t slot = pf.begin(st);
-  int k = launch_delta_level0(in, valid, base, level_a, st);
   int32_t* level = level_a;
-  int32_t* other = level_b;
-  for (int t = 1; t <= L; ++t) {
-    k += launch_delta_propagate(in, t, level, other, st);
-    int32_t* tmp = level; level = other; other = tmp;
+  int k = launch_delta_graphs(in, b->B, b->max_n, L, base, level, counts, cursor, st);
+  if (k < 0) {                                      // graphs beyond shared memory: pass by pass over all nodes
+    k = launch_delta_level0(in, valid, base, level_a, st);
+    int32_t* other = level_b;
+    for (int t = 1; t <= L; ++t) {
+      k += launch_delta_propagate(in, t, level, other, st);
+      int32_t* tmp = level; level = other; other = tmp;
+    }
+    k += launch_delta_count(N, L, level, counts, cursor, st);
   }
-  k += launch_delta_count(N, L, level, counts, cursor, st);
   k += launch_delta_assign(N, L, level, counts, cursor, rank, list, st);
   pf.end(FAM_PACK, slot, k, st);
   n_launch += k;

@@ -196,6 +196,8 @@ struct DeltaIn {
   int shape_bytes;                 // bytes of one node's shape features
   const int32_t* base_id;          // caller's hint
 };
+int launch_delta_graphs(const DeltaIn& in, int32_t B, int32_t max_n, int32_t L, int32_t* base, int32_t* level, int32_t* counts,
+                        int32_t* cursor, cudaStream_t st);
 int launch_delta_level0(const DeltaIn& in, int32_t* valid, int32_t* base, int32_t* level, cudaStream_t st);
 int launch_delta_propagate(const DeltaIn& in, int32_t t, const int32_t* level_in, int32_t* level_out,
                            cudaStream_t st);

@@ -1,0 +1,49 @@
+"""Delta encoding's levels by graph (shared memory) and, for a graph beyond that, pass by pass: both give the full encoder's
+embeddings, and the same number of reached rows per layer."""
+import numpy as np
+import pytest
+
+from workloads import dags
+import gpu_util
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(m, graphs, env_off, blob):
+    import torch
+    import paper_2304_14698_b200 as xrl
+    batch = dags.flatten(graphs, env_off, m["A_max"])
+    batch["model"] = m
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        full = torch.empty((len(graphs), m["H"]), device="cuda")
+        delta = torch.empty_like(full)
+        xrl.xrl_encode(ag.ctx, ag.batch, full)
+        xrl.xrl_encode_delta(ag.ctx, ag.batch, torch.from_numpy(batch["base_id"]).cuda(), delta)
+        torch.cuda.synchronize()
+        assert ag.device_status() == 0
+        return full.cpu().numpy(), delta.cpu().numpy(), xrl.xrl_delta_rows(ag.ctx, m["L"])
+    finally:
+        ag.close()
+
+
+@pytest.mark.parametrize("nodes", [2, 31, 257, 3000])
+@pytest.mark.parametrize("L", [0, 1, 5])
+def test_levels_by_graph_and_pass_by_pass(nodes, L):
+    m = dict(T=11, S=8, H=64, K=2, L=L, Hm=16, Dg=1, dtype="fp32", A_max=8)
+    rng = dags.make_rng(nodes + L)
+    graphs, env_off = [], [0]
+    for _ in range(2):
+        cur = dags.random_dag(rng, max(8, nodes), m["T"], 8, window=6)
+        graphs += [cur] + [dags.local_rewrite(rng, cur, m["T"]) for _ in range(4)]
+        env_off.append(len(graphs))
+    blob, _ = gpu_util.default_weights({"model": m, "n_nodes": np.array([max(8, nodes)])}, 6)
+    full, delta, rows = _run(m, graphs, env_off, blob)
+    gpu_util.assert_close(delta, full, "fp32", "by graph")
+    # the same environments beside one whose graph is too large for the per-graph kernel
+    big = dags.random_dag(rng, 16385, m["T"], 8, window=6)
+    full2, delta2, rows2 = _run(m, graphs + [big], env_off + [len(graphs) + 1], blob)
+    gpu_util.assert_close(delta2, full2, "fp32", "pass by pass")
+    assert [r + 16385 for r in rows] == rows2
