@@ -202,6 +202,7 @@ k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restri
 
 
 // ---- fp32 storage, many rows: the product on the tensor cores with every operand split in two ----------------
+// (the widths whose split W does not fit k_xform_tf32: 160, 224 and more than 256)
 // x = hi + lo with hi = tf32(x) and lo = tf32(x - hi); Z = sum hi_a hi_b + hi_a lo_b + lo_a hi_b in fp32
 // accumulators (mma.sync m16n8k8, the small terms first): the dropped lo_a lo_b term is below 2^-22 of the
 // product, i.e. the result is as good as an fp32 FMA chain in another order.  CTA tile 128 rows x 128 columns,
@@ -359,13 +360,16 @@ static bool fuse_scores(const Dims& d, const LayerWeights& lw, int tile_cols, co
 }
 
 int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void* Z, float* scores,
-                      Window win, cudaStream_t st) {
+                      Window win, int32_t* status, cudaStream_t st) {
   const int64_t rows = int64_t(win.row_end) - win.row_begin;
   if (rows <= 0) return 0;
   const size_t off = size_t(win.row_begin - win.win_base) * d.H;
   float2* sc = reinterpret_cast<float2*>(scores) + size_t(win.row_begin - win.win_base) * d.K;
   if (rows >= 8192 && d.dtype == XRL_FP32 && d.H % XK == 0) {
-    // fp32 storage: split operands on the tensor cores
+    // fp32 storage: split operands on the tensor cores (below 8,192 rows too few tiles for the SMs: FFMA)
+    const int k = launch_xform_tf32(d, static_cast<const float*>(h) + off, lw, static_cast<float*>(Z) + off, sc, rows, status, st);
+    if (k == 1) return 1;
+    if (k == 0) return 1 + launch_scores(d, Z, lw, scores, win, st);
     dim3 gx(unsigned((rows + XM - 1) / XM), unsigned((d.H + XN - 1) / XN));
     const size_t smem = sizeof(uint32_t) * 4 * XK * XS;
     const int w = d.H / d.K;

@@ -570,7 +570,7 @@ int run_node_layers(xrl_ctx* ctx, const xrl_batch* b, int layers, cudaStream_t s
                             ctx->status.as<int32_t>(), st);
     if (k < 0 && !d.zmerged)
       k = launch_xform_simt(d, h_in, ctx->dw.layer[l], Zl, Sl, win,
-                            st);
+                            ctx->status.as<int32_t>(), st);
     if (k < 0) return -1;                       // merged rows: only the tensor-core transform writes them
     pf.end(FAM_XFORM, slot, k, st);
     n += k;
@@ -1053,7 +1053,8 @@ xrl_status xrl_encode_delta(xrl_ctx* ctx, const xrl_batch* b, const int32_t* bas
       k = launch_xform_umma(d, ctx->h.p, ctx->dw.layer[l], ctx->Z.p, ctx->scores.as<float>(), wp,
                             ctx->status.as<int32_t>(), st);
     if (k < 0 && !d.zmerged)
-      k = launch_xform_simt(d, ctx->h.p, ctx->dw.layer[l], ctx->Z.p, ctx->scores.as<float>(), wp, st);
+      k = launch_xform_simt(d, ctx->h.p, ctx->dw.layer[l], ctx->Z.p, ctx->scores.as<float>(), wp,
+                            ctx->status.as<int32_t>(), st);
     if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
     pf.end(FAM_XFORM, slot, k, st);
     n_launch += k;

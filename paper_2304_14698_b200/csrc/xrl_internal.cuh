@@ -150,7 +150,9 @@ int launch_embed(const Dims& d, const int32_t* rowptr, const int32_t* col, const
                  const int32_t* row_list = nullptr, const void* eattr = nullptr);
 // scores: [N][K] pairs {s_src, s_dst} (float2), both already multiplied by log2(e)
 int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void* Z, float* scores,
-                      Window win, cudaStream_t st);
+                      Window win, int32_t* status, cudaStream_t st);
+int launch_xform_tf32(const Dims& d, const float* h, const LayerWeights& lw, float* Z, float2* scores, int64_t rows,
+                      int32_t* status, cudaStream_t st);
 int launch_rows_times_matrix(const Dims& d, const float* G, const void* Wt, float* out, int rows, cudaStream_t st);
 bool embed_umma_supported(const Dims& d);
 int embed_umma_kpad(const Dims& d);

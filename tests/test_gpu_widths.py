@@ -60,3 +60,35 @@ def test_bf16_widths_with_many_tiles_per_cta(xo, H, K):
                 assert (got[i] == got[0]).all()
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K", [(32, 4), (64, 1), (96, 3), (128, 16), (192, 6), (192, 1), (256, 8), (256, 2)])
+@pytest.mark.parametrize("copies", [6, 30])
+def test_fp32_widths_on_many_rows(xo, H, K, copies):
+    """The split-operand transform (8,192 rows and more): widths with one and several column slices, heads within a slice and
+    across, a last tile of 40 or 72 rows, one and several tiles per CTA."""
+    import paper_2304_14698_b200 as xrl
+    rng = dags.make_rng(H + K)
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=24, Dg=1, dtype="fp32", A_max=64)
+    n = 1372
+    g = dags.random_dag(rng, n, m["T"], 8)
+    batch = dags.flatten([g] * copies, [0, copies], 64)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 4)
+    one = dags.flatten([g], [0, 1], 64)
+    st, packed = xo.pack(one)
+    assert st == 0
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        for layer in (1, 2):
+            got = xrl.xrl_debug_node_features(ag.ctx, ag.batch, layer, H).reshape(copies, n, H)
+            want = xo.encode(m, blob, one, packed, dump_layer=layer, want_nodes=True)["nodes"]
+            # every copy against the definition (the attention kernel takes producers singly or in pairs as a copy's rows
+            # fall into its blocks, so copies agree within the fp32 bound, not bit for bit)
+            for i in range(copies):
+                gpu_util.assert_close(got[i], want, "fp32", f"copy {i} after stage {layer}")
+        assert ag.device_status() == 0
+    finally:
+        ag.close()
