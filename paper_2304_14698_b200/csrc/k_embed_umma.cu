@@ -44,7 +44,8 @@ template <int NS> struct ECfg {
   static constexpr int TMEM_COLS = 2 * ACC_COLS;
 };
 
-template <int NS>
+// SLICED: hidden above 256, a CTA per slice of NS columns (the last one may be narrower)
+template <int NS, bool SLICED>
 __global__ void __launch_bounds__(kThreads, 1)
 k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_h,
              const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -57,7 +58,8 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int num_tiles = (rows + BM - 1) / BM;
   const int kchunks = (ksteps + 3) / 4;
-  const int slice = int(blockIdx.x) % slices, first = int(blockIdx.x) / slices, step = int(gridDim.x) / slices;
+  const int slice = SLICED ? int(blockIdx.x) % slices : 0, first = SLICED ? int(blockIdx.x) / slices : int(blockIdx.x);
+  const int step = SLICED ? int(gridDim.x) / slices : int(gridDim.x);
   const int col0 = slice * NS, cols = min(NS, H - col0);
 
   if ((base & 1023u) != 0) {
@@ -143,11 +145,13 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
           for (int t = 0; t < 32; ++t) v[1][t] = 0u;
         }
         tc_wait_ld();
-        if (c * 64 >= cols) continue;            // columns that do not exist (the same for all threads)
-        // the two staging tiles alternate from store to store, across tiles too (a tile may have an odd number of chunks)
+        if (SLICED && c * 64 >= cols) continue;  // columns that do not exist (the same for all threads)
+        // the two staging tiles alternate from store to store, across tiles too (a tile may have an odd number of chunks; an
+        // even number starts every tile at the first)
+        const int sb = !SLICED && (NS + 63) / 64 % 2 == 0 ? c & 1 : int(stores & 1);
         if (leader) tma_wait_read<1>();
         epi_barrier();
-        uint8_t* stage = smem + C::OFF_OUT + (stores & 1) * CHUNK_BYTES + row_in_tile * 128;
+        uint8_t* stage = smem + C::OFF_OUT + sb * CHUNK_BYTES + row_in_tile * 128;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const uint32_t* z = &v[j >> 2][(j & 3) * 8];
@@ -161,7 +165,7 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
         fence_async_smem();
         epi_barrier();
         if (leader) {
-          tma_store_2d(&map_h, base + C::OFF_OUT + (stores & 1) * CHUNK_BYTES, col0 + c * 64, tile * BM);
+          tma_store_2d(&map_h, base + C::OFF_OUT + sb * CHUNK_BYTES, col0 + c * 64, tile * BM);
           tma_commit();
         }
         ++stores;
@@ -253,13 +257,13 @@ __global__ void k_build_w0ext(const bf16* __restrict__ W0, const float* __restri
   out[i] = __float2bfloat16_rn(v);
 }
 
-template <int NS>
+template <int NS, bool SLICED>
 int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int32_t* op,
              const void* shape, const void* w0ext_t, void* h, Window win, const int32_t* row_list,
              int32_t* status, cudaStream_t st, const void* eattr) {
   using C = ECfg<NS>;
   static bool attr_set[64] = {};
-  if (!ensure_dynamic_smem(k_embed_umma<NS>, C::SMEM_BYTES, attr_set)) return -1;
+  if (!ensure_dynamic_smem(k_embed_umma<NS, SLICED>, C::SMEM_BYTES, attr_set)) return -1;
   const int op_pieces = (d.T + 7) / 8;
   const int ksteps = (4 + op_pieces + 1) / 2;
   const int kpad = ((ksteps + 3) / 4) * KCH;
@@ -270,7 +274,7 @@ int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int
   const int tiles = int((rows + BM - 1) / BM);
   const int slices = (d.H + NS - 1) / NS, groups = kNumSMs / slices;
   const int grid = (tiles < groups ? tiles : groups) * slices;
-  k_embed_umma<NS><<<grid, kThreads, C::SMEM_BYTES, st>>>(mw, mh, rowptr, col, op,
+  k_embed_umma<NS, SLICED><<<grid, kThreads, C::SMEM_BYTES, st>>>(mw, mh, rowptr, col, op,
                                                          static_cast<const bf16*>(shape), row_list,
                                                          win.row_begin, int(rows), op_pieces, ksteps, status,
                                                          static_cast<const bf16*>(eattr), d.H, slices);
@@ -300,8 +304,10 @@ int launch_embed_umma(const Dims& d, const int32_t* rowptr, const int32_t* col, 
                       cudaStream_t st, const int32_t* row_list, const void* eattr) {
   if (int64_t(win.row_end) - win.row_begin <= 0) return 0;
 #define EMBED_CASE(NS_) \
-  case NS_: return launch_h<NS_>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
-  switch (d.H < 256 ? d.H : 256) {                // (above 256: slices of 256 columns, the rows gathered for each)
+  case NS_: return launch_h<NS_, false>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
+  if (d.H > 256)                                  // slices of 256 columns, the rows gathered for each
+    return launch_h<256, true>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
+  switch (d.H) {
     EMBED_CASE(32) EMBED_CASE(64) EMBED_CASE(96) EMBED_CASE(128) EMBED_CASE(160) EMBED_CASE(192) EMBED_CASE(224)
     EMBED_CASE(256)
     default: return -1;
