@@ -276,8 +276,8 @@ xrl_status xrl_sample(xrl_ctx* ctx, const float* probs, int32_t num_envs, int32_
  * The forward pass is that of xrl_encode and xrl_policy_value with every layer's input and Z kept; the reverse
  * pass runs layer by layer in fp32 (ReLU'(0) = 0, LeakyReLU'(0) = 0.2; where the clipped term of Eq. 3 is
  * the smaller one its slope is zero).  For a bf16 model the gradient of W0 and of the layer matrices is the
- * one with respect to the stored (rounded) values.  Sums over rows use floating-point atomics: the last
- * bits of a gradient may differ from run to run.
+ * one with respect to the stored (rounded) values.  Sums over rows use floating-point atomics (and the lists by
+ * producer are filled in the order the hardware serves them): the last bits of a gradient may differ from run to run.
  *   g0        DEVICE fp32 [B x Dg] or NULL            mask      DEVICE u8 [num_envs x A_max]
  *   action    DEVICE int32 [num_envs]  in [0, A_max], A_max = No-Op; an action the mask excludes raises
  *                                      XRL_ERR_INVALID_ARG in the device status word (results undefined)
@@ -286,7 +286,8 @@ xrl_status xrl_sample(xrl_ctx* ctx, const float* probs, int32_t num_envs, int32_
  *   grad      DEVICE fp32, laid out like the weight blob (xrl_weights_size bytes), overwritten
  *   logp_out  DEVICE fp32 [num_envs] or NULL: log pi(action_e) under the current weights
  * The first call allocates the workspace for the context's capacities ((L + 2) copies of the node features,
- * L of the transformed features Z and three fp32 ones) and therefore synchronises; later calls only enqueue.  Not recordable
+ * L of the transformed features Z, three fp32 ones, and for hidden 128 or 256 the lists by producer: 8 * heads
+ * bytes per node and edge and 12 more per edge) and therefore synchronises; later calls only enqueue.  Not recordable
  * (XRL_ERR_STATE between xrl_graph_begin and xrl_graph_launch).  XRL_ERR_UNSUPPORTED when
  * (T + 8) x H floats exceed one SM's shared memory (227 KB): the operator block of W0's gradient and a tile
  * of eight rows are kept there.
