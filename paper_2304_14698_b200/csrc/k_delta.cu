@@ -212,17 +212,20 @@ inline int grid(int64_t n) { return int((n + TB - 1) / TB); }
 
 }  // namespace
 
-// base, level, counts [L + 2] (cursor [L + 2] zeroed) of the whole batch in one launch; -1: graphs too large for it
+// base, level, counts [L + 2] (cursor [L + 2] zeroed) of the whole batch in one launch; -1: graphs too large for it, -2: the
+// launch failed (nothing that reads the levels may follow)
 int launch_delta_graphs(const DeltaIn& in, int32_t B, int32_t max_n, int32_t L, int32_t* base, int32_t* level, int32_t* counts,
                         int32_t* cursor, cudaStream_t st) {
   if (max_n > kGraphNodes || L > 64) return -1;
   static bool attr[64] = {};
   const size_t smem = (size_t(max_n) * 5 + 15) & ~size_t(15);
-  if (smem > 48 * 1024 && !ensure_dynamic_smem(k_delta_graph, 5 * kGraphNodes, attr)) return -1;
+  // (asked for whatever the size: without it the kernel's own arrays count against the 48 KB too)
+  if (!ensure_dynamic_smem(k_delta_graph, 5 * kGraphNodes, attr)) return -1;
   cudaMemsetAsync(counts, 0, sizeof(int32_t) * size_t(L + 2), st);
   cudaMemsetAsync(cursor, 0, sizeof(int32_t) * size_t(L + 2), st);
   if (in.N <= 0 || B <= 0) return 0;
   k_delta_graph<<<B, TB, smem, st>>>(in, L, max_n, base, level, counts);
+  if (cudaPeekAtLastError() != cudaSuccess) return -2;
   return 1;
 }
 int launch_delta_level0(const DeltaIn& in, int32_t* valid, int32_t* base, int32_t* level, cudaStream_t st) {
