@@ -182,7 +182,12 @@ k_delta_graph(DeltaIn in, int32_t L, int32_t cap_n, int32_t* __restrict__ base, 
       const int32_t e0 = in.rowptr[nb + i], m = in.rowptr[nb + i + 1] - e0, f0 = in.rowptr[b];
       if (m == in.rowptr[b + 1] - f0) {
         dirty = false;
-        for (int32_t k = 0; k < m && !dirty; ++k) dirty = base_s[in.col[e0 + k] - nb] != in.col[f0 + k];
+        // A producer outside the graph (a batch that was reported bad may hold one: the slots of a graph without nodes fall
+        // into the row before it) equals no node of the current graph; only rows whose producers all lie inside stay clean
+        for (int32_t k = 0; k < m && !dirty; ++k) {
+          const uint32_t j = uint32_t(in.col[e0 + k] - nb);
+          dirty = j >= uint32_t(n) || base_s[j] != in.col[f0 + k];
+        }
       }
     }
     lv[i] = dirty ? 0 : 127;
@@ -190,7 +195,7 @@ k_delta_graph(DeltaIn in, int32_t L, int32_t cap_n, int32_t* __restrict__ base, 
   for (int32_t t = 1; t <= L; ++t) {
     __syncthreads();
     for (int32_t i = tid; i < n; i += TB) {
-      if (lv[i] != 127) continue;
+      if (lv[i] != 127) continue;                     // (so its producers are nodes of this graph)
       for (int32_t e = in.rowptr[nb + i], e1 = in.rowptr[nb + i + 1]; e < e1; ++e)
         if (lv[in.col[e] - nb] < t) { lv[i] = int8_t(t); break; }
     }

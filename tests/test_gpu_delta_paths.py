@@ -68,3 +68,42 @@ def test_levels_by_graph_around_the_default_limit_of_shared_memory(nodes):
     full2, delta2, rows2 = _run(m, graphs + [big], [0, 3, 4], blob)
     gpu_util.assert_close(delta2, full2, "fp32", "pass by pass")
     assert [r + 16385 for r in rows] == rows2
+
+
+@pytest.mark.parametrize("extra", [1, 3])
+def test_batch_with_edges_on_an_empty_graph(extra):
+    """A graph without nodes that was given edges is reported; its slots fall into the last row of the graph before it, whose
+    node can then look like its twin by its number of producers.  Delta encoding of such a batch stays inside its arrays and
+    gives what the full encoder gives."""
+    import torch
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=11, S=8, H=64, K=2, L=3, Hm=16, Dg=1, dtype="fp32", A_max=4)
+    rng = dags.make_rng(40 + extra)
+    n = 300
+    cur = dags.random_dag(rng, n, m["T"], 8, window=6)
+    last = np.arange(n - 1 - extra, n - 1, dtype=np.int32)           # the last node reads `extra` nodes for certain
+    keep = cur["edge_dst"] != n - 1
+    cur["edge_src"] = np.concatenate([cur["edge_src"][keep], last])
+    cur["edge_dst"] = np.concatenate([cur["edge_dst"][keep], np.full(extra, n - 1, np.int32)])
+    twin = dict(cur, twin=np.arange(n, dtype=np.int32))
+    lost = dict(twin, edge_src=cur["edge_src"][:-extra], edge_dst=cur["edge_dst"][:-extra])
+    empty = dict(op=np.zeros(0, np.int32), shape=np.zeros((0, 8), np.float32), edge_src=np.zeros(extra, np.int32),
+                 edge_dst=np.ones(extra, np.int32), twin=np.zeros(0, np.int32))
+    batch = dags.flatten([cur, twin, lost, empty, twin], [0, 5], m["A_max"])
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights({"model": m, "n_nodes": np.array([n])}, 6)
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        full = torch.empty((5, m["H"]), device="cuda")
+        delta = torch.empty_like(full)
+        xrl.xrl_encode(ag.ctx, ag.batch, full)
+        xrl.xrl_encode_delta(ag.ctx, ag.batch, torch.from_numpy(batch["base_id"]).cuda(), delta)
+        torch.cuda.synchronize()
+        assert ag.device_status() == 2
+        gpu_util.assert_close(delta.cpu().numpy(), full.cpu().numpy(), "fp32", "delta of a bad batch")
+        rows = xrl.xrl_delta_rows(ag.ctx, m["L"])
+        assert rows == [n + 1] * (m["L"] + 1)            # the current graph and the one row that gained the slots
+    finally:
+        ag.close()
