@@ -27,11 +27,12 @@ constexpr int G = 2;                 // k_dz_gather: groups of four rows in flig
 constexpr int LIST = 96;             // list capacity per piece, a multiple of 8
 
 // ---- transposed lists ------------------------------------------------------------------------------------------
-// (the slots that rows own end at rowptr[N]: a batch that was reported bad may have been given more)
+// (the slots that rows own are rowptr[0] .. rowptr[N] - 1: a batch that was reported bad may have been given others, before
+// them when its first graph has edges and no nodes, or behind)
 __global__ void k_t_count(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int32_t N, int32_t E,
                           int32_t* __restrict__ cnt) {
   const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < E && e < __ldg(rowptr + N)) atomicAdd(&cnt[col[e]], 1);
+  if (e < E && e >= __ldg(rowptr) && e < __ldg(rowptr + N)) atomicAdd(&cnt[col[e]], 1);
 }
 // cnt holds the counts on entry and zeros on return; inv[e]: where the entry of slot e sits (every list is preceded by
 // its producer's own entry, so entry number = list position + producer + 1)

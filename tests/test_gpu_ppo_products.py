@@ -72,3 +72,39 @@ def _compare(xo, batch, m):
                         entrywise=BF16_ENTRYWISE if dtype == "bf16" else None)
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K,dtype,both,extra", [(128, 4, "fp32", False, 1), (128, 2, "bf16", True, 7),
+                                                  (256, 8, "bf16", False, 200), (256, 4, "bf16", True, 200)])
+def test_gradient_of_a_batch_whose_first_graph_has_edges_and_no_nodes(H, K, dtype, both, extra):
+    """Such a batch is reported; its first slots belong to no row.  The gradient is then that of the batch without them, up to
+    the order of its atomic sums (a few thousand fp32 terms: 1e-5 of the gradient)."""
+    import torch
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3, both_ways=both)
+    rng = dags.make_rng(H + extra)
+    rest = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (60, 64, 90, 61)]
+    got = []
+    for k in (extra, 0):
+        empty = dict(op=np.zeros(0, np.int32), shape=np.zeros((0, 8), np.float32), edge_src=np.zeros(k, np.int32),
+                     edge_dst=np.ones(k, np.int32))
+        batch = dags.flatten([empty] + rest, [0, 2, 5], 3)
+        batch["model"] = m
+        blob, _ = gpu_util.default_weights({"model": m, "n_nodes": np.array([60])}, 7)
+        ag = gpu_util.make_agent(batch)
+        try:
+            ag.set_weights(blob)
+            ag.pack(batch)
+            f32 = lambda *a: torch.tensor(a, device="cuda")
+            grad, loss = torch.empty(len(blob), device="cuda"), torch.empty(4, device="cuda")
+            xrl.xrl_ppo_grad(ag.ctx, ag.batch, torch.from_numpy(batch["mask"]).cuda(),
+                             torch.tensor([0, 3], dtype=torch.int32, device="cuda"), f32(-0.7, -1.0), f32(1.0, -0.5),
+                             f32(0.3, 0.1), loss, grad)
+            torch.cuda.synchronize()
+            assert ag.device_status() == (2 if k else 0)
+            got.append((loss.cpu().numpy(), grad.cpu().numpy().astype(np.float64)))
+        finally:
+            ag.close()
+    np.testing.assert_allclose(got[0][0], got[1][0], rtol=1e-5, atol=1e-6)
+    assert np.linalg.norm(got[1][1]) > 0
+    assert np.linalg.norm(got[0][1] - got[1][1]) <= 1e-5 * np.linalg.norm(got[1][1])
