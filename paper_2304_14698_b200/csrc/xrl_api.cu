@@ -1203,9 +1203,12 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   int n = run_node_layers(ctx, b, L, st, false, nullptr, 0, -1, hs, zs, ss);
   if (n < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
   const float* wb = ctx->w_f32.as<float>();
-  // Eq. 8's per-graph sums as in xrl_encode: readout chunks, added per graph by the next kernel
-  n += launch_readout(d, hs[L], b->d_chunk_row0, b->d_chunk_row1, 0, b->num_chunks, ctx->partial.as<float>(), 0, st);
-  const int kh = launch_ppo_heads(d, ctx->dw, grad, wb, hs[L], ctx->partial.as<float>(), b->d_graph_chunk_off,
+  // Eq. 8's per-graph sums as in xrl_encode: readout chunks, added per graph by the next kernel.  They wait in dz (a chunk has
+  // at least one row, and dz is not written before the heads are done): the context's own partial sums belong to
+  // xrl_encode, which may run on another stream meanwhile
+  float* readout = dz;
+  n += launch_readout(d, hs[L], b->d_chunk_row0, b->d_chunk_row1, 0, b->num_chunks, readout, 0, st);
+  const int kh = launch_ppo_heads(d, ctx->dw, grad, wb, hs[L], readout, b->d_graph_chunk_off,
                                   b->seg_id.as<int32_t>(), g0, b->d_env_off, mask, action, logp_old, adv, ret, eps, c1, c2, b->B,
                                   b->num_envs, b->N, heads_ws, loss_out, dh_a, logp_out, ctx->status.as<int32_t>(), st);
   if (kh < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }

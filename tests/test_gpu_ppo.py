@@ -280,3 +280,50 @@ def test_gradient_of_a_batch_packed_range_by_range(xo, monkeypatch):
         _check_grad(m, grad.cpu().numpy().astype(np.float64), mir["grad"], GRAD_TOL["bf16 mirrored"], "mirrored")
     finally:
         ag.close()
+
+
+def test_gradient_beside_an_encode_on_another_stream():
+    """The two calls share a context but no buffer they write: an encode beside training steps gives its embeddings bit for
+    bit, and the gradients stay what they are alone (up to the order of their atomic sums)."""
+    import torch
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=12, S=8, H=64, K=2, L=1, Hm=24, Dg=1, dtype="fp32", A_max=31)
+    rng = dags.make_rng(5)
+    g = dags.random_dag(rng, 200, m["T"], 8)
+    graphs = [g] + [dags.local_rewrite(rng, g, m["T"]) for _ in range(31)]
+    batch = dags.flatten(graphs, [0, 32], 31)
+    other = dags.flatten(graphs[::-1][:31] + [graphs[0]], [0, 20, 32], 31)
+    blob, _ = gpu_util.default_weights(dict(batch, model=m), 5)
+    ag = xrl.Agent(m, 32, 2, int(batch["n_nodes"].sum()), int(batch["n_edges"].sum()))
+    second = None
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        first, ag.batch = ag.batch, None
+        second = ag.pack(other)
+        mask = torch.from_numpy(other["mask"]).cuda()
+        action = torch.full((2,), 31, dtype=torch.int32, device="cuda")
+        f = lambda *a: torch.tensor(a, device="cuda")
+        logp, adv, ret = f(-2.0, -3.0), f(1.0, -1.0), f(0.5, 0.2)
+        loss = torch.empty(4, device="cuda")
+        grads = torch.empty((41, len(blob)), device="cuda")
+        embs = torch.empty((41, 32, 64), device="cuda")
+        train = lambda i: xrl.xrl_ppo_grad(ag.ctx, second, mask, action, logp, adv, ret, loss, grads[i])
+        train(40)
+        xrl.xrl_encode(ag.ctx, first, embs[40])
+        torch.cuda.synchronize()
+        sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+        for i in range(40):
+            with torch.cuda.stream(sa):
+                xrl.xrl_encode(ag.ctx, first, embs[i])
+            with torch.cuda.stream(sb):
+                train(i)
+        torch.cuda.synchronize()
+        assert ag.device_status() == 0
+        assert (embs[:40] == embs[40]).all()
+        far = (grads[:40] - grads[40]).norm(dim=1) / grads[40].norm()
+        assert far.max() < 1e-5
+    finally:
+        if second is not None:
+            xrl.xrl_batch_free(ag.ctx, first)
+        ag.close()
