@@ -110,6 +110,7 @@ struct xrl_ctx {
   bool capturing = false;
   // reverse pass: saved layer inputs and gradient scratch (allocated on the first xrl_ppo_grad)
   DeviceBuf bw;
+  bool bw_lists = false;    // with the lists by producer
   cudaStream_t last_pipe = nullptr;   // stream of the last batch that was packed range by range (its kernels
                                       // report bad graphs too: xrl_last_device_status waits for it as well)
 };
@@ -1160,20 +1161,28 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   const size_t heads_bytes = up(4 * ppo_heads_workspace_floats(d, c.max_graphs, c.max_envs));
   const size_t z_bytes = up(Nmax * z_row_bytes(d));
   // dz by producer: transposed neighbour lists (N + 1, E, E ints; scratch), one {alpha, score gradient} per entry and head
-  const bool gather = bwd_gather_supported(d);
   const size_t Emax = size_t(c.max_edges) * (c.neighbourhood ? 2 : 1);
   const size_t t_rows = up(4 * (Nmax + 1)), t_slots = up(4 * (Emax + 1)),
                t_scratch = up(4 * (Nmax + scan_workspace_ints(int64_t(Nmax) + 1))),
                t_entries = up(8 * size_t(c.heads) * (Nmax + Emax + 4));
-  const size_t lists_bytes = gather ? t_rows + 2 * t_slots + t_scratch + t_entries : 0;
   if (!ctx->bw.p) {
-    if (ctx->bw.alloc(lists_bytes + size_t(L + 2) * h_bytes + size_t(L) * (z_bytes + ds_bytes) + 3 * f_bytes + ds_bytes +
-                      heads_bytes) != cudaSuccess) {
+    const size_t bytes = size_t(L + 2) * h_bytes + size_t(L) * (z_bytes + ds_bytes) + 3 * f_bytes + ds_bytes + heads_bytes;
+    // without room for the lists dz is scattered with atomics: slower, but the call does not need them
+    ctx->bw_lists = bwd_gather_supported(d) && Nmax + Emax < (size_t(1) << 31);      // (entry numbers are 32 bits)
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (ctx->bw_lists) e = ctx->bw.alloc(bytes + t_rows + 2 * t_slots + t_scratch + t_entries);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      ctx->bw_lists = false;
+      e = ctx->bw.alloc(bytes);
+    }
+    if (e != cudaSuccess) {
       cudaGetLastError();
       ctx->bw.p = nullptr;
       return XRL_ERR_ALLOC;
     }
   }
+  const bool gather = ctx->bw_lists;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (b->nparts > 0) { const xrl_status j = join_parts(b, st); if (j != XRL_OK) return j; }
   char* p = ctx->bw.as<char>();

@@ -108,3 +108,39 @@ def test_gradient_of_a_batch_whose_first_graph_has_edges_and_no_nodes(H, K, dtyp
     np.testing.assert_allclose(got[0][0], got[1][0], rtol=1e-5, atol=1e-6)
     assert np.linalg.norm(got[1][1]) > 0
     assert np.linalg.norm(got[0][1] - got[1][1]) <= 1e-5 * np.linalg.norm(got[1][1])
+
+
+def test_gradient_where_the_lists_by_producer_do_not_fit():
+    """A context whose workspace fits the GPU's free memory without those lists and not with them: the call scatters instead
+    of refusing, with the same gradient (fp32 sums in another order: 1e-5)."""
+    import torch
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=9, S=8, H=128, K=16, L=1, Hm=20, Dg=1, dtype="fp32", A_max=3)
+    rng = dags.make_rng(8)
+    batch = dags.flatten([dags.random_dag(rng, n, m["T"], 8, window=6) for n in (60, 64, 90, 61)], [0, 4], 3)
+    blob, _ = gpu_util.default_weights(dict(batch, model=m), 7)
+    N, E = 50_000, 6_000_000
+    lists = 8 * m["K"] * (N + E)
+    f32 = lambda *a: torch.tensor(a, device="cuda")
+    mask, action = torch.from_numpy(batch["mask"]).cuda(), torch.tensor([1], dtype=torch.int32, device="cuda")
+    logp, adv, ret, loss = f32(-1.0), f32(1.0), f32(0.3), torch.empty(4, device="cuda")
+    grads, used, filler = [torch.empty(len(blob), device="cuda") for _ in range(2)], 0, None
+    for i in range(2):
+        ag = xrl.Agent(m, 4, 1, N, E)
+        try:
+            ag.set_weights(blob)
+            ag.pack(batch)
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            free = torch.cuda.mem_get_info()[0]
+            if i:
+                filler = torch.empty(free - used + lists // 2, dtype=torch.uint8, device="cuda")
+            xrl.xrl_ppo_grad(ag.ctx, ag.batch, mask, action, logp, adv, ret, loss, grads[i])
+            torch.cuda.synchronize()
+            used = free - torch.cuda.mem_get_info()[0]
+            assert ag.device_status() == 0
+        finally:
+            ag.close()
+    del filler
+    torch.cuda.empty_cache()
+    assert (grads[1] - grads[0]).norm() <= 1e-5 * grads[0].norm() and grads[0].norm() > 0
