@@ -5,9 +5,10 @@
 //   piece 0        bf16(ebar)            ebar = fp32 sum of the producers' shape features
 //   piece 1        the node's own shape features (already bf16)
 //   pieces 2..     the one-hot operator id
-//   next piece     bf16(ebar - bf16(ebar)): with it the product sees ebar to ~2^-17 relative
-//   next piece     (1, 1, 0, ...) against two rows holding b0 split the same way into high and low
-//                  bf16 parts, so that the bias enters with fp32-like accuracy
+//   next pieces    what the bf16 parts so far leave of ebar, rounded to bf16: one such piece (PARTS = 2) and the product
+//                  sees ebar to ~2^-17 relative, or two (PARTS = 3) and it sees every bit of it
+//   next piece     (1, 1, 0, ...) or (1, 1, 1, 0, ...) against two or three rows holding b0 split the same way
+// PARTS = 2 for hidden 128 and 256, 3 for the other widths.
 // W0ext^T (K-major, built once when the weights are set) stays resident in shared memory; three
 // gather groups of 128 threads fill three A stages in turn; one thread issues tcgen05.mma; four
 // epilogue warps apply the ReLU, round to bf16 and store the tile with TMA.  The layer writes H b
@@ -44,8 +45,8 @@ template <int NS> struct ECfg {
   static constexpr int TMEM_COLS = 2 * ACC_COLS;
 };
 
-// SLICED: hidden above 256, a CTA per slice of NS columns (the last one may be narrower)
-template <int NS, bool SLICED>
+// SLICED: hidden above 256, a CTA per slice of NS columns (the last one may be narrower).  PARTS: see the header
+template <int NS, bool SLICED, int PARTS>
 __global__ void __launch_bounds__(kThreads, 1)
 k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_h,
              const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -202,18 +203,23 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
           for (int s = 0; s < kS; ++s) e[s] += f[s];
         }
       }
-      float hi[kS], lo[kS];
+      float part[PARTS][kS];                   // (the last one is rounded where it is packed)
 #pragma unroll
       for (int s = 0; s < kS; ++s) {
-        hi[s] = __bfloat162float(__float2bfloat16_rn(e[s]));
-        lo[s] = e[s] - hi[s];
+        float rest = e[s];
+#pragma unroll
+        for (int q = 0; q < PARTS - 1; ++q) {
+          part[q][s] = __bfloat162float(__float2bfloat16_rn(rest));
+          rest = PARTS == 3 && rest == part[q][s] ? 0.f : rest - part[q][s];     // (an infinite sum leaves nothing)
+        }
+        part[PARTS - 1][s] = rest;
       }
       const uint32_t use = lt / GROUPS;
       if (use > 0 && !mbar_wait(bar_a_empty(g), (use - 1) & 1)) { raise(status, XRL_ERR_TIMEOUT); break; }
       uint8_t* arow = smem + C::OFF_A + g * A_STAGE_BYTES + r * 128;
       for (int pc = 0; pc < pieces; ++pc) {
         uint4 val = make_uint4(0, 0, 0, 0);
-        if (pc == 0) val = pack(hi);
+        if (pc == 0) val = pack(part[0]);
         else if (pc == 1) val = own;
         else if (pc < 2 + op_pieces) {
           if (o >= 0 && (o >> 3) == pc - 2) {                 // bf16 1.0 = 0x3F80 at element o % 8
@@ -222,8 +228,12 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
             val.x = w == 0 ? one : 0u; val.y = w == 1 ? one : 0u;
             val.z = w == 2 ? one : 0u; val.w = w == 3 ? one : 0u;
           }
-        } else if (pc == 2 + op_pieces) val = pack(lo);
-        else if (pc == 3 + op_pieces) val.x = (lrow < rows) ? 0x3F803F80u : 0u;
+        } else if (pc == 2 + op_pieces) val = pack(part[1]);
+        else if (PARTS == 3 && pc == 3 + op_pieces) val = pack(part[PARTS - 1]);
+        else if (pc == 1 + PARTS + op_pieces && lrow < rows) {
+          val.x = 0x3F803F80u;
+          if (PARTS == 3) val.y = 0x3F80u;
+        }
         *reinterpret_cast<uint4*>(arow + (pc >> 3) * CHUNK_BYTES + (((pc & 7) ^ (r & 7)) << 4)) = val;
       }
       fence_async_smem();
@@ -242,31 +252,38 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
 
 // W0ext^T [H x kpad] bf16, K-major: column k of node-update input piece layout (see the header).
 __global__ void k_build_w0ext(const bf16* __restrict__ W0, const float* __restrict__ b0,
-                              bf16* __restrict__ out, int H, int T, int op_pieces, int kpad) {
+                              bf16* __restrict__ out, int H, int T, int op_pieces, int kpad, int parts) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= H * kpad) return;
   const int n = i / kpad, k = i - n * kpad;
-  const int k_lo = 16 + 8 * op_pieces, k_b = k_lo + 8;
+  const int k_rest = 16 + 8 * op_pieces, k_b = k_rest + 8 * (parts - 1);
   float v = 0.f;
-  if (k < 8) v = __bfloat162float(W0[size_t(k) * H + n]);                          // edge aggregate (high)
+  if (k < 8) v = __bfloat162float(W0[size_t(k) * H + n]);                          // edge aggregate (first part)
   else if (k < 16) v = __bfloat162float(W0[size_t(kS + T + (k - 8)) * H + n]);     // own shape
   else if (k < 16 + T) v = __bfloat162float(W0[size_t(kS + (k - 16)) * H + n]);    // one-hot operator
-  else if (k >= k_lo && k < k_lo + 8) v = __bfloat162float(W0[size_t(k - k_lo) * H + n]);  // aggregate (low)
-  else if (k == k_b) v = __bfloat162float(__float2bfloat16_rn(b0[n]));
-  else if (k == k_b + 1) v = b0[n] - __bfloat162float(__float2bfloat16_rn(b0[n]));
+  else if (k >= k_rest && k < k_b) v = __bfloat162float(W0[size_t((k - k_rest) & 7) * H + n]);   // its other parts
+  else if (k >= k_b && k < k_b + parts) {
+    v = b0[n];
+    for (int q = k_b; q < k; ++q) v -= __bfloat162float(__float2bfloat16_rn(v));
+  }
   out[i] = __float2bfloat16_rn(v);
 }
 
-template <int NS, bool SLICED>
+// Parts of the edge aggregate and of the bias.  Widths 128 and 256 keep two (their features have always been those); the
+// others keep three, so that all 24 bits of both reach the product, as in the CUDA-core kernel.  The third costs one piece:
+// nothing with 33 to 40 operators (an even number of pieces either way), a k-step of four or five with 32.
+constexpr int parts_of(int H) { return H == 128 || H == 256 ? 2 : 3; }
+int op_pieces_of(const Dims& d) { return (d.T + 7) / 8; }
+int ksteps_of(const Dims& d) { return (2 + op_pieces_of(d) + parts_of(d.H) + 1) / 2; }
+
+template <int NS, bool SLICED, int PARTS>
 int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int32_t* op,
              const void* shape, const void* w0ext_t, void* h, Window win, const int32_t* row_list,
              int32_t* status, cudaStream_t st, const void* eattr) {
   using C = ECfg<NS>;
   static bool attr_set[64] = {};
-  if (!ensure_dynamic_smem(k_embed_umma<NS, SLICED>, C::SMEM_BYTES, attr_set)) return -1;
-  const int op_pieces = (d.T + 7) / 8;
-  const int ksteps = (4 + op_pieces + 1) / 2;
-  const int kpad = ((ksteps + 3) / 4) * KCH;
+  if (!ensure_dynamic_smem(k_embed_umma<NS, SLICED, PARTS>, C::SMEM_BYTES, attr_set)) return -1;
+  const int op_pieces = op_pieces_of(d), ksteps = ksteps_of(d), kpad = embed_umma_kpad(d);
   const int64_t rows = int64_t(win.row_end) - win.row_begin;
   bf16* hp = static_cast<bf16*>(h) + size_t(win.row_begin - win.win_base) * d.H;
   CUtensorMap mw, mh;
@@ -274,7 +291,7 @@ int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int
   const int tiles = int((rows + BM - 1) / BM);
   const int slices = (d.H + NS - 1) / NS, groups = kNumSMs / slices;
   const int grid = (tiles < groups ? tiles : groups) * slices;
-  k_embed_umma<NS, SLICED><<<grid, kThreads, C::SMEM_BYTES, st>>>(mw, mh, rowptr, col, op,
+  k_embed_umma<NS, SLICED, PARTS><<<grid, kThreads, C::SMEM_BYTES, st>>>(mw, mh, rowptr, col, op,
                                                          static_cast<const bf16*>(shape), row_list,
                                                          win.row_begin, int(rows), op_pieces, ksteps, status,
                                                          static_cast<const bf16*>(eattr), d.H, slices);
@@ -284,19 +301,19 @@ int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int
 }  // namespace
 
 bool embed_umma_supported(const Dims& d) {
-  return d.dtype == XRL_BF16 && d.H % 32 == 0 && d.H <= 512 && d.T <= 96 && encode_fn() != nullptr;
+  // (two chunks of eight pieces hold 96 operators beside two parts, 88 beside three)
+  return d.dtype == XRL_BF16 && d.H % 32 == 0 && d.H <= 512 && ksteps_of(d) <= 8 && encode_fn() != nullptr;
 }
 
 // Elements in one row of W0ext^T (a multiple of 64).
 int embed_umma_kpad(const Dims& d) {
-  const int op_pieces = (d.T + 7) / 8;
-  return (((4 + op_pieces + 1) / 2 + 3) / 4) * KCH;
+  return ((ksteps_of(d) + 3) / 4) * KCH;
 }
 
 void build_w0ext(const Dims& d, const void* W0_store, const float* b0, void* out, cudaStream_t st) {
   const int kpad = embed_umma_kpad(d), n = d.H * kpad;
   k_build_w0ext<<<(n + 255) / 256, 256, 0, st>>>(static_cast<const bf16*>(W0_store), b0,
-                                                  static_cast<bf16*>(out), d.H, d.T, (d.T + 7) / 8, kpad);
+                                                  static_cast<bf16*>(out), d.H, d.T, op_pieces_of(d), kpad, parts_of(d.H));
 }
 
 int launch_embed_umma(const Dims& d, const int32_t* rowptr, const int32_t* col, const int32_t* op,
@@ -304,9 +321,9 @@ int launch_embed_umma(const Dims& d, const int32_t* rowptr, const int32_t* col, 
                       cudaStream_t st, const int32_t* row_list, const void* eattr) {
   if (int64_t(win.row_end) - win.row_begin <= 0) return 0;
 #define EMBED_CASE(NS_) \
-  case NS_: return launch_h<NS_, false>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
+  case NS_: return launch_h<NS_, false, parts_of(NS_)>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
   if (d.H > 256)                                  // slices of 256 columns, the rows gathered for each
-    return launch_h<256, true>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
+    return launch_h<256, true, 3>(d, rowptr, col, op, shape, w0ext_t, h, win, row_list, status, st, eattr);
   switch (d.H) {
     EMBED_CASE(32) EMBED_CASE(64) EMBED_CASE(96) EMBED_CASE(128) EMBED_CASE(160) EMBED_CASE(192) EMBED_CASE(224)
     EMBED_CASE(256)

@@ -34,6 +34,40 @@ def test_bf16_widths(xo, H, K, nodes):
         ag.close()
 
 
+@pytest.mark.parametrize("T", [21, 32, 88, 89, 96])
+@pytest.mark.parametrize("H", [32, 64, 96, 160, 192, 224, 320, 512])
+def test_bf16_node_update_keeps_every_bit_of_the_edge_sum_and_of_the_bias(H, T):
+    """Eq. 6 where all but 2^-19 cancels: an edge sum of 1 + 2^-9 + 2^-19 (20 bits) against the node's own features in the even
+    columns, one of 1 + 2^-9 + 2^-18 in a second node against a bias of -(1 + 2^-9 + 2^-19) in the odd ones.  The operands
+    are exact, so is every partial sum in fp32: the result is 2^-19 exactly."""
+    import numpy as np
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=T, S=8, H=H, K=1, L=0, Hm=8, Dg=1, dtype="bf16", A_max=1)
+    shape = np.zeros((6, 8), np.float32)
+    shape[:4, 0] = [1, 2.0**-9, 2.0**-19, 2.0**-18]
+    shape[4, :2] = [1, 2.0**-9]
+    g = dict(op=np.array([0, 1, 2, 3, T - 1, T - 1], np.int32), shape=shape,
+             edge_src=np.array([0, 1, 2, 0, 1, 3], np.int32), edge_dst=np.array([4, 4, 4, 5, 5, 5], np.int32))
+    batch = dags.flatten([g], [0, 1], 1)
+    batch["model"] = m
+    W0, b0 = np.zeros((16 + T, H), np.float32), np.zeros(H, np.float32)
+    W0[0] = 1
+    W0[8 + T:10 + T, ::2] = -1
+    b0[1::2] = -(1 + 2.0**-9 + 2.0**-19)
+    ag = gpu_util.make_agent(batch)
+    try:
+        blob = np.zeros(xrl.xrl_weights_size(ag.ctx) // 4, np.float32)
+        blob[:W0.size + H] = np.concatenate([W0.ravel(), b0])
+        ag.set_weights(blob)
+        ag.pack(batch)
+        h = xrl.xrl_debug_node_features(ag.ctx, ag.batch, 0, H)
+        assert ag.device_status() == 0
+        assert (h[4, ::2] == 2.0**-19).all()
+        assert (h[5, 1::2] == 2.0**-19).all()
+    finally:
+        ag.close()
+
+
 @pytest.mark.parametrize("H,K", [(64, 2), (192, 6), (320, 2)])
 def test_bf16_widths_with_many_tiles_per_cta(xo, H, K):
     """Output tiles with an odd number of 64-column chunks, several tiles per CTA: the staging buffers of one tile's last
