@@ -147,7 +147,12 @@ __global__ void k_delta_remap(int32_t N, int32_t L, const int32_t* __restrict__ 
 // The kernels up to the counts in one, a CTA per graph with the graph's base nodes and levels in shared memory: validation of
 // the hints, level 0, every layer's propagation (in place: a level written in pass t is not below t) and the counts.  The
 // separate kernels read rowptr, col and the levels of all nodes once per layer (2 M nodes, 4 layers: 20 + 19 + 4 x 13 + 7 us).
-constexpr int32_t kGraphNodes = 16384;                // 5 bytes of shared memory per node
+// One CTA walks a graph, so graphs of thousands of nodes are a long serial chain per CTA unless there are enough of them to
+// fill the GPU.  Whole call at hidden 64 (random graphs), passes over all nodes against this kernel: 1 layer, 64 graphs of
+// 1,000 / 2,000 / 4,000 / 8,000 nodes 104 / 104 / 107 / 124 us against 93 / 105 / 126 / 166; 4 layers 192 / 192 / 201 / 232
+// against 159 / 178 / 211 / 291; 4,000 nodes, 256 graphs 140 and 258 us against 142 and 233, 512 graphs 199 and 353 against
+// 188 and 291; 8,000 nodes, 256 graphs 200 and 343 against 242 and 376.
+constexpr int32_t kGraphNodes = 2048, kGraphNodesMany = 4096, kManyGraphs = 256;
 __global__ void __launch_bounds__(TB)
 k_delta_graph(DeltaIn in, int32_t L, int32_t cap_n, int32_t* __restrict__ base, int32_t* __restrict__ level,
               int32_t* __restrict__ counts) {
@@ -217,15 +222,12 @@ inline int grid(int64_t n) { return int((n + TB - 1) / TB); }
 
 }  // namespace
 
-// base, level, counts [L + 2] (cursor [L + 2] zeroed) of the whole batch in one launch; -1: graphs too large for it, -2: the
-// launch failed (nothing that reads the levels may follow)
+// base, level, counts [L + 2] (cursor [L + 2] zeroed) of the whole batch in one launch; -1: the passes over all nodes are
+// faster, -2: the launch failed (nothing that reads the levels may follow)
 int launch_delta_graphs(const DeltaIn& in, int32_t B, int32_t max_n, int32_t L, int32_t* base, int32_t* level, int32_t* counts,
                         int32_t* cursor, cudaStream_t st) {
-  if (max_n > kGraphNodes || L > 64) return -1;
-  static bool attr[64] = {};
-  const size_t smem = (size_t(max_n) * 5 + 15) & ~size_t(15);
-  // (asked for whatever the size: without it the kernel's own arrays count against the 48 KB too)
-  if (!ensure_dynamic_smem(k_delta_graph, 5 * kGraphNodes, attr)) return -1;
+  if (max_n > (B >= kManyGraphs ? kGraphNodesMany : kGraphNodes) || L > 64) return -1;
+  const size_t smem = (size_t(max_n) * 5 + 15) & ~size_t(15);      // (at most 20 KB: no opt-in)
   cudaMemsetAsync(counts, 0, sizeof(int32_t) * size_t(L + 2), st);
   cudaMemsetAsync(cursor, 0, sizeof(int32_t) * size_t(L + 2), st);
   if (in.N <= 0 || B <= 0) return 0;

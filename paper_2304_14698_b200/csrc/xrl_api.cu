@@ -1009,7 +1009,7 @@ xrl_status xrl_encode_delta(xrl_ctx* ctx, const xrl_batch* b, const int32_t* bas
   int32_t* level = level_a;
   int k = launch_delta_graphs(in, b->B, b->max_n, L, base, level, counts, cursor, st);
   if (k < -1) { cudaGetLastError(); return XRL_ERR_CUDA; }
-  if (k < 0) {                                      // graphs beyond shared memory: pass by pass over all nodes
+  if (k < 0) {                                      // large graphs: pass by pass over all nodes
     k = launch_delta_level0(in, valid, base, level_a, st);
     int32_t* other = level_b;
     for (int t = 1; t <= L; ++t) {

@@ -49,23 +49,25 @@ def test_levels_by_graph_and_pass_by_pass(nodes, L):
     assert [r + 16385 for r in rows] == rows2
 
 
-@pytest.mark.parametrize("nodes", [9777, 9830, 9831, 16384])
-def test_levels_by_graph_around_the_default_limit_of_shared_memory(nodes):
-    """The per-graph kernel's shared memory at sizes that need the opt-in only with the kernel's own arrays counted, just
-    beyond, and at its largest."""
-    m = dict(T=11, S=8, H=32, K=2, L=2, Hm=16, Dg=1, dtype="fp32", A_max=2)
+@pytest.mark.parametrize("nodes,copies", [(2048, 2), (2049, 2), (9777, 2), (9830, 2), (16384, 2), (4096, 255), (4097, 255),
+                                          (4096, 254)])
+def test_levels_at_the_lines_between_the_two(nodes, copies):
+    """Graphs at and beyond the sizes up to which a CTA takes a graph (fewer nodes for few graphs), and sizes whose shared
+    memory at five bytes a node would need the opt-in: valid batches all, whichever kernels take them."""
+    m = dict(T=11, S=8, H=32, K=2, L=2, Hm=16, Dg=1, dtype="fp32", A_max=copies)
     cur = dags.random_dag(dags.make_rng(nodes), nodes, m["T"], 8, window=6)
     graphs = [cur]
-    for i in (1, nodes // 2):                           # a candidate of the same size: one operator changed
+    for c in range(copies):                             # a candidate of the same size: one operator changed
         op = cur["op"].copy()
+        i = 1 + c * (nodes // copies)
         op[i] = (op[i] + 1) % m["T"]
         graphs.append(dict(cur, op=op, twin=np.arange(nodes, dtype=np.int32)))
     blob, _ = gpu_util.default_weights({"model": m, "n_nodes": np.array([nodes])}, 6)
-    full, delta, rows = _run(m, graphs, [0, 3], blob)
-    gpu_util.assert_close(delta, full, "fp32", "by graph")
-    assert nodes < rows[0] <= rows[1] <= rows[2] < 2 * nodes
+    full, delta, rows = _run(m, graphs, [0, len(graphs)], blob)
+    gpu_util.assert_close(delta, full, "fp32", "by graph, or pass by pass")
+    assert nodes < rows[0] <= rows[1] <= rows[2] < nodes * (1 + copies / 2)
     big = dags.random_dag(dags.make_rng(1), 16385, m["T"], 8, window=6)
-    full2, delta2, rows2 = _run(m, graphs + [big], [0, 3, 4], blob)
+    full2, delta2, rows2 = _run(m, graphs + [big], [0, len(graphs), len(graphs) + 1], blob)
     gpu_util.assert_close(delta2, full2, "fp32", "pass by pass")
     assert [r + 16385 for r in rows] == rows2
 
