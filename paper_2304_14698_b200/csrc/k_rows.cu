@@ -304,7 +304,7 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
 
     if constexpr (VPL == 1) {
       // One vector per lane.  The 32 / LPR rows of a warp go through one code path together: producers two at a time up to
-      // the largest count among the rows (absent ones weigh 0), the first two asked for together with the row's own
+      // the largest count among the rows, the first two asked for together with the row's own
       // vector, packed fp32 arithmetic, a reference exponent that moves only when a score exceeds it by 32.  Rows of
       // different degrees taking their own branches through groups of 1 to 4 producers executed 115 warp instructions
       // per row at 58 % issue utilisation (hidden 128 bf16, 299 k rows of mean degree 1.1: 0.057 ms; now
@@ -351,7 +351,8 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
           if (t > 0) pair(t);
           const float ev0 = lrelu(ea + sd), ev1 = lrelu(eo + sd), evm = fmaxf(ev0, ev1);
           if (evm > m + 32.f) aggtma::raise_reference<NP>(evm, m, l, acc);
-          const float p0 = fast_exp2(ev0 - m), p1 = fast_exp2(ev1 - m);
+          // (absent producers weigh 0 by their place and not by their score, which is no number where the row's is infinite)
+          const float p0 = t < n ? fast_exp2(ev0 - m) : 0.f, p1 = t + 1 < n ? fast_exp2(ev1 - m) : 0.f;
           l += p0 + p1;
           aggtma::F2 z[NP];
           aggtma::to_pairs(qa, z);

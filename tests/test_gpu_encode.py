@@ -305,3 +305,37 @@ def test_bf16_model_takes_shape_features_off_the_bf16_grid(xo):
             gpu_util.assert_close(o[k].cpu().numpy(), want[k], "bf16", k)
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,dtype", [(32, "fp32"), (64, "fp32"), (64, "bf16"), (128, "bf16"), (192, "bf16")])
+def test_rows_without_producers_beside_others_when_scores_overflow(H, dtype):
+    """A half-score beyond fp32's range (2 x 2e38) leaves no number where it meets a producer's; a node without producers is
+    its own whole neighbourhood and gives ReLU(Z + b) whatever its score, also beside rows that have producers."""
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=5, S=8, H=H, K=1, L=1, Hm=8, Dg=1, dtype=dtype, A_max=1)
+    n = 64
+    src, dst = [], []
+    for i in range(0, n, 4):                            # rows 1, 2 and 3 of every four have 1, 2 and 3 producers, row 0 none
+        for j in range(1, 4):
+            src += list(range(i, i + j)); dst += [i + j] * j
+    g = dict(op=np.zeros(n, np.int32), shape=np.zeros((n, 8), np.float32), edge_src=np.array(src, np.int32),
+             edge_dst=np.array(dst, np.int32))
+    batch = dags.flatten([g], [0, 1], 1)
+    batch["model"] = m
+    W0, b0, W, a_src, a_dst, b = (np.zeros(v, np.float32) for v in ((16 + 5, H), H, (H, H), H, H, H))
+    b0[:] = 1
+    W[np.arange(H), np.arange(H)] = 1                   # Z = 1 everywhere
+    a_dst[:2] = 2e38
+    b[:] = 0.5
+    ag = gpu_util.make_agent(batch)
+    try:
+        blob = np.zeros(xrl.xrl_weights_size(ag.ctx) // 4, np.float32)
+        parts = np.concatenate([a.ravel() for a in (W0, b0, W, a_src, a_dst, b)])
+        blob[:len(parts)] = parts
+        ag.set_weights(blob)
+        ag.pack(batch)
+        h = xrl.xrl_debug_node_features(ag.ctx, ag.batch, 1, H)
+        assert ag.device_status() == 0
+        assert (h[::4] == 1.5).all()
+    finally:
+        ag.close()
