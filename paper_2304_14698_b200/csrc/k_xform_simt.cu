@@ -1,9 +1,8 @@
 // Dense node transform of a graph-attention layer, Z = h W (paper Eq. 7, the "W h_j" term), on
-// the CUDA cores with fp32 accumulation.  This is the path for fp32 storage (whose tolerance a
-// single-pass reduced-precision tensor-core product cannot guarantee) and for the bf16 models the
-// tensor-core kernel is kept off for (XRL_FORCE_SIMT_TRANSFORM).  The attention half-scores are taken from the accumulators in the
-// kernel's last step when one tile spans all H columns, the storage is fp32 and a head is 4, 8, ... 128 columns
-// wide (SCORES); otherwise from Z by k_scores.
+// the CUDA cores with fp32 accumulation.  This is the path for fp32 storage of few rows (for many rows see
+// k_xform_tf32) and for the bf16 models the tensor-core kernel is kept off for (XRL_FORCE_SIMT_TRANSFORM).  The attention
+// half-scores are taken from the accumulators in the kernel's last step when one tile spans all H columns, the
+// storage is fp32 and a head is 4, 8, ... 64 columns wide (SCORES); otherwise from Z by k_scores.
 #include "xrl_internal.cuh"
 
 namespace xrl {
@@ -115,10 +114,9 @@ __device__ __forceinline__ void load4<bf16>(const bf16* p, bool ok, float (&v)[4
 
 // (TA, TW, TZ: element types of the rows, of the matrix and of the result: the reverse pass multiplies fp32 gradients
 // with matrices in the storage type)
-template <typename TA, typename TW, typename TZ, bool SCORES>
+template <typename TA, typename TW, typename TZ>
 __global__ void __launch_bounds__(256)
-k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restrict__ Z, int H, int rows,
-                const float* __restrict__ a_src, const float* __restrict__ a_dst, float2* __restrict__ scores, int K) {
+k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restrict__ Z, int H, int rows) {
   __shared__ __align__(16) float As[TK][TM];
   __shared__ __align__(16) float Bs[TK][TN];
   const int tid = threadIdx.x;
@@ -167,28 +165,6 @@ k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restri
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int64_t r = row0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
-    if (SCORES) {                               // (every lane takes part in the shuffles)
-      const int d = H / K;
-      float ss[2], sd[2];
-#pragma unroll
-      for (int jg = 0; jg < 2; ++jg) {
-        const int c = jg * 64 + tx * 4;
-        const float z[4] = {acc[i][jg * 4], acc[i][jg * 4 + 1], acc[i][jg * 4 + 2], acc[i][jg * 4 + 3]};
-        head_partial(z, a_src, a_dst, c < H ? c : 0, d >= 64 ? 16 : (d >> 2), ss[jg], sd[jg]);   // (columns >= H hold 0)
-      }
-      if (r < rows) {
-        if (d == 128) {                         // one head over both column groups
-          if (tx == 0) scores[size_t(r) * K] = make_float2((ss[0] + ss[1]) * kLog2e, (sd[0] + sd[1]) * kLog2e);
-        } else {
-          const int g = d >= 64 ? 16 : (d >> 2);
-#pragma unroll
-          for (int jg = 0; jg < 2; ++jg) {
-            const int c = jg * 64 + tx * 4;
-            if (c < H && (tx & (g - 1)) == 0) scores[size_t(r) * K + c / d] = make_float2(ss[jg] * kLog2e, sd[jg] * kLog2e);
-          }
-        }
-      }
-    }
     if (r >= rows) continue;
 #pragma unroll
     for (int jg = 0; jg < 2; ++jg) {
@@ -200,15 +176,14 @@ k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restri
   }
 }
 
-
 // ---- fp32 storage, many rows: the product on the tensor cores with every operand split in two ----------------
-// (the widths whose split W does not fit k_xform_tf32: 160, 224 and more than 256)
+// (the widths whose split W does not fit k_xform_tf32: 160, 224 and more than 256; any other where its set-up fails)
 // x = hi + lo with hi = tf32(x) and lo = tf32(x - hi); Z = sum hi_a hi_b + hi_a lo_b + lo_a hi_b in fp32
 // accumulators (mma.sync m16n8k8, the small terms first): the dropped lo_a lo_b term is below 2^-22 of the
 // product, i.e. the result is as good as an fp32 FMA chain in another order.  CTA tile 128 rows x 128 columns,
 // 8 warps as 4 (rows) x 2 (columns), warp tile 32 x 64 = 2 x 8 MMA tiles; K advanced 16 at a time; both splits of a
 // slice are made once, when it is written to shared memory (stored k-major: fragment reads are conflict-free
-// with a row stride of 136 words).  Half-scores from the accumulators when a head is 8 ... 64 columns wide.
+// with a row stride of 136 words).
 constexpr int XM = 128, XN = 128, XK = 16, XS = 136;
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -223,10 +198,8 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-template <bool SCORES>
 __global__ void __launch_bounds__(256, 2)
-k_xform_tf32x3(const float* __restrict__ h, const float* __restrict__ W, float* __restrict__ Z, int H, int rows,
-               const float* __restrict__ a_src, const float* __restrict__ a_dst, float2* __restrict__ scores, int K) {
+k_xform_tf32x3(const float* __restrict__ h, const float* __restrict__ W, float* __restrict__ Z, int H, int rows) {
   extern __shared__ __align__(16) uint32_t xs[];          // A hi, A lo, B hi, B lo: each [XK][XS]
   uint32_t* Ah = xs;
   uint32_t* Al = Ah + XK * XS;
@@ -320,25 +293,6 @@ k_xform_tf32x3(const float* __restrict__ h, const float* __restrict__ W, float* 
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       const int64_t r = row0 + wm + i * 16 + g + half * 8;
-      if (SCORES) {                             // (every lane takes part in the shuffles)
-        const int d = H / K, tiles = d >> 3;    // MMA tiles per head: 1, 2, 4 or 8
-        float ss = 0.f, sd = 0.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int c = col0 + wn + j * 8 + 2 * t;
-          const int cc = c < H ? c : 0;         // (columns >= H hold 0)
-          const float2 s = __ldg(reinterpret_cast<const float2*>(a_src + cc));
-          const float2 u = __ldg(reinterpret_cast<const float2*>(a_dst + cc));
-          ss = fmaf(acc[i][j][2 * half + 1], s.y, fmaf(acc[i][j][2 * half], s.x, ss));
-          sd = fmaf(acc[i][j][2 * half + 1], u.y, fmaf(acc[i][j][2 * half], u.x, sd));
-          if (((j + 1) & (tiles - 1)) == 0) {   // the head ends with this tile
-            ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1); sd += __shfl_xor_sync(0xFFFFFFFFu, sd, 1);
-            ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 2); sd += __shfl_xor_sync(0xFFFFFFFFu, sd, 2);
-            if (t == 0 && r < rows && c < H) scores[size_t(r) * K + c / d] = make_float2(ss * kLog2e, sd * kLog2e);
-            ss = 0.f; sd = 0.f;
-          }
-        }
-      }
       if (r >= rows) continue;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -351,12 +305,12 @@ k_xform_tf32x3(const float* __restrict__ h, const float* __restrict__ W, float* 
 
 }  // namespace
 
-// SCORES variant: fp32 storage, one tile across all H columns, heads 4 ... 128 columns wide (a power of two)
-static bool fuse_scores(const Dims& d, const LayerWeights& lw, int tile_cols, const float* scores, int min_width = 4) {
-  if (d.dtype != XRL_FP32 || d.zmerged || scores == nullptr || d.H > tile_cols || (d.H & 3) || d.K < 1 || d.H % d.K) return false;
+// SCORES variant: fp32 storage, one tile across all H columns, heads 4 ... 64 columns wide (a power of two)
+static bool fuse_scores(const Dims& d, const LayerWeights& lw, const float* scores) {
+  if (d.dtype != XRL_FP32 || d.zmerged || scores == nullptr || d.H > BN || (d.H & 3) || d.K < 1 || d.H % d.K) return false;
   if ((reinterpret_cast<uintptr_t>(lw.a_src) | reinterpret_cast<uintptr_t>(lw.a_dst)) & 15) return false;   // vector loads
   const int w = d.H / d.K;
-  return w >= min_width && w <= tile_cols && (w & (w - 1)) == 0;
+  return w >= 4 && w <= BN && (w & (w - 1)) == 0;
 }
 
 int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void* Z, float* scores,
@@ -365,43 +319,22 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
   if (rows <= 0) return 0;
   const size_t off = size_t(win.row_begin - win.win_base) * d.H;
   float2* sc = reinterpret_cast<float2*>(scores) + size_t(win.row_begin - win.win_base) * d.K;
-  if (rows >= 8192 && d.dtype == XRL_FP32 && d.H % XK == 0) {
+  if (rows >= 8192 && d.dtype == XRL_FP32) {
     // fp32 storage: split operands on the tensor cores (below 8,192 rows too few tiles for the SMs: FFMA)
-    const int k = launch_xform_tf32(d, static_cast<const float*>(h) + off, lw, static_cast<float*>(Z) + off, sc, rows, status, st);
+    const float* hp = static_cast<const float*>(h) + off;
+    float* zp = static_cast<float*>(Z) + off;
+    const int k = launch_xform_tf32(d, hp, lw, zp, sc, rows, status, st);
     if (k == 1) return 1;
-    if (k == 0) return 1 + launch_scores(d, Z, lw, scores, win, st);
-    dim3 gx(unsigned((rows + XM - 1) / XM), unsigned((d.H + XN - 1) / XN));
-    const size_t smem = sizeof(uint32_t) * 4 * XK * XS;
-    const int w = d.H / d.K;
-    if (fuse_scores(d, lw, XN, scores, 8) && w <= 64) {
-      k_xform_tf32x3<true><<<gx, 256, smem, st>>>(static_cast<const float*>(h) + off, static_cast<const float*>(lw.W),
-                                                 static_cast<float*>(Z) + off, d.H, int(rows), lw.a_src, lw.a_dst, sc, d.K);
-      return 1;
+    if (k < 0) {
+      const dim3 gx(unsigned((rows + XM - 1) / XM), unsigned((d.H + XN - 1) / XN));
+      k_xform_tf32x3<<<gx, 256, sizeof(uint32_t) * 4 * XK * XS, st>>>(hp, static_cast<const float*>(lw.W), zp, d.H, int(rows));
     }
-    k_xform_tf32x3<false><<<gx, 256, smem, st>>>(static_cast<const float*>(h) + off, static_cast<const float*>(lw.W),
-                                                static_cast<float*>(Z) + off, d.H, int(rows), nullptr, nullptr, nullptr,
-                                                d.K);
     return 1 + launch_scores(d, Z, lw, scores, win, st);
   }
   if (rows >= 8192) {
-    dim3 g128(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
-    if (d.dtype == XRL_BF16) {
-      k_xform_simt128<bf16, bf16, bf16, false><<<g128, 256, 0, st>>>(static_cast<const bf16*>(h) + off,
-                                                         static_cast<const bf16*>(lw.W),
-                                                         static_cast<bf16*>(Z) + off, d.H, int(rows), nullptr, nullptr,
-                                                         nullptr, d.K);
-    } else if (fuse_scores(d, lw, TN, scores)) {
-      k_xform_simt128<float, float, float, true><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
-                                                         static_cast<const float*>(lw.W),
-                                                         static_cast<float*>(Z) + off, d.H, int(rows), lw.a_src, lw.a_dst,
-                                                         sc, d.K);
-      return 1;
-    } else {
-      k_xform_simt128<float, float, float, false><<<g128, 256, 0, st>>>(static_cast<const float*>(h) + off,
-                                                          static_cast<const float*>(lw.W),
-                                                          static_cast<float*>(Z) + off, d.H, int(rows), nullptr, nullptr,
-                                                          nullptr, d.K);
-    }
+    const dim3 g128(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
+    k_xform_simt128<bf16, bf16, bf16><<<g128, 256, 0, st>>>(static_cast<const bf16*>(h) + off, static_cast<const bf16*>(lw.W),
+                                                            static_cast<bf16*>(Z) + off, d.H, int(rows));
     return 1 + launch_scores(d, Z, lw, scores, win, st);
   }
   dim3 grid(unsigned((rows + BM - 1) / BM), unsigned((d.H + BN - 1) / BN));
@@ -410,7 +343,7 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
                                                    static_cast<const bf16*>(lw.W),
                                                    static_cast<bf16*>(Z) + off, d.H, int(rows), nullptr, nullptr, nullptr,
                                                    d.K);
-  } else if (fuse_scores(d, lw, BN, scores)) {
+  } else if (fuse_scores(d, lw, scores)) {
     k_xform_simt<float, true><<<grid, 256, 0, st>>>(static_cast<const float*>(h) + off,
                                                    static_cast<const float*>(lw.W),
                                                    static_cast<float*>(Z) + off, d.H, int(rows), lw.a_src, lw.a_dst, sc,
@@ -430,11 +363,9 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
 int launch_rows_times_matrix(const Dims& d, const float* G, const void* Wt, float* out, int rows, cudaStream_t st) {
   dim3 g(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
   if (d.dtype == XRL_BF16)
-    k_xform_simt128<float, bf16, float, false><<<g, 256, 0, st>>>(G, static_cast<const bf16*>(Wt), out, d.H, rows, nullptr,
-                                                                  nullptr, nullptr, d.K);
+    k_xform_simt128<float, bf16, float><<<g, 256, 0, st>>>(G, static_cast<const bf16*>(Wt), out, d.H, rows);
   else
-    k_xform_simt128<float, float, float, false><<<g, 256, 0, st>>>(G, static_cast<const float*>(Wt), out, d.H, rows, nullptr,
-                                                                   nullptr, nullptr, d.K);
+    k_xform_simt128<float, float, float><<<g, 256, 0, st>>>(G, static_cast<const float*>(Wt), out, d.H, rows);
   return 1;
 }
 
