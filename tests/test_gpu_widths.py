@@ -126,3 +126,32 @@ def test_fp32_widths_on_many_rows(xo, H, K, copies):
         assert ag.device_status() == 0
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K", [(32, 2), (64, 2), (96, 3), (128, 4), (160, 5), (192, 6), (224, 7), (256, 4), (320, 5)])
+def test_fp32_transform_of_many_rows_keeps_fp32_accuracy(xo, H, K):
+    """Both split-operand products (8,192 rows and more) against 64 bits.  Their sums take 3 H / 8 steps, each cut at the 24th
+    bit of a running sum that is half its final size on average: (3 H / 16) 2^-24 of the result, and 4 x 2^-24 for Eq. 6,
+    the softmax and the weighted sum.  One dropped part of an operand is 2^-12 of a product and far outside."""
+    import numpy as np
+    import paper_2304_14698_b200 as xrl
+    m = dict(T=9, S=8, H=H, K=K, L=1, Hm=24, Dg=1, dtype="fp32", A_max=64)
+    n, copies = 1372, 6
+    g = dags.random_dag(dags.make_rng(H), n, m["T"], 8)
+    batch = dags.flatten([g] * copies, [0, copies], 64)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 4)
+    one = dags.flatten([g], [0, 1], 64)
+    st, packed = xo.pack(one)
+    assert st == 0
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        got = xrl.xrl_debug_node_features(ag.ctx, ag.batch, 1, H).reshape(copies, n, H)
+        want = np.asarray(xo.encode(m, blob, one, packed, dump_layer=1, want_nodes=True)["nodes"], np.float64)
+        for i in range(copies):
+            assert np.linalg.norm(got[i] - want) <= (3 * H / 16 + 4) * 2.0**-24 * np.linalg.norm(want)
+        assert ag.device_status() == 0
+    finally:
+        ag.close()
