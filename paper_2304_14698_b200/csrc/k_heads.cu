@@ -72,7 +72,8 @@ k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ o
                 float* __restrict__ emb, float* __restrict__ U_out, int H, int Dg, int B) {
   extern __shared__ __align__(16) float u[];     // [GP][xs], then scratch
   const int xs = row_stride(H + Dg), nt = blockDim.x, tid = threadIdx.x;
-  float* part = u + GP * xs;
+  int32_t* filled = reinterpret_cast<int32_t*>(u + GP * xs);       // [GP] parts of each graph that hold any row
+  float* part = u + GP * xs + row_stride(GP);
   const int32_t first = blockIdx.x * GP;
   const int HV = H >> 2, NG = nt / HV, P = NG >= GP ? NG / GP : 1;
   const int cv = tid % HV, grp = tid / HV;
@@ -95,6 +96,7 @@ k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ o
       if (first + gl >= B) break;
       int32_t b0, b1;
       range(first + gl, b0, b1);
+      if (p == 0 && cv == 0) filled[gl] = min(P, max(0, b1 - b0 + 1));
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int32_t b = b0 + p; b <= b1; b += 8 * P) {
         float4 v[8];
@@ -118,7 +120,7 @@ k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ o
         const int32_t start = off[g];
         if (off[g + 1] > start && (start & ((1 << bshift) - 1))) v = partial[size_t(nblocks + g) * H + c];
       }
-      for (int q = 0; q < P; ++q) v += part[size_t(gl * P + q) * H + c];
+      for (int q = 0, n = filled[gl]; q < n; ++q) v += part[size_t(gl * P + q) * H + c];
     } else if (g < B && c < H + Dg) {
       v = g0 ? g0[size_t(g) * Dg + (c - H)] : 0.f;
     }
@@ -429,10 +431,10 @@ int launch_readout(const Dims& d, const void* h, const int32_t* chunk_row0, cons
 namespace {
 template <int GP, bool BLOCKS>
 int global_update(const Dims& d, const float* partial, const int32_t* off, int32_t nblocks, int shift, const float* g0,
-                  const DevWeights& w, float* emb, float* U_out, int32_t B, size_t smem, cudaStream_t st) {
+                  const DevWeights& w, float* emb, float* U_out, int32_t B, size_t smem, cudaStream_t st, int nt = kThreads) {
   static bool attr[64] = {};
   if (smem > 48 * 1024 && !ensure_dynamic_smem(k_global_update<GP, BLOCKS>, 227 * 1024, attr)) return -1;
-  k_global_update<GP, BLOCKS><<<(B + GP - 1) / GP, kThreads, smem, st>>>(partial, off, nblocks, shift, g0, w.Wg, w.bg, emb,
+  k_global_update<GP, BLOCKS><<<(B + GP - 1) / GP, nt, smem, st>>>(partial, off, nblocks, shift, g0, w.Wg, w.bg, emb,
                                                                          U_out, d.H, d.Dg, B);
   return 1;
 }
@@ -443,11 +445,17 @@ int launch_update(const Dims& d, const float* partial, const int32_t* off, int32
   // rows of u, then scratch: the parts of the block sums (max(groups, GP) rows of H), the parts of the dense map
   auto bytes = [&](int gp) {
     const size_t rows = size_t(std::max(kThreads / (d.H / 4), gp)) * d.H, parts = size_t(gp) * kThreads;
-    return sizeof(float) * (size_t(gp) * row_stride(d.H + d.Dg) + std::max(rows, parts));
+    return sizeof(float) * (size_t(gp) * row_stride(d.H + d.Dg) + row_stride(gp) + std::max(rows, parts));
   };
-  const int gp = graphs_per_cta(B, bytes);
+  int gp = graphs_per_cta(B, bytes);
+  // two graphs per CTA (up to two per SM) are slower than four, and than one each on fewer threads where W_g is small: 220
+  // graphs, hidden 64 / 128 / 256 / 512: 5.4 / 7.4 / 12.6 / 32.9 us, four 5.2 / 6.8 / 11.5 / 27.9, one 4.3 / 6.2 / 12.2 / 36.8
+  if (gp == 2) {
+    if (d.H <= 128) return global_update<1, BLOCKS>(d, partial, off, nblocks, shift, g0, w, emb, U_out, B, bytes(1), st, 256);
+    gp = 4;
+  }
 #define UPDATE_CASE(G_) case G_: return global_update<G_, BLOCKS>(d, partial, off, nblocks, shift, g0, w, emb, U_out, B, bytes(G_), st);
-  switch (gp) { UPDATE_CASE(1) UPDATE_CASE(2) UPDATE_CASE(4) UPDATE_CASE(8) default: UPDATE_CASE(16) }
+  switch (gp) { UPDATE_CASE(1) UPDATE_CASE(4) UPDATE_CASE(8) default: UPDATE_CASE(16) }
 #undef UPDATE_CASE
 }
 template <int GP>
