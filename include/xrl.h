@@ -286,11 +286,12 @@ xrl_status xrl_sample(xrl_ctx* ctx, const float* probs, int32_t num_envs, int32_
  *   grad      DEVICE fp32, laid out like the weight blob (xrl_weights_size bytes), overwritten
  *   logp_out  DEVICE fp32 [num_envs] or NULL: log pi(action_e) under the current weights
  * The first call allocates the workspace for the context's capacities ((L + 2) copies of the node features,
- * L of the transformed features Z, three fp32 ones, and for hidden 128 or 256 the lists by producer: 8 * heads
- * bytes per node and edge and 12 more per edge) and therefore synchronises; later calls only enqueue.  Not recordable
- * (XRL_ERR_STATE between xrl_graph_begin and xrl_graph_launch).  XRL_ERR_UNSUPPORTED when
- * (T + 8) x H floats exceed one SM's shared memory (227 KB): the operator block of W0's gradient and a tile
- * of eight rows are kept there.
+ * L of the transformed features Z, three fp32 ones, and for hidden 128 or 256 with an even number of heads that divides
+ * 32 the lists by producer: 8 * heads bytes per node and edge and 12 more per edge; where only the lists do not fit, the
+ * context works without them) and therefore synchronises; later calls only enqueue.  The call writes no buffer that
+ * xrl_encode or xrl_policy_value use, so it may run beside them on another stream.  Not recordable
+ * (XRL_ERR_STATE between xrl_graph_begin and xrl_graph_launch).  XRL_ERR_UNSUPPORTED for models whose operator
+ * block of W0's gradient and eight rows of features, (T + 8) x H floats, exceed 227 KB.
  * Errors: INVALID_ARG, STATE, UNSUPPORTED, ALLOC, CUDA. */
 xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* batch, const float* g0, const uint8_t* mask,
                         const int32_t* action, const float* logp_old, const float* adv, const float* ret,

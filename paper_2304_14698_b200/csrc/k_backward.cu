@@ -1202,8 +1202,8 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   return 4;
 }
 
-// The model shapes Eq. 6's reverse takes: a copy of the one-hot block of W0's gradient ([T x H]) and eight rows of all
-// columns within one SM's shared memory (the kernel itself keeps 64 columns of it per warp).
+// The model shapes xrl_ppo_grad takes: a copy of the one-hot block of W0's gradient ([T x H]) and eight rows of all columns
+// within 227 KB.  A limit of the interface: the kernel below keeps 64 columns of that block per warp and would take any.
 size_t embed_bwd_smem_bytes(const Dims& d) {
   return sizeof(float) * (size_t(d.T) * d.H + 8 * size_t(d.H) + 8 * 2 * kS) + sizeof(int32_t) * 8;
 }
