@@ -45,6 +45,7 @@ k_aggregate_tma(const __grid_constant__ CUtensorMap map_z, const __grid_constant
                 const float* __restrict__ bias, T* __restrict__ h_out, Window win,
                 const int32_t* __restrict__ seg_id, float* __restrict__ partial, int32_t nblocks,
                 const int32_t* __restrict__ self_idx, int32_t* status, int32_t br_shift) {
+  enter();
   using Smem = WarpSmem<K, MERGED, G, GQ>;
   extern __shared__ __align__(128) uint8_t tma_smem_raw[];
   Smem& sm = reinterpret_cast<Smem*>(tma_smem_raw)[threadIdx.x >> 5];
@@ -112,7 +113,7 @@ int launch_k_seq(const int32_t* rowptr, const int32_t* col, const void* Z, const
   const int64_t nblocks = (rows + br - 1) / br;
   int64_t nb = (rows + br * TW - 1) / (br * TW);
   if (nb > int64_t(kNumSMs) * XRL_AGG_CTAS) nb = int64_t(kNumSMs) * XRL_AGG_CTAS;
-  k_aggregate_tma<T, K, READOUT, MERGED, SEQ><<<int(nb), TW * 32, smem, st>>>(
+  launch(k_aggregate_tma<T, K, READOUT, MERGED, SEQ>, int(nb), TW * 32, smem, st,
       mz, ms, rowptr, col, static_cast<const T*>(Z), reinterpret_cast<const float2*>(scores), bias,
       static_cast<T*>(h_out), win, seg_id, partial, int32_t(nblocks), self_idx, status, int32_t(shift));
   return 1;

@@ -51,6 +51,7 @@ k_aggregate_bwd(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ 
                 const T* __restrict__ h_out, const float* __restrict__ dh_out, float* __restrict__ dz,
                 float* __restrict__ ds_src, float* __restrict__ ds_dst, float* __restrict__ db, int N, int H,
                 int K) {
+  enter();
   extern __shared__ float sm_db[];                 // [H] per-CTA sums of dpre
   for (int c = threadIdx.x; c < H; c += blockDim.x) sm_db[c] = 0.f;
   __syncthreads();
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(256)
 k_scores_bwd(ZView<T> zv, const float* __restrict__ ds_src, const float* __restrict__ ds_dst,
              const float* __restrict__ a_src, const float* __restrict__ a_dst, float* __restrict__ dz,
              float* __restrict__ da_src, float* __restrict__ da_dst, int N, int H, int K) {
+  enter();
   extern __shared__ float sm_da[];                 // [2H]
   for (int c = threadIdx.x; c < 2 * H; c += blockDim.x) sm_da[c] = 0.f;
   __syncthreads();
@@ -209,6 +211,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
                      const T* __restrict__ h_out, float* __restrict__ dh_out, bool masked, float* __restrict__ dz,
                      float* __restrict__ ds_src, float* __restrict__ ds_dst, float* __restrict__ db, int N, int K,
                      BwdLists tl) {
+  enter();
   constexpr int H = 32 * NF;
   __shared__ float sm_db[H];
   for (int c = threadIdx.x; c < H; c += blockDim.x) sm_db[c] = 0.f;
@@ -348,6 +351,7 @@ __global__ void __launch_bounds__(256)
 k_scores_bwd_rows(ZView<T> zv, const float* __restrict__ ds_src, const float* __restrict__ ds_dst,
                   const float* __restrict__ a_src, const float* __restrict__ a_dst, float* __restrict__ dz,
                   bf16* __restrict__ dzb, float* __restrict__ da_src, float* __restrict__ da_dst, int N, int K) {
+  enter();
   constexpr int H = 32 * NF;
   __shared__ float sm_da[2 * H];
   for (int c = threadIdx.x; c < 2 * H; c += blockDim.x) sm_da[c] = 0.f;
@@ -403,6 +407,7 @@ constexpr int kMaxTasks = 8;
 struct GradTasks { GradTask t[kMaxTasks]; int n; };
 __global__ void __launch_bounds__(256)
 k_head_grads(const __grid_constant__ GradTasks tasks) {
+  enter();
   __shared__ float As[16][64 + 1];
   __shared__ float Bs[16][64 + 1];
   int which = 0;
@@ -476,6 +481,7 @@ template <typename TA, int TILE>
 __global__ void __launch_bounds__((TILE / 8) * (TILE / 8))
 k_atb_tile(const TA* __restrict__ A, const float* __restrict__ Bm, float* __restrict__ Cout, int rows, int H,
            int rows_per_chunk, bool vec) {
+  enter();
   constexpr int NTX = TILE / 8, NT = NTX * NTX;
   constexpr int PIECES = kAtbRows * TILE / 4 / NT;     // 4-wide pieces per thread, operand and step
   __shared__ __align__(16) float As[kAtbRows][TILE];
@@ -548,6 +554,7 @@ k_atb_tile(const TA* __restrict__ A, const float* __restrict__ Bm, float* __rest
 template <typename TW>
 __global__ void __launch_bounds__(256)
 k_gwt(const float* __restrict__ G, const TW* __restrict__ W, float* __restrict__ out, int rows, int Hk, int Hn) {
+  enter();
   __shared__ float Gs[64][16 + 1];
   __shared__ float Ws[64][16 + 1];
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -586,6 +593,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_embed_inputs(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, const T* __restrict__ shape,
                const T* __restrict__ eattr, float* __restrict__ xs, int N) {
+  enter();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   float x[2 * kS];
@@ -615,6 +623,7 @@ template <typename T>
 __global__ void __launch_bounds__(128)
 k_embed_bwd(const float* __restrict__ xs, const int32_t* __restrict__ op, const T* __restrict__ h0,
             const float* __restrict__ dh0, bool masked, float* __restrict__ dW0, float* __restrict__ db0, int N, int H, int Tn) {
+  enter();
   extern __shared__ __align__(16) float sm_embed[];
   const int warps = blockDim.x >> 5, wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   EmbBwdStage& stg = reinterpret_cast<EmbBwdStage*>(sm_embed)[wib];
@@ -759,6 +768,7 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
           const float* __restrict__ adv, const float* __restrict__ ret, float eps, float c1, float c2, Mlp vm,
           EnvBufs eb, int H, int A, int num_envs, float* __restrict__ loss, float* __restrict__ dlogit,
           float* __restrict__ demb, float* __restrict__ logp_out, int32_t* status) {
+  enter();
   extern __shared__ __align__(16) float sm[];
   const int e = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   float* scratch = sm;                              // [4 blockDim]
@@ -860,6 +870,7 @@ k_graph_bwd(const float* __restrict__ emb, const float* __restrict__ dlogit, Mlp
             const float* __restrict__ py1, const float* __restrict__ py2, const float* __restrict__ demb,
             const float* __restrict__ Wg, float* __restrict__ pd1, float* __restrict__ pd2,
             float* __restrict__ dpre, float* __restrict__ dr, int H, int B) {
+  enter();
   extern __shared__ float sm[];
   const int tid = threadIdx.x, nt = blockDim.x;
   float* d1 = sm;                                   // [GP][hid]
@@ -911,6 +922,7 @@ k_graph_bwd(const float* __restrict__ emb, const float* __restrict__ dlogit, Mlp
 template <typename T>
 __global__ void k_readout_bwd(const float* __restrict__ dr, const int32_t* __restrict__ seg_id, const T* __restrict__ h,
                               float* __restrict__ dh, int64_t n_quads, int H) {
+  enter();
   const int q = H >> 2;
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_quads; t += int64_t(gridDim.x) * blockDim.x) {
     const int64_t i = t / q;
@@ -950,7 +962,7 @@ int graph_bwd(const Dims& d, const float* emb, const float* dlogit, const Mlp& p
   static bool attr[64] = {};
   const size_t smem = sizeof(float) * size_t(GP) * (d.H + d.Hm + d.Hm2);
   if (smem > 48 * 1024 && !ensure_dynamic_smem(k_graph_bwd<GP>, 227 * 1024, attr)) return -1;
-  k_graph_bwd<GP><<<(B + GP - 1) / GP, 1024, smem, st>>>(emb, dlogit, pm, py1, py2, demb, Wg, pd1, pd2, dpre, dr, d.H, B);
+  launch(k_graph_bwd<GP>, (B + GP - 1) / GP, 1024, smem, st, emb, dlogit, pm, py1, py2, demb, Wg, pd1, pd2, dpre, dr, d.H, B);
   return 1;
 }
 
@@ -959,6 +971,7 @@ int graph_bwd(const Dims& d, const float* emb, const float* dlogit, const Mlp& p
 __global__ void k_gae(const float* __restrict__ reward, const float* __restrict__ values,
                       const uint8_t* __restrict__ done, float gamma, float lambda, int T, int M,
                       float* __restrict__ adv, float* __restrict__ ret) {
+  enter();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
   float run = 0.f, vnext = values[size_t(T) * M + j];
@@ -982,6 +995,7 @@ namespace {
 template <typename F>
 __global__ void k_grad_weigh(const F* __restrict__ grad, int64_t count, const F* __restrict__ loss, F n,
                              F* __restrict__ buf) {
+  enter();
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < count) buf[i] = grad[i] * n;
   else if (i < count + 4) buf[i] = loss[i - count] * n;
@@ -989,6 +1003,7 @@ __global__ void k_grad_weigh(const F* __restrict__ grad, int64_t count, const F*
 }
 template <typename F>
 __global__ void k_grad_unweigh(const F* __restrict__ buf, int64_t count, F* __restrict__ grad, F* __restrict__ loss) {
+  enter();
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const F total = buf[count + 4];
   if (i < count) grad[i] = buf[i] / total;
@@ -1000,20 +1015,20 @@ int launch_grad_weigh(int elem_bytes, const void* grad, int64_t count, const voi
                       cudaStream_t st) {
   const unsigned blocks = unsigned((count + 5 + 255) / 256);
   if (elem_bytes == 8)
-    k_grad_weigh<double><<<blocks, 256, 0, st>>>(static_cast<const double*>(grad), count,
+    launch(k_grad_weigh<double>, blocks, 256, 0, st, static_cast<const double*>(grad), count,
                                                  static_cast<const double*>(loss), double(n), static_cast<double*>(buf));
   else
-    k_grad_weigh<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(grad), count,
+    launch(k_grad_weigh<float>, blocks, 256, 0, st, static_cast<const float*>(grad), count,
                                                 static_cast<const float*>(loss), float(n), static_cast<float*>(buf));
   return 1;
 }
 int launch_grad_unweigh(int elem_bytes, const void* buf, int64_t count, void* grad, void* loss, cudaStream_t st) {
   const unsigned blocks = unsigned((count + 4 + 255) / 256);
   if (elem_bytes == 8)
-    k_grad_unweigh<double><<<blocks, 256, 0, st>>>(static_cast<const double*>(buf), count, static_cast<double*>(grad),
+    launch(k_grad_unweigh<double>, blocks, 256, 0, st, static_cast<const double*>(buf), count, static_cast<double*>(grad),
                                                    static_cast<double*>(loss));
   else
-    k_grad_unweigh<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(buf), count, static_cast<float*>(grad),
+    launch(k_grad_unweigh<float>, blocks, 256, 0, st, static_cast<const float*>(buf), count, static_cast<float*>(grad),
                                                   static_cast<float*>(loss));
   return 1;
 }
@@ -1021,7 +1036,7 @@ int launch_grad_unweigh(int elem_bytes, const void* buf, int64_t count, void* gr
 int launch_gae(const float* reward, const float* values, const uint8_t* done, float gamma, float lambda, int32_t T,
                int32_t M, float* adv, float* ret, cudaStream_t st) {
   if (T <= 0 || M <= 0) return 0;
-  k_gae<<<unsigned((M + 127) / 128), 128, 0, st>>>(reward, values, done, gamma, lambda, T, M, adv, ret);
+  launch(k_gae, unsigned((M + 127) / 128), 128, 0, st, reward, values, done, gamma, lambda, T, M, adv, ret);
   return 1;
 }
 
@@ -1075,7 +1090,7 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
   if (k < 0) return -1;
   n += k;
   const size_t env_smem = sizeof(float) * (4 * 1024 + 4 * H + 2 * heads::row_stride(d.Hm) + 2 * heads::row_stride(d.Hm2));
-  k_ppo_env<<<num_envs, 1024, env_smem, st>>>(emb, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
+  launch(k_ppo_env, num_envs, 1024, env_smem, st, emb, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
                                               d.A, num_envs, loss, dlogit, demb, logp_out, status);
   ++n;
   // graphs per CTA: as few as leave every CTA an SM of its own, at most eight
@@ -1091,13 +1106,13 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
              gp(w.pb2));
   tl.add_mlp(eb.vu, 2 * d.H, num_envs, d.Hm, d.Hm2, eb.vy1, eb.vy2, eb.vd1, eb.vd2, eb.vdout, gp(w.vW1), gp(w.vb1), gp(w.vWh),
              gp(w.vbh), gp(w.vw2), gp(w.vb2));
-  k_head_grads<<<tl.ctas, 256, 0, st>>>(tl.tasks);
+  launch(k_head_grads, tl.ctas, 256, 0, st, tl.tasks);
   ++n;
   const int64_t ne = N * (d.H / 4);
   if (ne > 0) {
     const unsigned grid = unsigned(std::min<int64_t>((ne + 255) / 256, int64_t(kNumSMs) * 64));
-    if (d.dtype == XRL_BF16) k_readout_bwd<bf16><<<grid, 256, 0, st>>>(dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
-    else k_readout_bwd<float><<<grid, 256, 0, st>>>(dr, seg_id, static_cast<const float*>(hL), dh, ne, d.H);
+    if (d.dtype == XRL_BF16) launch(k_readout_bwd<bf16>, grid, 256, 0, st, dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
+    else launch(k_readout_bwd<float>, grid, 256, 0, st, dr, seg_id, static_cast<const float*>(hL), dh, ne, d.H);
     ++n;
   }
   return n;
@@ -1144,15 +1159,15 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   bf16* dzb = mma ? static_cast<bf16*>(dz_store) : nullptr;
 #define BWD_ROWS(TY_, NF_)                                                                                     \
   do {                                                                                                         \
-    k_aggregate_bwd_rows<TY_, NF_, false><<<grid_rows, 256, 0, st>>>(                                          \
+    launch(k_aggregate_bwd_rows<TY_, NF_, false>, grid_rows, 256, 0, st,                                           \
         rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, dz, ds_src, ds_dst, gb, N, K, BwdLists{});  \
-    k_scores_bwd_rows<TY_, NF_><<<grid_rows, 256, 0, st>>>(zv, ds_src, ds_dst, lw.a_src, lw.a_dst, dz, dzb,    \
+    launch(k_scores_bwd_rows<TY_, NF_>, grid_rows, 256, 0, st, zv, ds_src, ds_dst, lw.a_src, lw.a_dst, dz, dzb,    \
                                                            ga_src, ga_dst, N, K);                              \
   } while (0)
 #define BWD_GATHER(TY_, NF_)                                                                                   \
   do {                                                                                                         \
     if (launch_rows_gather(d, *lists, rowptr, col, Z, scores, h_out, dh_out, masked, ds_dst, gb, N, status, st) < 0) \
-      k_aggregate_bwd_rows<TY_, NF_, true><<<grid_rows, 256, 0, st>>>(                                         \
+      launch(k_aggregate_bwd_rows<TY_, NF_, true>, grid_rows, 256, 0, st,                                          \
           rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, nullptr, nullptr, ds_dst, gb, N, K, *lists); \
     if (launch_dz_gather(d, *lists, dh_out, Z, zrow, ds_dst, lw, mma ? dz_store : static_cast<void*>(dz), ga_src, ga_dst, \
                          N, status, st) < 0)                                                                   \
@@ -1176,23 +1191,23 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
         default: BWD_ROWS(TY_, 16); break;                                                                     \
       }                                                                                                        \
     } else {                                                                                                   \
-      k_aggregate_bwd<TY_><<<grid_rows, 256, sizeof(float) * H, st>>>(                                         \
+      launch(k_aggregate_bwd<TY_>, grid_rows, 256, sizeof(float) * H, st,                                          \
           rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, dz, ds_src, ds_dst, gb, N, H, K);           \
-      k_scores_bwd<TY_><<<grid_cols, 256, sizeof(float) * 2 * H, st>>>(zv, ds_src, ds_dst, lw.a_src, lw.a_dst, \
+      launch(k_scores_bwd<TY_>, grid_cols, 256, sizeof(float) * 2 * H, st, zv, ds_src, ds_dst, lw.a_src, lw.a_dst, \
                                                                        dz, ga_src, ga_dst, N, H, K);           \
     }                                                                                                          \
     if (mma) {                                                                                                 \
       if (launch_bwd_umma(d, h_in, dzb, lw.W, dh_in, gW, N, status, st) < 0) return -1;                        \
     } else {                                                                                                   \
       if (wide_atb)                                                                                            \
-        k_atb_tile<TY_, 128><<<g_atb, 256, 0, st>>>(static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);  \
+        launch(k_atb_tile<TY_, 128>, g_atb, 256, 0, st, static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);  \
       else                                                                                                     \
-        k_atb_tile<TY_, 64><<<g_atb, 64, 0, st>>>(static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);    \
+        launch(k_atb_tile<TY_, 64>, g_atb, 64, 0, st, static_cast<const TY_*>(h_in), dz, gW, N, H, chunk, vec);    \
       /* from 8,192 rows on the 128 x 128 tiles of the forward product have CTAs for every SM */               \
       if (N >= 8192 && H > 64)                                                                                 \
         launch_rows_times_matrix(d, dz, lw.Wt, dh_in, N, st);                                                  \
       else                                                                                                     \
-        k_gwt<TY_><<<g_gwt, 256, 0, st>>>(dz, static_cast<const TY_*>(lw.W), dh_in, N, H, H);                  \
+        launch(k_gwt<TY_>, g_gwt, 256, 0, st, dz, static_cast<const TY_*>(lw.W), dh_in, N, H, H);                  \
     }                                                                                                          \
   } while (0)
   if (d.dtype == XRL_BF16) BWD_BODY(bf16); else BWD_BODY(float);
@@ -1226,15 +1241,15 @@ int launch_embed_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, c
   if (d.dtype == XRL_BF16) {
     static bool attr[64] = {};
     if (!ensure_dynamic_smem(k_embed_bwd<bf16>, kSmemCeiling, attr)) return -1;
-    k_embed_inputs<bf16><<<grid_x, 256, 0, st>>>(rowptr, col, static_cast<const bf16*>(shape),
+    launch(k_embed_inputs<bf16>, grid_x, 256, 0, st, rowptr, col, static_cast<const bf16*>(shape),
                                                  static_cast<const bf16*>(eattr), xs, N);
-    k_embed_bwd<bf16><<<grid, 32 * warps, smem, st>>>(xs, op, static_cast<const bf16*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
+    launch(k_embed_bwd<bf16>, grid, 32 * warps, smem, st, xs, op, static_cast<const bf16*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
   } else {
     static bool attr[64] = {};
     if (!ensure_dynamic_smem(k_embed_bwd<float>, kSmemCeiling, attr)) return -1;
-    k_embed_inputs<float><<<grid_x, 256, 0, st>>>(rowptr, col, static_cast<const float*>(shape),
+    launch(k_embed_inputs<float>, grid_x, 256, 0, st, rowptr, col, static_cast<const float*>(shape),
                                                   static_cast<const float*>(eattr), xs, N);
-    k_embed_bwd<float><<<grid, 32 * warps, smem, st>>>(xs, op, static_cast<const float*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
+    launch(k_embed_bwd<float>, grid, 32 * warps, smem, st, xs, op, static_cast<const float*>(h0), dh0, masked, gW0, gb0, N, d.H, d.T);
   }
   return 2;
 }

@@ -31,6 +31,7 @@ constexpr int LIST = 96;             // list capacity per piece, a multiple of 8
 // them when its first graph has edges and no nodes, or behind)
 __global__ void k_t_count(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int32_t N, int32_t E,
                           int32_t* __restrict__ cnt) {
+  enter();
   const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e < E && e >= __ldg(rowptr) && e < __ldg(rowptr + N)) atomicAdd(&cnt[col[e]], 1);
 }
@@ -39,6 +40,7 @@ __global__ void k_t_count(const int32_t* __restrict__ rowptr, const int32_t* __r
 __global__ void k_t_fill(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int32_t N,
                          const int32_t* __restrict__ rowptr_t, int32_t* __restrict__ cnt, int32_t* __restrict__ col_t,
                          int32_t* __restrict__ inv) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   for (int32_t e = rowptr[i]; e < rowptr[i + 1]; ++e) {
@@ -83,6 +85,7 @@ k_dz_gather(const __grid_constant__ CUtensorMap map_dp, const float* __restrict_
             size_t z_row, const float* __restrict__ ds_dst, const float* __restrict__ a_src,
             const float* __restrict__ a_dst, T* __restrict__ dz, float* __restrict__ da_src, float* __restrict__ da_dst,
             int32_t N, int32_t K, int32_t br_shift, int32_t* status) {
+  enter();
   constexpr int H = 128 * NV;
   using L = Layout<NV>;
   extern __shared__ __align__(128) uint8_t gsm[];
@@ -294,6 +297,7 @@ k_rows_gather(const __grid_constant__ CUtensorMap map_z, const __grid_constant__
               const float2* __restrict__ scores, const T* __restrict__ h_out, float* __restrict__ dh, bool masked,
               const BwdLists tl, float* __restrict__ ds_dst, float* __restrict__ db, int32_t N, int32_t br_shift,
               int32_t* status) {
+  enter();
   using Smem = RowSmem<K, MERGED>;
   constexpr int VEC = VecOf<T>::N, NP = VEC / 2, H = 32 * VEC, LPH = 32 / K;
   constexpr uint32_t ZR = Smem::ROW, SR = MERGED ? ZR : 8 * K;
@@ -578,7 +582,7 @@ int launch_rows_k(const BwdLists& t, const int32_t* rowptr, const int32_t* col, 
     return -1;
   }
   const int shift = aggregate_block_shift(N);
-  k_rows_gather<T, K, MERGED><<<gather_grid(N, shift), TW * 32, smem, st>>>(
+  launch(k_rows_gather<T, K, MERGED>, gather_grid(N, shift), TW * 32, smem, st,
       mz, ms, rowptr, col, static_cast<const T*>(Z), reinterpret_cast<const float2*>(scores), static_cast<const T*>(h_out), dh,
       masked, t, ds_dst, gb, N, shift, status);
   return 1;
@@ -596,7 +600,7 @@ int launch_nv(const BwdLists& t, const float* dpre, const void* Z, size_t z_row,
   CUtensorMap m;
   if (!make_gather_map(&m, dpre, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, uint64_t(N), 128 * NV)) return -1;
   const int shift = aggregate_block_shift(N);
-  k_dz_gather<T, NV><<<gather_grid(N, shift), TW * 32, smem, st>>>(
+  launch(k_dz_gather<T, NV>, gather_grid(N, shift), TW * 32, smem, st,
       m, dpre, t.entry, t.rowptr, t.col, static_cast<const char*>(Z), z_row, ds_dst, lw.a_src, lw.a_dst, static_cast<T*>(dz),
       ga_src, ga_dst, N, K, shift, status);
   return 1;
@@ -616,9 +620,9 @@ int launch_bwd_lists(const int32_t* rowptr, const int32_t* col, int32_t N, int32
   if (N <= 0) return 0;
   int32_t* cnt = scratch;
   cudaMemsetAsync(cnt, 0, sizeof(int32_t) * size_t(N), st);
-  if (E > 0) k_t_count<<<(E + 255) / 256, 256, 0, st>>>(rowptr, col, N, E, cnt);
+  if (E > 0) launch(k_t_count, (E + 255) / 256, 256, 0, st, rowptr, col, N, E, cnt);
   const int n = launch_exclusive_scan(cnt, t.rowptr, N, scratch + N, st);
-  k_t_fill<<<(N + 255) / 256, 256, 0, st>>>(rowptr, col, N, t.rowptr, cnt, t.col, t.inv);
+  launch(k_t_fill, (N + 255) / 256, 256, 0, st, rowptr, col, N, t.rowptr, cnt, t.col, t.inv);
   return n + 2;
 }
 

@@ -69,6 +69,7 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
   if (warp == 0) {
     if (lane == 0) {
       load_w<C>(base, &map_w, col0);
+      enter();
       uint32_t it = 0;
       if (!produce_tiles<C>(base, &map_g, first, step, num_tiles, it)) {
         raise(status, XRL_ERR_TIMEOUT);
@@ -85,6 +86,7 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
     const bool leader = threadIdx.x == 64;
     volatile uint32_t* abort_flag = tmem_slot + 1;
     uint32_t lt = 0;
+    enter();
     // The features whose ReLU masks the result: this thread's row of a tile, 32 columns (64 bytes) per chunk, asked for a
     // whole tile ahead (2 NS bytes of them in registers: asked for one chunk ahead the four warps wait for them,
     // 0.448 instead of 0.351 ms at 990 k rows and hidden 256).
@@ -208,6 +210,7 @@ k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  enter();
   const int nblk = blk1 - blk0;            // >= 1: the launch has at most one part per block
 
   if (warp == 0) {
@@ -322,7 +325,7 @@ int launch_dh(int H, const void* h, const void* dzb, const void* W, float* dh, i
   if (!make_map(&mg, dzb, uint64_t(rows), H, BM) || !make_map(&mw, W, H, H, NS) || !make_map_f32(&mo, dh, uint64_t(rows), H))
     return -1;
   const int slices = (H + NS - 1) / NS, tiles = (rows + BM - 1) / BM, groups = kNumSMs / slices;
-  k_dh_umma<NS, KP><<<(tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st>>>(
+  launch(k_dh_umma<NS, KP>, (tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st,
       mg, mw, mo, static_cast<const bf16*>(h), rows, H, slices, status);
   return 1;
 }
@@ -340,7 +343,7 @@ int launch_dw(int H, const void* h, const void* dzb, float* dW, int32_t rows, in
   const int side = H / S, squares = side * side;
   // at least eight blocks per CTA: every CTA ends with a reduction of its whole square of dW into the gradient
   const int blocks = (rows + RB - 1) / RB, want = (blocks + 7) / 8, most = kNumSMs / squares;
-  k_dw_umma<S><<<(want < most ? want : most) * squares, kThreads, C::SMEM_BYTES, st>>>(
+  launch(k_dw_umma<S>, (want < most ? want : most) * squares, kThreads, C::SMEM_BYTES, st,
       mh, mg, mo, dW, rows, H, side, aligned, status);
   return 1;
 }

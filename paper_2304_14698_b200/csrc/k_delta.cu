@@ -20,6 +20,7 @@ constexpr int TB = 256;
 // with the same operator and bit-identical shape features; base[i] = that node, else -1.
 // Nodes of current graphs are never valid (they are always computed).
 __global__ void k_delta_valid(DeltaIn in, int32_t* __restrict__ valid, int32_t* __restrict__ base) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= in.N) return;
   const int32_t g = in.seg_id[i];
@@ -45,6 +46,7 @@ constexpr int32_t kNever = 1 << 20;   // level of a node no change reaches withi
 // producer k); kNever otherwise (for now).
 __global__ void k_delta_level0(DeltaIn in, const int32_t* __restrict__ valid, const int32_t* __restrict__ base,
                                int32_t* __restrict__ level) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= in.N) return;
   int32_t dirty = 1;
@@ -68,6 +70,7 @@ __global__ void k_delta_level0(DeltaIn in, const int32_t* __restrict__ valid, co
 // a node must not depend on the order in which threads run).
 __global__ void k_delta_propagate(DeltaIn in, int32_t t, const int32_t* __restrict__ lin,
                                   int32_t* __restrict__ lout) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= in.N) return;
   int32_t lv = lin[i];
@@ -79,6 +82,7 @@ __global__ void k_delta_propagate(DeltaIn in, int32_t t, const int32_t* __restri
 
 // counts[v] = number of nodes with level v (v <= L); warp-aggregated atomics
 __global__ void k_delta_count(int32_t N, const int32_t* __restrict__ level, int32_t* __restrict__ counts) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const int32_t lv = (i < N) ? level[i] : kNever;
   const uint32_t peers = __match_any_sync(0xFFFFFFFFu, lv);
@@ -91,6 +95,7 @@ __global__ void k_delta_count(int32_t N, const int32_t* __restrict__ level, int3
 __global__ void k_delta_assign(int32_t N, int32_t L, const int32_t* __restrict__ level,
                                const int32_t* __restrict__ counts, int32_t* __restrict__ cursor,
                                int32_t* __restrict__ rank, int32_t* __restrict__ list) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const int32_t lv = (i < N) ? level[i] : kNever;
   const uint32_t peers = __match_any_sync(0xFFFFFFFFu, lv);
@@ -110,6 +115,7 @@ __global__ void k_delta_assign(int32_t N, int32_t L, const int32_t* __restrict__
 
 __global__ void k_delta_degrees(DeltaIn in, int32_t n, const int32_t* __restrict__ list,
                                 int32_t* __restrict__ deg) {
+  enter();
   const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const int32_t i = list[r];
@@ -128,6 +134,7 @@ __global__ void k_delta_fill(DeltaIn in, int32_t n, int32_t t, const int32_t* __
                              const int32_t* __restrict__ rowptr_c, const int32_t* __restrict__ level,
                              const int32_t* __restrict__ rank, const int32_t* __restrict__ base,
                              int32_t* __restrict__ col_c, int32_t* __restrict__ self_c) {
+  enter();
   const int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const int32_t i = list[r];
@@ -140,6 +147,7 @@ __global__ void k_delta_fill(DeltaIn in, int32_t n, int32_t t, const int32_t* __
 __global__ void k_delta_remap(int32_t N, int32_t L, const int32_t* __restrict__ level,
                               const int32_t* __restrict__ rank, const int32_t* __restrict__ base,
                               int32_t* __restrict__ remap) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) remap[i] = dense_row(i, L + 1, level, rank, base);
 }
@@ -156,6 +164,7 @@ constexpr int32_t kGraphNodes = 2048, kGraphNodesMany = 4096, kManyGraphs = 256;
 __global__ void __launch_bounds__(TB)
 k_delta_graph(DeltaIn in, int32_t L, int32_t cap_n, int32_t* __restrict__ base, int32_t* __restrict__ level,
               int32_t* __restrict__ counts) {
+  enter();
   extern __shared__ int32_t dsm[];
   int32_t* base_s = dsm;                              // [cap_n]
   int8_t* lv = reinterpret_cast<int8_t*>(base_s + cap_n);   // [cap_n], 127 = not reached
@@ -231,20 +240,20 @@ int launch_delta_graphs(const DeltaIn& in, int32_t B, int32_t max_n, int32_t L, 
   cudaMemsetAsync(counts, 0, sizeof(int32_t) * size_t(L + 2), st);
   cudaMemsetAsync(cursor, 0, sizeof(int32_t) * size_t(L + 2), st);
   if (in.N <= 0 || B <= 0) return 0;
-  k_delta_graph<<<B, TB, smem, st>>>(in, L, max_n, base, level, counts);
+  launch(k_delta_graph, B, TB, smem, st, in, L, max_n, base, level, counts);
   if (cudaPeekAtLastError() != cudaSuccess) return -2;
   return 1;
 }
 int launch_delta_level0(const DeltaIn& in, int32_t* valid, int32_t* base, int32_t* level, cudaStream_t st) {
   if (in.N <= 0) return 0;
-  k_delta_valid<<<grid(in.N), TB, 0, st>>>(in, valid, base);
-  k_delta_level0<<<grid(in.N), TB, 0, st>>>(in, valid, base, level);
+  launch(k_delta_valid, grid(in.N), TB, 0, st, in, valid, base);
+  launch(k_delta_level0, grid(in.N), TB, 0, st, in, valid, base, level);
   return 2;
 }
 int launch_delta_propagate(const DeltaIn& in, int32_t t, const int32_t* level_in, int32_t* level_out,
                            cudaStream_t st) {
   if (in.N <= 0) return 0;
-  k_delta_propagate<<<grid(in.N), TB, 0, st>>>(in, t, level_in, level_out);
+  launch(k_delta_propagate, grid(in.N), TB, 0, st, in, t, level_in, level_out);
   return 1;
 }
 // counts / cursor: [L + 2] ints each, zeroed here
@@ -253,31 +262,31 @@ int launch_delta_count(int32_t N, int32_t L, const int32_t* level, int32_t* coun
   cudaMemsetAsync(counts, 0, sizeof(int32_t) * size_t(L + 2), st);
   cudaMemsetAsync(cursor, 0, sizeof(int32_t) * size_t(L + 2), st);
   if (N <= 0) return 0;
-  k_delta_count<<<grid(N), TB, 0, st>>>(N, level, counts);
+  launch(k_delta_count, grid(N), TB, 0, st, N, level, counts);
   return 1;
 }
 int launch_delta_assign(int32_t N, int32_t L, const int32_t* level, const int32_t* counts, int32_t* cursor,
                         int32_t* rank, int32_t* list, cudaStream_t st) {
   if (N <= 0) return 0;
-  k_delta_assign<<<grid(N), TB, 0, st>>>(N, L, level, counts, cursor, rank, list);
+  launch(k_delta_assign, grid(N), TB, 0, st, N, L, level, counts, cursor, rank, list);
   return 1;
 }
 int launch_delta_degrees(const DeltaIn& in, int32_t n, const int32_t* list, int32_t* deg, cudaStream_t st) {
   if (n <= 0) return 0;
-  k_delta_degrees<<<grid(n), TB, 0, st>>>(in, n, list, deg);
+  launch(k_delta_degrees, grid(n), TB, 0, st, in, n, list, deg);
   return 1;
 }
 int launch_delta_fill(const DeltaIn& in, int32_t n, int32_t t, const int32_t* list, const int32_t* rowptr_c,
                       const int32_t* level, const int32_t* rank, const int32_t* base, int32_t* col_c,
                       int32_t* self_c, cudaStream_t st) {
   if (n <= 0) return 0;
-  k_delta_fill<<<grid(n), TB, 0, st>>>(in, n, t, list, rowptr_c, level, rank, base, col_c, self_c);
+  launch(k_delta_fill, grid(n), TB, 0, st, in, n, t, list, rowptr_c, level, rank, base, col_c, self_c);
   return 1;
 }
 int launch_delta_remap(int32_t N, int32_t L, const int32_t* level, const int32_t* rank, const int32_t* base,
                        int32_t* remap, cudaStream_t st) {
   if (N <= 0) return 0;
-  k_delta_remap<<<grid(N), TB, 0, st>>>(N, L, level, rank, base, remap);
+  launch(k_delta_remap, grid(N), TB, 0, st, N, L, level, rank, base, remap);
   return 1;
 }
 

@@ -126,6 +126,7 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
     const bool leader = (threadIdx.x == 32);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     uint32_t lt = 0, stores = 0;
+    enter();
     for (int tile = first; tile < num_tiles; tile += step, ++lt) {
       const int buf = lt & 1;
       uint32_t okw = 1;
@@ -181,6 +182,7 @@ k_embed_umma(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ 
     const int r = ((warp - 5) & 3) * 32 + lane;               // row inside the tile
     const int pieces = 2 * ksteps;                            // 16-byte pieces per row actually read
     uint32_t lt = 0;
+    enter();
     for (int tile = first; tile < num_tiles; tile += step, ++lt) {
       if (int(lt % GROUPS) != g) continue;
       const int lrow = tile * BM + r;
@@ -291,7 +293,7 @@ int launch_h(const Dims& d, const int32_t* rowptr, const int32_t* col, const int
   const int tiles = int((rows + BM - 1) / BM);
   const int slices = (d.H + NS - 1) / NS, groups = kNumSMs / slices;
   const int grid = (tiles < groups ? tiles : groups) * slices;
-  k_embed_umma<NS, SLICED, PARTS><<<grid, kThreads, C::SMEM_BYTES, st>>>(mw, mh, rowptr, col, op,
+  launch(k_embed_umma<NS, SLICED, PARTS>, grid, kThreads, C::SMEM_BYTES, st, mw, mh, rowptr, col, op,
                                                          static_cast<const bf16*>(shape), row_list,
                                                          win.row_begin, int(rows), op_pieces, ksteps, status,
                                                          static_cast<const bf16*>(eattr), d.H, slices);

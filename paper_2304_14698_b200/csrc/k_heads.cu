@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(kRoThreads)
 k_readout(const T* __restrict__ h, const int32_t* __restrict__ chunk_row0,
           const int32_t* __restrict__ chunk_row1, int32_t chunk_begin, float* __restrict__ partial,
           int H, int32_t win_base, const int32_t* __restrict__ remap) {
+  enter();
   constexpr int VEC = VecOf<T>::N;
   extern __shared__ float red[];                 // [RG][H]
   const int NV = H / VEC;
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(kThreads)
 k_global_update(const float* __restrict__ partial, const int32_t* __restrict__ off, int32_t nblocks, int bshift,
                 const float* __restrict__ g0, const float* __restrict__ Wg, const float* __restrict__ bg,
                 float* __restrict__ emb, float* __restrict__ U_out, int H, int Dg, int B) {
+  enter();
   extern __shared__ __align__(16) float u[];     // [GP][xs], then scratch
   const int xs = row_stride(H + Dg), nt = blockDim.x, tid = threadIdx.x;
   int32_t* filled = reinterpret_cast<int32_t*>(u + GP * xs);       // [GP] parts of each graph that hold any row
@@ -157,6 +159,7 @@ k_policy_value_hidden(const float* __restrict__ emb, const Mlp pm, float* __rest
                       int policy_ctas, float* __restrict__ y1_out, float* __restrict__ y2_out,
                       const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask, int A, const Mlp vm,
                       float* __restrict__ y1v, int VC) {
+  enter();
   extern __shared__ __align__(16) float sm[];
   const int nt = blockDim.x, tid = threadIdx.x;
   if (int(blockIdx.x) < policy_ctas) {
@@ -288,6 +291,7 @@ __global__ void __launch_bounds__(1024)
 k_env_policy(const float* __restrict__ logit, const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask,
              const Mlp vmlp, float* __restrict__ probs, float* __restrict__ value, int32_t* __restrict__ action, int A,
              uint64_t seed, uint64_t step, int32_t* status, const float* __restrict__ y1v) {
+  enter();
   extern __shared__ __align__(16) unsigned long long sm64[];   // [nt + 2] u64, then floats
   const int nt = blockDim.x, tid = threadIdx.x;
   float* scratch = reinterpret_cast<float*>(sm64 + nt + 2);   // [nt]
@@ -356,6 +360,7 @@ k_env_policy(const float* __restrict__ logit, const int32_t* __restrict__ env_of
 __global__ void __launch_bounds__(1024)
 k_sample(const float* __restrict__ probs, int A1, uint64_t seed, uint64_t step,
          int32_t* __restrict__ action) {
+  enter();
   extern __shared__ unsigned long long sm64[];
   const int32_t e = blockIdx.x;
   const int32_t act = sample_row(probs + size_t(e) * A1, A1, seed, step, uint32_t(e), sm64);
@@ -418,11 +423,11 @@ int launch_readout(const Dims& d, const void* h, const int32_t* chunk_row0, cons
   if (n <= 0) return 0;
   if (d.dtype == XRL_BF16) {
     const int RG = kRoThreads / (d.H / 8);
-    k_readout<bf16><<<n, kRoThreads, sizeof(float) * size_t(RG) * d.H, st>>>(
+    launch(k_readout<bf16>, n, kRoThreads, sizeof(float) * size_t(RG) * d.H, st,
         static_cast<const bf16*>(h), chunk_row0, chunk_row1, chunk_begin, partial, d.H, win_base, remap);
   } else {
     const int RG = kRoThreads / (d.H / 4);
-    k_readout<float><<<n, kRoThreads, sizeof(float) * size_t(RG) * d.H, st>>>(
+    launch(k_readout<float>, n, kRoThreads, sizeof(float) * size_t(RG) * d.H, st,
         static_cast<const float*>(h), chunk_row0, chunk_row1, chunk_begin, partial, d.H, win_base, remap);
   }
   return 1;
@@ -434,7 +439,7 @@ int global_update(const Dims& d, const float* partial, const int32_t* off, int32
                   const DevWeights& w, float* emb, float* U_out, int32_t B, size_t smem, cudaStream_t st, int nt = kThreads) {
   static bool attr[64] = {};
   if (smem > 48 * 1024 && !ensure_dynamic_smem(k_global_update<GP, BLOCKS>, 227 * 1024, attr)) return -1;
-  k_global_update<GP, BLOCKS><<<(B + GP - 1) / GP, nt, smem, st>>>(partial, off, nblocks, shift, g0, w.Wg, w.bg, emb,
+  launch(k_global_update<GP, BLOCKS>, (B + GP - 1) / GP, nt, smem, st, partial, off, nblocks, shift, g0, w.Wg, w.bg, emb,
                                                                          U_out, d.H, d.Dg, B);
   return 1;
 }
@@ -465,7 +470,7 @@ int policy_value(const Dims& d, const Mlp& pm, const Mlp& vm, const float* emb, 
   static bool attr[64] = {};
   if (smem > 48 * 1024 && !ensure_dynamic_smem(k_policy_value_hidden<GP>, 227 * 1024, attr)) return -1;
   const int pc = (B + GP - 1) / GP;
-  k_policy_value_hidden<GP><<<pc + num_envs * VC, kThreads, smem, st>>>(emb, pm, logit, d.H, B, pc, y1_out, y2_out, env_off,
+  launch(k_policy_value_hidden<GP>, pc + num_envs * VC, kThreads, smem, st, emb, pm, logit, d.H, B, pc, y1_out, y2_out, env_off,
                                                                         mask, d.A, vm, y1v, VC);
   return 1;
 }
@@ -514,7 +519,7 @@ int launch_heads(const Dims& d, const DevWeights& w, const float* emb, const int
   if (num_envs <= kNumSMs && d.Hm2 > 0) want = 1024;     // (an SM per environment: more parts, shorter chains)
   const int nt = pow2_threads(want);
   const size_t smem = sizeof(unsigned long long) * size_t(nt + 2) + sizeof(float) * size_t(nt + d.Hm);
-  k_env_policy<<<num_envs, nt, smem, st>>>(logit_ws, env_off, mask, vm, probs, value, action, d.A, seed, step, status, y1v);
+  launch(k_env_policy, num_envs, nt, smem, st, logit_ws, env_off, mask, vm, probs, value, action, d.A, seed, step, status, y1v);
   return 2;
 }
 
@@ -522,7 +527,7 @@ int launch_sample(const float* probs, int32_t num_envs, int32_t A1, uint64_t see
                   int32_t* action, cudaStream_t st) {
   if (num_envs <= 0) return 0;
   const int nt = pow2_threads(A1);
-  k_sample<<<num_envs, nt, sizeof(unsigned long long) * size_t(nt + 1), st>>>(probs, A1, seed, step,
+  launch(k_sample, num_envs, nt, sizeof(unsigned long long) * size_t(nt + 1), st, probs, A1, seed, step,
                                                                               action);
   return 1;
 }

@@ -17,6 +17,7 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_tile(const int32_t* __restrict__ in, int32_t* __restrict__ out, int32_t n_in, int32_t n_out,
             int32_t* __restrict__ block_sums) {
+  enter();
   __shared__ int32_t warp_tot[kScanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(tid) * kScanItems;
@@ -54,6 +55,7 @@ k_scan_tile(const int32_t* __restrict__ in, int32_t* __restrict__ out, int32_t n
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_add(int32_t* __restrict__ out, int32_t n_out, const int32_t* __restrict__ block_offsets) {
+  enter();
   const int32_t add = block_offsets[blockIdx.x];
   const int64_t base = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanItems;
 #pragma unroll
@@ -70,16 +72,16 @@ int exclusive_scan(const int32_t* in, int32_t* out, int32_t n_in, int32_t* ws, c
   const int tiles = num_tiles(n_out);
   int launches = 0;
   if (tiles == 1) {
-    k_scan_tile<<<1, kScanThreads, 0, st>>>(in, out, n_in, n_out, nullptr);
+    launch(k_scan_tile, 1, kScanThreads, 0, st, in, out, n_in, n_out, nullptr);
     return 1;
   }
   int32_t* sums = ws;
   int32_t* sums_scanned = ws + tiles;
-  k_scan_tile<<<tiles, kScanThreads, 0, st>>>(in, out, n_in, n_out, sums);
+  launch(k_scan_tile, tiles, kScanThreads, 0, st, in, out, n_in, n_out, sums);
   ++launches;
   // scan of the tile sums (tiles outputs are enough; the recursion writes tiles + 1)
   launches += exclusive_scan(sums, sums_scanned, tiles, ws + 2 * tiles + 2, st);
-  k_scan_add<<<tiles, kScanThreads, 0, st>>>(out, n_out, sums_scanned);
+  launch(k_scan_add, tiles, kScanThreads, 0, st, out, n_out, sums_scanned);
   return launches + 1;
 }
 
@@ -99,6 +101,7 @@ __device__ __forceinline__ int32_t upper_segment(const int32_t* __restrict__ off
 constexpr int kCoarseShift = 10;
 __global__ void k_edge_coarse(const int32_t* __restrict__ edge_off, int32_t B, int32_t E,
                               int32_t* __restrict__ coarse) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if ((int64_t(i) << kCoarseShift) < E) coarse[i] = upper_segment(edge_off, B, i << kCoarseShift);
 }
@@ -113,6 +116,7 @@ __global__ void k_node_segments(const int32_t* __restrict__ node_off, int32_t B,
                                 const int32_t* __restrict__ op, int32_t T,
                                 int32_t* __restrict__ seg_id, int32_t* __restrict__ deg,
                                 int32_t* status) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   seg_id[i] = upper_segment(node_off, B, i);
@@ -123,6 +127,7 @@ __global__ void k_node_segments(const int32_t* __restrict__ node_off, int32_t B,
 
 __global__ void k_graph_envs(const int32_t* __restrict__ env_off, int32_t num_envs, int32_t B,
                              int32_t* __restrict__ graph_env) {
+  enter();
   const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g < B) graph_env[g] = upper_segment(env_off, num_envs, g);
 }
@@ -132,6 +137,7 @@ __global__ void k_edge_count(const int32_t* __restrict__ edge_src, const int32_t
                              const int32_t* __restrict__ edge_off, const int32_t* __restrict__ node_off,
                              const int32_t* __restrict__ coarse, int32_t B, int32_t E,
                              int32_t* __restrict__ deg, int32_t* status) {
+  enter();
   const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   const int32_t g = graph_of_edge(edge_off, coarse, B, e);
@@ -148,6 +154,7 @@ __global__ void k_edge_scatter(const int32_t* __restrict__ edge_src, const int32
                                const int32_t* __restrict__ coarse, const int32_t* __restrict__ rowptr,
                                int32_t B, int32_t E, int32_t* __restrict__ cursor,
                                int2* __restrict__ tmp) {
+  enter();
   const int32_t e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   const int32_t g = graph_of_edge(edge_off, coarse, B, e);
@@ -167,6 +174,7 @@ constexpr int kShortRow = 32;
 __global__ void k_row_order(const int32_t* __restrict__ rowptr, const int2* __restrict__ tmp, int32_t N,
                             int32_t* __restrict__ col, int32_t* __restrict__ long_rows,
                             int32_t* __restrict__ long_count, int32_t* __restrict__ eid) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int32_t b = rowptr[i], n = rowptr[i + 1] - b;
@@ -187,6 +195,7 @@ __global__ void __launch_bounds__(256)
 k_row_order_long(const int32_t* __restrict__ rowptr, const int2* __restrict__ tmp,
                  int32_t* __restrict__ col, const int32_t* __restrict__ long_rows,
                  const int32_t* __restrict__ long_count, int32_t* __restrict__ eid) {
+  enter();
   const int lane = threadIdx.x & 31;
   const int32_t warps = (gridDim.x * blockDim.x) >> 5;
   const int32_t count = *long_count;
@@ -229,6 +238,7 @@ k_pack_graph(int32_t* __restrict__ node_off, int32_t* __restrict__ edge_off,
              const int32_t* __restrict__ n_nodes, const int32_t* __restrict__ n_edges,
              const int32_t* __restrict__ env_off, int32_t num_envs, int32_t* __restrict__ graph_env,
              int32_t* __restrict__ op_copy, const uint4* __restrict__ shape, uint4* __restrict__ shape_copy, int32_t pieces) {
+  enter();
   extern __shared__ __align__(16) int32_t psm[];
   int32_t* deg = psm;                         // [cap_n + 1] in-degree, then exclusive row starts
   int32_t* cur = psm + cap_n + 1;             // [cap_n]     row cursors
@@ -389,6 +399,7 @@ size_t pack_graph_smem(int32_t cap_n, int32_t cap_m) {
 namespace {
 __global__ void k_permute_rows(const uint4* __restrict__ src, const int32_t* __restrict__ eid,
                                uint4* __restrict__ dst, int64_t E, int pieces) {
+  enter();
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= E * pieces) return;
   const int64_t k = i / pieces;
@@ -402,7 +413,7 @@ int launch_permute_edge_rows(const void* src, const int32_t* eid, void* dst, int
   if (E <= 0) return 0;
   const int pieces = row_bytes / 16;
   const int64_t n = E * pieces;
-  k_permute_rows<<<unsigned((n + 255) / 256), 256, 0, st>>>(static_cast<const uint4*>(src), eid,
+  launch(k_permute_rows, unsigned((n + 255) / 256), 256, 0, st, static_cast<const uint4*>(src), eid,
                                                              static_cast<uint4*>(dst), E, pieces);
   return 1;
 }
@@ -413,6 +424,7 @@ namespace {
 __global__ void k_merge_csr(const int32_t* __restrict__ rp_a, const int32_t* __restrict__ col_a,
                             const int32_t* __restrict__ rp_b, const int32_t* __restrict__ col_b, int32_t N,
                             int32_t* __restrict__ rp_m, int32_t* __restrict__ col_m) {
+  enter();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i > N) return;
   const int32_t a0 = rp_a[i], b0 = rp_b[i];
@@ -427,7 +439,7 @@ __global__ void k_merge_csr(const int32_t* __restrict__ rp_a, const int32_t* __r
 
 int launch_merge_csr(const int32_t* rp_a, const int32_t* col_a, const int32_t* rp_b, const int32_t* col_b,
                      int32_t N, int32_t* rp_m, int32_t* col_m, cudaStream_t st) {
-  k_merge_csr<<<(N + 1 + 255) / 256, 256, 0, st>>>(rp_a, col_a, rp_b, col_b, N, rp_m, col_m);
+  launch(k_merge_csr, (N + 1 + 255) / 256, 256, 0, st, rp_a, col_a, rp_b, col_b, N, rp_m, col_m);
   return 1;
 }
 
@@ -459,7 +471,7 @@ int launch_pack_offsets(const PackIn& in, const PackOut& out, cudaStream_t st) {
   launches += exclusive_scan(in.n_nodes, out.node_off, in.B, out.scan_ws, st);
   launches += exclusive_scan(in.n_edges, out.edge_off, in.B, out.scan_ws, st);
   if (in.B > 0) {
-    k_graph_envs<<<(in.B + TB - 1) / TB, TB, 0, st>>>(in.env_off, in.num_envs, in.B, out.graph_env);
+    launch(k_graph_envs, (in.B + TB - 1) / TB, TB, 0, st, in.env_off, in.num_envs, in.B, out.graph_env);
     ++launches;
   }
   return launches;
@@ -475,7 +487,7 @@ int launch_pack_graphs(const PackIn& in, const PackOut& out, int T, int32_t g0, 
 #define PACK_GRAPH(NT_, OFF_, ATTR_)                                                                              \
   do {                                                                                                            \
     ensure_dynamic_smem(k_pack_graph<NT_, OFF_>, 160 * 1024, ATTR_);                                              \
-    k_pack_graph<NT_, OFF_><<<g1 - g0, NT_, smem, st>>>(out.node_off, out.edge_off, in.op, in.edge_src,           \
+    launch(k_pack_graph<NT_, OFF_>, g1 - g0, NT_, smem, st, out.node_off, out.edge_off, in.op, in.edge_src,           \
                                                         in.edge_dst, T, in.B, in.max_n, out.seg_id, out.rowptr,   \
                                                         out.col, status, g0, out.eid, in.n_nodes, in.n_edges,     \
                                                         in.env_off, in.num_envs, out.graph_env, out.op_copy,      \
@@ -500,14 +512,14 @@ int launch_pack(const PackIn& in, const PackOut& out, int T, int32_t* status, cu
   const int TB = 256;
   if (pack_per_graph(in)) return launches + launch_pack_graphs(in, out, T, 0, in.B, status, st);
   if (in.N > 0) {
-    k_node_segments<<<(in.N + TB - 1) / TB, TB, 0, st>>>(out.node_off, in.B, in.N, in.op, T,
+    launch(k_node_segments, (in.N + TB - 1) / TB, TB, 0, st, out.node_off, in.B, in.N, in.op, T,
                                                           out.seg_id, out.deg, status);
     ++launches;
   }
   if (in.E > 0) {
     const int nc = (in.E >> kCoarseShift) + 1;
-    k_edge_coarse<<<(nc + TB - 1) / TB, TB, 0, st>>>(out.edge_off, in.B, in.E, out.coarse);
-    k_edge_count<<<(in.E + TB - 1) / TB, TB, 0, st>>>(in.edge_src, in.edge_dst, out.edge_off,
+    launch(k_edge_coarse, (nc + TB - 1) / TB, TB, 0, st, out.edge_off, in.B, in.E, out.coarse);
+    launch(k_edge_count, (in.E + TB - 1) / TB, TB, 0, st, in.edge_src, in.edge_dst, out.edge_off,
                                                        out.node_off, out.coarse, in.B, in.E, out.deg, status);
     launches += 2;
   }
@@ -516,12 +528,12 @@ int launch_pack(const PackIn& in, const PackOut& out, int T, int32_t* status, cu
     cudaMemsetAsync(out.deg, 0, sizeof(int32_t) * size_t(in.N), st);      // reused as the row cursors
     cudaMemsetAsync(out.long_count, 0, sizeof(int32_t), st);
     int2* tmp = reinterpret_cast<int2*>(out.tmp_eid);
-    k_edge_scatter<<<(in.E + TB - 1) / TB, TB, 0, st>>>(in.edge_src, in.edge_dst, out.edge_off,
+    launch(k_edge_scatter, (in.E + TB - 1) / TB, TB, 0, st, in.edge_src, in.edge_dst, out.edge_off,
                                                          out.node_off, out.coarse, out.rowptr, in.B, in.E,
                                                          out.deg, tmp);
-    k_row_order<<<(in.N + TB - 1) / TB, TB, 0, st>>>(out.rowptr, tmp, in.N, out.col, out.long_rows,
+    launch(k_row_order, (in.N + TB - 1) / TB, TB, 0, st, out.rowptr, tmp, in.N, out.col, out.long_rows,
                                                       out.long_count, out.eid);
-    k_row_order_long<<<kNumSMs, 256, 0, st>>>(out.rowptr, tmp, out.col, out.long_rows, out.long_count, out.eid);
+    launch(k_row_order_long, kNumSMs, 256, 0, st, out.rowptr, tmp, out.col, out.long_rows, out.long_count, out.eid);
     launches += 3;
   }
   return launches;

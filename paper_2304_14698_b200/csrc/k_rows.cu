@@ -37,6 +37,7 @@ k_embed(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
         const int32_t* __restrict__ op, const T* __restrict__ shape, const T* __restrict__ W0,
         const float* __restrict__ b0, T* __restrict__ h, int H, int Tn, Window win,
         const int32_t* __restrict__ row_list, const T* __restrict__ eattr) {
+  enter();
   constexpr int VEC = VecOf<T>::N;
   constexpr int RPW = 32 / LPR;
   extern __shared__ __align__(16) float smem[];
@@ -157,6 +158,7 @@ template <typename T, int LPR, int VPL>
 __global__ void __launch_bounds__(kRowThreads)
 k_scores(const T* __restrict__ Z, const float* __restrict__ a_src, const float* __restrict__ a_dst,
          float2* __restrict__ scores, int H, int K, Window win) {
+  enter();
   constexpr int VEC = VecOf<T>::N;
   constexpr int RPW = 32 / LPR;
   constexpr int WARPS = kRowThreads / 32;
@@ -263,6 +265,7 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
             const T* __restrict__ Z, const float2* __restrict__ scores,
             const float* __restrict__ bias, T* __restrict__ h_out, int H, int K, Window win,
             const int32_t* __restrict__ self_idx, int block_rows) {
+  enter();
   constexpr int VEC = VecOf<T>::N;
   constexpr int RPW = 32 / LPR;
   constexpr int WARPS = kRowThreads / 32;
@@ -449,7 +452,7 @@ int launch_embed(const Dims& d, const int32_t* rowptr, const int32_t* col, const
 #define CALL(TY_, LPR, VPL)                                                                        \
   if (smem > 48 * 1024 &&                                                                          \
       !ensure_dynamic_smem(k_embed<TY_, LPR, VPL>, int(smem), attr_set[embed_slot(sizeof(TY_), LPR, VPL)])) return -1; \
-  k_embed<TY_, LPR, VPL><<<row_grid(rows, kEmbedRows), kRowThreads, smem, st>>>(                           \
+  launch(k_embed<TY_, LPR, VPL>, row_grid(rows, kEmbedRows), kRowThreads, smem, st,                            \
       rowptr, col, op, static_cast<const TY_*>(shape), static_cast<const TY_*>(w.W0), w.b0,   \
       static_cast<TY_*>(h), d.H, d.T, win, row_list, static_cast<const TY_*>(eattr))
   if (d.dtype == XRL_BF16) XRL_ROW_DISPATCH(bf16, d.H, CALL);
@@ -463,7 +466,7 @@ int launch_scores(const Dims& d, const void* Z, const LayerWeights& lw, float* s
   const int64_t rows = int64_t(win.row_end) - win.row_begin;
   if (rows <= 0) return 0;
 #define CALL(TY_, LPR, VPL)                                                                        \
-  k_scores<TY_, LPR, VPL><<<row_grid(rows, 32 / LPR), kRowThreads, 0, st>>>(                       \
+  launch(k_scores<TY_, LPR, VPL>, row_grid(rows, 32 / LPR), kRowThreads, 0, st,                        \
       static_cast<const TY_*>(Z), lw.a_src, lw.a_dst, reinterpret_cast<float2*>(scores), d.H, d.K, win)
   if (d.dtype == XRL_BF16) XRL_ROW_DISPATCH(bf16, d.H, CALL);
   else XRL_ROW_DISPATCH(float, d.H, CALL);
@@ -491,7 +494,7 @@ int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, c
     int64_t br_ = (rows + warps_avail - 1) / warps_avail;                                          \
     br_ = ((br_ + rpw_ - 1) / rpw_) * rpw_;                                                        \
     if (br_ > kAggBlockRows) br_ = kAggBlockRows;                                                  \
-    k_aggregate<TY_, LPR, VPL><<<row_grid(rows, int(br_)), kRowThreads, 0, st>>>(                  \
+    launch(k_aggregate<TY_, LPR, VPL>, row_grid(rows, int(br_)), kRowThreads, 0, st,                   \
         rowptr, col, static_cast<const TY_*>(Z), reinterpret_cast<const float2*>(scores), bias,    \
         static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_));                              \
   } while (0)

@@ -30,6 +30,7 @@ template <typename T, bool SCORES>
 __global__ void __launch_bounds__(256)
 k_xform_simt(const T* __restrict__ h, const T* __restrict__ W, T* __restrict__ Z, int H, int rows,
              const float* __restrict__ a_src, const float* __restrict__ a_dst, float2* __restrict__ scores, int K) {
+  enter();
   __shared__ float As[BK][BM + 4];
   __shared__ float Bs[BK][BN + 4];
   const int tid = threadIdx.x;
@@ -117,6 +118,7 @@ __device__ __forceinline__ void load4<bf16>(const bf16* p, bool ok, float (&v)[4
 template <typename TA, typename TW, typename TZ>
 __global__ void __launch_bounds__(256)
 k_xform_simt128(const TA* __restrict__ h, const TW* __restrict__ W, TZ* __restrict__ Z, int H, int rows) {
+  enter();
   __shared__ __align__(16) float As[TK][TM];
   __shared__ __align__(16) float Bs[TK][TN];
   const int tid = threadIdx.x;
@@ -200,6 +202,7 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 
 __global__ void __launch_bounds__(256, 2)
 k_xform_tf32x3(const float* __restrict__ h, const float* __restrict__ W, float* __restrict__ Z, int H, int rows) {
+  enter();
   extern __shared__ __align__(16) uint32_t xs[];          // A hi, A lo, B hi, B lo: each [XK][XS]
   uint32_t* Ah = xs;
   uint32_t* Al = Ah + XK * XS;
@@ -327,30 +330,30 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
     if (k == 1) return 1;
     if (k < 0) {
       const dim3 gx(unsigned((rows + XM - 1) / XM), unsigned((d.H + XN - 1) / XN));
-      k_xform_tf32x3<<<gx, 256, sizeof(uint32_t) * 4 * XK * XS, st>>>(hp, static_cast<const float*>(lw.W), zp, d.H, int(rows));
+      launch(k_xform_tf32x3, gx, 256, sizeof(uint32_t) * 4 * XK * XS, st, hp, static_cast<const float*>(lw.W), zp, d.H, int(rows));
     }
     return 1 + launch_scores(d, Z, lw, scores, win, st);
   }
   if (rows >= 8192) {
     const dim3 g128(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
-    k_xform_simt128<bf16, bf16, bf16><<<g128, 256, 0, st>>>(static_cast<const bf16*>(h) + off, static_cast<const bf16*>(lw.W),
+    launch(k_xform_simt128<bf16, bf16, bf16>, g128, 256, 0, st, static_cast<const bf16*>(h) + off, static_cast<const bf16*>(lw.W),
                                                             static_cast<bf16*>(Z) + off, d.H, int(rows));
     return 1 + launch_scores(d, Z, lw, scores, win, st);
   }
   dim3 grid(unsigned((rows + BM - 1) / BM), unsigned((d.H + BN - 1) / BN));
   if (d.dtype == XRL_BF16) {
-    k_xform_simt<bf16, false><<<grid, 256, 0, st>>>(static_cast<const bf16*>(h) + off,
+    launch(k_xform_simt<bf16, false>, grid, 256, 0, st, static_cast<const bf16*>(h) + off,
                                                    static_cast<const bf16*>(lw.W),
                                                    static_cast<bf16*>(Z) + off, d.H, int(rows), nullptr, nullptr, nullptr,
                                                    d.K);
   } else if (fuse_scores(d, lw, scores)) {
-    k_xform_simt<float, true><<<grid, 256, 0, st>>>(static_cast<const float*>(h) + off,
+    launch(k_xform_simt<float, true>, grid, 256, 0, st, static_cast<const float*>(h) + off,
                                                    static_cast<const float*>(lw.W),
                                                    static_cast<float*>(Z) + off, d.H, int(rows), lw.a_src, lw.a_dst, sc,
                                                    d.K);
     return 1;
   } else {
-    k_xform_simt<float, false><<<grid, 256, 0, st>>>(static_cast<const float*>(h) + off,
+    launch(k_xform_simt<float, false>, grid, 256, 0, st, static_cast<const float*>(h) + off,
                                                     static_cast<const float*>(lw.W),
                                                     static_cast<float*>(Z) + off, d.H, int(rows), nullptr, nullptr,
                                                     nullptr, d.K);
@@ -363,9 +366,9 @@ int launch_xform_simt(const Dims& d, const void* h, const LayerWeights& lw, void
 int launch_rows_times_matrix(const Dims& d, const float* G, const void* Wt, float* out, int rows, cudaStream_t st) {
   dim3 g(unsigned((rows + TM - 1) / TM), unsigned((d.H + TN - 1) / TN));
   if (d.dtype == XRL_BF16)
-    k_xform_simt128<float, bf16, float><<<g, 256, 0, st>>>(G, static_cast<const bf16*>(Wt), out, d.H, rows);
+    launch(k_xform_simt128<float, bf16, float>, g, 256, 0, st, G, static_cast<const bf16*>(Wt), out, d.H, rows);
   else
-    k_xform_simt128<float, float, float><<<g, 256, 0, st>>>(G, static_cast<const float*>(Wt), out, d.H, rows);
+    launch(k_xform_simt128<float, float, float>, g, 256, 0, st, G, static_cast<const float*>(Wt), out, d.H, rows);
   return 1;
 }
 

@@ -112,6 +112,7 @@ k_xform_tf32(const float* __restrict__ h, const float* __restrict__ Wt, const __
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  enter();
 
   if (warp == 0) {
     // ---- MMA issuer -------------------------------------------------------------------------------
@@ -272,7 +273,7 @@ int launch_h(const Dims& d, const float* h, const LayerWeights& lw, float* Z, fl
   const int slices = K / NS, tiles = int((rows + BM - 1) / BM), groups = kNumSMs / slices;
   const int head = d.H / d.K;
   const bool whole = slices == 1 || NS % head == 0;      // else a head crosses a slice's end: half-scores from Z afterwards
-  k_xform_tf32<NS, K><<<(tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st>>>(
+  launch(k_xform_tf32<NS, K>, (tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st,
       h, static_cast<const float*>(lw.Wt), mz, lw.a_src, lw.a_dst, whole ? scores : nullptr, d.K, int(rows), head, slices, status);
   return whole ? 1 : 0;
 }

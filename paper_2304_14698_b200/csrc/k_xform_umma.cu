@@ -76,6 +76,7 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
     // ---- TMA producer ---------------------------------------------------------------------------
     if (lane == 0) {
       load_w<C>(base, &map_w, col0);
+      enter();
       uint32_t it = 0;
       if (!produce_tiles<C>(base, &map_h, first, step, num_tiles, it)) {
         raise(status, XRL_ERR_TIMEOUT);
@@ -85,12 +86,14 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
   } else if (warp == 1) {
     // ---- MMA issuer -----------------------------------------------------------------------------
     if (lane == 0) {
+      enter();
       uint32_t it = 0, lt = 0;
       if (!mma_tiles<C, NS>(base, tmem_base, first, step, num_tiles, it, lt, 0)) raise(status, XRL_ERR_TIMEOUT);
     }
   } else {
     // ---- epilogue: 4 warps ------------------------------------------------------------------------
     uint32_t lt = 0;
+    enter();
     epilogue_tiles<C, NS, ROUNDED>(smem, base, tmem_base, &map_z, scores ? scores + col0 / d : nullptr, score_stride, rows,
                                    d, first, step, num_tiles, lt, threadIdx.x == 64, status, col0, cols);
   }
@@ -130,7 +133,7 @@ int launch_h(const Dims& d, const void* h, const LayerWeights& lw, void* Z, floa
     return -1;
   const int tiles = int((rows + BM - 1) / BM);
   const int groups = kNumSMs / slices, grid = (tiles < groups ? tiles : groups) * slices;
-  k_xform_umma<NS, KP, kRounded><<<grid, kThreads, C::SMEM_BYTES, st>>>(
+  launch(k_xform_umma<NS, KP, kRounded>, grid, kThreads, C::SMEM_BYTES, st,
       mh, mw, mz, lw.a_src, lw.a_dst, whole_heads ? sc : nullptr, sc_stride, int(rows), d.H, head, slices, status);
   return whole_heads ? 1 : 1 + launch_scores(d, Z, lw, scores, win, st);
 }
