@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_w,
           const __grid_constant__ CUtensorMap map_o, const bf16* __restrict__ h, int rows, int H, int slices,
           int32_t* status) {
-  using C = Cfg<NS, KP>;
+  using C = Cfg<NS, KP, true>;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -55,7 +55,7 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM);
   if (threadIdx.x == 0) {
     tmem_slot[1] = 0;
-    init_barriers<C>(base);
+    init_barriers<C>(base, 128);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -318,7 +318,7 @@ bool make_map_f32(CUtensorMap* m, void* ptr, uint64_t rows, uint64_t cols) {
 
 template <int NS, int KP>
 int launch_dh(int H, const void* h, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
-  using C = Cfg<NS, KP>;
+  using C = Cfg<NS, KP, true>;
   static bool attr_set[64] = {};
   if (!ensure_dynamic_smem(k_dh_umma<NS, KP>, C::SMEM_BYTES, attr_set)) return -1;
   CUtensorMap mg, mw, mo;

@@ -5,7 +5,7 @@
 // tiles per SM at most; launched layer by layer it is bound by the fill and drain of 2 L small kernels.
 // Here one persistent CTA per SM owns the tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... for the
 // whole stack and alternates between two phases per layer:
-//   transform   Z = h W (+ half-scores) of its tiles: TMA producer, tcgen05 issuer and four epilogue
+//   transform   Z = h W (+ half-scores) of its tiles: TMA producer, tcgen05 issuer and eight epilogue
 //               warps, exactly the roles of the one-layer kernel;
 //   attention   score / softmax / aggregate of the rows of the same tiles: every warp takes blocks of
 //               destination rows and gathers the producers' Z rows with the TMA unit.
@@ -32,7 +32,7 @@ using namespace umma;
 namespace {
 
 constexpr int H = 256;
-constexpr int kWarps = 16;             // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue; all 16 in the attention phase
+constexpr int kWarps = 16;             // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue; all 16 in the attention phase
 constexpr int kThreads = 32 * kWarps;
 #ifndef XRL_COOP_RING_GROUPS
 #define XRL_COOP_RING_GROUPS 2
@@ -50,8 +50,7 @@ using XC = xform::Cfg<H>;
 
 struct CoopParams {
   CUtensorMap map_h;                   // node features [rows x H] bf16: A tiles of the transform
-  CUtensorMap map_zs[2];               // the two Z buffers as [rows x H] bf16 with the merged row stride: stores
-  CUtensorMap map_zg[2];               // the same buffers as merged rows of 32-bit words: gathers
+  CUtensorMap map_zg[2];               // the two Z buffers as merged rows of 32-bit words: gathers
   CUtensorMap map_w[kMaxLayers];       // W^T of each layer
   const float* a_src[kMaxLayers];
   const float* a_dst[kMaxLayers];
@@ -110,7 +109,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
     tmem_slot[1] = 0;
     tmem_slot[2] = (base & 1023u) != 0 ? 1u : 0u;
     if (tmem_slot[2]) raise(p.status, XRL_ERR_UNSUPPORTED);
-    xform::init_barriers<XC>(base);
+    xform::init_barriers<XC>(base, 4 * xform::epilogue_groups(H, H / K));
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -152,13 +151,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
           raise(p.status, XRL_ERR_TIMEOUT);
           *abort_role = 1;
         }
-      } else if (warp < 6) {
-        float2* pairs = reinterpret_cast<float2*>(reinterpret_cast<char*>(p.Z[zb]) + size_t(H) * 2);
-        xform::epilogue_tiles<XC, H, false>(smem, base, tmem_base, &p.map_zs[zb], pairs, p.z_row_bytes / 8, p.rows, H / K,
-                                 blockIdx.x, gridDim.x, num_tiles, epi_lt, threadIdx.x == 64, p.status);
+      } else if (warp < 10) {
+        char* z = reinterpret_cast<char*>(p.Z[zb]);
+        xform::epilogue_tiles<XC, H, false, H / K>(smem, base, tmem_base, z, p.z_row_bytes, reinterpret_cast<float2*>(z + H * 2),
+                                                   p.z_row_bytes / 8, p.rows, H / K, xform::epilogue_groups(H, H / K), blockIdx.x,
+                                                   gridDim.x, num_tiles, epi_lt, p.status);
       }
     }
-    // the pairs were written with plain stores and are gathered by other CTAs' TMA units
+    // the rows were written with plain stores and are gathered by other CTAs' TMA units
     fence_async_all();
     tc_fence_before();
     if (!grid_barrier(p.sync, uint32_t(l + 1), gridDim.x, tmem_slot + 3) && threadIdx.x == 0) {
@@ -270,9 +270,7 @@ int launch_layers_coop(const Dims& d, const DevWeights& dw, int layers, void* h,
   void* Zs[2] = {Z0, Z1};
   if (!make_map(&p.map_h, h, uint64_t(rows), H, xform::BM)) return -1;
   for (int i = 0; i < 2; ++i) {
-    if (!make_map(&p.map_zs[i], Zs[i], uint64_t(rows), H, xform::BM, zrow) ||
-        !aggtma::make_merged_map(&p.map_zg[i], Zs[i], uint64_t(rows), uint32_t(zrow)))
-      return -1;
+    if (!aggtma::make_merged_map(&p.map_zg[i], Zs[i], uint64_t(rows), uint32_t(zrow))) return -1;
     p.Z[i] = static_cast<bf16*>(Zs[i]);
   }
   for (int l = 0; l < kMaxLayers; ++l) {

@@ -5,8 +5,8 @@
 //
 // One persistent CTA per SM.  W^T (the K-major B operand, bf16) stays resident in shared memory; 128-row tiles of h
 // stream through a ring of TMA-loaded, 128-byte-swizzled stages; one thread issues tcgen05.mma (M = 128, N = NS,
-// K = 16) into one of two accumulator buffers in tensor memory; four epilogue warps read the accumulators back
-// (tcgen05.ld), form the half-scores, round Z to bf16 into a swizzled staging tile and hand it to a TMA store.
+// K = 16) into one of two accumulator buffers in tensor memory; eight epilogue warps read the accumulators back
+// (tcgen05.ld), form the half-scores, round Z to bf16 and write it from registers, whole sectors per lane.
 // The op moves 2 H b bytes per node against 2 H^2 flops: up to hidden 256 it is bound by HBM, not by the tensor
 // pipe, so the design goal is to keep loads and stores streaming.
 //
@@ -16,7 +16,7 @@
 // to fourth reading of h comes from L2.  Widths that are not a multiple of 64 leave the last chunk to the TMA
 // unit's bounds: zeros on the way in, nothing written on the way out.
 // Measured: hidden 192, 124 k rows, 0.286 ms per layer with the CUDA-core product plus 0.052 ms for the half-scores
-// -> 0.026 ms (95 MB: 3.6 TB/s); hidden 256, 4.1 M rows, 0.80 ms (4.5 GB: 5.6 TB/s).
+// -> 0.022 ms (95 MB: 4.3 TB/s); hidden 256, 4.1 M rows, 0.73 ms (4.5 GB: 6.2 TB/s), 2.8 M rows 0.58 -> 0.49 ms.
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records XRL_ERR_TIMEOUT, drains its
 // own copies in flight, frees its tensor memory and returns.
@@ -29,12 +29,12 @@ using namespace xform;
 
 namespace {
 
-constexpr int kThreads = 192;           // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+constexpr int kThreads = 320;           // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
 
-template <int NS, int KP, bool ROUNDED>
+template <int NS, int KP, bool ROUNDED, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
-             const __grid_constant__ CUtensorMap map_z, const float* __restrict__ a_src,
+             char* __restrict__ Z, int z_row, const float* __restrict__ a_src,
              const float* __restrict__ a_dst, float2* __restrict__ scores, int score_stride,
              int rows, int H, int d, int slices, int32_t* status) {
   using C = Cfg<NS, KP>;
@@ -55,7 +55,7 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
 
   if (threadIdx.x == 0) {
     tmem_slot[1] = 0;
-    init_barriers<C>(base);
+    init_barriers<C>(base, 4 * epilogue_groups(NS, d));
   }
   // attention vectors pre-multiplied by log2(e): the half-scores are consumed by an exp2 softmax
   for (int t = threadIdx.x; t < NS; t += kThreads) {
@@ -94,8 +94,8 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
     // ---- epilogue: 4 warps ------------------------------------------------------------------------
     uint32_t lt = 0;
     enter();
-    epilogue_tiles<C, NS, ROUNDED>(smem, base, tmem_base, &map_z, scores ? scores + col0 / d : nullptr, score_stride, rows,
-                                   d, first, step, num_tiles, lt, threadIdx.x == 64, status, col0, cols);
+    epilogue_tiles<C, NS, ROUNDED, HD>(smem, base, tmem_base, Z + col0 * 2, z_row, scores ? scores + col0 / d : nullptr,
+                                       score_stride, rows, d, epilogue_groups(NS, d), first, step, num_tiles, lt, status, cols);
   }
 
   tc_fence_before();
@@ -109,13 +109,13 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
 
 // Widths 128 and 256 take the half-scores from the fp32 accumulators, the others from Z as it is stored (both are
 // fixed per model, so that the forward and the reverse pass of a model see the same scores).
-template <int NS, int KP>
+template <int NS, int KP, int HD = 0>
 int launch_h(const Dims& d, const void* h, const LayerWeights& lw, void* Z, float* scores,
              Window win, int32_t* status, cudaStream_t st) {
   using C = Cfg<NS, KP>;
   constexpr bool kRounded = !(NS == KP && (NS == 128 || NS == 256));
   static bool attr_set[64] = {};
-  if (!ensure_dynamic_smem(k_xform_umma<NS, KP, kRounded>, C::SMEM_BYTES, attr_set)) return -1;
+  if (!ensure_dynamic_smem(k_xform_umma<NS, KP, kRounded, HD>, C::SMEM_BYTES, attr_set)) return -1;
   const int64_t rows = int64_t(win.row_end) - win.row_begin;
   const size_t off = size_t(win.row_begin - win.win_base), H = size_t(d.H);
   const bf16* hp = static_cast<const bf16*>(h) + off * H;
@@ -127,14 +127,12 @@ int launch_h(const Dims& d, const void* h, const LayerWeights& lw, void* Z, floa
   const int head = d.H / d.K, slices = (d.H + NS - 1) / NS;
   // a head that crosses a slice's end has its half-scores taken from Z afterwards
   const bool whole_heads = slices == 1 || NS % head == 0;
-  CUtensorMap mh, mw, mz;
-  if (!make_map(&mh, hp, uint64_t(rows), H, BM) || !make_map(&mw, lw.Wt, H, H, NS) ||
-      !make_map(&mz, zp, uint64_t(rows), H, BM, zrow))
-    return -1;
+  CUtensorMap mh, mw;
+  if (!make_map(&mh, hp, uint64_t(rows), H, BM) || !make_map(&mw, lw.Wt, H, H, NS)) return -1;
   const int tiles = int((rows + BM - 1) / BM);
   const int groups = kNumSMs / slices, grid = (tiles < groups ? tiles : groups) * slices;
-  launch(k_xform_umma<NS, KP, kRounded>, grid, kThreads, C::SMEM_BYTES, st,
-      mh, mw, mz, lw.a_src, lw.a_dst, whole_heads ? sc : nullptr, sc_stride, int(rows), d.H, head, slices, status);
+  launch(k_xform_umma<NS, KP, kRounded, HD>, grid, kThreads, C::SMEM_BYTES, st,
+      mh, mw, zp, int(zrow), lw.a_src, lw.a_dst, whole_heads ? sc : nullptr, sc_stride, int(rows), d.H, head, slices, status);
   return whole_heads ? 1 : 1 + launch_scores(d, Z, lw, scores, win, st);
 }
 
@@ -150,6 +148,11 @@ int launch_xform_umma(const Dims& d, const void* h, const LayerWeights& lw, void
   if (int64_t(win.row_end) - win.row_begin <= 0) return 0;
 #define XFORM_CASE(H_, NS_, KP_) \
   case H_: return launch_h<NS_, KP_>(d, h, lw, Z, scores, win, status, st);
+  // heads of 16, 32 or 64 columns in the usual widths (their half-scores leave in 32-byte pieces)
+#define XFORM_HEADS(H_, HD_) \
+  if (d.H == H_ && d.H / d.K == HD_) return launch_h<H_, H_, HD_>(d, h, lw, Z, scores, win, status, st);
+  XFORM_HEADS(128, 16) XFORM_HEADS(128, 32) XFORM_HEADS(128, 64) XFORM_HEADS(256, 16) XFORM_HEADS(256, 32) XFORM_HEADS(256, 64)
+#undef XFORM_HEADS
   switch (d.H) {
     XFORM_CASE(32, 32, 64) XFORM_CASE(64, 64, 64) XFORM_CASE(96, 96, 128) XFORM_CASE(128, 128, 128)
     XFORM_CASE(160, 160, 192) XFORM_CASE(192, 192, 192) XFORM_CASE(224, 224, 256) XFORM_CASE(256, 256, 256)

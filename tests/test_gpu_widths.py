@@ -155,3 +155,32 @@ def test_fp32_transform_of_many_rows_keeps_fp32_accuracy(xo, H, K):
         assert ag.device_status() == 0
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K", [(128, 1), (128, 2), (128, 4), (128, 8), (256, 1), (256, 2), (256, 4), (256, 8), (256, 16)])
+@pytest.mark.parametrize("nodes", [1, 127, 129])
+@pytest.mark.parametrize("fused", [True, False])
+def test_bf16_heads_of_every_width(xo, monkeypatch, H, K, nodes, fused):
+    """The transform's epilogue at 128 and 256 columns: heads of 32 and 64 columns leave in pieces, the others one by one, a
+    head of the whole width keeps the columns with one group of warps."""
+    import paper_2304_14698_b200 as xrl
+    if not fused:
+        monkeypatch.setenv("XRL_NO_FUSED_LAYERS", "1")
+    rng = dags.make_rng(H + nodes + K)
+    m = dict(T=21, S=8, H=H, K=K, L=2, Hm=24, Dg=1, dtype="bf16", A_max=2)
+    batch = dags.flatten([dags.random_dag(rng, n, m["T"], 8, True) for n in (nodes, 1)], [0, 2], 2)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 3)
+    st, packed = xo.pack(batch)
+    assert st == 0
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        for layer in range(m["L"] + 1):
+            got = xrl.xrl_debug_node_features(ag.ctx, ag.batch, layer, H)
+            want = xo.encode(m, blob, batch, packed, dump_layer=layer, want_nodes=True)
+            gpu_util.assert_close(got, want["nodes"], "bf16", f"nodes after stage {layer}")
+        assert ag.device_status() == 0
+    finally:
+        ag.close()
