@@ -1,5 +1,6 @@
 // The two dense products of an attention layer's reverse pass (paper Section 3.3.4's gradient through Eq. 7) on the
-// 5th-generation tensor cores, for bf16 models: with dz the gradient of Z = h W in bf16,
+// 5th-generation tensor cores, for bf16 models: with dz the gradient of Z = h W in bf16 (hidden 128 and 256: both in one
+// kernel, k_dhw_umma; hidden 512, whose dW no tensor memory holds beside dh, one after the other),
 //   dh = dz W^T   the transform kernel's roles and tiles (xrl_xform_umma.cuh) with W itself as the K-major operand
 //                 and an fp32 result, which leaves masked by the ReLU of h (what the next layer down needs);
 //   dW += h^T dz  reduces over the rows, so both operands are used as they lie in memory: a 64-row block of h and one
@@ -7,7 +8,8 @@
 //                 the whole H x H result (H = 256: all 512 columns of tensor memory) stays in tensor memory
 //                 while the CTA walks its range of rows.  The CTAs' results meet in the gradient by TMA
 //                 reductions (fp32 add in L2).
-// Both are bound by HBM: 8 H bytes per row (dh: 4 H in, 4 H out) and 4 H bytes per row (dW).
+// Both are bound by HBM: 8 H bytes per row (dh: 4 H in, 4 H out) and 4 H bytes per row (dW); together, with dz and h read
+// once, 8 H.
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records XRL_ERR_TIMEOUT, drains its own copies in
 // flight, frees its tensor memory and returns.
@@ -150,7 +152,7 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
 }
 
 // ---- dW += h^T dz ----------------------------------------------------------------------------------------------
-// S: side of the square of dW a CTA accumulates (128: H = 128; 256: H = 256, and a quarter of H = 512).
+// S: side of the square of dW a CTA accumulates (256: a quarter of H = 512).
 constexpr int RB = 64;                   // rows per stage
 template <int S> struct WCfg {
   static constexpr int CHUNK = RB * 128;                 // 64 rows x 64 columns
@@ -303,6 +305,229 @@ k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
   }
 }
 
+// ---- both products in one pass: dh = dz W^T and dW += h^T dz for H = 128 and 256 -----------------------------------
+// A CTA takes 128 columns of h (H / 128 CTAs side by side per tile of rows): their 128 x H part of dW stays in tensor memory
+// for the whole range of tiles, and the same 128 columns of dh are computed tile by tile into two more accumulators.  A
+// 128-row tile of dz (64-column chunks through a ring) is then read once from memory for both products - as the K-major
+// operand of dh and, the same bytes, as the MN-major operand of dW - and so is the tile of h, which is dW's other operand
+// and the ReLU mask of dh.  W's 128 rows are resident.  One kernel per product read both twice: 990 k rows of 256,
+// 0.163 + 0.365 -> 0.341 ms per layer; 183 k rows 41 + 65 -> 66 us.
+template <int H> struct PCfg {
+  static constexpr int KC = H / KCH, HALVES = H / 128;
+  static constexpr int W_CHUNK = 128 * 128, W_BYTES = KC * W_CHUNK;
+  static constexpr int RING = 4, H_STAGES = 2, H_STAGE = 2 * STAGE_BYTES;
+  static constexpr int OFF_DZ = W_BYTES;
+  static constexpr int OFF_H = OFF_DZ + RING * STAGE_BYTES;
+  static constexpr int OFF_OUT = OFF_H + H_STAGES * H_STAGE;
+  static constexpr int OFF_BAR = OFF_OUT + 2 * STAGE_BYTES;
+  static constexpr int NUM_BARS = 2 + 2 * RING + 2 * H_STAGES + 4;
+  static constexpr int OFF_TMEM = OFF_BAR + 8 * NUM_BARS;
+  static constexpr int SMEM_BYTES = OFF_TMEM + 16;
+  static constexpr int TMEM_COLS = 512;                  // dW: H columns, then two accumulators of 128
+  static_assert(SMEM_BYTES <= 227 * 1024 && H + 256 <= 512, "shared and tensor memory of one SM");
+};
+
+template <int H>
+__global__ void __launch_bounds__(kThreads, 1)
+k_dhw_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_h,
+           const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_dh,
+           const __grid_constant__ CUtensorMap map_dw, float* __restrict__ dW, int rows, bool use_tma, int32_t* status) {
+  using C = PCfg<H>;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const uint32_t base = smem_u32(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((base & 1023u) != 0) {
+    if (threadIdx.x == 0) raise(status, XRL_ERR_UNSUPPORTED);
+    return;
+  }
+  const int num_tiles = (rows + BM - 1) / BM;
+  const int a0 = int(blockIdx.x) % C::HALVES * 128, first = int(blockIdx.x) / C::HALVES, step = int(gridDim.x) / C::HALVES;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM);
+  const uint32_t bars = base + C::OFF_BAR, bar_w = bars, bar_done = bars + 8;
+  auto dz_full = [&](uint32_t s) { return bars + 8u * (2 + s); };
+  auto dz_empty = [&](uint32_t s) { return bars + 8u * (2 + C::RING + s); };
+  auto h_full = [&](uint32_t s) { return bars + 8u * (2 + 2 * C::RING + s); };
+  auto h_empty = [&](uint32_t s) { return bars + 8u * (2 + 2 * C::RING + C::H_STAGES + s); };
+  auto acc_full = [&](uint32_t b) { return bars + 8u * (2 + 2 * C::RING + 2 * C::H_STAGES + b); };
+  auto acc_empty = [&](uint32_t b) { return bars + 8u * (2 + 2 * C::RING + 2 * C::H_STAGES + 2 + b); };
+  if (threadIdx.x == 0) {
+    tmem_slot[1] = 0;
+    mbar_init(bar_w, 1);
+    mbar_init(bar_done, 1);
+    for (uint32_t s = 0; s < C::RING; ++s) { mbar_init(dz_full(s), 1); mbar_init(dz_empty(s), 1); }
+    // a tile of h is free once the products have read it and each epilogue warp has taken its mask
+    for (uint32_t s = 0; s < C::H_STAGES; ++s) { mbar_init(h_full(s), 1); mbar_init(h_empty(s), 5); }
+    for (uint32_t b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), 128); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      mbar_expect_tx(bar_w, C::W_BYTES);
+      for (int kc = 0; kc < C::KC; ++kc) tma_load_2d(base + kc * C::W_CHUNK, &map_w, kc * KCH, a0, bar_w);
+      enter();
+      bool ok = true;
+      uint32_t it = 0, lt = 0;
+      for (int tile = first; tile < num_tiles && ok; tile += step, ++lt) {
+        const uint32_t hs = lt % C::H_STAGES, hr = lt / C::H_STAGES;
+        if (hr > 0 && !mbar_wait(h_empty(hs), (hr - 1) & 1)) { ok = false; break; }
+        mbar_expect_tx(h_full(hs), C::H_STAGE);
+        for (int c = 0; c < 2; ++c)
+          tma_load_2d(base + C::OFF_H + hs * C::H_STAGE + c * STAGE_BYTES, &map_h, a0 + c * KCH, tile * BM, h_full(hs));
+        for (int kc = 0; kc < C::KC; ++kc, ++it) {
+          const uint32_t s = it % C::RING, round = it / C::RING;
+          if (round > 0 && !mbar_wait(dz_empty(s), (round - 1) & 1)) { ok = false; break; }
+          mbar_expect_tx(dz_full(s), STAGE_BYTES);
+          tma_load_2d(base + C::OFF_DZ + s * STAGE_BYTES, &map_g, kc * KCH, tile * BM, dz_full(s));
+        }
+      }
+      if (!ok) {                             // let the loads already issued land before the shared memory goes away
+        raise(status, XRL_ERR_TIMEOUT);
+        for (uint32_t j = it > C::RING ? it - C::RING : 0; j < it; ++j) mbar_wait(dz_full(j % C::RING), (j / C::RING) & 1);
+        for (uint32_t j = lt > C::H_STAGES ? lt - C::H_STAGES : 0; j < lt; ++j)
+          mbar_wait(h_full(j % C::H_STAGES), (j / C::H_STAGES) & 1);
+        mbar_wait(bar_w, 0);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // fp32 accumulators, bf16 x bf16: dh K-major both, M = N = 128; dW MN-major both (bits 15, 16), M = 128, N = 64
+      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(128 >> 4) << 24);
+      constexpr uint32_t idesc_dh = idesc | (uint32_t(128 >> 3) << 17);
+      constexpr uint32_t idesc_dw = idesc | (1u << 15) | (1u << 16) | (uint32_t(64 >> 3) << 17);
+      bool ok = mbar_wait(bar_w, 0);
+      uint32_t it = 0, lt = 0;
+      for (int tile = first; tile < num_tiles && ok; tile += step, ++lt) {
+        const uint32_t hs = lt % C::H_STAGES, buf = lt & 1, use = lt >> 1;
+        if (use > 0 && !mbar_wait(acc_empty(buf), (use - 1) & 1)) { ok = false; break; }
+        if (!mbar_wait(h_full(hs), (lt / C::H_STAGES) & 1)) { ok = false; break; }
+        const uint32_t acc = tmem_base + uint32_t(H) + buf * 128u, h_at = base + C::OFF_H + hs * C::H_STAGE;
+        for (int kc = 0; kc < C::KC; ++kc, ++it) {
+          const uint32_t s = it % C::RING, at = base + C::OFF_DZ + s * STAGE_BYTES;
+          if (!mbar_wait(dz_full(s), (it / C::RING) & 1)) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll
+          for (int k = 0; k < KCH / 16; ++k)
+            tc_mma(acc, smem_desc(at + k * 32), smem_desc(base + kc * C::W_CHUNK + k * 32), idesc_dh, (kc | k) != 0 ? 1u : 0u);
+#pragma unroll
+          for (int ks = 0; ks < BM / 16; ++ks)         // 16 rows = two 8-row groups per instruction
+            tc_mma(tmem_base + uint32_t(kc * KCH), smem_desc_mn(h_at + ks * 2048, STAGE_BYTES),
+                   smem_desc_mn(at + ks * 2048, STAGE_BYTES), idesc_dw, (lt | uint32_t(ks)) != 0 ? 1u : 0u);
+          tc_commit(dz_empty(s));
+        }
+        if (!ok) break;
+        tc_commit(h_empty(hs));
+        tc_commit(acc_full(buf));
+      }
+      if (ok) tc_commit(bar_done);
+      else raise(status, XRL_ERR_TIMEOUT);
+    }
+  } else {
+    const int q = warp & 3, row = q * 32 + lane;
+    const bool leader = threadIdx.x == 64;
+    volatile uint32_t* abort_flag = tmem_slot + 1;
+    uint32_t lt = 0, stores = 0;
+    enter();
+    // a 32-column piece of a thread's row, out through the staging tile whose store of two pieces ago has read it
+    auto stage_out = [&](const uint32_t (&v)[32], auto store) {
+      if (leader) tma_wait_read<1>();
+      epi_barrier();
+      stage_row(smem + C::OFF_OUT + (stores & 1) * STAGE_BYTES, row, v);
+      fence_async_smem();
+      epi_barrier();
+      if (leader) {
+        store(base + C::OFF_OUT + (stores & 1) * STAGE_BYTES);
+        tma_commit();
+      }
+      ++stores;
+    };
+    // the outcome of a wait, agreed on by the four warps
+    auto agreed = [&](bool ok) {
+      if (!ok && lane == 0) { *abort_flag = 1; raise(status, XRL_ERR_TIMEOUT); }
+      epi_barrier();
+      return *abort_flag == 0;
+    };
+    bool run = true;
+    for (int tile = first; tile < num_tiles; tile += step, ++lt) {
+      const uint32_t hs = lt % C::H_STAGES, buf = lt & 1;
+      // this thread's 128 features of h (every lane waits: each has to see the copy's bytes itself)
+      run = agreed(mbar_wait(h_full(hs), (lt / C::H_STAGES) & 1));
+      if (!run) break;
+      uint4 f[2][8];
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          f[c][j] = *reinterpret_cast<const uint4*>(smem + C::OFF_H + hs * C::H_STAGE + c * STAGE_BYTES + row * 128 + ((j ^ (row & 7)) << 4));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(h_empty(hs));
+      bool ok = true;
+      if (lane == 0) ok = mbar_wait(acc_full(buf), (lt >> 1) & 1);
+      run = agreed(__shfl_sync(0xFFFFFFFFu, int(ok), 0) != 0);
+      if (!run) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(H) + buf * 128u;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t v[32];
+        tc_ld32(taddr + c * 32, v);
+        tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float x[8];
+          unpack(f[c >> 1][(c & 1) * 4 + j], x);
+#pragma unroll
+          for (int t = 0; t < 8; ++t) v[8 * j + t] = x[t] > 0.f ? v[8 * j + t] : 0u;
+        }
+        if (c == 3) {
+          tc_fence_before();
+          mbar_arrive(acc_empty(buf));
+        }
+        stage_out(v, [&](uint32_t src) { tma_store_2d(&map_dh, src, a0 + c * 32, tile * BM); });
+      }
+    }
+    if (run) {
+      bool ok = true;
+      if (lane == 0) ok = mbar_wait(bar_done, 0);
+      run = agreed(__shfl_sync(0xFFFFFFFFu, int(ok), 0) != 0);
+    }
+    if (run) {
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + (uint32_t(q * 32) << 16);
+      for (int c = 0; c < H / 32; ++c) {
+        uint32_t v[32];
+        tc_ld32(taddr + c * 32, v);
+        tc_wait_ld();
+        if (use_tma) {
+          stage_out(v, [&](uint32_t src) { tma_reduce_add_2d(&map_dw, src, c * 32, a0); });
+        } else {
+          float* o = dW + size_t(a0 + row) * H + c * 32;
+#pragma unroll
+          for (int t = 0; t < 32; ++t) atomicAdd(o + t, __uint_as_float(v[t]));
+        }
+      }
+    }
+    if (leader) tma_wait_all();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                 ::"r"(tmem_base), "r"(uint32_t(C::TMEM_COLS)) : "memory");
+  }
+}
+
 // 2-D fp32 tensor [rows x cols] row-major, box [128 rows x 32 columns], 128-byte swizzle
 bool make_map_f32(CUtensorMap* m, void* ptr, uint64_t rows, uint64_t cols) {
   EncodeTiledFn fn = encode_fn();
@@ -348,6 +573,25 @@ int launch_dw(int H, const void* h, const void* dzb, float* dW, int32_t rows, in
   return 1;
 }
 
+template <int H>
+int launch_dhw(const void* h, const void* dzb, const void* W, float* dh, float* dW, int32_t rows, int32_t* status, cudaStream_t st) {
+  using C = PCfg<H>;
+  static bool attr_set[64] = {};
+  if (!ensure_dynamic_smem(k_dhw_umma<H>, C::SMEM_BYTES, attr_set)) return -1;
+  const bool aligned = (reinterpret_cast<uintptr_t>(dW) & 15) == 0;    // the caller's buffer may sit on any 4-byte boundary
+  CUtensorMap mg, mh, mw, mo, md;
+  if (!make_map(&mg, dzb, uint64_t(rows), H, BM) || !make_map(&mh, h, uint64_t(rows), H, BM) ||
+      !make_map(&mw, W, H, H, 128) || !make_map_f32(&mo, dh, uint64_t(rows), H))
+    return -1;
+  if (aligned) { if (!make_map_f32(&md, dW, H, H)) return -1; }
+  else md = mo;
+  // at least two tiles per CTA: every CTA ends with a reduction of its part of dW into the gradient
+  const int tiles = (rows + BM - 1) / BM, want = (tiles + 1) / 2, most = kNumSMs / C::HALVES;
+  launch(k_dhw_umma<H>, (want < most ? want : most) * C::HALVES, kThreads, C::SMEM_BYTES, st,
+         mg, mh, mw, mo, md, dW, rows, aligned, status);
+  return 1;
+}
+
 }  // namespace
 
 // bf16 models of hidden 128, 256 or 512 (the widths whose dz is kept in bf16 for these products)
@@ -361,13 +605,9 @@ int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W
   int a, b;
   switch (d.H) {
     case 128:
-      a = launch_dw<128>(128, h, dzb, dW, rows, status, st);
-      b = launch_dh<128, 128>(128, h, dzb, W, dh, rows, status, st);
-      break;
+      return launch_dhw<128>(h, dzb, W, dh, dW, rows, status, st);
     case 256:
-      a = launch_dw<256>(256, h, dzb, dW, rows, status, st);
-      b = launch_dh<256, 256>(256, h, dzb, W, dh, rows, status, st);
-      break;
+      return launch_dhw<256>(h, dzb, W, dh, dW, rows, status, st);
     case 512:
       a = launch_dw<256>(512, h, dzb, dW, rows, status, st);
       b = launch_dh<128, 512>(512, h, dzb, W, dh, rows, status, st);

@@ -144,3 +144,13 @@ def test_gradient_where_the_lists_by_producer_do_not_fit():
     del filler
     torch.cuda.empty_cache()
     assert (grads[1] - grads[0]).norm() <= 1e-5 * grads[0].norm() and grads[0].norm() > 0
+
+
+@pytest.mark.parametrize("H,K,nodes", [(256, 8, 30), (256, 8, 31), (256, 4, 63), (128, 8, 31), (128, 2, 127), (256, 8, 9600)])
+def test_gradient_of_both_products_at_the_edges_of_their_tiles(xo, H, K, nodes):
+    """125, 129, 257, 513 rows (one to five tiles of 128, one or two CTAs per half) and 38,405 (several tiles per CTA, an odd
+    number of rows)."""
+    m = dict(T=9, S=8, H=H, K=K, L=1 if nodes > 1000 else 2, Hm=20, Dg=1, dtype="bf16", A_max=3)
+    rng = dags.make_rng(H + nodes)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, True, window=6) for n in (nodes, nodes + 3, nodes, 1, nodes + 1)]
+    _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
