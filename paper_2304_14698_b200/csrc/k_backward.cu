@@ -1049,13 +1049,15 @@ size_t ppo_heads_workspace_floats(const Dims& d, int64_t B, int64_t num_envs) {
 }
 
 // Forward from the readout's chunk sums to the logits, Eq. 3-5, and the reverse pass down to the gradient of the last
-// layer's node features (dh [N x H]).  ws: ppo_heads_workspace_floats floats.
+// layer's node features (dh [N x H]), or, without dh, to that of the graphs' sums (*dr_out [B x H], in ws).  ws:
+// ppo_heads_workspace_floats floats.
 int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const float* w_base, const void* hL,
                      const float* partial, const int32_t* graph_chunk_off, const int32_t* seg_id, const float* g0,
                      const int32_t* env_off,
                      const uint8_t* mask, const int32_t* action, const float* logp_old, const float* adv,
                      const float* ret, float eps, float c1, float c2, int32_t B, int32_t num_envs, int64_t N,
-                     float* ws, float* loss, float* dh, float* logp_out, int32_t* status, cudaStream_t st) {
+                     float* ws, float* loss, float* dh, const float** dr_out, float* logp_out, int32_t* status,
+                     cudaStream_t st) {
   if (B <= 0 || num_envs <= 0) return 0;
   const size_t H = d.H, Hm = d.Hm, Hm2 = d.Hm2, HU = H + d.Dg;
   float* p = ws;
@@ -1108,7 +1110,8 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
              gp(w.vbh), gp(w.vw2), gp(w.vb2));
   launch(k_head_grads, tl.ctas, 256, 0, st, tl.tasks);
   ++n;
-  const int64_t ne = N * (d.H / 4);
+  *dr_out = dr;
+  const int64_t ne = dh != nullptr ? N * (d.H / 4) : 0;
   if (ne > 0) {
     const unsigned grid = unsigned(std::min<int64_t>((ne + 255) / 256, int64_t(kNumSMs) * 64));
     if (d.dtype == XRL_BF16) launch(k_readout_bwd<bf16>, grid, 256, 0, st, dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
@@ -1125,10 +1128,11 @@ static bool bwd_rows_kernels(const Dims& d) {
 bool bwd_leaves_masked(const Dims& d) { return bwd_rows_kernels(d) && bwd_umma_supported(d); }
 
 // One attention layer backwards: dh_out -> (dW, da_src, da_dst, db) and dh_in.  Z / scores hold the layer's
-// forward transform of h_in; dz [N x H] and ds [2 N K] are scratch.
+// forward transform of h_in; dz [N x H] and ds [2 N K] are scratch.  With dr (rows_gather_supported models with lists only)
+// the gradient of a row's output is its graph's row of dr, and dh_out is scratch.
 int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores,
-                         const void* h_in, const void* h_out, float* dh_out, bool masked, float* dh_in, float* dz,
-                         float* ds, void* dz_store, const BwdLists* lists, const LayerWeights& lw, float* gW, float* ga_src,
+                         const void* h_in, const void* h_out, float* dh_out, bool masked, const float* dr,
+                         const int32_t* seg_id, float* dh_in, float* dz, float* ds, void* dz_store, const BwdLists* lists, const LayerWeights& lw, float* gW, float* ga_src,
                          float* ga_dst, float* gb, int32_t N, int32_t* status, cudaStream_t st) {
   if (N <= 0) return 0;
   const int H = d.H, K = d.K;
@@ -1166,7 +1170,10 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   } while (0)
 #define BWD_GATHER(TY_, NF_)                                                                                   \
   do {                                                                                                         \
-    if (launch_rows_gather(d, *lists, rowptr, col, Z, scores, h_out, dh_out, masked, ds_dst, gb, N, status, st) < 0) \
+    const int k_ = launch_rows_gather(d, *lists, rowptr, col, Z, scores, h_out, dh_out, masked, dr, seg_id, ds_dst, gb, N, \
+                                      status, st);                                                             \
+    if (k_ < 0 && dr != nullptr) return -1;                                                                    \
+    if (k_ < 0)                                                                                                \
       launch(k_aggregate_bwd_rows<TY_, NF_, true>, grid_rows, 256, 0, st,                                          \
           rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, nullptr, nullptr, ds_dst, gb, N, K, *lists); \
     if (launch_dz_gather(d, *lists, dh_out, Z, zrow, ds_dst, lw, mma ? dz_store : static_cast<void*>(dz), ga_src, ga_dst, \

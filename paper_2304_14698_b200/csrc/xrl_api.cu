@@ -1220,9 +1220,13 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   // xrl_encode, which may run on another stream meanwhile
   float* readout = dz;
   n += launch_readout(d, hs[L], b->d_chunk_row0, b->d_chunk_row1, 0, b->num_chunks, readout, 0, st);
+  // the last layer's softmax reverse takes its rows' gradients from the graphs' where it can, else they are written out first
+  const bool from_graphs = gather && L > 0 && rows_gather_supported(d);
+  const float* dr = nullptr;
   const int kh = launch_ppo_heads(d, ctx->dw, grad, wb, hs[L], readout, b->d_graph_chunk_off,
                                   b->seg_id.as<int32_t>(), g0, b->d_env_off, mask, action, logp_old, adv, ret, eps, c1, c2, b->B,
-                                  b->num_envs, b->N, heads_ws, loss_out, dh_a, logp_out, ctx->status.as<int32_t>(), st);
+                                  b->num_envs, b->N, heads_ws, loss_out, from_graphs ? nullptr : dh_a, &dr, logp_out,
+                                  ctx->status.as<int32_t>(), st);
   if (kh < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
   n += kh;
   const int32_t* gat_rowptr = c.neighbourhood ? b->rowptr_nbr.as<int32_t>() : b->rowptr.as<int32_t>();
@@ -1235,8 +1239,8 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
     const LayerWeights& lw = ctx->dw.layer[l];
     float* ga_src = grad + (lw.a_src - wb);
     const int k = launch_gat_layer_bwd(d, gat_rowptr, gat_col, zs[l], ss[l], hs[l], hs[l + 1], dh_cur,
-                             l == L - 1 || bwd_leaves_masked(d),   // (the readout's reverse masks too)
-                             dh_nxt, dz, ds, dz_store, gather ? &lists : nullptr, lw, ga_src - H * H, ga_src, grad + (lw.a_dst - wb),
+                             l == L - 1 ? !from_graphs : bwd_leaves_masked(d),   // (the readout's reverse masks too)
+                             l == L - 1 && from_graphs ? dr : nullptr, b->seg_id.as<int32_t>(), dh_nxt, dz, ds, dz_store, gather ? &lists : nullptr, lw, ga_src - H * H, ga_src, grad + (lw.a_dst - wb),
                              grad + (lw.b - wb), b->N, ctx->status.as<int32_t>(), st);
     if (k < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
     n += k;

@@ -258,7 +258,8 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
                      const int32_t* env_off,
                      const uint8_t* mask, const int32_t* action, const float* logp_old, const float* adv,
                      const float* ret, float eps, float c1, float c2, int32_t B, int32_t num_envs, int64_t N,
-                     float* ws, float* loss, float* dh, float* logp_out, int32_t* status, cudaStream_t st);
+                     float* ws, float* loss, float* dh, const float** dr_out, float* logp_out, int32_t* status,
+                     cudaStream_t st);
 // Transposed neighbour lists of the reverse pass: rowptr [N + 1], col [E] (the rows that read a producer), inv [E] (the
 // entry of a CSR slot), entry [(N + E + 4) x K] = {alpha, score gradient} per entry, a producer's own entry first.
 struct BwdLists { int32_t *rowptr, *col, *inv; float2* entry; };
@@ -266,8 +267,9 @@ bool bwd_gather_supported(const Dims& d);
 int launch_bwd_lists(const int32_t* rowptr, const int32_t* col, int32_t N, int32_t E, const BwdLists& t, int32_t* scratch,
                      cudaStream_t st);
 int launch_rows_gather(const Dims& d, const BwdLists& t, const int32_t* rowptr, const int32_t* col, const void* Z,
-                       const float* scores, const void* h_out, float* dh, bool masked, float* ds_dst, float* gb, int32_t N,
-                       int32_t* status, cudaStream_t st);
+                       const float* scores, const void* h_out, float* dh, bool masked, const float* dr, const int32_t* seg_id,
+                       float* ds_dst, float* gb, int32_t N, int32_t* status, cudaStream_t st);
+bool rows_gather_supported(const Dims& d);
 int launch_dz_gather(const Dims& d, const BwdLists& t, const float* dpre, const void* Z, size_t z_row, const float* ds_dst,
                      const LayerWeights& lw, void* dz, float* ga_src, float* ga_dst, int32_t N, int32_t* status,
                      cudaStream_t st);
@@ -277,8 +279,8 @@ bool bwd_leaves_masked(const Dims& d);
 int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W, float* dh, float* dW, int32_t rows,
                     int32_t* status, cudaStream_t st);
 int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores,
-                         const void* h_in, const void* h_out, float* dh_out, bool masked, float* dh_in, float* dz,
-                         float* ds, void* dz_store, const BwdLists* lists, const LayerWeights& lw, float* gW, float* ga_src,
+                         const void* h_in, const void* h_out, float* dh_out, bool masked, const float* dr,
+                         const int32_t* seg_id, float* dh_in, float* dz, float* ds, void* dz_store, const BwdLists* lists, const LayerWeights& lw, float* gW, float* ga_src,
                          float* ga_dst, float* gb, int32_t N, int32_t* status, cudaStream_t st);
 int launch_gae(const float* reward, const float* values, const uint8_t* done, float gamma, float lambda, int32_t T,
                int32_t M, float* adv, float* ret, cudaStream_t st);
