@@ -135,8 +135,8 @@ int launch_k(const int32_t* rowptr, const int32_t* col, const void* Z, const flo
 }  // namespace
 
 // buf_rows: rows of the Z / scores buffers reachable from this window (indices are window-relative).
-// partial != nullptr selects the variant fused with the per-graph sum (then h_out is not written and
-// the window must start at row 0).  Returns kernels launched, or -1 when this shape is not handled here.
+// partial != nullptr selects the variant fused with the per-graph sum (then h_out may be nullptr: rows not stored; the
+// window must start at row 0).  Returns kernels launched, or -1 when this shape is not handled here.
 int launch_aggregate_tma(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z,
                          const float* scores, const float* bias, void* h_out, Window win, int64_t buf_rows,
                          const int32_t* seg_id, float* partial, int32_t* status, cudaStream_t st,

@@ -1048,11 +1048,13 @@ size_t ppo_heads_workspace_floats(const Dims& d, int64_t B, int64_t num_envs) {
          up4(e * 2 * H) + 2 * up4(e * Hm) + 2 * up4(e * Hm2) + up4(e);
 }
 
-// Forward from the readout's chunk sums to the logits, Eq. 3-5, and the reverse pass down to the gradient of the last
+// Forward from the readout's sums (of chunks: partial_off = the graphs' first chunks, nblocks = 0; or of the last layer's
+// blocks of rows: partial_off = the graphs' first rows) to the logits, Eq. 3-5, and the reverse pass down to the gradient of the last
 // layer's node features (dh [N x H]), or, without dh, to that of the graphs' sums (*dr_out [B x H], in ws).  ws:
 // ppo_heads_workspace_floats floats.
 int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const float* w_base, const void* hL,
-                     const float* partial, const int32_t* graph_chunk_off, const int32_t* seg_id, const float* g0,
+                     const float* partial, const int32_t* partial_off, int32_t nblocks, int block_shift,
+                     const int32_t* seg_id, const float* g0,
                      const int32_t* env_off,
                      const uint8_t* mask, const int32_t* action, const float* logp_old, const float* adv,
                      const float* ret, float eps, float c1, float c2, int32_t B, int32_t num_envs, int64_t N,
@@ -1085,7 +1087,8 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
   const Mlp pm{w.pW1, w.pb1, w.pWh, w.pbh, w.pw2, w.pb2, d.Hm, d.Hm2};
   int n = 0;
   cudaMemsetAsync(ws, 0, sizeof(float) * size_t(cleared_end - ws), st);
-  int k = launch_global_update(d, partial, graph_chunk_off, g0, w, emb, B, st, U);
+  int k = nblocks > 0 ? launch_global_update_blocks(d, partial, partial_off, nblocks, block_shift, g0, w, emb, B, st, U)
+                      : launch_global_update(d, partial, partial_off, g0, w, emb, B, st, U);
   if (k < 0) return -1;
   n += k;
   k = launch_policy_value_hidden(d, w, emb, logit, B, py1, py2, nullptr, nullptr, 0, nullptr, st);

@@ -483,8 +483,8 @@ int launch_global_update(const Dims& d, const float* partial, const int32_t* gra
 
 int launch_global_update_blocks(const Dims& d, const float* partial, const int32_t* node_off, int32_t nblocks,
                                 int block_shift, const float* g0, const DevWeights& w, float* emb, int32_t B,
-                                cudaStream_t st) {
-  return launch_update<true>(d, partial, node_off, nblocks, block_shift, g0, w, emb, nullptr, B, st);
+                                cudaStream_t st, float* U_out) {
+  return launch_update<true>(d, partial, node_off, nblocks, block_shift, g0, w, emb, U_out, B, st);
 }
 
 // Policy scores of all graphs (logit [B]; y1_out / y2_out optional) and, for num_envs > 0, the first layer of the value

@@ -94,7 +94,8 @@ __device__ __forceinline__ void to_pairs(const uint4& raw, F2 (&z)[2]) {        
 }
 
 // out = ReLU(acc * inv + bias), stored in the feature type
-__device__ __forceinline__ void finish_row(bf16* dst, const F2 (&acc)[4], float inv, const float (&bs)[8]) {
+// (the row as stored is returned)
+__device__ __forceinline__ uint4 finish_row(bf16* dst, const F2 (&acc)[4], float inv, const float (&bs)[8]) {
   uint32_t w[4];
   const F2 i2 = make_f2(inv, inv);
 #pragma unroll
@@ -105,9 +106,11 @@ __device__ __forceinline__ void finish_row(bf16* dst, const F2 (&acc)[4], float 
     split_f2(o, lo, hi);
     asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(w[t]) : "f"(hi), "f"(lo));   // ReLU inside the rounding
   }
-  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  const uint4 raw = make_uint4(w[0], w[1], w[2], w[3]);
+  *reinterpret_cast<uint4*>(dst) = raw;
+  return raw;
 }
-__device__ __forceinline__ void finish_row(float* dst, const F2 (&acc)[2], float inv, const float (&bs)[4]) {
+__device__ __forceinline__ uint4 finish_row(float* dst, const F2 (&acc)[2], float inv, const float (&bs)[4]) {
   float o[4];
 #pragma unroll
   for (int t = 0; t < 2; ++t) {
@@ -116,7 +119,9 @@ __device__ __forceinline__ void finish_row(float* dst, const F2 (&acc)[2], float
     o[2 * t] = fmaxf(fmaf(lo, inv, bs[2 * t]), 0.f);
     o[2 * t + 1] = fmaxf(fmaf(hi, inv, bs[2 * t + 1]), 0.f);
   }
-  *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+  const uint4 raw = make_uint4(__float_as_uint(o[0]), __float_as_uint(o[1]), __float_as_uint(o[2]), __float_as_uint(o[3]));
+  *reinterpret_cast<uint4*>(dst) = raw;
+  return raw;
 }
 
 // out = ReLU(acc * inv + bias) kept in fp32, as register pairs (for the fused per-graph readout)
@@ -150,8 +155,8 @@ __device__ __forceinline__ void raise_reference(float ev, float& m, float& l, F2
 
 // One warp's share of a layer.  `next_block()` returns the first row of the warp's next block of up to
 // 2^br_shift destination rows, or a negative value when there is none left.  READOUT = true is the last
-// attention layer fused with the per-graph sum of Eq. 8: the layer output is not stored; the warp adds
-// the rows of its block per graph, in row order, and writes
+// attention layer fused with the per-graph sum of Eq. 8: the layer output is stored only where h_out is given (the
+// training step keeps it; the sum is then of the rows as stored, as its reverse pass reads them); the warp adds the rows of its block per graph, in row order, and writes
 //   partial[b]           the rows of block b that belong to the graph of the block's first row
 //   partial[nblocks + g] the rows of graph g inside the block in which g starts, when that is not at
 //                        the block's first row
@@ -291,7 +296,8 @@ __device__ __forceinline__ bool aggregate_warp(
         }
         if (READOUT) {
           F2 o[NP];
-          finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
+          if (h_out != nullptr) to_pairs(finish_row(h_out + size_t(lrow) * H + c0, acc, __fdividef(1.f, l), bs), o);
+          else finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
           add_row(rs, o);
         } else {
           finish_row(h_out + size_t(lrow) * H + c0, acc, __fdividef(1.f, l), bs);
@@ -412,7 +418,9 @@ __device__ __forceinline__ bool aggregate_warp(
         }
         if (READOUT) {
           F2 o[NP];
-          finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
+          if (h_out != nullptr)
+            to_pairs(finish_row(h_out + size_t(int32_t(r0) + rs + rr - win.win_base) * H + c0, acc, __fdividef(1.f, l), bs), o);
+          else finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
           add_row(rs + rr, o);
         } else {
           finish_row(h_out + size_t(int32_t(r0) + rs + rr - win.win_base) * H + c0, acc, __fdividef(1.f, l), bs);

@@ -524,11 +524,13 @@ xrl_status pack_common(xrl_ctx* ctx, const xrl_graph* graphs, int32_t where, int
 // ctx->partial instead of node features in ctx->h; *fused tells whether it did.
 // With `hs` (layers + 1 buffers of N x H storage-type values) every layer's input is kept: Eq. 6 writes hs[0],
 // layer l reads hs[l] and writes hs[l + 1]; with `zs` / `ss` layer l's Z rows and half-scores go to zs[l] / ss[l]
-// instead of the context's one buffer each.
+// instead of the context's one buffer each.  partial: where the sums go instead of ctx->partial (with hs the last layer's
+// rows are stored too).
 int run_node_layers(xrl_ctx* ctx, const xrl_batch* b, int layers, cudaStream_t st, bool fuse_readout = false,
                     bool* fused = nullptr, int32_t row_begin = 0, int32_t row_end = -1, void* const* hs = nullptr,
-                    void* const* zs = nullptr, float* const* ss = nullptr) {
+                    void* const* zs = nullptr, float* const* ss = nullptr, float* partial = nullptr) {
   const Dims& d = ctx->dims;
+  if (partial == nullptr) partial = ctx->partial.as<float>();
   const Window win{row_begin, row_end < 0 ? b->N : row_end, 0};   // graphs are independent: any range of whole graphs
   Profiler& pf = ctx->prof;
   const void* eattr = b->has_eattr ? b->eattr.p : nullptr;      // attributes on the edges, in slot order
@@ -583,8 +585,8 @@ int run_node_layers(xrl_ctx* ctx, const xrl_batch* b, int layers, cudaStream_t s
     bool fused_here = false;
     if (fuse_readout && l == layers - 1) {
       k = launch_aggregate_tma(d, gat_rowptr, gat_col, Zl,
-                               Sl, ctx->dw.layer[l].b, h_out, win, b->N,
-                               b->seg_id.as<int32_t>(), ctx->partial.as<float>(),
+                               Sl, ctx->dw.layer[l].b, hs ? h_out : nullptr, win, b->N,
+                               b->seg_id.as<int32_t>(), partial,
                                ctx->status.as<int32_t>(), st);
       if (k >= 0) { fused_here = true; if (fused) *fused = true; }
     }
@@ -1212,19 +1214,24 @@ xrl_status xrl_ppo_grad(xrl_ctx* ctx, const xrl_batch* b, const float* g0, const
   XRL_CUDA(cudaMemsetAsync(grad, 0, 4 * ctx->weight_floats, st));
   XRL_CUDA(cudaMemsetAsync(loss_out, 0, 16, st));
   if (b->B == 0 || b->num_envs == 0) return XRL_OK;
-  int n = run_node_layers(ctx, b, L, st, false, nullptr, 0, -1, hs, zs, ss);
+  // Eq. 8's per-graph sums as in xrl_encode: from the last layer's own launch where the model has it and its blocks' sums
+  // fit, else readout chunks, added per graph by the next kernel.  They wait in dz (a chunk has at least one row, and dz is
+  // not written before the heads are done): the context's own partial sums belong to xrl_encode, which may run on another
+  // stream meanwhile.  (A pass of its own over 990 k stored rows of 256 read 0.08 ms, over 183 k 16 us beside its launch: the
+  // mini-batches 7,420 -> 7,338 us and 1,837 -> 1,811.)
+  float* readout = dz;
+  bool fused = false;
+  const int32_t nblocks = aggregate_readout_blocks(b->N);
+  int n = run_node_layers(ctx, b, L, st, int64_t(nblocks) + b->B <= c.max_nodes, &fused, 0, -1, hs, zs, ss, readout);
   if (n < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }
   const float* wb = ctx->w_f32.as<float>();
-  // Eq. 8's per-graph sums as in xrl_encode: readout chunks, added per graph by the next kernel.  They wait in dz (a chunk has
-  // at least one row, and dz is not written before the heads are done): the context's own partial sums belong to
-  // xrl_encode, which may run on another stream meanwhile
-  float* readout = dz;
-  n += launch_readout(d, hs[L], b->d_chunk_row0, b->d_chunk_row1, 0, b->num_chunks, readout, 0, st);
+  if (!fused) n += launch_readout(d, hs[L], b->d_chunk_row0, b->d_chunk_row1, 0, b->num_chunks, readout, 0, st);
   // the last layer's softmax reverse takes its rows' gradients from the graphs' where it can, else they are written out first
   const bool from_graphs = gather && L > 0 && rows_gather_supported(d);
   const float* dr = nullptr;
-  const int kh = launch_ppo_heads(d, ctx->dw, grad, wb, hs[L], readout, b->d_graph_chunk_off,
-                                  b->seg_id.as<int32_t>(), g0, b->d_env_off, mask, action, logp_old, adv, ret, eps, c1, c2, b->B,
+  const int kh = launch_ppo_heads(d, ctx->dw, grad, wb, hs[L], readout,
+                                  fused ? b->node_off.as<int32_t>() : b->d_graph_chunk_off, fused ? nblocks : 0,
+                                  aggregate_block_shift(b->N), b->seg_id.as<int32_t>(), g0, b->d_env_off, mask, action, logp_old, adv, ret, eps, c1, c2, b->B,
                                   b->num_envs, b->N, heads_ws, loss_out, from_graphs ? nullptr : dh_a, &dr, logp_out,
                                   ctx->status.as<int32_t>(), st);
   if (kh < 0) { cudaGetLastError(); return XRL_ERR_CUDA; }

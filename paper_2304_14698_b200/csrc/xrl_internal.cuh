@@ -211,7 +211,7 @@ int32_t aggregate_readout_blocks(int64_t rows);
 // block_shift: aggregate_block_shift of the launch that wrote `partial`
 int launch_global_update_blocks(const Dims& d, const float* partial, const int32_t* node_off, int32_t nblocks,
                                 int block_shift, const float* g0, const DevWeights& w, float* emb, int32_t B,
-                                cudaStream_t st);
+                                cudaStream_t st, float* U_out = nullptr);
 int launch_readout(const Dims& d, const void* h, const int32_t* chunk_row0, const int32_t* chunk_row1,
                    int32_t chunk_begin, int32_t chunk_end, float* partial, int32_t win_base,
                    cudaStream_t st, const int32_t* remap = nullptr);
@@ -254,7 +254,8 @@ int launch_sample(const float* probs, int32_t num_envs, int32_t A1, uint64_t see
 // ---- reverse pass (Section 3.3.4) --------------------------------------------------------------------
 size_t ppo_heads_workspace_floats(const Dims& d, int64_t B, int64_t num_envs);
 int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const float* w_base, const void* hL,
-                     const float* partial, const int32_t* graph_chunk_off, const int32_t* seg_id, const float* g0,
+                     const float* partial, const int32_t* partial_off, int32_t nblocks, int block_shift,
+                     const int32_t* seg_id, const float* g0,
                      const int32_t* env_off,
                      const uint8_t* mask, const int32_t* action, const float* logp_old, const float* adv,
                      const float* ret, float eps, float c1, float c2, int32_t B, int32_t num_envs, int64_t N,

@@ -154,3 +154,22 @@ def test_gradient_of_both_products_at_the_edges_of_their_tiles(xo, H, K, nodes):
     rng = dags.make_rng(H + nodes)
     graphs = [dags.random_dag(rng, n, m["T"], 8, True, window=6) for n in (nodes, nodes + 3, nodes, 1, nodes + 1)]
     _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
+
+
+def _no_nodes():
+    return dict(op=np.zeros(0, np.int32), shape=np.zeros((0, 8), np.float32), edge_src=np.zeros(0, np.int32),
+                edge_dst=np.zeros(0, np.int32))
+
+
+@pytest.mark.parametrize("H,K,dtype,sizes", [
+    (H, K, dtype, sizes) for H, K, dtype in ((256, 4, "bf16"), (256, 8, "bf16"), (256, 16, "bf16"), (128, 4, "fp32"),
+                                             (128, 8, "fp32"), (128, 4, "bf16"))
+    for sizes in ((1, 1, 1, 1), (7, 8, 9, 1, 15, 17), (0, 5, 0, 33), (300, 0, 1, 700))
+    if dtype == "fp32" or sum(sizes) > 4])    # (four bf16 nodes: one rounded ReLU is a matrix column)
+def test_gradient_of_the_readout_fused_with_the_last_layer(xo, H, K, dtype, sizes):
+    """Graphs that begin and end inside, at and across the last layer's blocks of eight rows, graphs without nodes, and more
+    graphs than blocks (their sums then do not fit and the readout runs on its own)."""
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=len(sizes))
+    rng = dags.make_rng(H + K + len(sizes))
+    graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) if n else _no_nodes() for n in sizes]
+    _compare(xo, dags.flatten(graphs, [0, len(graphs)], m["A_max"]), m)
