@@ -259,12 +259,18 @@ __device__ __forceinline__ void agg_group(const int32_t* __restrict__ js, int32_
   }
 }
 
-template <typename T, int LPR, int VPL>
+// READOUT (several rows per warp only): the last layer fused with the per-graph sum of Eq. 8 (hidden 128 in bf16, 299 k rows:
+// 51 + 19 -> 51 us; with a row per warp, hidden 192, 124 k rows, 46 + 10 -> 59 us: the sums do not fit the registers of four
+// CTAs per SM), in the layout of the TMA kernel's fused variant (blocks of `block_rows` = 2^k rows from row 0 on: the rows of
+// a block's first graph to partial[block], those of a graph that starts inside it to partial[nblocks + graph]).  READOUT = 2
+// stores the rows as well, and the sum is then of the rows as stored.
+template <typename T, int LPR, int VPL, int READOUT>
 __global__ void __launch_bounds__(kRowThreads, (VPL == 1 ? 4 : 2))
 k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
             const T* __restrict__ Z, const float2* __restrict__ scores,
             const float* __restrict__ bias, T* __restrict__ h_out, int H, int K, Window win,
-            const int32_t* __restrict__ self_idx, int block_rows) {
+            const int32_t* __restrict__ self_idx, int block_rows, const int32_t* __restrict__ seg_id,
+            float* __restrict__ partial, int32_t nblocks) {
   enter();
   constexpr int VEC = VecOf<T>::N;
   constexpr int RPW = 32 / LPR;
@@ -315,6 +321,32 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
       constexpr int NP = VEC / 2;
       const T* zlane = Z + c0[0];
       const float2* slane = scores + head[0];
+      // (READOUT) the running sum of the current graph's rows, one per row group of the warp
+      const int32_t myseg = READOUT && lane < nr ? __ldg(seg_id + r0 + lane) : 0;
+      int32_t cur = -1;
+      bool first_seg = true;
+      aggtma::F2 sum[NP];
+      auto clear = [&]() {
+#pragma unroll
+        for (int t = 0; t < NP; ++t) sum[t] = aggtma::make_f2(0.f, 0.f);
+      };
+      auto flush = [&]() {
+        float* dst = partial + size_t(first_seg ? int32_t(r0 / block_rows) : nblocks + cur) * H + c0[0];
+#pragma unroll
+        for (int t = 0; t < NP; ++t) {
+          float lo, hi;
+          aggtma::split_f2(sum[t], lo, hi);
+#pragma unroll
+          for (int o = LPR; o < 32; o <<= 1) {
+            lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+            hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+          }
+          if (sub == 0 && on[0]) *reinterpret_cast<float2*>(dst + 2 * t) = make_float2(lo, hi);
+        }
+        first_seg = false;
+        clear();
+      };
+      if (READOUT) clear();
       for (int base = 0; base < nr; base += RPW) {
         const int rr = base + sub;
         const bool live = on[0] && rr < nr;
@@ -366,8 +398,33 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
 #pragma unroll
           for (int q = 0; q < NP; ++q) aggtma::fma2(acc[q], w1, z[q]);
         }
-        if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, __fdividef(1.f, l), bs[0]);
+        const float inv = __fdividef(1.f, l);
+        if constexpr (READOUT == 0) {
+          if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]);
+        } else {
+          aggtma::F2 o[NP];
+          if constexpr (READOUT == 1) aggtma::finish_row_f32<NP>(acc, inv, bs[0], o);
+          else if (live) aggtma::to_pairs(aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]), o);
+          const int32_t g0 = __shfl_sync(0xFFFFFFFFu, myseg, base), g1 = __shfl_sync(0xFFFFFFFFu, myseg, min(base + RPW, nr) - 1);
+          if (g0 == cur && g1 == cur) {
+            if (live)
+#pragma unroll
+              for (int t = 0; t < NP; ++t) aggtma::add2(sum[t], o[t]);
+          } else {                                 // a graph begins here: row by row
+            for (int s = 0; s < RPW && base + s < nr; ++s) {
+              const int32_t g = __shfl_sync(0xFFFFFFFFu, myseg, base + s);
+              if (g != cur) {
+                if (cur >= 0) flush();
+                cur = g;
+              }
+              if (live && sub == s)
+#pragma unroll
+                for (int t = 0; t < NP; ++t) aggtma::add2(sum[t], o[t]);
+            }
+          }
+        }
       }
+      if (READOUT && cur >= 0) flush();
       r0 += int64_t(warps_total) * block_rows;
       continue;
     }
@@ -413,10 +470,12 @@ template <typename T>
 RowGeom row_geom(int H) {
   const int nv = H / VecOf<T>::N;
   if (nv <= 8) return {8, 1};
-  if (nv == 16) return {16, 1};
+  if (nv <= 16) return {16, 1};        // (12 vectors, hidden 96: a row per warp took 66 us per layer of 194 k rows, two 43)
   const int vpl = (nv + 31) / 32;
   return {32, vpl <= 1 ? 1 : (vpl == 2 ? 2 : 4)};
 }
+
+RowGeom row_geom_of(const Dims& d) { return d.dtype == XRL_BF16 ? row_geom<bf16>(d.H) : row_geom<float>(d.H); }
 
 int row_grid(int64_t rows, int rpw) {
   const int64_t warps = (rows + rpw - 1) / rpw;
@@ -477,30 +536,38 @@ int launch_scores(const Dims& d, const void* Z, const LayerWeights& lw, float* s
 int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z,
                      const float* scores, const float* bias, void* h_out,
                      Window win, int64_t buf_rows, int32_t* status, cudaStream_t st,
-                     const int32_t* self_idx) {
+                     const int32_t* self_idx, const int32_t* seg_id, float* partial) {
   const int64_t rows = int64_t(win.row_end) - win.row_begin;
   if (rows <= 0) return 0;
   {   // 512-byte rows with 4 | K: gathers by the TMA engine
-    const int k = launch_aggregate_tma(d, rowptr, col, Z, scores, bias, h_out, win, buf_rows, nullptr, nullptr, status, st,
+    const int k = launch_aggregate_tma(d, rowptr, col, Z, scores, bias, h_out, win, buf_rows, seg_id, partial, status, st,
                                        self_idx);
     if (k >= 0 || d.zmerged) return k;       // with merged rows there is no other kernel to fall back to
   }
+  if (partial != nullptr && (win.row_begin != 0 || win.win_base != 0 || row_geom_of(d).lpr > 16)) return -1;
   // rows per warp and pass: the 32 of a full block, fewer for small batches (a multiple of the rows a
-  // warp holds at once)
+  // warp holds at once); with the sums the blocks that their layout has
   const int64_t warps_avail = int64_t(kNumSMs) * 8 * (kRowThreads / 32);
+  const int64_t sum_rows = int64_t(1) << aggregate_block_shift(rows);
+#define CALL_(TY_, LPR, VPL, RO_, br_)                                                             \
+  launch(k_aggregate<TY_, LPR, VPL, RO_>, row_grid(rows, int(br_)), kRowThreads, 0, st,            \
+         rowptr, col, static_cast<const TY_*>(Z), reinterpret_cast<const float2*>(scores), bias,   \
+         static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_), seg_id, partial,             \
+         int32_t((rows + sum_rows - 1) / sum_rows))
 #define CALL(TY_, LPR, VPL)                                                                        \
   do {                                                                                             \
     const int rpw_ = 32 / LPR;                                                                     \
     int64_t br_ = (rows + warps_avail - 1) / warps_avail;                                          \
     br_ = ((br_ + rpw_ - 1) / rpw_) * rpw_;                                                        \
     if (br_ > kAggBlockRows) br_ = kAggBlockRows;                                                  \
-    launch(k_aggregate<TY_, LPR, VPL>, row_grid(rows, int(br_)), kRowThreads, 0, st,                   \
-        rowptr, col, static_cast<const TY_*>(Z), reinterpret_cast<const float2*>(scores), bias,    \
-        static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_));                              \
+    if (LPR > 16 || partial == nullptr) CALL_(TY_, LPR, VPL, 0, br_);                              \
+    else if (h_out == nullptr) CALL_(TY_, LPR, VPL, (LPR <= 16 ? 1 : 0), sum_rows);                \
+    else CALL_(TY_, LPR, VPL, (LPR <= 16 ? 2 : 0), sum_rows);                                      \
   } while (0)
   if (d.dtype == XRL_BF16) XRL_ROW_DISPATCH(bf16, d.H, CALL);
   else XRL_ROW_DISPATCH(float, d.H, CALL);
 #undef CALL
+#undef CALL_
   return 1;
 }
 

@@ -584,10 +584,8 @@ int run_node_layers(xrl_ctx* ctx, const xrl_batch* b, int layers, cudaStream_t s
     k = -1;
     bool fused_here = false;
     if (fuse_readout && l == layers - 1) {
-      k = launch_aggregate_tma(d, gat_rowptr, gat_col, Zl,
-                               Sl, ctx->dw.layer[l].b, hs ? h_out : nullptr, win, b->N,
-                               b->seg_id.as<int32_t>(), partial,
-                               ctx->status.as<int32_t>(), st);
+      k = launch_aggregate(d, gat_rowptr, gat_col, Zl, Sl, ctx->dw.layer[l].b, hs ? h_out : nullptr, win, b->N, ctx->status.as<int32_t>(), st,
+                           nullptr, b->seg_id.as<int32_t>(), partial);
       if (k >= 0) { fused_here = true; if (fused) *fused = true; }
     }
     if (k < 0)

@@ -194,7 +194,7 @@ int launch_scores(const Dims& d, const void* Z, const LayerWeights& lw, float* s
 int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z,
                      const float* scores, const float* bias, void* h_out,
                      Window win, int64_t buf_rows, int32_t* status, cudaStream_t st,
-                     const int32_t* self_idx = nullptr);
+                     const int32_t* self_idx = nullptr, const int32_t* seg_id = nullptr, float* partial = nullptr);
 int launch_aggregate_tma(const Dims& d, const int32_t* rowptr, const int32_t* col, const void* Z,
                          const float* scores, const float* bias, void* h_out, Window win, int64_t buf_rows,
                          const int32_t* seg_id, float* partial, int32_t* status, cudaStream_t st,
