@@ -551,31 +551,41 @@ k_atb_tile(const TA* __restrict__ A, const float* __restrict__ Bm, float* __rest
 }
 
 // ---- out = G W^T: G [rows x Hn] fp32, W [Hk x Hn] (storage type, row-major [in x out]) -> out [rows x Hk] ----
+// (k_xform_simt's order of loads: 5.4 k rows of 512, 149 -> 96 us)
 template <typename TW>
 __global__ void __launch_bounds__(256)
 k_gwt(const float* __restrict__ G, const TW* __restrict__ W, float* __restrict__ out, int rows, int Hk, int Hn) {
   enter();
-  __shared__ float Gs[64][16 + 1];
-  __shared__ float Ws[64][16 + 1];
+  __shared__ __align__(16) float Gs[16][64 + 4];
+  __shared__ __align__(16) float Ws[16][64 + 4];
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int r0 = blockIdx.x * 64, k0 = blockIdx.y * 64;
   float acc[4][4] = {};
+  // four columns of one row of each operand per thread and step (the widths are multiples of 32), the next step's in flight
+  // during the arithmetic
+  const int rr = tid >> 2, cc0 = (tid & 3) * 4;
+  const bool g_ok = r0 + rr < rows, w_ok = k0 + rr < Hk;
+  const float* gp = G + size_t(g_ok ? r0 + rr : 0) * Hn + cc0;
+  const TW* wp = W + size_t(w_ok ? k0 + rr : 0) * Hn + cc0;
+  float g[4] = {}, w[4] = {};
+  if (g_ok) load_chunk<float, 4>(gp, g);
+  if (w_ok) load_chunk<TW, 4>(wp, w);
   for (int c0 = 0; c0 < Hn; c0 += 16) {
-    for (int t = tid; t < 64 * 16; t += 256) {
-      const int rr = t >> 4, cc = t & 15;
-      Gs[rr][cc] = (r0 + rr < rows && c0 + cc < Hn) ? G[size_t(r0 + rr) * Hn + c0 + cc] : 0.f;
-      Ws[rr][cc] = (k0 + rr < Hk && c0 + cc < Hn) ? to_float(W[size_t(k0 + rr) * Hn + c0 + cc]) : 0.f;
-    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) { Gs[cc0 + t][rr] = g[t]; Ws[cc0 + t][rr] = w[t]; }
     __syncthreads();
+    if (c0 + 16 < Hn) {
+      if (g_ok) load_chunk<float, 4>(gp + c0 + 16, g);
+      if (w_ok) load_chunk<TW, 4>(wp + c0 + 16, w);
+    }
 #pragma unroll
     for (int cc = 0; cc < 16; ++cc) {
-      float g[4], w[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { g[u] = Gs[ty * 4 + u][cc]; w[u] = Ws[tx * 4 + u][cc]; }
+      const float4 a4 = *reinterpret_cast<const float4*>(&Gs[cc][ty * 4]), b4 = *reinterpret_cast<const float4*>(&Ws[cc][tx * 4]);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(g[u], w[v], acc[u][v]);
+        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
     }
     __syncthreads();
   }
