@@ -263,7 +263,7 @@ __device__ __forceinline__ void agg_group(const int32_t* __restrict__ js, int32_
 // 51 + 19 -> 51 us; with a row per warp, hidden 192, 124 k rows, 46 + 10 -> 59 us: the sums do not fit the registers of four
 // CTAs per SM), in the layout of the TMA kernel's fused variant (blocks of `block_rows` = 2^k rows from row 0 on: the rows of
 // a block's first graph to partial[block], those of a graph that starts inside it to partial[nblocks + graph]).  READOUT = 2
-// stores the rows as well, and the sum is then of the rows as stored.
+// stores the rows as well; the sum is of the rows as they are stored either way, as the readout's and the delta path's are.
 template <typename T, int LPR, int VPL, int READOUT>
 __global__ void __launch_bounds__(kRowThreads, (VPL == 1 ? 4 : 2))
 k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -403,7 +403,7 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
           if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]);
         } else {
           aggtma::F2 o[NP];
-          if constexpr (READOUT == 1) aggtma::finish_row_f32<NP>(acc, inv, bs[0], o);
+          if constexpr (READOUT == 1) aggtma::to_pairs(aggtma::row_as_stored(acc, inv, bs[0]), o);
           else if (live) aggtma::to_pairs(aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]), o);
           const int32_t g0 = __shfl_sync(0xFFFFFFFFu, myseg, base), g1 = __shfl_sync(0xFFFFFFFFu, myseg, min(base + RPW, nr) - 1);
           if (g0 == cur && g1 == cur) {

@@ -93,9 +93,8 @@ __device__ __forceinline__ void to_pairs(const uint4& raw, F2 (&z)[2]) {        
   z[1] = make_f2(__uint_as_float(raw.z), __uint_as_float(raw.w));
 }
 
-// out = ReLU(acc * inv + bias), stored in the feature type
-// (the row as stored is returned)
-__device__ __forceinline__ uint4 finish_row(bf16* dst, const F2 (&acc)[4], float inv, const float (&bs)[8]) {
+// out = ReLU(acc * inv + bias) in the feature type, as it is stored
+__device__ __forceinline__ uint4 row_as_stored(const F2 (&acc)[4], float inv, const float (&bs)[8]) {        // 8 bf16
   uint32_t w[4];
   const F2 i2 = make_f2(inv, inv);
 #pragma unroll
@@ -106,20 +105,22 @@ __device__ __forceinline__ uint4 finish_row(bf16* dst, const F2 (&acc)[4], float
     split_f2(o, lo, hi);
     asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(w[t]) : "f"(hi), "f"(lo));   // ReLU inside the rounding
   }
-  const uint4 raw = make_uint4(w[0], w[1], w[2], w[3]);
-  *reinterpret_cast<uint4*>(dst) = raw;
-  return raw;
+  return make_uint4(w[0], w[1], w[2], w[3]);
 }
-__device__ __forceinline__ uint4 finish_row(float* dst, const F2 (&acc)[2], float inv, const float (&bs)[4]) {
-  float o[4];
+__device__ __forceinline__ uint4 row_as_stored(const F2 (&acc)[2], float inv, const float (&bs)[4]) {        // 4 fp32
+  uint32_t o[4];
 #pragma unroll
   for (int t = 0; t < 2; ++t) {
     float lo, hi;
     split_f2(acc[t], lo, hi);
-    o[2 * t] = fmaxf(fmaf(lo, inv, bs[2 * t]), 0.f);
-    o[2 * t + 1] = fmaxf(fmaf(hi, inv, bs[2 * t + 1]), 0.f);
+    o[2 * t] = __float_as_uint(fmaxf(fmaf(lo, inv, bs[2 * t]), 0.f));
+    o[2 * t + 1] = __float_as_uint(fmaxf(fmaf(hi, inv, bs[2 * t + 1]), 0.f));
   }
-  const uint4 raw = make_uint4(__float_as_uint(o[0]), __float_as_uint(o[1]), __float_as_uint(o[2]), __float_as_uint(o[3]));
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+template <typename T, int NP>
+__device__ __forceinline__ uint4 finish_row(T* dst, const F2 (&acc)[NP], float inv, const float (&bs)[2 * NP]) {
+  const uint4 raw = row_as_stored(acc, inv, bs);
   *reinterpret_cast<uint4*>(dst) = raw;
   return raw;
 }
