@@ -92,50 +92,70 @@ __device__ __forceinline__ void dense_rows(const float* x, int xs, int in, const
   }
 }
 
-// out[g][k] = sum_c W[k * ncols + c] v[g][c] for the GP rows of v (in shared memory, vs floats apart): a warp per two rows of
-// W, lanes along the columns.  emit(g, k, value) runs in one lane; ends with a barrier.
+// The sums over a warp's lanes of V = 2^k values each: value i ends up in lanes i * 32 / V and up.  Every step
+// halves the values that a lane carries: V - 1 + log2(32 / V) shuffles where a tree per value takes 5 V, the same additions.
+template <int V>
+__device__ __forceinline__ float warp_sums(float (&v)[V], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int n = V / 2; n > 0; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+      v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+    }
+  }
+  float s = v[0];
+  for (; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  return s;
+}
+
+// out[g][k] = sum_c W[k * ncols + c] v[g][c] for the GP rows of v (in shared memory, vs floats apart): a warp per R rows of
+// W, lanes along the columns, 4 R loads in flight.  The chain of passes over W's rows bounds it, then the shuffles
+// (two rows a warp and a tree per sum: k_graph_bwd of 324 graphs of 256 33 us, now 16; k_ppo_env 37 -> 32).
+// emit(g, k, value) runs in one lane; ends with a barrier.
 template <int GP, typename Emit>
 __device__ __forceinline__ void rows_dot(const float* __restrict__ W, int nrows, int ncols, const float* v, int vs, Emit emit) {
+  constexpr int R = GP == 1 ? 8 : GP <= 4 ? 4 : 2, V = R * GP;
+  static_assert((V & (V - 1)) == 0 && V <= 32, "");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = 2 * warp; k < nrows; k += 2 * nw) {
+  for (int k = R * warp; k < nrows; k += R * nw) {
     const float* w0 = W + size_t(k) * ncols;
-    const float* w1 = k + 1 < nrows ? w0 + ncols : w0;
-    float a0[GP], a1[GP];
+    const int last = nrows - 1 - k;                   // (rows past the end: the last one again)
+    float a[V];
 #pragma unroll
-    for (int g = 0; g < GP; ++g) a0[g] = a1[g] = 0.f;
+    for (int i = 0; i < V; ++i) a[i] = 0.f;
     int c = lane;
     for (; c + 96 < ncols; c += 128) {
-      float p[4], q[4];
+      float p[R][4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) { p[t] = __ldg(w0 + c + 32 * t); q[t] = __ldg(w1 + c + 32 * t); }
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) p[r][t] = __ldg(w0 + size_t(min(r, last)) * ncols + c + 32 * t);
 #pragma unroll
       for (int g = 0; g < GP; ++g)
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const float x = v[g * vs + c + 32 * t];
-          a0[g] = fmaf(p[t], x, a0[g]);
-          a1[g] = fmaf(q[t], x, a1[g]);
+#pragma unroll
+          for (int r = 0; r < R; ++r) a[r * GP + g] = fmaf(p[r][t], x, a[r * GP + g]);
         }
     }
     for (; c < ncols; c += 32) {
-      const float p = __ldg(w0 + c), q = __ldg(w1 + c);
+      float p[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) p[r] = __ldg(w0 + size_t(min(r, last)) * ncols + c);
 #pragma unroll
       for (int g = 0; g < GP; ++g) {
         const float x = v[g * vs + c];
-        a0[g] = fmaf(p, x, a0[g]);
-        a1[g] = fmaf(q, x, a1[g]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r * GP + g] = fmaf(p[r], x, a[r * GP + g]);
       }
     }
-#pragma unroll
-    for (int g = 0; g < GP; ++g) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        a0[g] += __shfl_xor_sync(0xFFFFFFFFu, a0[g], o);
-        a1[g] += __shfl_xor_sync(0xFFFFFFFFu, a1[g], o);
-      }
-      if (lane == 0) emit(g, k, a0[g]);
-      if (lane == 1 && k + 1 < nrows) emit(g, k + 1, a1[g]);
-    }
+    const float s = warp_sums<V>(a, lane);
+    const int i = lane / (32 / V), r = i / GP;
+    if (lane % (32 / V) == 0 && r <= last) emit(i % GP, k + r, s);
   }
   __syncthreads();
 }
