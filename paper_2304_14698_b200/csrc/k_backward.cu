@@ -772,7 +772,8 @@ __device__ __forceinline__ void mlp_hidden_bwd(const Mlp& m, const float* y1, co
 // ---- per environment: Eq. 3-5, d J / d logit of its graphs, value head forward and reverse -----------------
 // loss[4] += {J, L_clip, L_vf, L_ent} (atomics); dlogit [B]; demb [B x H] = the value head's share (plain
 // stores: a graph belongs to one environment); the value head's per-row buffers vu [2H], vy1, vy2, vd1, vd2,
-// vdout; logp_out [num_envs].
+// vdout; logp_out [num_envs].  Two CTAs per environment, side by side: blockIdx.y 0 the policy's part, 1 the value head's
+// (one after the other: 19 us instead of 16 at 6 environments of hidden 128, 32 instead of 29.5 at hidden 256).
 struct EnvBufs { float *vu, *vy1, *vy2, *vd1, *vd2, *vdout; };
 
 __global__ void __launch_bounds__(1024)
@@ -797,39 +798,48 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
   const float inv_ne = 1.f / float(num_envs);
   auto valid = [&](int a) { return a == A || (a < C && mk[a]); };
   auto lg = [&](int a) { return logit[a == A ? cur : cur + 1 + a]; };
-  // masked softmax statistics
-  float mx = -INFINITY;
-  for (int a = tid; a <= A; a += nt)
-    if (valid(a)) mx = fmaxf(mx, lg(a));
-  mx = heads::block_max(mx, scratch);
-  float se = 0.f;
-  for (int a = tid; a <= A; a += nt)
-    if (valid(a)) se += expf(lg(a) - mx);
-  const float sum = heads::block_sum(se, scratch);
-  const float lsum = logf(sum);
-  float pl = 0.f;                                   // sum_a p_a log p_a
-  for (int a = tid; a <= A; a += nt)
-    if (valid(a)) { const float lp = lg(a) - mx - lsum; pl += expf(lp) * lp; }
-  const float plogp = heads::block_sum(pl, scratch);
   const int act = action[e];
-  if (act < 0 || act > A || !valid(act)) {          // the same for every thread of the CTA
-    if (tid == 0) raise(status, XRL_ERR_INVALID_ARG);
+  if (act < 0 || act > A || !valid(act)) {          // the same for every thread of both CTAs
+    if (tid == 0 && blockIdx.y == 0) raise(status, XRL_ERR_INVALID_ARG);
     return;
   }
-  const float logp = lg(act) - mx - lsum;
-  const float ratio = expf(logp - logp_old[e]);
-  const float clipped = fminf(fmaxf(ratio, 1.f - eps), 1.f + eps);
-  const float t1 = ratio * adv[e], t2 = clipped * adv[e];
-  const float dlogp = (t1 <= t2) ? -adv[e] * ratio * inv_ne : 0.f;
-  for (int a = tid; a <= A; a += nt) {
-    if (a < A && a >= C) continue;                  // no graph behind a padded slot
-    const int32_t g = a == A ? cur : cur + 1 + a;
-    float dl = 0.f;
-    if (valid(a)) {
-      const float lp = lg(a) - mx - lsum, p = expf(lp);
-      dl = dlogp * ((a == act ? 1.f : 0.f) - p) + c2 * inv_ne * p * (lp - plogp);
+  if (blockIdx.y == 0) {
+    // masked softmax statistics
+    float mx = -INFINITY;
+    for (int a = tid; a <= A; a += nt)
+      if (valid(a)) mx = fmaxf(mx, lg(a));
+    mx = heads::block_max(mx, scratch);
+    float se = 0.f;
+    for (int a = tid; a <= A; a += nt)
+      if (valid(a)) se += expf(lg(a) - mx);
+    const float sum = heads::block_sum(se, scratch);
+    const float lsum = logf(sum);
+    float pl = 0.f;                                   // sum_a p_a log p_a
+    for (int a = tid; a <= A; a += nt)
+      if (valid(a)) { const float lp = lg(a) - mx - lsum; pl += expf(lp) * lp; }
+    const float plogp = heads::block_sum(pl, scratch);
+    const float logp = lg(act) - mx - lsum;
+    const float ratio = expf(logp - logp_old[e]);
+    const float clipped = fminf(fmaxf(ratio, 1.f - eps), 1.f + eps);
+    const float t1 = ratio * adv[e], t2 = clipped * adv[e];
+    const float dlogp = (t1 <= t2) ? -adv[e] * ratio * inv_ne : 0.f;
+    for (int a = tid; a <= A; a += nt) {
+      if (a < A && a >= C) continue;                  // no graph behind a padded slot
+      const int32_t g = a == A ? cur : cur + 1 + a;
+      float dl = 0.f;
+      if (valid(a)) {
+        const float lp = lg(a) - mx - lsum, p = expf(lp);
+        dl = dlogp * ((a == act ? 1.f : 0.f) - p) + c2 * inv_ne * p * (lp - plogp);
+      }
+      dlogit[g] = dl;
     }
-    dlogit[g] = dl;
+    if (tid == 0) {
+      const float lc = -(t1 <= t2 ? t1 : t2) * inv_ne, le = plogp * inv_ne;
+      atomicAdd(&loss[1], lc); atomicAdd(&loss[3], le);
+      atomicAdd(&loss[0], lc + c2 * le);
+      if (logp_out) logp_out[e] = logp;
+    }
+    return;
   }
   // value head over [ current graph | mean of the valid candidates ]
   const float nv = heads::value_input(emb, cur, C, mk, A, H, u, scratch);
@@ -867,10 +877,9 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
   }
   if (tid == 0) {
     eb.vdout[e] = dv;
-    const float lc = -(t1 <= t2 ? t1 : t2) * inv_ne, lv = (v - ret[e]) * (v - ret[e]) * inv_ne, le = plogp * inv_ne;
-    atomicAdd(&loss[1], lc); atomicAdd(&loss[2], lv); atomicAdd(&loss[3], le);
-    atomicAdd(&loss[0], lc + c1 * lv + c2 * le);
-    if (logp_out) logp_out[e] = logp;
+    const float lv = (v - ret[e]) * (v - ret[e]) * inv_ne;
+    atomicAdd(&loss[2], lv);
+    atomicAdd(&loss[0], c1 * lv);
   }
 }
 
@@ -1108,7 +1117,7 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
   if (k < 0) return -1;
   n += k;
   const size_t env_smem = sizeof(float) * (4 * 1024 + 4 * H + 2 * heads::row_stride(d.Hm) + 2 * heads::row_stride(d.Hm2));
-  launch(k_ppo_env, num_envs, 1024, env_smem, st, emb, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
+  launch(k_ppo_env, dim3(unsigned(num_envs), 2), 1024, env_smem, st, emb, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
                                               d.A, num_envs, loss, dlogit, demb, logp_out, status);
   ++n;
   // graphs per CTA: as few as leave every CTA an SM of its own, at most eight
