@@ -174,6 +174,10 @@ k_scores_bwd(ZView<T> zv, const float* __restrict__ ds_src, const float* __restr
 // A lane owns NF consecutive features, all of one head (32 / K lanes per head): a head's reductions stay inside
 // its group of lanes, all heads proceed at once, rows move as 4- to 16-byte pieces, and the scattered sums
 // go out as vector atomics.
+// Both add the columns that a CTA's warps keep (db; da_src, da_dst) from a slot per warp, and the second kernel gives a warp two
+// rows at least: additions into one shared row, and one global one per column and eight rows, took 56 us for 7 k rows of 512
+// (now 11; the first kernel 32 -> 23).
+constexpr int kBwdWarps = 8;
 // (NF values side by side, on the boundary that every lane's have: the power of two in their size, 16 at most)
 constexpr int chunk_align(int bytes) { return bytes % 16 == 0 ? 16 : bytes % 8 == 0 ? 8 : bytes % 4 == 0 ? 4 : 2; }
 template <typename T, int NF> struct alignas(chunk_align(int(sizeof(T)) * NF)) Chunk { T v[NF]; };
@@ -216,9 +220,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
                      BwdLists tl) {
   enter();
   constexpr int H = 32 * NF;
-  __shared__ float sm_db[H];
-  for (int c = threadIdx.x; c < H; c += blockDim.x) sm_db[c] = 0.f;
-  __syncthreads();
+  __shared__ __align__(16) float sm_db[kBwdWarps][H];             // each warp's sums
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int lph = 32 / K, k = lane / lph;            // lanes per head, this lane's head
@@ -339,12 +341,14 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
     }
     if (leader) ds_dst[size_t(i) * K + k] = dsd;
   }
-#pragma unroll
-  for (int f = 0; f < NF; ++f)
-    if (dbr[f] != 0.f) atomicAdd(&sm_db[lane * NF + f], dbr[f]);
+  store_chunk<NF>(&sm_db[threadIdx.x >> 5][lane * NF], dbr);
   __syncthreads();
-  for (int c = threadIdx.x; c < H; c += blockDim.x)
-    if (sm_db[c] != 0.f) atomicAdd(&db[c], sm_db[c]);
+  for (int c = threadIdx.x; c < H; c += blockDim.x) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < kBwdWarps; ++w) v += sm_db[w][c];
+    if (v != 0.f) atomicAdd(&db[c], v);
+  }
 }
 
 // dz += ds_src a_src + ds_dst a_dst per row and head, da_src / da_dst += ds z.  With `dzb` (tensor-core
@@ -356,9 +360,7 @@ k_scores_bwd_rows(ZView<T> zv, const float* __restrict__ ds_src, const float* __
                   bf16* __restrict__ dzb, float* __restrict__ da_src, float* __restrict__ da_dst, int N, int K) {
   enter();
   constexpr int H = 32 * NF;
-  __shared__ float sm_da[2 * H];
-  for (int c = threadIdx.x; c < 2 * H; c += blockDim.x) sm_da[c] = 0.f;
-  __syncthreads();
+  __shared__ __align__(16) float sm_da[kBwdWarps][2 * H];         // each warp's sums
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int k = lane / (32 / K);
@@ -388,15 +390,14 @@ k_scores_bwd_rows(ZView<T> zv, const float* __restrict__ ds_src, const float* __
       *reinterpret_cast<Chunk<bf16, NF>*>(dzb + size_t(i) * H + lane * NF) = c;
     }
   }
-#pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    atomicAdd(&sm_da[lane * NF + f], accs[f]);
-    atomicAdd(&sm_da[H + lane * NF + f], accd[f]);
-  }
+  store_chunk<NF>(&sm_da[threadIdx.x >> 5][lane * NF], accs);
+  store_chunk<NF>(&sm_da[threadIdx.x >> 5][H + lane * NF], accd);
   __syncthreads();
-  for (int c = threadIdx.x; c < H; c += blockDim.x) {
-    if (sm_da[c] != 0.f) atomicAdd(&da_src[c], sm_da[c]);
-    if (sm_da[H + c] != 0.f) atomicAdd(&da_dst[c], sm_da[H + c]);
+  for (int c = threadIdx.x; c < 2 * H; c += blockDim.x) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < kBwdWarps; ++w) v += sm_da[w][c];
+    if (v != 0.f) atomicAdd(c < H ? &da_src[c] : &da_dst[c - H], v);
   }
 }
 
@@ -1169,6 +1170,7 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   float* ds_dst = ds + size_t(N) * K;
   const size_t zrow = z_row_bytes(d);
   const int grid_rows = int(std::min<int64_t>((int64_t(N) + 7) / 8, int64_t(kNumSMs) * 8));
+  const int grid_sums = int(std::min<int64_t>((int64_t(N) + 15) / 16, int64_t(kNumSMs) * 4));
   const int grid_cols = int(std::min<int64_t>((int64_t(N) + 255) / 256, int64_t(kNumSMs) * 2));
   // dW on CUDA cores: 128-wide tiles where they fit H (one CTA of 256 threads per SM: 160 registers; held to 128
   // registers and two CTAs the launch takes 35.6 us instead of 33.6 at 36 k rows), else 64-wide ones (six CTAs of 64
@@ -1189,7 +1191,7 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   do {                                                                                                         \
     launch(k_aggregate_bwd_rows<TY_, NF_, false>, grid_rows, 256, 0, st,                                           \
         rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, dz, ds_src, ds_dst, gb, N, K, BwdLists{});  \
-    launch(k_scores_bwd_rows<TY_, NF_>, grid_rows, 256, 0, st, zv, ds_src, ds_dst, lw.a_src, lw.a_dst, dz, dzb,    \
+    launch(k_scores_bwd_rows<TY_, NF_>, grid_sums, 256, 0, st, zv, ds_src, ds_dst, lw.a_src, lw.a_dst, dz, dzb,    \
                                                            ga_src, ga_dst, N, K);                              \
   } while (0)
 #define BWD_GATHER(TY_, NF_)                                                                                   \
