@@ -253,9 +253,7 @@ k_scores(const T* __restrict__ Z, const float* __restrict__ a_src, const float* 
 // whole block are fetched with a few coalesced loads into shared memory, so that the per-row work
 // starts straight at the gathers of Z.  The half-scores arrive already multiplied by log2(e)
 // (LeakyReLU commutes with a positive factor), so the softmax weights are plain exp2.  Producers
-// are taken in groups of up to four: all their loads are issued first, the running maximum is
-// updated once per group and the partial sum rescaled only if it grew.  Every Z row and every
-// score is read once.
+// are taken two at a time, the first two asked for with the row's own vector.
 constexpr int kAggBlockRows = 32;
 constexpr int kAggColCap = 224;       // producer ids cached per block of rows
 
@@ -266,53 +264,17 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-// One group of NB (1..4) producers of a row: loads, then maximum, weights, accumulation.
-template <typename T, int NB>
-__device__ __forceinline__ void agg_group(const int32_t* __restrict__ js, int32_t win_base,
-                                          const T* __restrict__ zlane, const float2* __restrict__ slane,
-                                          int H, int K, float sd, float& m, float& l,
-                                          float (&acc)[VecOf<T>::N]) {
-  constexpr int VEC = VecOf<T>::N;
-  float ev[NB];
-  uint4 raw[NB];
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const int32_t j = js[b] - win_base;
-    ev[b] = __ldg(&slane[size_t(j) * K].x);
-    raw[b] = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(j) * H));
-  }
-  float mx = m;
-#pragma unroll
-  for (int b = 0; b < NB; ++b) { ev[b] = lrelu(ev[b] + sd); mx = fmaxf(mx, ev[b]); }
-  if (mx > m) {
-    const float scale = fast_exp2(m - mx);
-    l *= scale;
-#pragma unroll
-    for (int t = 0; t < VEC; ++t) acc[t] *= scale;
-    m = mx;
-  }
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const float p = fast_exp2(ev[b] - m);
-    l += p;
-    float z[VEC];
-    unpack(raw[b], z);
-#pragma unroll
-    for (int t = 0; t < VEC; ++t) acc[t] = fmaf(p, z[t], acc[t]);
-  }
-}
-
 // READOUT (several rows per warp only): the last layer fused with the per-graph sum of Eq. 8 (hidden 128 in bf16, 299 k rows:
 // 51 + 19 -> 51 us; with a row per warp, hidden 192, 124 k rows, 46 + 10 -> 59 us: the sums do not fit the registers of four
 // CTAs per SM), in the layout of the TMA kernel's fused variant (blocks of `block_rows` = 2^k rows from row 0 on: the rows of
 // a block's first graph to partial[block], those of a graph that starts inside it to partial[nblocks + graph]).  READOUT = 2
 // stores the rows as well; the sum is of the rows as they are stored either way, as the readout's and the delta path's are.
-template <typename T, int LPR, int VPL, int READOUT>
-__global__ void __launch_bounds__(kRowThreads, (VPL == 1 ? 4 : 2))
+template <typename T, int LPR, int READOUT>
+__global__ void __launch_bounds__(kRowThreads, 4)
 k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
             const T* __restrict__ Z, const float2* __restrict__ scores,
             const float* __restrict__ bias, T* __restrict__ h_out, int H, int K, Window win,
-            const int32_t* __restrict__ self_idx, int block_rows, const int32_t* __restrict__ seg_id,
+            const int32_t* __restrict__ self_idx, int block_rows, int slab_vecs, const int32_t* __restrict__ seg_id,
             float* __restrict__ partial, int32_t nblocks) {
   enter();
   constexpr int VEC = VecOf<T>::N;
@@ -325,18 +287,15 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
   const int warps_total = (gridDim.x * blockDim.x) >> 5;
   const int warp_id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
 
-  int c0[VPL], head[VPL];
-  bool on[VPL];
-  float bs[VPL][VEC];
+  // one vector per lane; rows of more than 32 vectors are split into gridDim.y slabs of columns (every slab weighs the
+  // producers anew; two vectors per lane one after the other, in groups of one to four producers, took 356 us per layer of
+  // 323 k rows of 512 with one head, slabs 240)
+  const int vi = int(blockIdx.y) * slab_vecs + sl;
+  const bool on = sl < slab_vecs && vi < NV;
+  const int c0 = on ? vi * VEC : 0, head = c0 / d;
+  float bs[VEC];
 #pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int vi = v * LPR + sl;
-    on[v] = vi < NV;
-    c0[v] = on[v] ? vi * VEC : 0;
-    head[v] = c0[v] / d;
-#pragma unroll
-    for (int t = 0; t < VEC; ++t) bs[v][t] = __ldg(bias + c0[v] + t);
-  }
+  for (int t = 0; t < VEC; ++t) bs[t] = __ldg(bias + c0 + t);
 
   // blocks of rows: as many rows (up to 32) as keep the block's producer ids within the cache;
   // a single row with more producers than that is walked straight from global memory
@@ -354,154 +313,119 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     for (int t = lane; t < ne; t += 32) s_col[wib][t] = __ldg(col + eb + t);
     __syncwarp();
 
-    if constexpr (VPL == 1) {
-      // One vector per lane.  The 32 / LPR rows of a warp go through one code path together: producers two at a time up to
-      // the largest count among the rows, the first two asked for together with the row's own
-      // vector, packed fp32 arithmetic, a reference exponent that moves only when a score exceeds it by 32.  Rows of
-      // different degrees taking their own branches through groups of 1 to 4 producers executed 115 warp instructions
-      // per row at 58 % issue utilisation (hidden 128 bf16, 299 k rows of mean degree 1.1: 0.057 ms; now
-      // 0.053.  Asking for the next rows' vectors one step ahead costs a resident CTA per SM: 0.066).
-      constexpr int NP = VEC / 2;
-      const T* zlane = Z + c0[0];
-      const float2* slane = scores + head[0];
-      // (READOUT) the running sum of the current graph's rows, one per row group of the warp
-      const int32_t myseg = READOUT && lane < nr ? __ldg(seg_id + r0 + lane) : 0;
-      int32_t cur = -1;
-      bool first_seg = true;
-      aggtma::F2 sum[NP];
-      auto clear = [&]() {
+    // The 32 / LPR rows of a warp go through one code path together: producers two at a time up to
+    // the largest count among the rows, the first two asked for together with the row's own
+    // vector, packed fp32 arithmetic, a reference exponent that moves only when a score exceeds it by 32.  Rows of
+    // different degrees taking their own branches through groups of 1 to 4 producers executed 115 warp instructions
+    // per row at 58 % issue utilisation (hidden 128 bf16, 299 k rows of mean degree 1.1: 0.057 ms; now
+    // 0.053.  Asking for the next rows' vectors one step ahead costs a resident CTA per SM: 0.066).
+    constexpr int NP = VEC / 2;
+    const T* zlane = Z + c0;
+    const float2* slane = scores + head;
+    // (READOUT) the running sum of the current graph's rows, one per row group of the warp
+    const int32_t myseg = READOUT && lane < nr ? __ldg(seg_id + r0 + lane) : 0;
+    int32_t cur = -1;
+    bool first_seg = true;
+    aggtma::F2 sum[NP];
+    auto clear = [&]() {
 #pragma unroll
-        for (int t = 0; t < NP; ++t) sum[t] = aggtma::make_f2(0.f, 0.f);
+      for (int t = 0; t < NP; ++t) sum[t] = aggtma::make_f2(0.f, 0.f);
+    };
+    auto flush = [&]() {
+      float* dst = partial + size_t(first_seg ? int32_t(r0 / block_rows) : nblocks + cur) * H + c0;
+#pragma unroll
+      for (int t = 0; t < NP; ++t) {
+        float lo, hi;
+        aggtma::split_f2(sum[t], lo, hi);
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) {
+          lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+          hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
+        }
+        if (sub == 0 && on) *reinterpret_cast<float2*>(dst + 2 * t) = make_float2(lo, hi);
+      }
+      first_seg = false;
+      clear();
+    };
+    if (READOUT) clear();
+    for (int base = 0; base < nr; base += RPW) {
+      const int rr = base + sub;
+      const bool live = on && rr < nr;
+      int e0 = 0, n = 0;
+      if (live) { e0 = s_rp[wib][rr] - eb; n = s_rp[wib][rr + 1] - eb - e0; }
+      const int nmax = RPW == 1 ? n : __reduce_max_sync(0xFFFFFFFFu, n);
+      const int32_t lrow = int32_t(r0) + rr - win.win_base;
+      const int32_t* js = e0 + n <= kAggColCap ? &s_col[wib][e0] : col + eb + e0;
+      float2 self = make_float2(0.f, 0.f);
+      uint4 raw = make_uint4(0u, 0u, 0u, 0u), qa, qb;
+      float ea, eo;
+      if (live) {
+        const int32_t srow = self_idx ? __ldg(self_idx + int32_t(r0) + rr) : lrow;   // where the row's own Z lives
+        self = __ldg(slane + size_t(srow) * K);
+        raw = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(srow) * H));
+      }
+      auto pair = [&](int t) {                        // producers t, t + 1
+        ea = eo = -INFINITY;
+        qa = qb = make_uint4(0u, 0u, 0u, 0u);
+        if (t < n) {
+          const int32_t j = js[t] - win.win_base;
+          ea = __ldg(&slane[size_t(j) * K].x);
+          qa = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(j) * H));
+        }
+        if (t + 1 < n) {
+          const int32_t j = js[t + 1] - win.win_base;
+          eo = __ldg(&slane[size_t(j) * K].x);
+          qb = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(j) * H));
+        }
       };
-      auto flush = [&]() {
-        float* dst = partial + size_t(first_seg ? int32_t(r0 / block_rows) : nblocks + cur) * H + c0[0];
+      if (nmax > 0) pair(0);
+      const float sd = self.y;
+      float m = lrelu(self.x + sd), l = 1.f;          // the self term opens the softmax
+      aggtma::F2 acc[NP];
+      aggtma::to_pairs(raw, acc);
+      for (int t = 0; t < nmax; t += 2) {
+        if (t > 0) pair(t);
+        const float ev0 = lrelu(ea + sd), ev1 = lrelu(eo + sd), evm = fmaxf(ev0, ev1);
+        if (evm > m + 32.f) aggtma::raise_reference<NP>(evm, m, l, acc);
+        // (absent producers weigh 0 by their place and not by their score, which is no number where the row's is infinite)
+        const float p0 = t < n ? fast_exp2(ev0 - m) : 0.f, p1 = t + 1 < n ? fast_exp2(ev1 - m) : 0.f;
+        l += p0 + p1;
+        aggtma::F2 z[NP];
+        aggtma::to_pairs(qa, z);
+        const aggtma::F2 w0 = aggtma::make_f2(p0, p0), w1 = aggtma::make_f2(p1, p1);
 #pragma unroll
-        for (int t = 0; t < NP; ++t) {
-          float lo, hi;
-          aggtma::split_f2(sum[t], lo, hi);
+        for (int q = 0; q < NP; ++q) aggtma::fma2(acc[q], w0, z[q]);
+        aggtma::to_pairs(qb, z);
 #pragma unroll
-          for (int o = LPR; o < 32; o <<= 1) {
-            lo += __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-            hi += __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-          }
-          if (sub == 0 && on[0]) *reinterpret_cast<float2*>(dst + 2 * t) = make_float2(lo, hi);
-        }
-        first_seg = false;
-        clear();
-      };
-      if (READOUT) clear();
-      for (int base = 0; base < nr; base += RPW) {
-        const int rr = base + sub;
-        const bool live = on[0] && rr < nr;
-        int e0 = 0, n = 0;
-        if (live) { e0 = s_rp[wib][rr] - eb; n = s_rp[wib][rr + 1] - eb - e0; }
-        const int nmax = RPW == 1 ? n : __reduce_max_sync(0xFFFFFFFFu, n);
-        const int32_t lrow = int32_t(r0) + rr - win.win_base;
-        const int32_t* js = e0 + n <= kAggColCap ? &s_col[wib][e0] : col + eb + e0;
-        float2 self = make_float2(0.f, 0.f);
-        uint4 raw = make_uint4(0u, 0u, 0u, 0u), qa, qb;
-        float ea, eo;
-        if (live) {
-          const int32_t srow = self_idx ? __ldg(self_idx + int32_t(r0) + rr) : lrow;   // where the row's own Z lives
-          self = __ldg(slane + size_t(srow) * K);
-          raw = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(srow) * H));
-        }
-        auto pair = [&](int t) {                        // producers t, t + 1
-          ea = eo = -INFINITY;
-          qa = qb = make_uint4(0u, 0u, 0u, 0u);
-          if (t < n) {
-            const int32_t j = js[t] - win.win_base;
-            ea = __ldg(&slane[size_t(j) * K].x);
-            qa = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(j) * H));
-          }
-          if (t + 1 < n) {
-            const int32_t j = js[t + 1] - win.win_base;
-            eo = __ldg(&slane[size_t(j) * K].x);
-            qb = __ldg(reinterpret_cast<const uint4*>(zlane + size_t(j) * H));
-          }
-        };
-        if (nmax > 0) pair(0);
-        const float sd = self.y;
-        float m = lrelu(self.x + sd), l = 1.f;          // the self term opens the softmax
-        aggtma::F2 acc[NP];
-        aggtma::to_pairs(raw, acc);
-        for (int t = 0; t < nmax; t += 2) {
-          if (t > 0) pair(t);
-          const float ev0 = lrelu(ea + sd), ev1 = lrelu(eo + sd), evm = fmaxf(ev0, ev1);
-          if (evm > m + 32.f) aggtma::raise_reference<NP>(evm, m, l, acc);
-          // (absent producers weigh 0 by their place and not by their score, which is no number where the row's is infinite)
-          const float p0 = t < n ? fast_exp2(ev0 - m) : 0.f, p1 = t + 1 < n ? fast_exp2(ev1 - m) : 0.f;
-          l += p0 + p1;
-          aggtma::F2 z[NP];
-          aggtma::to_pairs(qa, z);
-          const aggtma::F2 w0 = aggtma::make_f2(p0, p0), w1 = aggtma::make_f2(p1, p1);
+        for (int q = 0; q < NP; ++q) aggtma::fma2(acc[q], w1, z[q]);
+      }
+      const float inv = __fdividef(1.f, l);
+      if constexpr (READOUT == 0) {
+        if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0, acc, inv, bs);
+      } else {
+        aggtma::F2 o[NP];
+        if constexpr (READOUT == 1) aggtma::to_pairs(aggtma::row_as_stored(acc, inv, bs), o);
+        else if (live) aggtma::to_pairs(aggtma::finish_row(h_out + size_t(lrow) * H + c0, acc, inv, bs), o);
+        const int32_t g0 = __shfl_sync(0xFFFFFFFFu, myseg, base), g1 = __shfl_sync(0xFFFFFFFFu, myseg, min(base + RPW, nr) - 1);
+        if (g0 == cur && g1 == cur) {
+          if (live)
 #pragma unroll
-          for (int q = 0; q < NP; ++q) aggtma::fma2(acc[q], w0, z[q]);
-          aggtma::to_pairs(qb, z);
-#pragma unroll
-          for (int q = 0; q < NP; ++q) aggtma::fma2(acc[q], w1, z[q]);
-        }
-        const float inv = __fdividef(1.f, l);
-        if constexpr (READOUT == 0) {
-          if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]);
-        } else {
-          aggtma::F2 o[NP];
-          if constexpr (READOUT == 1) aggtma::to_pairs(aggtma::row_as_stored(acc, inv, bs[0]), o);
-          else if (live) aggtma::to_pairs(aggtma::finish_row(h_out + size_t(lrow) * H + c0[0], acc, inv, bs[0]), o);
-          const int32_t g0 = __shfl_sync(0xFFFFFFFFu, myseg, base), g1 = __shfl_sync(0xFFFFFFFFu, myseg, min(base + RPW, nr) - 1);
-          if (g0 == cur && g1 == cur) {
-            if (live)
+            for (int t = 0; t < NP; ++t) aggtma::add2(sum[t], o[t]);
+        } else {                                 // a graph begins here: row by row
+          for (int s = 0; s < RPW && base + s < nr; ++s) {
+            const int32_t g = __shfl_sync(0xFFFFFFFFu, myseg, base + s);
+            if (g != cur) {
+              if (cur >= 0) flush();
+              cur = g;
+            }
+            if (live && sub == s)
 #pragma unroll
               for (int t = 0; t < NP; ++t) aggtma::add2(sum[t], o[t]);
-          } else {                                 // a graph begins here: row by row
-            for (int s = 0; s < RPW && base + s < nr; ++s) {
-              const int32_t g = __shfl_sync(0xFFFFFFFFu, myseg, base + s);
-              if (g != cur) {
-                if (cur >= 0) flush();
-                cur = g;
-              }
-              if (live && sub == s)
-#pragma unroll
-                for (int t = 0; t < NP; ++t) aggtma::add2(sum[t], o[t]);
-            }
           }
         }
       }
-      if (READOUT && cur >= 0) flush();
-      r0 += int64_t(warps_total) * block_rows;
-      continue;
     }
-
-    for (int rr = sub; rr < nr; rr += RPW) {
-      const int32_t lrow = int32_t(r0) + rr - win.win_base;
-      const int e0 = s_rp[wib][rr] - eb;              // edge offsets relative to the block
-      const int n = s_rp[wib][rr + 1] - eb - e0;
-      const bool cached = e0 + n <= kAggColCap;
-      const int32_t* js = cached ? &s_col[wib][e0] : col + eb + e0;
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        if (!on[v]) continue;
-        const T* zlane = Z + c0[v];
-        const float2* slane = scores + head[v];
-        const int32_t srow = self_idx ? __ldg(self_idx + int32_t(r0) + rr) : lrow;   // where the row's own Z lives
-        const float2 self = __ldg(slane + size_t(srow) * K);
-        const float sd = self.y;
-        float m = lrelu(self.x + sd);                               // the self term opens the softmax
-        float l = 1.f, acc[VEC];
-        load_vec(zlane + size_t(srow) * H, acc);
-        int t = 0;
-        for (; t + 4 <= n; t += 4) agg_group<T, 4>(js + t, win.win_base, zlane, slane, H, K, sd, m, l, acc);
-        const int rem = n - t;                          // the same for all lanes of a row group
-        if (rem == 1) agg_group<T, 1>(js + t, win.win_base, zlane, slane, H, K, sd, m, l, acc);
-        else if (rem == 2) agg_group<T, 2>(js + t, win.win_base, zlane, slane, H, K, sd, m, l, acc);
-        else if (rem == 3) agg_group<T, 3>(js + t, win.win_base, zlane, slane, H, K, sd, m, l, acc);
-        const float inv = __fdividef(1.f, l);
-        float o[VEC];
-#pragma unroll
-        for (int t2 = 0; t2 < VEC; ++t2) o[t2] = fmaxf(fmaf(acc[t2], inv, bs[v][t2]), 0.f);
-        store_vec(h_out + size_t(lrow) * H + c0[v], o);
-      }
-    }
+    if (READOUT && cur >= 0) flush();
     r0 += int64_t(warps_total) * block_rows;
   }
 }
@@ -592,20 +516,22 @@ int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, c
   // warp holds at once); with the sums the blocks that their layout has
   const int64_t warps_avail = int64_t(kNumSMs) * 8 * (kRowThreads / 32);
   const int64_t sum_rows = int64_t(1) << aggregate_block_shift(rows);
-#define CALL_(TY_, LPR, VPL, RO_, br_)                                                             \
-  launch(k_aggregate<TY_, LPR, VPL, RO_>, row_grid(rows, int(br_)), kRowThreads, 0, st,            \
+  const int nv = d.H / (d.dtype == XRL_BF16 ? VecOf<bf16>::N : VecOf<float>::N), slabs = (nv + 31) / 32,
+            slab_vecs = (nv + slabs - 1) / slabs;
+#define CALL_(TY_, LPR, RO_, br_)                                                                  \
+  launch(k_aggregate<TY_, LPR, RO_>, dim3(unsigned(row_grid(rows, int(br_))), unsigned(slabs)), kRowThreads, 0, st, \
          rowptr, col, static_cast<const TY_*>(Z), reinterpret_cast<const float2*>(scores), bias,   \
-         static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_), seg_id, partial,             \
+         static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_), slab_vecs, seg_id, partial,  \
          int32_t((rows + sum_rows - 1) / sum_rows))
 #define CALL(TY_, LPR, VPL)                                                                        \
   do {                                                                                             \
     const int rpw_ = 32 / LPR;                                                                     \
-    int64_t br_ = (rows + warps_avail - 1) / warps_avail;                                          \
+    int64_t br_ = (rows * slabs + warps_avail - 1) / warps_avail;                                          \
     br_ = ((br_ + rpw_ - 1) / rpw_) * rpw_;                                                        \
     if (br_ > kAggBlockRows) br_ = kAggBlockRows;                                                  \
-    if (LPR > 16 || partial == nullptr) CALL_(TY_, LPR, VPL, 0, br_);                              \
-    else if (h_out == nullptr) CALL_(TY_, LPR, VPL, (LPR <= 16 ? 1 : 0), sum_rows);                \
-    else CALL_(TY_, LPR, VPL, (LPR <= 16 ? 2 : 0), sum_rows);                                      \
+    if (LPR > 16 || partial == nullptr) CALL_(TY_, LPR, 0, br_);                              \
+    else if (h_out == nullptr) CALL_(TY_, LPR, (LPR <= 16 ? 1 : 0), sum_rows);                \
+    else CALL_(TY_, LPR, (LPR <= 16 ? 2 : 0), sum_rows);                                      \
   } while (0)
   if (d.dtype == XRL_BF16) XRL_ROW_DISPATCH(bf16, d.H, CALL);
   else XRL_ROW_DISPATCH(float, d.H, CALL);
