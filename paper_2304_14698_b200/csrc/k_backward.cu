@@ -778,7 +778,7 @@ __device__ __forceinline__ void mlp_hidden_bwd(const Mlp& m, const float* y1, co
 struct EnvBufs { float *vu, *vy1, *vy2, *vd1, *vd2, *vdout; };
 
 __global__ void __launch_bounds__(1024)
-k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const int32_t* __restrict__ env_off,
+k_ppo_env(const float* __restrict__ logit, const int32_t* __restrict__ env_off,
           const uint8_t* __restrict__ mask, const int32_t* __restrict__ action, const float* __restrict__ logp_old,
           const float* __restrict__ adv, const float* __restrict__ ret, float eps, float c1, float c2, Mlp vm,
           EnvBufs eb, int H, int A, int num_envs, float* __restrict__ loss, float* __restrict__ dlogit,
@@ -787,8 +787,7 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
   extern __shared__ __align__(16) float sm[];
   const int e = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   float* scratch = sm;                              // [4 blockDim]
-  float* u = scratch + 4 * nt;                      // [2H]
-  float* du = u + 2 * H;                            // [2H]
+  float* du = scratch + 4 * nt;                     // [2H]
   float* y1 = du + 2 * H;                           // [hid], padded
   float* y2 = y1 + heads::row_stride(vm.hid);       // [hid2], padded
   float* d1 = y2 + heads::row_stride(vm.hid2);      // [hid], padded
@@ -842,9 +841,12 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
     }
     return;
   }
-  // value head over [ current graph | mean of the valid candidates ]
-  const float nv = heads::value_input(emb, cur, C, mk, A, H, u, scratch);
-  heads::dense_rows<1>(u, 0, 2 * H, vm.W1, vm.hid, vm.hid, vm.b1, scratch, [&](int, int c, float y) { y1[c] = fmaxf(y, 0.f); });
+  // value head over [ current graph | mean of the valid candidates ]: its input and first layer come from the launch that
+  // scores the policy, whose CTAs share the layer (one CTA here read all of its weights)
+  float cnt = 0.f;
+  for (int a = tid; a < min(C, A); a += nt) cnt += mk[a] ? 1.f : 0.f;
+  for (int c = tid; c < vm.hid; c += nt) y1[c] = eb.vy1[size_t(e) * vm.hid + c];
+  const float nv = heads::block_sum(cnt, scratch);
   float contrib = 0.f;
   if (vm.hid2 <= 0) {
     for (int c = tid; c < vm.hid; c += nt) contrib += y1[c] * vm.w2[c];
@@ -858,11 +860,7 @@ k_ppo_env(const float* __restrict__ emb, const float* __restrict__ logit, const 
   const float dv = c1 * 2.f * (v - ret[e]) * inv_ne;
   mlp_hidden_bwd(vm, y1, y2, dv, d1, d2);
   heads::rows_dot<1>(vm.W1, 2 * H, vm.hid, d1, 0, [&](int, int k, float x) { du[k] = x; });
-  for (int c = tid; c < 2 * H; c += nt) eb.vu[size_t(e) * 2 * H + c] = u[c];
-  for (int c = tid; c < vm.hid; c += nt) {
-    eb.vy1[size_t(e) * vm.hid + c] = y1[c];
-    eb.vd1[size_t(e) * vm.hid + c] = d1[c];
-  }
+  for (int c = tid; c < vm.hid; c += nt) eb.vd1[size_t(e) * vm.hid + c] = d1[c];
   for (int c = tid; c < vm.hid2; c += nt) {
     eb.vy2[size_t(e) * vm.hid2 + c] = y2[c];
     eb.vd2[size_t(e) * vm.hid2 + c] = d2[c];
@@ -1114,11 +1112,11 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
                       : launch_global_update(d, partial, partial_off, g0, w, emb, B, st, U);
   if (k < 0) return -1;
   n += k;
-  k = launch_policy_value_hidden(d, w, emb, logit, B, py1, py2, nullptr, nullptr, 0, nullptr, st);
+  k = launch_policy_value_hidden(d, w, emb, logit, B, py1, py2, env_off, mask, num_envs, eb.vy1, st, eb.vu);
   if (k < 0) return -1;
   n += k;
-  const size_t env_smem = sizeof(float) * (4 * 1024 + 4 * H + 2 * heads::row_stride(d.Hm) + 2 * heads::row_stride(d.Hm2));
-  launch(k_ppo_env, dim3(unsigned(num_envs), 2), 1024, env_smem, st, emb, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
+  const size_t env_smem = sizeof(float) * (4 * 1024 + 2 * H + 2 * heads::row_stride(d.Hm) + 2 * heads::row_stride(d.Hm2));
+  launch(k_ppo_env, dim3(unsigned(num_envs), 2), 1024, env_smem, st, logit, env_off, mask, action, logp_old, adv, ret, eps, c1, c2, vm, eb, d.H,
                                               d.A, num_envs, loss, dlogit, demb, logp_out, status);
   ++n;
   // graphs per CTA: as few as leave every CTA an SM of its own, at most eight

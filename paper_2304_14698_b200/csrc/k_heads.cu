@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kThreads)
 k_policy_value_hidden(const float* __restrict__ emb, const Mlp pm, float* __restrict__ logit, int H, int32_t B,
                       int policy_ctas, float* __restrict__ y1_out, float* __restrict__ y2_out,
                       const int32_t* __restrict__ env_off, const uint8_t* __restrict__ mask, int A, const Mlp vm,
-                      float* __restrict__ y1v, int VC) {
+                      float* __restrict__ y1v, int VC, float* __restrict__ u_out) {
   enter();
   extern __shared__ __align__(16) float sm[];
   const int nt = blockDim.x, tid = threadIdx.x;
@@ -202,6 +202,8 @@ k_policy_value_hidden(const float* __restrict__ emb, const Mlp pm, float* __rest
   const int32_t e = (int32_t(blockIdx.x) - policy_ctas) / VC, ch = (int32_t(blockIdx.x) - policy_ctas) % VC;
   const int32_t cur = env_off[e];
   value_input(emb, cur, env_off[e + 1] - cur - 1, mask + size_t(e) * A, A, H, u, scratch);
+  if (u_out != nullptr && ch == 0)
+    for (int c = tid; c < 2 * H; c += nt) u_out[size_t(e) * 2 * H + c] = u[c];
   const int CW = (vm.hid + VC - 1) / VC, c_lo = ch * CW, ncols = min(CW, vm.hid - c_lo);
   if (ncols > 0)
     dense_rows<1>(u, 0, 2 * H, vm.W1 + c_lo, vm.hid, ncols, vm.b1 + c_lo, scratch,
@@ -466,12 +468,12 @@ int launch_update(const Dims& d, const float* partial, const int32_t* off, int32
 template <int GP>
 int policy_value(const Dims& d, const Mlp& pm, const Mlp& vm, const float* emb, float* logit, int32_t B, float* y1_out,
                  float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v, int VC, size_t smem,
-                 cudaStream_t st) {
+                 cudaStream_t st, float* u_out) {
   static bool attr[64] = {};
   if (smem > 48 * 1024 && !ensure_dynamic_smem(k_policy_value_hidden<GP>, 227 * 1024, attr)) return -1;
   const int pc = (B + GP - 1) / GP;
   launch(k_policy_value_hidden<GP>, pc + num_envs * VC, kThreads, smem, st, emb, pm, logit, d.H, B, pc, y1_out, y2_out, env_off,
-                                                                        mask, d.A, vm, y1v, VC);
+                                                                        mask, d.A, vm, y1v, VC, u_out);
   return 1;
 }
 }  // namespace
@@ -488,10 +490,10 @@ int launch_global_update_blocks(const Dims& d, const float* partial, const int32
 }
 
 // Policy scores of all graphs (logit [B]; y1_out / y2_out optional) and, for num_envs > 0, the first layer of the value
-// head (y1v [num_envs x Hm]).
+// head (y1v [num_envs x Hm]; its input u_out [num_envs x 2 H] is optional).
 int launch_policy_value_hidden(const Dims& d, const DevWeights& w, const float* emb, float* logit, int32_t B, float* y1_out,
                                float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v,
-                               cudaStream_t st) {
+                               cudaStream_t st, float* u_out) {
   const Mlp pm{w.pW1, w.pb1, w.pWh, w.pbh, w.pw2, w.pb2, d.Hm, d.Hm2};
   const Mlp vm{w.vW1, w.vb1, w.vWh, w.vbh, w.vw2, w.vb2, d.Hm, d.Hm2};
   auto bytes = [&](int gp) {
@@ -502,7 +504,7 @@ int launch_policy_value_hidden(const Dims& d, const DevWeights& w, const float* 
   // the value CTAs of an environment share its first layer: eight while they find SMs of their own beside the others'
   const int VC = num_envs <= 8 ? 8 : num_envs <= 32 ? 4 : num_envs <= 128 ? 2 : 1;
 #define POLICY_CASE(G_) \
-  case G_: return policy_value<G_>(d, pm, vm, emb, logit, B, y1_out, y2_out, env_off, mask, num_envs, y1v, VC, bytes(G_), st);
+  case G_: return policy_value<G_>(d, pm, vm, emb, logit, B, y1_out, y2_out, env_off, mask, num_envs, y1v, VC, bytes(G_), st, u_out);
   switch (gp) { POLICY_CASE(1) POLICY_CASE(2) POLICY_CASE(4) POLICY_CASE(8) default: POLICY_CASE(16) }
 #undef POLICY_CASE
 }

@@ -244,7 +244,7 @@ int launch_global_update(const Dims& d, const float* partial, const int32_t* gra
                          float* U_out = nullptr);
 int launch_policy_value_hidden(const Dims& d, const DevWeights& w, const float* emb, float* logit, int32_t B, float* y1_out,
                                float* y2_out, const int32_t* env_off, const uint8_t* mask, int32_t num_envs, float* y1v,
-                               cudaStream_t st);
+                               cudaStream_t st, float* u_out = nullptr);
 int launch_heads(const Dims& d, const DevWeights& w, const float* emb, const int32_t* env_off,
                  const uint8_t* mask, int32_t B, int32_t num_envs, float* logit_ws, float* probs,
                  float* value, int32_t* action, uint64_t seed, uint64_t step, int32_t* status,
