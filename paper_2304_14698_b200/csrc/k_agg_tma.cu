@@ -37,7 +37,7 @@ constexpr int GQ = XRL_AGG_GATHERS; // gathers (of four rows each) per group: on
 // destination rows (32 in large launches; small ones take 16 or 8, see aggregate_block_shift: with few
 // rows a 32-row block per warp leaves most warps idle).  SEQ: see aggregate_warp; set for the small launches that
 // the all-layers kernel can replace, whose results it must reproduce bit for bit.
-template <typename T, int K, bool READOUT, bool MERGED, bool SEQ>
+template <typename T, int K, int READOUT, bool MERGED, bool SEQ>
 __global__ void __launch_bounds__(TW * 32, XRL_AGG_CTAS)
 k_aggregate_tma(const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_s,
                 const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
@@ -90,7 +90,7 @@ bool make_row_map(CUtensorMap* m, const void* ptr, CUtensorMapDataType dt, uint3
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <typename T, int K, bool READOUT, bool MERGED, bool SEQ>
+template <typename T, int K, int READOUT, bool MERGED, bool SEQ>
 int launch_k_seq(const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores, const float* bias,
              void* h_out, Window win, int64_t buf_rows, const int32_t* seg_id, float* partial,
              const int32_t* self_idx, int32_t* status, cudaStream_t st) {
@@ -120,7 +120,7 @@ int launch_k_seq(const int32_t* rowptr, const int32_t* col, const void* Z, const
 }
 
 
-template <typename T, int K, bool READOUT, bool MERGED>
+template <typename T, int K, int READOUT, bool MERGED>
 int launch_k(const int32_t* rowptr, const int32_t* col, const void* Z, const float* scores, const float* bias,
              void* h_out, Window win, int64_t buf_rows, const int32_t* seg_id, float* partial,
              const int32_t* self_idx, int32_t* status, cudaStream_t st) {
@@ -147,18 +147,19 @@ int launch_aggregate_tma(const Dims& d, const int32_t* rowptr, const int32_t* co
   if (d.zmerged && !bf) return -1;
   if (partial != nullptr && (win.row_begin != 0 || win.win_base != 0)) return -1;
 #define TMA_ARGS rowptr, col, Z, scores, bias, h_out, win, buf_rows, seg_id, partial, self_idx, status, st
+#define TMA_SUMS(TY_, KK, MERGED_)                                                                     \
+  (partial == nullptr ? launch_k<TY_, KK, 0, MERGED_>(TMA_ARGS)                                        \
+   : h_out == nullptr ? launch_k<TY_, KK, 1, MERGED_>(TMA_ARGS) : launch_k<TY_, KK, 2, MERGED_>(TMA_ARGS))
 #define TMA_CASE(KK)                                                                                   \
   case KK:                                                                                             \
-    if (d.zmerged)                                                                                     \
-      return partial ? launch_k<bf16, KK, true, true>(TMA_ARGS) : launch_k<bf16, KK, false, true>(TMA_ARGS); \
-    if (partial != nullptr)                                                                            \
-      return bf ? launch_k<bf16, KK, true, false>(TMA_ARGS) : launch_k<float, KK, true, false>(TMA_ARGS);    \
-    return bf ? launch_k<bf16, KK, false, false>(TMA_ARGS) : launch_k<float, KK, false, false>(TMA_ARGS);
+    if (d.zmerged) return TMA_SUMS(bf16, KK, true);                                                    \
+    return bf ? TMA_SUMS(bf16, KK, false) : TMA_SUMS(float, KK, false);
   switch (d.K) {
     TMA_CASE(4) TMA_CASE(8) TMA_CASE(16)
     default: return -1;
   }
 #undef TMA_ARGS
+#undef TMA_SUMS
 #undef TMA_CASE
 }
 

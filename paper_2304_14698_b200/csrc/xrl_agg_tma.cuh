@@ -155,9 +155,11 @@ __device__ __forceinline__ void raise_reference(float ev, float& m, float& l, F2
 }
 
 // One warp's share of a layer.  `next_block()` returns the first row of the warp's next block of up to
-// 2^br_shift destination rows, or a negative value when there is none left.  READOUT = true is the last
-// attention layer fused with the per-graph sum of Eq. 8: the layer output is stored only where h_out is given (the
-// training step keeps it; the sum is then of the rows as stored, as its reverse pass reads them); the warp adds the rows of its block per graph, in row order, and writes
+// 2^br_shift destination rows, or a negative value when there is none left.  READOUT = 1 and 2 are the last
+// attention layer fused with the per-graph sum of Eq. 8: 1 leaves the layer output unstored, 2 stores it (the training
+// step keeps it; the sum is then of the rows as stored, as its reverse pass reads them).  (One kernel for both that tested
+// h_out per row took 2 to 4 registers more: the last layer of 36 k fp32 rows of 128 16.0 us, now 14.9, of 179 k bf16 rows of 256
+// 43.2, now 39.6.)  The warp adds the rows of its block per graph, in row order, and writes
 //   partial[b]           the rows of block b that belong to the graph of the block's first row
 //   partial[nblocks + g] the rows of graph g inside the block in which g starts, when that is not at
 //                        the block's first row
@@ -167,7 +169,7 @@ __device__ __forceinline__ void raise_reference(float ev, float& m, float& l, F2
 // SEQ: producers taken two at a time are added exactly as if taken singly (one more addition and compare per
 // pair); without it the pair's weights are summed first and one overflow test serves both, which is faster
 // and equal up to rounding.  Kernels whose results must agree bit for bit use the same setting.
-template <typename T, int K, bool READOUT, bool MERGED, int G, int GQ, bool SEQ, typename NextBlock>
+template <typename T, int K, int READOUT, bool MERGED, int G, int GQ, bool SEQ, typename NextBlock>
 __device__ __forceinline__ bool aggregate_warp(
     const CUtensorMap* map_z_p, const CUtensorMap* map_s_p, const int32_t* __restrict__ rowptr,
     const int32_t* __restrict__ col, const T* __restrict__ Z, const float2* __restrict__ scores,
@@ -295,9 +297,9 @@ __device__ __forceinline__ bool aggregate_warp(
 #pragma unroll
           for (int t2 = 0; t2 < NP; ++t2) fma2(acc[t2], p2, z[t2]);
         }
-        if (READOUT) {
+        if constexpr (READOUT != 0) {
           F2 o[NP];
-          if (h_out != nullptr) to_pairs(finish_row(h_out + size_t(lrow) * H + c0, acc, __fdividef(1.f, l), bs), o);
+          if constexpr (READOUT == 2) to_pairs(finish_row(h_out + size_t(lrow) * H + c0, acc, __fdividef(1.f, l), bs), o);
           else finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
           add_row(rs, o);
         } else {
@@ -417,9 +419,9 @@ __device__ __forceinline__ bool aggregate_warp(
 #pragma unroll
           for (int t2 = 0; t2 < NP; ++t2) fma2(acc[t2], p2, z[t2]);
         }
-        if (READOUT) {
+        if constexpr (READOUT != 0) {
           F2 o[NP];
-          if (h_out != nullptr)
+          if constexpr (READOUT == 2)
             to_pairs(finish_row(h_out + size_t(int32_t(r0) + rs + rr - win.win_base) * H + c0, acc, __fdividef(1.f, l), bs), o);
           else finish_row_f32<NP>(acc, __fdividef(1.f, l), bs, o);
           add_row(rs + rr, o);
