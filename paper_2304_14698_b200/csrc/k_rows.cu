@@ -37,7 +37,6 @@ k_embed(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
         const int32_t* __restrict__ op, const T* __restrict__ shape, const T* __restrict__ W0,
         const float* __restrict__ b0, T* __restrict__ h, int H, int Tn, Window win,
         const int32_t* __restrict__ row_list, const T* __restrict__ eattr) {
-  enter();
   constexpr int VEC = VecOf<T>::N;
   constexpr int RPW = 32 / LPR;
   extern __shared__ __align__(16) float smem[];
@@ -50,6 +49,9 @@ k_embed(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
     Wd[t] = to_float(W0[size_t(src_row) * H + c]);
   }
   for (int t = threadIdx.x; t < H; t += blockDim.x) bs[t] = b0[t];
+  // only weights are read above; as the kernel's first statement the wait cost the one-vector bf16 kernels 47 registers and their
+  // third CTA per SM (179 k rows of hidden 64 65.9 us instead of 59.8, of 128 171.9 instead of 166.5)
+  enter();
   __syncthreads();
 
   const int NV = H / VEC;
