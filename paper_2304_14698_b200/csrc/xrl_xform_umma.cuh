@@ -127,13 +127,17 @@ __device__ __forceinline__ float pair_sum(unsigned long long a) {
   return lo + hi;
 }
 
-// Whether two groups of four epilogue warps can share the columns of a tile: halves of whole 32-column pieces and heads.
+// Groups of four epilogue warps on one tile: two where its halves are whole 32-column pieces and heads, else one.
 __host__ __device__ constexpr int epilogue_groups(int NS, int d) { return NS % 64 == 0 && (NS / 2) % d == 0 ? 2 : 1; }
 
 // The epilogue warps (two groups of four from CTA warp 2 on; warp q = warp & 3 of a group reads tensor-memory lanes
 // [32 q, 32 q + 32)): per tile the half-scores from the fp32 accumulators and Z rounded to bf16, a lane per row, written
-// straight from registers in whole 32-byte sectors.  With `groups` = 2 a group takes half of the columns, else the second
-// group has nothing to do.  No barrier between the warps: each waits for the accumulator and frees it on its own.
+// straight from registers in whole 32-byte sectors.  With `groups` = 2 a group takes half of every tile's columns.  With one
+// group per tile the two take tiles in turn, an accumulator each, where a CTA has all of a power of two of columns (one head at
+// 64, 128 or 256: 1.02 M rows 58, 93 and 184 us per layer with an idle second group, 51, 89 and 178 in turn; four warps and
+// TMA stores 76, 95 and 180); elsewhere the second group has nothing to do (both storing rows of other lengths at once: 192 with
+// three heads 134 -> 140 us, 160, 224, 96 and 32 +1 to +3 %, slices of 320 to 512 +1 to +3 %).  No barrier between the
+// warps: each waits for the accumulator and frees it on its own.
 // (Through swizzled staging tiles and TMA stores, two CTA barriers and a proxy fence per 64 columns, four warps took 3.3 us
 // per 128 x 256 tile, which held the large steps' transform to what 148 such epilogues can do: 2.8 M rows 0.58 -> 0.49 ms,
 // 4.1 M 0.79 -> 0.73, 124 k rows of 192 26.6 -> 22.1 us, the all-layers kernel of a small step 65.5 -> 61.8.  Eight warps
@@ -151,13 +155,15 @@ __device__ __forceinline__ void epilogue_tiles(uint8_t* smem, uint32_t base, uin
                                                int cols_left = NS) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3, grp = (warp - 2) >> 2;
-  if (grp >= groups) { lt += num_tiles > first ? (num_tiles - first + step - 1) / step : 0; return; }
+  constexpr bool kTurns = NS == C::KC * KCH && (NS & (NS - 1)) == 0;
+  if (!kTurns && grp >= groups) { lt += num_tiles > first ? (num_tiles - first + step - 1) / step : 0; return; }
   const int row_in_tile = q * 32 + lane;
-  const int c0 = grp * (NS / 2), c1 = groups == 2 ? c0 + NS / 2 : NS;
+  const int c0 = groups == 2 ? grp * (NS / 2) : 0, c1 = groups == 2 ? c0 + NS / 2 : NS;
   const float* avec = reinterpret_cast<const float*>(smem + C::OFF_AVEC);
   volatile uint32_t* abort_flag = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM) + 1;
   for (int tile = first; tile < num_tiles; tile += step, ++lt) {
     const int buf = lt & 1;
+    if (kTurns && groups == 1 && buf != grp) continue;
     uint32_t ok = 1;
     if (lane == 0) ok = mbar_wait(C::bar_acc_full(base, buf), (lt >> 1) & 1) ? 1u : 0u;
     ok = __shfl_sync(0xFFFFFFFFu, ok, 0);

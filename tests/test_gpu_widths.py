@@ -184,3 +184,10 @@ def test_bf16_heads_of_every_width(xo, monkeypatch, H, K, nodes, fused):
         assert ag.device_status() == 0
     finally:
         ag.close()
+
+
+@pytest.mark.parametrize("H,K", [(64, 1), (128, 1), (256, 1), (32, 2), (96, 3), (160, 4), (192, 3), (224, 7), (512, 4)])
+def test_bf16_heads_that_two_groups_of_epilogue_warps_cannot_halve(xo, H, K):
+    """64, 128 and 256 columns with one head: a group takes every other tile (three or four tiles per CTA, so both numbers of
+    turns); the other widths leave all tiles to one group."""
+    test_bf16_widths_with_many_tiles_per_cta(xo, H, K)
