@@ -1069,6 +1069,17 @@ size_t ppo_heads_workspace_floats(const Dims& d, int64_t B, int64_t num_envs) {
          up4(e * 2 * H) + 2 * up4(e * Hm) + 2 * up4(e * Hm2) + up4(e);
 }
 
+// The gradient of every row of the last layer's features, masked by their ReLU, from that of the graphs' sums.
+static int launch_readout_bwd(const Dims& d, const float* dr, const int32_t* seg_id, const void* hL, float* dh, int64_t N,
+                              cudaStream_t st) {
+  const int64_t ne = N * (d.H / 4);
+  if (ne <= 0) return 0;
+  const unsigned grid = unsigned(std::min<int64_t>((ne + 255) / 256, int64_t(kNumSMs) * 64));
+  if (d.dtype == XRL_BF16) launch(k_readout_bwd<bf16>, grid, 256, 0, st, dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
+  else launch(k_readout_bwd<float>, grid, 256, 0, st, dr, seg_id, static_cast<const float*>(hL), dh, ne, d.H);
+  return 1;
+}
+
 // Forward from the readout's sums (of chunks: partial_off = the graphs' first chunks, nblocks = 0; or of the last layer's
 // blocks of rows: partial_off = the graphs' first rows) to the logits, Eq. 3-5, and the reverse pass down to the gradient of the last
 // layer's node features (dh [N x H]), or, without dh, to that of the graphs' sums (*dr_out [B x H], in ws).  ws:
@@ -1135,13 +1146,7 @@ int launch_ppo_heads(const Dims& d, const DevWeights& w, float* grad_base, const
   launch(k_head_grads, tl.ctas, 256, 0, st, tl.tasks);
   ++n;
   *dr_out = dr;
-  const int64_t ne = dh != nullptr ? N * (d.H / 4) : 0;
-  if (ne > 0) {
-    const unsigned grid = unsigned(std::min<int64_t>((ne + 255) / 256, int64_t(kNumSMs) * 64));
-    if (d.dtype == XRL_BF16) launch(k_readout_bwd<bf16>, grid, 256, 0, st, dr, seg_id, static_cast<const bf16*>(hL), dh, ne, d.H);
-    else launch(k_readout_bwd<float>, grid, 256, 0, st, dr, seg_id, static_cast<const float*>(hL), dh, ne, d.H);
-    ++n;
-  }
+  if (dh != nullptr) n += launch_readout_bwd(d, dr, seg_id, hL, dh, N, st);
   return n;
 }
 
@@ -1196,10 +1201,11 @@ int launch_gat_layer_bwd(const Dims& d, const int32_t* rowptr, const int32_t* co
   do {                                                                                                         \
     const int k_ = launch_rows_gather(d, *lists, rowptr, col, Z, scores, h_out, dh_out, masked, dr, seg_id, ds_dst, gb, N, \
                                       status, st);                                                             \
-    if (k_ < 0 && dr != nullptr) return -1;                                                                    \
-    if (k_ < 0)                                                                                                \
-      launch(k_aggregate_bwd_rows<TY_, NF_, true>, grid_rows, 256, 0, st,                                          \
-          rowptr, col, zv, static_cast<const TY_*>(h_out), dh_out, masked, nullptr, nullptr, ds_dst, gb, N, K, *lists); \
+    if (k_ < 0) {                            /* (it reads rows: the graphs' gradients are written out first) */   \
+      if (dr != nullptr) launch_readout_bwd(d, dr, seg_id, h_out, dh_out, N, st);                              \
+      launch(k_aggregate_bwd_rows<TY_, NF_, true>, grid_rows, 256, 0, st, rowptr, col, zv,                     \
+             static_cast<const TY_*>(h_out), dh_out, masked || dr != nullptr, nullptr, nullptr, ds_dst, gb, N, K, *lists); \
+    }                                                                                                          \
     if (launch_dz_gather(d, *lists, dh_out, Z, zrow, ds_dst, lw, mma ? dz_store : static_cast<void*>(dz), ga_src, ga_dst, \
                          N, status, st) < 0)                                                                   \
       return -1;                                                                                               \

@@ -173,3 +173,35 @@ def test_gradient_of_the_readout_fused_with_the_last_layer(xo, H, K, dtype, size
     rng = dags.make_rng(H + K + len(sizes))
     graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) if n else _no_nodes() for n in sizes]
     _compare(xo, dags.flatten(graphs, [0, len(graphs)], m["A_max"]), m)
+
+
+def _library_that_declines(name, out):
+    """libxrl.so with the launcher `name` replaced by one that declines every call, as it does where a tensor map is refused."""
+    import glob
+    import os
+    import subprocess
+    from paper_2304_14698_b200 import build
+    sources = [os.path.basename(s)[:-3] for s in sorted(glob.glob(os.path.join(build.CSRC, "*.cu")))]
+    objects = [os.path.join(build.OBJ, s + ".o") for s in sources]
+    if not all(map(os.path.exists, objects)):
+        build.build()
+    symbols = subprocess.run(["nm", *objects], capture_output=True, text=True, check=True).stdout.split()
+    symbol, = {s for s in symbols if s.startswith(f"_ZN3xrl{len(name)}{name}E")}
+    stub, lib = str(out / "stub.cpp"), str(out / "libxrl_declines.so")
+    with open(stub, "w") as f:
+        f.write(f'extern "C" int __wrap_{symbol}() {{ return -1; }}\n')
+    subprocess.run([build._nvcc(), "-shared", "-Xcompiler", "-fPIC", "-o", lib, *objects, stub, "-Xlinker", f"--wrap={symbol}",
+                    "-gencode", "arch=compute_100a,code=sm_100a"], check=True)
+    return lib
+
+
+@pytest.mark.parametrize("H,K,dtype", [(256, 8, "bf16"), (128, 4, "fp32")])
+def test_gradient_where_the_gather_of_the_softmax_reverse_declines(xo, monkeypatch, tmp_path, H, K, dtype):
+    """The kernel without TMA reads rows of gradients, which the last layer then has to have written."""
+    from paper_2304_14698_b200 import binding
+    monkeypatch.setattr(binding, "_LIB_PATH", _library_that_declines("launch_rows_gather", tmp_path))
+    monkeypatch.setattr(binding, "_lib", None)
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3)
+    rng = dags.make_rng(H)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (65, 70, 65, 33, 66)]
+    _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
