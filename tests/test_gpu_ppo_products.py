@@ -205,3 +205,17 @@ def test_gradient_where_the_gather_of_the_softmax_reverse_declines(xo, monkeypat
     rng = dags.make_rng(H)
     graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (65, 70, 65, 33, 66)]
     _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
+
+
+@pytest.mark.parametrize("H,K,dtype,nodes", [
+    (H, K, dtype, nodes) for H, K in ((96, 1), (96, 4), (160, 2), (192, 4), (192, 8), (224, 4), (288, 4), (320, 8), (352, 1),
+                                      (384, 4), (416, 2), (448, 8), (480, 4))
+    for dtype, nodes in (("fp32", 3), ("fp32", 40), ("bf16", 130))] + [(96, 2, "bf16", 2500), (192, 4, "fp32", 2500),
+                                                                     (384, 12, "fp32", 40), (192, 12, "bf16", 130)])
+def test_gradient_of_widths_without_a_power_of_two(xo, H, K, dtype, nodes):
+    """Every number of features per lane that is no power of two (pieces on 2- to 16-byte boundaries): CTAs whose warps have no
+    row, one, two, and (10,000 rows) several; then heads that do not divide a warp."""
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3)
+    rng = dags.make_rng(H + K + nodes)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (nodes, nodes + 3, nodes, 1, nodes + 1)]
+    _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
