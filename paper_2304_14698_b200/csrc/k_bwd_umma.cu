@@ -1,13 +1,12 @@
 // The two dense products of an attention layer's reverse pass (paper Section 3.3.4's gradient through Eq. 7) on the
 // 5th-generation tensor cores, for bf16 models: with dz the gradient of Z = h W in bf16 (hidden 128 and 256: both in one
-// kernel, k_dhw_umma; hidden 512, whose dW no tensor memory holds beside dh, one after the other),
+// kernel, k_dhw_umma; hidden 512, whose dW takes the tensor memory of four SMs, one after the other),
 //   dh = dz W^T   the transform kernel's roles and tiles (xrl_xform_umma.cuh) with W itself as the K-major operand
 //                 and an fp32 result, which leaves masked by the ReLU of h (what the next layer down needs);
-//   dW += h^T dz  reduces over the rows, so both operands are used as they lie in memory: a 64-row block of h and one
-//                 of dz come in as TMA boxes of 64 columns, which tcgen05.mma reads as MN-major operands, and
-//                 the whole H x H result (H = 256: all 512 columns of tensor memory) stays in tensor memory
-//                 while the CTA walks its range of rows.  The CTAs' results meet in the gradient by TMA
-//                 reductions (fp32 add in L2).
+//   dW += h^T dz  reduces over the rows, so both operands are used as they lie in memory, which tcgen05.mma reads as
+//                 MN-major operands, and the result stays in tensor memory while the CTA walks its range of rows
+//                 (hidden 512: a 256 x 256 quarter per CTA, all 512 columns).  The CTAs' results meet in the gradient by
+//                 TMA reductions (fp32 add in L2).
 // Both are bound by HBM: 8 H bytes per row (dh: 4 H in, 4 H out) and 4 H bytes per row (dW); together, with dz and h read
 // once, 8 H.
 //
@@ -37,19 +36,19 @@ __device__ __forceinline__ void stage_row(uint8_t* tile, int row, const uint32_t
     *reinterpret_cast<uint4*>(p + ((j ^ (row & 7)) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
 }
 
-// ---- dh = dz W^T ---------------------------------------------------------------------------------------------
-template <int NS, int KP>
+// ---- dh = dz W^T at hidden 512 ----------------------------------------------------------------------------------
+// (a CTA: 128 columns of dh for every 128-row tile of its share, four CTAs side by side)
+constexpr int WIDE = 512, NS = 128, SLICES = WIDE / NS;
+using DhCfg = Cfg<NS, WIDE, true>;
 __global__ void __launch_bounds__(kThreads, 1)
 k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_w,
-          const __grid_constant__ CUtensorMap map_o, const bf16* __restrict__ h, int rows, int H, int slices,
-          int32_t* status) {
-  using C = Cfg<NS, KP, true>;
+          const __grid_constant__ CUtensorMap map_o, const bf16* __restrict__ h, int rows, int32_t* status) {
+  using C = DhCfg;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int num_tiles = (rows + BM - 1) / BM;
-  const int slice = int(blockIdx.x) % slices, first = int(blockIdx.x) / slices, step = int(gridDim.x) / slices;
-  const int col0 = slice * NS, cols = min(NS, H - col0);
+  const int col0 = int(blockIdx.x) % SLICES * NS, first = int(blockIdx.x) / SLICES, step = int(gridDim.x) / SLICES;
   if ((base & 1023u) != 0) {
     if (threadIdx.x == 0) raise(status, XRL_ERR_UNSUPPORTED);
     return;
@@ -90,16 +89,16 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
     uint32_t lt = 0;
     enter();
     // The features whose ReLU masks the result: this thread's row of a tile, 32 columns (64 bytes) per chunk, asked for a
-    // whole tile ahead (2 NS bytes of them in registers: asked for one chunk ahead the four warps wait for them,
-    // 0.448 instead of 0.351 ms at 990 k rows and hidden 256).
+    // whole tile ahead (2 NS bytes of them in registers: asked for one chunk ahead the four warps wait for them; 256
+    // columns per CTA, 990 k rows: 0.448 instead of 0.351 ms).
     uint4 hn[NS / 32][4];
     auto features = [&](int tile, int c, uint4 (&f)[4]) {
       const int64_t r = int64_t(tile) * BM + row_in_tile;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         f[j] = make_uint4(0u, 0u, 0u, 0u);
-        if (tile < num_tiles && r < rows && c * 32 < cols)
-          f[j] = __ldg(reinterpret_cast<const uint4*>(h + size_t(r) * H + col0 + c * 32) + j);
+        if (tile < num_tiles && r < rows)
+          f[j] = __ldg(reinterpret_cast<const uint4*>(h + size_t(r) * WIDE + col0 + c * 32) + j);
       }
     };
 #pragma unroll
@@ -132,7 +131,7 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
         stage_row(smem + C::OFF_OUT + (c & 1) * STAGE_BYTES, row_in_tile, v);
         fence_async_smem();
         epi_barrier();
-        if (leader && c * 32 < cols) {
+        if (leader) {
           tma_store_2d(&map_o, base + C::OFF_OUT + (c & 1) * STAGE_BYTES, col0 + c * 32, tile * BM);
           tma_commit();
         }
@@ -151,13 +150,13 @@ k_dh_umma(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUt
   }
 }
 
-// ---- dW += h^T dz ----------------------------------------------------------------------------------------------
-// S: side of the square of dW a CTA accumulates (256: a quarter of H = 512).
-constexpr int RB = 64;                   // rows per stage
-template <int S> struct WCfg {
+// ---- dW += h^T dz at hidden 512 ---------------------------------------------------------------------------------
+constexpr int RB = 64;                   // rows per stage: 64-row blocks of h and of dz, in boxes of 64 columns
+constexpr int S = 256, SIDE = WIDE / S;  // side of the square of dW a CTA accumulates
+struct DwCfg {
   static constexpr int CHUNK = RB * 128;                 // 64 rows x 64 columns
   static constexpr int OPERAND = (S / 64) * CHUNK;       // one operand of a stage
-  static constexpr int STAGES = S == 256 ? 3 : 5;
+  static constexpr int STAGES = 3;
   static constexpr int OFF_OUT = STAGES * 2 * OPERAND;
   static constexpr int OFF_BAR = OFF_OUT + 2 * STAGE_BYTES;
   static constexpr int OFF_TMEM = OFF_BAR + 8 * (2 * STAGES + 1);
@@ -174,12 +173,10 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t chunk) 
          (uint64_t(1) << 46) | (uint64_t(2) << 61);
 }
 
-template <int S>
 __global__ void __launch_bounds__(kThreads, 1)
 k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_g,
-          const __grid_constant__ CUtensorMap map_o, float* __restrict__ dW, int rows, int H, int side, bool use_tma,
-          int32_t* status) {
-  using C = WCfg<S>;
+          const __grid_constant__ CUtensorMap map_o, float* __restrict__ dW, int rows, bool use_tma, int32_t* status) {
+  using C = DwCfg;
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -188,8 +185,9 @@ k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     return;
   }
   // CTA = (range of 64-row blocks, square of dW); the squares of a range side by side
-  const int squares = side * side, part = int(blockIdx.x) / squares, parts = int(gridDim.x) / squares;
-  const int a0 = (int(blockIdx.x) % squares) / side * S, b0 = int(blockIdx.x) % side * S;
+  constexpr int squares = SIDE * SIDE;
+  const int part = int(blockIdx.x) / squares, parts = int(gridDim.x) / squares;
+  const int a0 = (int(blockIdx.x) % squares) / SIDE * S, b0 = int(blockIdx.x) % SIDE * S;
   const int blocks = (rows + RB - 1) / RB;
   const int blk0 = int(int64_t(blocks) * part / parts), blk1 = int(int64_t(blocks) * (part + 1) / parts);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_TMEM);
@@ -288,7 +286,7 @@ k_dw_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
             tma_commit();
           }
         } else {
-          float* o = dW + size_t(a0 + m * 128 + row) * H + b0 + cc * 32;
+          float* o = dW + size_t(a0 + m * 128 + row) * WIDE + b0 + cc * 32;
 #pragma unroll
           for (int t = 0; t < 32; ++t) atomicAdd(o + t, __uint_as_float(v[t]));
         }
@@ -541,35 +539,32 @@ bool make_map_f32(CUtensorMap* m, void* ptr, uint64_t rows, uint64_t cols) {
          CUDA_SUCCESS;
 }
 
-template <int NS, int KP>
-int launch_dh(int H, const void* h, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
-  using C = Cfg<NS, KP, true>;
+int launch_dh(const void* h, const void* dzb, const void* W, float* dh, int32_t rows, int32_t* status, cudaStream_t st) {
   static bool attr_set[64] = {};
-  if (!ensure_dynamic_smem(k_dh_umma<NS, KP>, C::SMEM_BYTES, attr_set)) return -1;
+  if (!ensure_dynamic_smem(k_dh_umma, DhCfg::SMEM_BYTES, attr_set)) return -1;
   CUtensorMap mg, mw, mo;
-  if (!make_map(&mg, dzb, uint64_t(rows), H, BM) || !make_map(&mw, W, H, H, NS) || !make_map_f32(&mo, dh, uint64_t(rows), H))
+  if (!make_map(&mg, dzb, uint64_t(rows), WIDE, BM) || !make_map(&mw, W, WIDE, WIDE, NS) ||
+      !make_map_f32(&mo, dh, uint64_t(rows), WIDE))
     return -1;
-  const int slices = (H + NS - 1) / NS, tiles = (rows + BM - 1) / BM, groups = kNumSMs / slices;
-  launch(k_dh_umma<NS, KP>, (tiles < groups ? tiles : groups) * slices, kThreads, C::SMEM_BYTES, st,
-      mg, mw, mo, static_cast<const bf16*>(h), rows, H, slices, status);
+  const int tiles = (rows + BM - 1) / BM, groups = kNumSMs / SLICES;
+  launch(k_dh_umma, (tiles < groups ? tiles : groups) * SLICES, kThreads, DhCfg::SMEM_BYTES, st,
+         mg, mw, mo, static_cast<const bf16*>(h), rows, status);
   return 1;
 }
 
-template <int S>
-int launch_dw(int H, const void* h, const void* dzb, float* dW, int32_t rows, int32_t* status, cudaStream_t st) {
-  using C = WCfg<S>;
+int launch_dw(const void* h, const void* dzb, float* dW, int32_t rows, int32_t* status, cudaStream_t st) {
   static bool attr_set[64] = {};
-  if (!ensure_dynamic_smem(k_dw_umma<S>, C::SMEM_BYTES, attr_set)) return -1;
+  if (!ensure_dynamic_smem(k_dw_umma, DwCfg::SMEM_BYTES, attr_set)) return -1;
   const bool aligned = (reinterpret_cast<uintptr_t>(dW) & 15) == 0;    // the caller's buffer may sit on any 4-byte boundary
   CUtensorMap mh, mg, mo;
-  if (!make_map(&mh, h, uint64_t(rows), H, RB) || !make_map(&mg, dzb, uint64_t(rows), H, RB)) return -1;
-  if (aligned) { if (!make_map_f32(&mo, dW, H, H)) return -1; }
+  if (!make_map(&mh, h, uint64_t(rows), WIDE, RB) || !make_map(&mg, dzb, uint64_t(rows), WIDE, RB)) return -1;
+  if (aligned) { if (!make_map_f32(&mo, dW, WIDE, WIDE)) return -1; }
   else mo = mh;
-  const int side = H / S, squares = side * side;
+  constexpr int squares = SIDE * SIDE;
   // at least eight blocks per CTA: every CTA ends with a reduction of its whole square of dW into the gradient
   const int blocks = (rows + RB - 1) / RB, want = (blocks + 7) / 8, most = kNumSMs / squares;
-  launch(k_dw_umma<S>, (want < most ? want : most) * squares, kThreads, C::SMEM_BYTES, st,
-      mh, mg, mo, dW, rows, H, side, aligned, status);
+  launch(k_dw_umma, (want < most ? want : most) * squares, kThreads, DwCfg::SMEM_BYTES, st,
+         mh, mg, mo, dW, rows, aligned, status);
   return 1;
 }
 
@@ -608,9 +603,9 @@ int launch_bwd_umma(const Dims& d, const void* h, const void* dzb, const void* W
       return launch_dhw<128>(h, dzb, W, dh, dW, rows, status, st);
     case 256:
       return launch_dhw<256>(h, dzb, W, dh, dW, rows, status, st);
-    case 512:
-      a = launch_dw<256>(512, h, dzb, dW, rows, status, st);
-      b = launch_dh<128, 512>(512, h, dzb, W, dh, rows, status, st);
+    case WIDE:
+      a = launch_dw(h, dzb, dW, rows, status, st);
+      b = launch_dh(h, dzb, W, dh, rows, status, st);
       break;
     default: return -1;
   }
