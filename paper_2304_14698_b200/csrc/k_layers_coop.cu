@@ -15,7 +15,7 @@
 // transform reads only rows this CTA has just written, so a CTA barrier is enough there.  Z alternates between two buffers: a CTA that is already
 // transforming layer l + 1 must not overwrite rows a slower CTA still gathers for layer l.  W of the
 // next layer streams into shared memory during the attention phase, whose gather rings live where the
-// transform's A stages and output staging are.  Tensor memory is allocated once.
+// transform's A stages are.  Tensor memory is allocated once.
 //
 // Arithmetic, summation order and (for the last layer fused with the Eq. 8 sum) the layout of the
 // partial sums are those of the one-layer kernels: the results are bit-identical.
@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int num_tiles = (p.rows + xform::BM - 1) / xform::BM;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + XC::OFF_TMEM);
-  // [1] is set by the epilogue warps between their own barriers (they read it there), [2] by every other role,
-  // [3] holds the outcome of the last grid barrier
+  // [1] is set by an epilogue warp whose wait ran out (it stops on its own, the others at their own waits), [2] by every
+  // other role; both are read behind the next CTA or grid barrier only.  [3] holds the outcome of the last grid barrier
   volatile uint32_t* abort_role = tmem_slot + 2;
   auto aborted = [&]() { return (abort_role[-1] | abort_role[0]) != 0; };    // read between CTA barriers only
   float* avec = reinterpret_cast<float*>(smem + XC::OFF_AVEC);
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_layers_coop(const __grid_consta
     // (Issued only now: a thread's proxy fence waits for the copies it has in flight.)
     if (threadIdx.x == 0 && l + 1 < p.layers && !aborted()) xform::load_w<XC>(base, &p.map_w[l + 1]);
 
-    // ---- attention phase: rows of the same tiles; the rings take the place of the A stages and staging ---
+    // ---- attention phase: rows of the same tiles; the rings take the place of the A stages ---------------
     if (!aborted() && warp < kAttWarps) {
       Ring& sm = reinterpret_cast<Ring*>(smem + XC::OFF_A)[warp];
       const int total_blocks = my_tiles << blk_bits;

@@ -1,7 +1,8 @@
 // Row-wise kernels of the encoder (paper Section 3.4): the node-update layer (Eq. 6), the
 // attention half-scores, and the edge-score / segment-softmax / weighted-aggregate step of a
-// graph-attention layer (Eq. 7).  One group of LPR lanes owns one destination row and moves it
-// as 16-byte vectors (VPL vectors per lane); 32 / LPR rows share a warp.
+// graph-attention layer (Eq. 7).  One group of LPR lanes owns one destination row and moves it as 16-byte vectors: VPL per
+// lane in the first two, one in the attention kernel (which splits longer rows into slabs of columns); 32 / LPR rows share
+// a warp.
 #include "xrl_agg_tma.cuh"
 
 namespace xrl {

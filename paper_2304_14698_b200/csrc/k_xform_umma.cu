@@ -13,8 +13,8 @@
 // Hidden sizes: every multiple of 32 up to 512 (what the library supports).  Up to 256 a CTA holds all of W (128 KB at
 // 256) and computes whole rows.  Above, W no longer fits one SM (512 KB at 512): a CTA keeps a slice of 128 output columns
 // (128 KB at 512) for the whole launch and the CTAs of a row tile's slices run side by side, so that its second
-// to fourth reading of h comes from L2.  Widths that are not a multiple of 64 leave the last chunk to the TMA
-// unit's bounds: zeros on the way in, nothing written on the way out.
+// to fourth reading of h comes from L2.  Widths that are not a multiple of 64 leave the last chunk
+// of the way in to the TMA unit's bounds (zeros); on the way out pieces of 32 columns beyond the width are not written.
 // Measured: hidden 192, 124 k rows, 0.286 ms per layer with the CUDA-core product plus 0.052 ms for the half-scores
 // -> 0.022 ms (95 MB: 4.3 TB/s); hidden 256, 4.1 M rows, 0.73 ms (4.5 GB: 6.2 TB/s), 2.8 M rows 0.58 -> 0.49 ms.
 //
@@ -91,7 +91,7 @@ k_xform_umma(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ 
       if (!mma_tiles<C, NS>(base, tmem_base, first, step, num_tiles, it, lt, 0)) raise(status, XRL_ERR_TIMEOUT);
     }
   } else {
-    // ---- epilogue: 4 warps ------------------------------------------------------------------------
+    // ---- epilogue: two groups of four warps ----------------------------------------------------------
     uint32_t lt = 0;
     enter();
     epilogue_tiles<C, NS, ROUNDED, HD>(smem, base, tmem_base, Z + col0 * 2, z_row, scores ? scores + col0 / d : nullptr,
