@@ -272,7 +272,9 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // CTAs per SM), in the layout of the TMA kernel's fused variant (blocks of `block_rows` = 2^k rows from row 0 on: the rows of
 // a block's first graph to partial[block], those of a graph that starts inside it to partial[nblocks + graph]).  READOUT = 2
 // stores the rows as well; the sum is of the rows as they are stored either way, as the readout's and the delta path's are.
-template <typename T, int LPR, int READOUT>
+// ZERO (bf16 rows of more than 32 vectors): the ReLU of what is no number - a row that an infinite feature has reached - is 0, as
+// in the definition; the one inside the rounding, which shorter bf16 rows have, keeps it.
+template <typename T, int LPR, int READOUT, bool ZERO>
 __global__ void __launch_bounds__(kRowThreads, 4)
 k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
             const T* __restrict__ Z, const float2* __restrict__ scores,
@@ -404,7 +406,20 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
       }
       const float inv = __fdividef(1.f, l);
       if constexpr (READOUT == 0) {
-        if (live) aggtma::finish_row(h_out + size_t(lrow) * H + c0, acc, inv, bs);
+        if constexpr (ZERO) {
+          aggtma::F2 o[NP];
+          aggtma::finish_row_f32<NP>(acc, inv, bs, o);
+          uint32_t w[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            float lo, hi;
+            aggtma::split_f2(o[t], lo, hi);
+            w[t] = pack_bf16x2(lo, hi);
+          }
+          if (live) *reinterpret_cast<uint4*>(h_out + size_t(lrow) * H + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+        } else if (live) {
+          aggtma::finish_row(h_out + size_t(lrow) * H + c0, acc, inv, bs);
+        }
       } else {
         aggtma::F2 o[NP];
         if constexpr (READOUT == 1) aggtma::to_pairs(aggtma::row_as_stored(acc, inv, bs), o);
@@ -521,8 +536,8 @@ int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, c
   const int64_t sum_rows = int64_t(1) << aggregate_block_shift(rows);
   const int nv = d.H / (d.dtype == XRL_BF16 ? VecOf<bf16>::N : VecOf<float>::N), slabs = (nv + 31) / 32,
             slab_vecs = (nv + slabs - 1) / slabs;
-#define CALL_(TY_, LPR, RO_, br_)                                                                  \
-  launch(k_aggregate<TY_, LPR, RO_>, dim3(unsigned(row_grid(rows, int(br_))), unsigned(slabs)), kRowThreads, 0, st, \
+#define CALL_(TY_, LPR, RO_, ZERO_, br_)                                                           \
+  launch(k_aggregate<TY_, LPR, RO_, ZERO_>, dim3(unsigned(row_grid(rows, int(br_))), unsigned(slabs)), kRowThreads, 0, st, \
          rowptr, col, static_cast<const TY_*>(Z), reinterpret_cast<const float2*>(scores), bias,   \
          static_cast<TY_*>(h_out), d.H, d.K, win, self_idx, int(br_), slab_vecs, seg_id, partial,  \
          int32_t((rows + sum_rows - 1) / sum_rows))
@@ -532,9 +547,10 @@ int launch_aggregate(const Dims& d, const int32_t* rowptr, const int32_t* col, c
     int64_t br_ = (rows * slabs + warps_avail - 1) / warps_avail;                                          \
     br_ = ((br_ + rpw_ - 1) / rpw_) * rpw_;                                                        \
     if (br_ > kAggBlockRows) br_ = kAggBlockRows;                                                  \
-    if (LPR > 16 || partial == nullptr) CALL_(TY_, LPR, 0, br_);                              \
-    else if (h_out == nullptr) CALL_(TY_, LPR, (LPR <= 16 ? 1 : 0), sum_rows);                \
-    else CALL_(TY_, LPR, (LPR <= 16 ? 2 : 0), sum_rows);                                      \
+    if (slabs > 1) CALL_(TY_, 32, 0, sizeof(TY_) == 2, br_);                                       \
+    else if (LPR > 16 || partial == nullptr) CALL_(TY_, LPR, 0, false, br_);                       \
+    else if (h_out == nullptr) CALL_(TY_, LPR, (LPR <= 16 ? 1 : 0), false, sum_rows);              \
+    else CALL_(TY_, LPR, (LPR <= 16 ? 2 : 0), false, sum_rows);                                    \
   } while (0)
   if (d.dtype == XRL_BF16) XRL_ROW_DISPATCH(bf16, d.H, CALL);
   else XRL_ROW_DISPATCH(float, d.H, CALL);

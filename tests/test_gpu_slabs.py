@@ -34,3 +34,22 @@ def test_rows_of_several_vectors_per_lane(xo, H, K, dtype, nodes):
     want = xo.forward(m, blob, batch)
     for k in ("emb", "probs", "value"):
         gpu_util.assert_close(got[k], want[k], dtype, k)
+
+
+@pytest.mark.parametrize("H,K", [(288, 3), (320, 8), (384, 4), (480, 2), (512, 1), (512, 8), (512, 64)])
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_infinite_feature_in_rows_of_several_vectors_per_lane(xo, H, K, dtype):
+    """One infinite shape feature: rows of the layers that are no numbers leave their ReLU as 0, as in the definition (a ReLU
+    that kept them made the graph's embedding 0)."""
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype=dtype, A_max=3)
+    rng = dags.make_rng(H + K)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (33, 40, 36, 1, 35)]
+    graphs[2]["shape"][5, 3] = np.inf
+    batch = dags.flatten(graphs, [0, 3, 5], 3)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 5)
+    got = gpu_util.run_gpu(batch, blob)
+    want = xo.forward(m, blob, batch)
+    assert np.linalg.norm(want["emb"][2]) > 0.1 and np.isfinite(want["emb"]).all()
+    for k in ("emb", "probs", "value"):
+        gpu_util.assert_close(got[k], want[k], dtype, k)
