@@ -180,6 +180,10 @@ k_scores_bwd(ZView<T> zv, const float* __restrict__ ds_src, const float* __restr
 constexpr int kBwdWarps = 8;
 // (NF values side by side, on the boundary that every lane's have: the power of two in their size, 16 at most)
 constexpr int chunk_align(int bytes) { return bytes % 16 == 0 ? 16 : bytes % 8 == 0 ? 8 : bytes % 4 == 0 ? 4 : 2; }
+// Rows whose units are all off, lanes whose are, and half-scores without a gradient add nothing and are passed over at the
+// widths of a power of two.  The other widths, which the generic pair served first, take them as that pair does: 0 times an
+// infinite feature is no number, and the gradient shows it.
+template <int NF> constexpr bool kPassOver = (NF & (NF - 1)) == 0;
 template <typename T, int NF> struct alignas(chunk_align(int(sizeof(T)) * NF)) Chunk { T v[NF]; };
 
 template <typename T, int NF>
@@ -241,7 +245,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
     bool live = false;
 #pragma unroll
     for (int f = 0; f < NF; ++f) live = live || dp[f] != 0.f;
-    if (!GATHER && !__any_sync(0xFFFFFFFFu, live)) continue;   // a row whose units are all off: nothing flows (ds is zeroed)
+    if (!GATHER && kPassOver<NF> && !__any_sync(0xFFFFFFFFu, live)) continue;   // (ds is zeroed)
     const int32_t e0 = rowptr[i], deg = rowptr[i + 1] - e0;
     const int32_t self_entry = GATHER ? tl.rowptr[i] + i : 0;
     const float sd = zv.pair(i, k).y;
@@ -268,7 +272,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
       const float e = lrelu(eraw);
       if (e > mx) {
         const float sc = exp2f(mx - e);
-        sum = fmaf(sum, sc, 1.f); dotu = fmaf(dotu, sc, dal); mx = e;
+        sum = fmaf(sum, sc, kPassOver<NF> ? 1.f : 1.f + (e - e)); dotu = fmaf(dotu, sc, dal); mx = e;
       } else {
         const float w = exp2f(e - mx);
         sum += w; dotu = fmaf(w, dal, dotu);
@@ -318,7 +322,7 @@ k_aggregate_bwd_rows(const int32_t* __restrict__ rowptr, const int32_t* __restri
         return;
       }
       if (leader && de != 0.f) atomicAdd(&ds_src[size_t(j) * K + k], de);
-      if (live) {
+      if (live || (!kPassOver<NF> && al != al)) {
         float v[NF];
 #pragma unroll
         for (int f = 0; f < NF; ++f) v[f] = al * dp[f];
@@ -373,7 +377,7 @@ k_scores_bwd_rows(ZView<T> zv, const float* __restrict__ ds_src, const float* __
     const float gs = ds_src[size_t(i) * K + k], gd = ds_dst[size_t(i) * K + k];
     float z[NF], g[NF];
     load_chunk<float, NF>(dz + size_t(i) * H + lane * NF, g);
-    if (gs != 0.f || gd != 0.f) {
+    if (!kPassOver<NF> || gs != 0.f || gd != 0.f) {
       load_chunk<T, NF>(zv.row(i) + lane * NF, z);
 #pragma unroll
       for (int f = 0; f < NF; ++f) {

@@ -219,3 +219,43 @@ def test_gradient_of_widths_without_a_power_of_two(xo, H, K, dtype, nodes):
     rng = dags.make_rng(H + K + nodes)
     graphs = [dags.random_dag(rng, n, m["T"], 8, dtype == "bf16", window=6) for n in (nodes, nodes + 3, nodes, 1, nodes + 1)]
     _compare(xo, dags.flatten(graphs, [0, 3, 5], 3), m)
+
+
+@pytest.mark.parametrize("H,K", [(96, 1), (96, 4), (160, 4), (192, 1), (192, 8), (320, 2), (384, 4), (480, 2)])
+def test_gradient_of_an_infinite_feature_shows_it(xo, H, K):
+    """One infinite shape feature: the first layer's matrix, attention vectors and Eq. 6's bias have gradients that are no
+    numbers where the definition's are (rows and half-scores passed over as zeros gave finite ones)."""
+    import torch
+    import paper_2304_14698_b200 as xrl
+    from workloads import configs
+    m = dict(T=9, S=8, H=H, K=K, L=2, Hm=20, Dg=1, dtype="fp32", A_max=3)
+    rng = dags.make_rng(H + K)
+    graphs = [dags.random_dag(rng, n, m["T"], 8, window=6) for n in (33, 40, 36, 1, 35)]
+    graphs[2]["shape"][5, 3] = np.inf
+    batch = dags.flatten(graphs, [0, 3, 5], 3)
+    batch["model"] = m
+    blob, _ = gpu_util.default_weights(batch, 5)
+    st, packed = xo.pack(batch)
+    assert st == 0
+    action, logp, adv, ret = np.array([3, 3], np.int32), np.array([-0.7, -1.0]), np.array([1.0, -0.5]), np.array([0.3, 0.1])
+    want = xo.ppo_grad(m, blob, batch, packed, action, logp, adv, ret)["grad"]
+    ag = gpu_util.make_agent(batch)
+    try:
+        ag.set_weights(blob)
+        ag.pack(batch)
+        f32 = lambda a: torch.from_numpy(a.astype(np.float32)).cuda()
+        grad, loss = torch.empty(len(blob), device="cuda"), torch.empty(4, device="cuda")
+        xrl.xrl_ppo_grad(ag.ctx, ag.batch, torch.from_numpy(batch["mask"]).cuda(), torch.from_numpy(action).cuda(), f32(logp),
+                         f32(adv), f32(ret), loss, grad)
+        got = grad.cpu().numpy()
+        assert ag.device_status() == 0
+    finally:
+        ag.close()
+    off, seen = 0, 0
+    for name, shape in configs.weight_layout(m):
+        part = slice(off, off + int(np.prod(shape)))
+        off = part.stop
+        if name in ("b0", "W1", "a_src1", "a_dst1"):
+            assert np.array_equal(np.isnan(got[part]), np.isnan(want[part])), name
+            seen += int(np.isnan(want[part]).sum())
+    assert seen > H
