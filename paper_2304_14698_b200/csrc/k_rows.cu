@@ -407,14 +407,15 @@ k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
       const float inv = __fdividef(1.f, l);
       if constexpr (READOUT == 0) {
         if constexpr (ZERO) {
-          aggtma::F2 o[NP];
-          aggtma::finish_row_f32<NP>(acc, inv, bs, o);
           uint32_t w[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
+            aggtma::F2 v = aggtma::make_f2(bs[2 * t], bs[2 * t + 1]);
+            aggtma::fma2(v, acc[t], aggtma::make_f2(inv, inv));
             float lo, hi;
-            aggtma::split_f2(o[t], lo, hi);
+            aggtma::split_f2(v, lo, hi);
             w[t] = pack_bf16x2(lo, hi);
+            asm("max.bf16x2 %0, %0, %1;" : "+r"(w[t]) : "r"(0u));      // (of a number and none: the number)
           }
           if (live) *reinterpret_cast<uint4*>(h_out + size_t(lrow) * H + c0) = make_uint4(w[0], w[1], w[2], w[3]);
         } else if (live) {
