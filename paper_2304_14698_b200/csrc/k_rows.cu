@@ -273,7 +273,8 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // a block's first graph to partial[block], those of a graph that starts inside it to partial[nblocks + graph]).  READOUT = 2
 // stores the rows as well; the sum is of the rows as they are stored either way, as the readout's and the delta path's are.
 // ZERO (bf16 rows of more than 32 vectors): the ReLU of what is no number - a row that an infinite feature has reached - is 0, as
-// in the definition; the one inside the rounding, which shorter bf16 rows have, keeps it.
+// in the definition; the one inside the rounding, which shorter bf16 rows have, keeps it (a step of 256 k rows of 320 1,139 us
+// with that one, 1,144 with this).
 template <typename T, int LPR, int READOUT, bool ZERO>
 __global__ void __launch_bounds__(kRowThreads, 4)
 k_aggregate(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
